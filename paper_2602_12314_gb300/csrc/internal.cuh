@@ -340,12 +340,6 @@ latentam_status paper_prepare(latentam_ctx* ctx, const PaperArgs& a, const Paper
 latentam_status paper_chain(latentam_ctx* ctx, const PaperArgs& a, const PaperBuffers& b, float* dQ, float* dW,
                             float* dD, cudaStream_t st);
 
-// C = scale A B^T on the FP32 tiled GEMM: A (m x k) and B (n x k) row-major with row stride k,
-// C row stride ldc.  k and ldc multiples of 4, pointers 16-byte aligned, C rows padded to a
-// multiple of 4 columns (the tile stores float4).
-latentam_status sgemm_abt(const float* A, int64_t m, const float* B, int64_t n, int64_t k, float* C, int64_t ldc,
-                          float scale, cudaStream_t st);
-
 // Streaming K-means update of the dictionary (see latentam_stream_kmeans).
 struct KMeansArgs {
     const float* F;          // n x D embeddings of the new keyframe

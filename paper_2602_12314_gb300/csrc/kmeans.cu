@@ -4,15 +4,15 @@
 // dictionary size K.  Global centres keep their slots (row j stays row j); weight 0 marks an
 // empty slot, and the empty slots take the heaviest micro-centres first.
 //
-// Local phase (n rows, k <= 32 centres): one warp per row finds the nearest centre against the
-// centres staged in shared memory (squared distance as |c|^2 - 2 <x, c>, ties to the lower
-// index); each block then sums its row range per cluster with every thread owning fixed
-// columns of a per-row-group accumulator (no atomics), and the cluster means are formed by
-// summing the blocks' partials in block order, so the result does not depend on scheduling.
-// Global phase (at most K + k weighted points against K centres): the dot products of all
-// points with all centres come from the FP32 tiled GEMM, one warp per point takes the argmin
-// over the occupied slots, and one block per centre gathers its points' weighted sum in point
-// order.
+// Local phase (n rows, k <= 32 centres): one pass over the rows per Lloyd iteration.  A warp
+// holds four rows in registers (two past D = 512), finds each one's nearest centre against the
+// centres staged in shared memory (squared distance as |c|^2 - 2 <x, c>, ties to the lower index)
+// and adds the rows to its own copy of the cluster sums in shared memory; copies and blocks are
+// summed in a fixed order (no atomics), so the result does not depend on scheduling.
+// Global phase (at most K + k weighted points against K centres): an FP32 tiled product of the
+// points with the centres whose epilogue keeps each point's nearest occupied slot as one 64-bit
+// atomic minimum of (distance, slot), then one block per centre gathers its points' weighted sum
+// in point order.
 #include <algorithm>
 
 #include "internal.cuh"
@@ -21,12 +21,21 @@ namespace lat {
 namespace {
 
 constexpr int kMaxMicro = 32;
+constexpr int kRowWarps = 8;                // warps per block of the local pass, at most
+constexpr size_t kRowSmem = 220 * 1024;     // shared memory one block of it may take
 constexpr int kAccumThreads = 256;
 
 __device__ __forceinline__ float warp_allsum(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
+}
+
+// |x|^2 of a row, every lane (lane l takes x[l], x[l + 32], ... in order).
+__device__ __forceinline__ float warp_norm2(const float* x, int D, int lane) {
+    float s = 0.f;
+    for (int j = lane; j < D; j += 32) s += x[j] * x[j];
+    return warp_allsum(s);
 }
 
 // ---- local phase ------------------------------------------------------------------------
@@ -40,8 +49,149 @@ __global__ void local_init(const float* __restrict__ F, int64_t n, int D, const 
     for (int j = threadIdx.x; j < D; j += blockDim.x) C[(int64_t)c * D + j] = ok ? F[(int64_t)r * D + j] : 0.f;
 }
 
+// Warps (each with a copy of the k x D sums beside the staged centres) of a block of local_pass;
+// 0: not even one copy fits.
+int local_warps(int k, int D) {
+    const size_t copy = sizeof(float) * (size_t)k * D, norms = 256;
+    if (2 * copy + norms > kRowSmem) return 0;
+    return (int)std::min<size_t>(kRowWarps, (kRowSmem - norms) / copy - 1);
+}
+
+// One Lloyd pass: every valid row's nearest centre and the block's sums of its rows per cluster,
+// part[block] (k x D) and pcnt[block] (k).  Bound by the read of the embeddings (HBM, once per
+// iteration; the earlier assign / accumulate pair read them twice and held one row per warp).
+// R rows per warp: each centre quad read from shared memory meets 4 R products, and the R dot
+// products leave the butterfly together (log2 R scatter steps, then the R lane groups each finish
+// one row), in the summation tree of a plain butterfly.  Rows of one group that share their
+// cluster are added together before the read-modify-write of the sums.  NV: quads per lane
+// (D <= 128 NV).  `warps` of the block's eight take rows (as many as the sums' copies leave room
+// for, or as there are rows); all of them stage the centres and add up the copies.
+template <int NV, int R>
+__global__ void __launch_bounds__(32 * kRowWarps, 2) local_pass(const float* __restrict__ F, int64_t n, int D,
+                                                                const uint8_t* __restrict__ valid,
+                                                                const float* __restrict__ C, int k,
+                                                                int warps, int32_t* __restrict__ assign,
+                                                                float* __restrict__ part, int32_t* __restrict__ pcnt) {
+    extern __shared__ __align__(16) float sm[];
+    __shared__ int s_cnt[kRowWarps][kMaxMicro];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int D4 = D / 4;
+    float4* sC = reinterpret_cast<float4*>(sm);        // k x D
+    float4* sS = sC + (size_t)k * D4;                  // warps x k x D
+    float* sN = sm + (size_t)(warps + 1) * k * D;      // k
+    for (int i = threadIdx.x; i < k * D4; i += blockDim.x) sC[i] = reinterpret_cast<const float4*>(C)[i];
+    for (int i = threadIdx.x; i < warps * k * D4; i += blockDim.x) sS[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    __syncthreads();
+    for (int c = warp; c < k; c += kRowWarps) {
+        const float s = warp_norm2(sm + (size_t)c * D, D, lane);
+        if (lane == 0) sN[c] = s;
+    }
+    __syncthreads();
+    float4* own = sS + (size_t)warp * k * D4;  // lane l only touches quads l, l + 32, ...
+    int cnt = 0;                               // rows of cluster `lane`
+    constexpr int G = 32 / R;                  // lanes that end with one row's dot product
+    const float4* F4 = reinterpret_cast<const float4*>(F);
+    const int64_t step = (int64_t)gridDim.x * warps * R;
+    for (int64_t r0 = ((int64_t)blockIdx.x * warps + warp) * R; warp < warps && r0 < n; r0 += step) {
+        float4 x[R][NV];
+        bool ok[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) ok[r] = r0 + r < n && (!valid || valid[r0 + r]);
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int i = 0; i < NV; ++i) {
+                const int q = lane + 32 * i;
+                x[r][i] = ok[r] && q < D4 ? __ldcs(F4 + (r0 + r) * D4 + q) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+        float best = INFINITY;
+        int bi = 0;
+        for (int c = 0; c < k; ++c) {
+            float s[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) s[r] = 0.f;
+#pragma unroll
+            for (int i = 0; i < NV; ++i) {
+                const int q = lane + 32 * i;
+                if (q < D4) {
+                    const float4 cc = sC[c * D4 + q];
+#pragma unroll
+                    for (int r = 0; r < R; ++r)
+                        s[r] += x[r][i].x * cc.x + x[r][i].y * cc.y + x[r][i].z * cc.z + x[r][i].w * cc.w;
+                }
+            }
+#pragma unroll
+            for (int half = R / 2, o = 16; half >= 1; half >>= 1, o >>= 1) {
+                const bool upper = (lane & o) != 0;
+#pragma unroll
+                for (int r = 0; r < half; ++r) {
+                    const float send = upper ? s[r] : s[r + half], keep = upper ? s[r + half] : s[r];
+                    s[r] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                }
+            }
+#pragma unroll
+            for (int o = G / 2; o >= 1; o >>= 1) s[0] += __shfl_xor_sync(0xffffffffu, s[0], o);
+            const float v = sN[c] - 2.0f * s[0];
+            if (v < best) best = v, bi = c;
+        }
+        int a[R];
+        bool same = true;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            a[r] = __shfl_sync(0xffffffffu, bi, G * r);
+            if (!ok[r]) a[r] = -1;
+            same = same && a[r] == a[0];
+            cnt += a[r] == lane ? 1 : 0;
+            if (assign && lane == 0 && r0 + r < n) assign[r0 + r] = a[r];
+        }
+        auto add = [&](int c, const float4 (&y)[NV]) {
+#pragma unroll
+            for (int i = 0; i < NV; ++i) {
+                const int q = lane + 32 * i;
+                if (q < D4) {
+                    float4 t = own[c * D4 + q];
+                    t.x += y[i].x, t.y += y[i].y, t.z += y[i].z, t.w += y[i].w;
+                    own[c * D4 + q] = t;
+                }
+            }
+        };
+        if (same) {
+            if (a[0] >= 0) {
+#pragma unroll
+                for (int r = 1; r < R; ++r)
+#pragma unroll
+                    for (int i = 0; i < NV; ++i) {
+                        x[0][i].x += x[r][i].x, x[0][i].y += x[r][i].y;
+                        x[0][i].z += x[r][i].z, x[0][i].w += x[r][i].w;
+                    }
+                add(a[0], x[0]);
+            }
+        } else {
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if (a[r] >= 0) add(a[r], x[r]);
+        }
+    }
+    s_cnt[warp][lane] = cnt;
+    __syncthreads();
+    for (int i = threadIdx.x; i < k * D4; i += blockDim.x) {
+        float4 t = sS[i];
+        for (int w = 1; w < warps; ++w) {
+            const float4 u = sS[(size_t)w * k * D4 + i];
+            t.x += u.x, t.y += u.y, t.z += u.z, t.w += u.w;
+        }
+        reinterpret_cast<float4*>(part + (size_t)blockIdx.x * k * D)[i] = t;
+    }
+    if (threadIdx.x < k) {
+        int t = 0;
+        for (int w = 0; w < warps; ++w) t += s_cnt[w][threadIdx.x];
+        pcnt[(size_t)blockIdx.x * k + threadIdx.x] = t;
+    }
+}
+
 // assign[r] = nearest of the k centres (-1 for an invalid row); warp per row.  Shared memory:
-// the centres (k x D) and their squared norms.  D % 4 == 0, D <= 1024.
+// the centres (k x D) and their squared norms.  D % 4 == 0, D <= 1024.  With local_accum, the
+// form for k x D past what local_pass holds twice in shared memory (k = 32 at D > 860).
 __global__ void __launch_bounds__(256) local_assign(const float* __restrict__ F, int64_t n, int D,
                                                     const uint8_t* __restrict__ valid, const float* __restrict__ C,
                                                     int k, int32_t* __restrict__ assign) {
@@ -55,9 +205,7 @@ __global__ void __launch_bounds__(256) local_assign(const float* __restrict__ F,
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int c = warp; c < k; c += 8) {
-        float s = 0.f;
-        for (int j = lane; j < D; j += 32) s += sC[(size_t)c * D + j] * sC[(size_t)c * D + j];
-        s = warp_allsum(s);
+        const float s = warp_norm2(sC + (size_t)c * D, D, lane);
         if (lane == 0) sN[c] = s;
     }
     __syncthreads();
@@ -102,14 +250,14 @@ __global__ void __launch_bounds__(256) local_assign(const float* __restrict__ F,
 // group order into part[b] (k x D); pcnt[b] (k) counts the rows.
 __global__ void __launch_bounds__(kAccumThreads) local_accum(const float* __restrict__ F, int64_t n, int D,
                                                              const int32_t* __restrict__ assign, int k, int64_t R,
-                                                             float* __restrict__ part, float* __restrict__ pcnt) {
+                                                             float* __restrict__ part, int32_t* __restrict__ pcnt) {
     extern __shared__ __align__(16) float acc[];  // G x k x D
-    __shared__ float cnt[kMaxMicro];
+    __shared__ int cnt[kMaxMicro];
     const int D4 = D / 4;
     const int G = kAccumThreads / D4;  // row groups; threads past G * D4 (D4 not dividing 256) idle
     const int t = threadIdx.x, g = t / D4, q = t % D4;
     for (int i = t; i < G * k * D; i += kAccumThreads) acc[i] = 0.f;
-    if (t < k) cnt[t] = 0.f;
+    if (t < k) cnt[t] = 0;
     __syncthreads();
     const int64_t r0 = (int64_t)blockIdx.x * R, r1 = min(n, r0 + R);
     const float4* F4 = reinterpret_cast<const float4*>(F);
@@ -135,7 +283,7 @@ __global__ void __launch_bounds__(kAccumThreads) local_accum(const float* __rest
     if (t == 0) {  // row counts, in row order
         for (int64_t r = r0; r < r1; ++r) {
             const int c = assign[r];
-            if (c >= 0) cnt[c] += 1.f;
+            if (c >= 0) ++cnt[c];
         }
     }
     __syncthreads();
@@ -147,20 +295,34 @@ __global__ void __launch_bounds__(kAccumThreads) local_accum(const float* __rest
     if (t < k) pcnt[(int64_t)blockIdx.x * k + t] = cnt[t];
 }
 
-// C[c][j] = (sum over blocks, in order, of part[b][c][j]) / count_c, kept when the cluster is
-// empty; W[c] = count_c.
-__global__ void local_finish(const float* __restrict__ part, const float* __restrict__ pcnt, int nb, int k, int D,
-                             float* __restrict__ C, float* __restrict__ W) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)k * D) return;
-    const int c = (int)(i / D), j = (int)(i % D);
-    float s = 0.f, m = 0.f;
-    for (int b = 0; b < nb; ++b) {
-        s += part[(int64_t)b * k * D + i];
-        m += pcnt[(int64_t)b * k + c];
+// C[c][j] = (sum over blocks of part[b][c][j]) / count_c, kept when the cluster is empty;
+// W[c] = count_c.  Block per 32 columns of the k x D sums, warp w takes blocks w, w + 8, ... and the
+// warps' sums are added in order.  (One thread per column walking all blocks took 43 us over 304
+// blocks at k = 5, D = 512.)
+__global__ void __launch_bounds__(256) local_finish(const float* __restrict__ part, const int32_t* __restrict__ pcnt,
+                                                    int nb, int k, int D, float* __restrict__ C,
+                                                    float* __restrict__ W) {
+    __shared__ float s_sum[8][32];
+    __shared__ long long s_cnt[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + lane, kD = k * D;
+    const int c = min(i, kD - 1) / D;
+    float s = 0.f;
+    long long m = 0;
+    if (i < kD) {
+#pragma unroll 8
+        for (int b = warp; b < nb; b += 8) {
+            s += part[(size_t)b * kD + i];
+            m += pcnt[(size_t)b * k + c];
+        }
     }
-    if (m > 0.f) C[i] = s / m;
-    if (j == 0) W[c] = m;
+    s_sum[warp][lane] = s;
+    s_cnt[warp][lane] = m;
+    __syncthreads();
+    if (warp != 0 || i >= kD) return;
+    for (int w = 1; w < 8; ++w) s += s_sum[w][lane], m += s_cnt[w][lane];
+    if (m > 0) C[i] = s / (float)m;
+    if (i == c * D) W[c] = (float)m;
 }
 
 // ---- global phase -----------------------------------------------------------------------
@@ -245,112 +407,268 @@ __global__ void __launch_bounds__(1024) global_merge(const float* __restrict__ w
     if (t == 0) b.n_points[0] = U + n_live;
 }
 
-// Pm[p] = the point's row (an occupied slot of C, or a micro-centre), p < |P|.
-__global__ void global_points(const float* __restrict__ C, const float* __restrict__ mC, int D, MergeBufs b,
-                              float* __restrict__ Pm) {
-    const int p = blockIdx.x;
-    if (p >= b.n_points[0]) return;
-    const int s = b.pt_src[p];
-    const float* src = s >= 0 ? C + (int64_t)s * D : mC + (int64_t)(-1 - s) * D;
-    for (int j = threadIdx.x; j < D; j += blockDim.x) Pm[(int64_t)p * D + j] = src[j];
+// Rows and keys of the re-clustering.  Block b: point b (an occupied slot of C, or a micro-centre;
+// zero past the last one) into Pm, its assignment and keys cleared; slot b: an empty slot that takes
+// a micro-centre starts there, and the slot's squared norm.
+__global__ void __launch_bounds__(256) global_setup(float* __restrict__ C, const float* __restrict__ mC, int K, int KP,
+                                                    int D, MergeBufs b, float* __restrict__ Pm,
+                                                    float* __restrict__ nrm, uint64_t* __restrict__ keys,
+                                                    int32_t* __restrict__ pa) {
+    const int i = blockIdx.x, t = threadIdx.x;
+    if (i < KP) {
+        const int s = i < b.n_points[0] ? b.pt_src[i] : 0;
+        const bool live = i < b.n_points[0];
+        const float* src = s >= 0 ? C + (int64_t)s * D : mC + (int64_t)(-1 - s) * D;
+        for (int j = t; j < D; j += 256) Pm[(int64_t)i * D + j] = live ? src[j] : 0.f;
+        if (t == 0) {
+            keys[i] = keys[KP + i] = ~0ull;
+            if (pa) pa[i] = -1;
+        }
+    }
+    if (i < K) {
+        const int c = b.slot_fill[i];
+        const float* src = c >= 0 ? mC + (int64_t)c * D : C + (int64_t)i * D;
+        if (c >= 0)
+            for (int j = t; j < D; j += 256) C[(int64_t)i * D + j] = src[j];
+        if (t < 32) {
+            const float s = warp_norm2(src, D, t);
+            if (t == 0) nrm[i] = s;
+        }
+    }
 }
 
-// The empty slots that take a micro-centre start there.
-__global__ void global_fill(const float* __restrict__ mC, int D, MergeBufs b, float* __restrict__ C) {
-    const int j = blockIdx.x;
-    const int c = b.slot_fill[j];
-    if (c < 0) return;
-    for (int i = threadIdx.x; i < D; i += blockDim.x) C[(int64_t)j * D + i] = mC[(int64_t)c * D + i];
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool in) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    const int bytes = in ? 16 : 0;  // the rest is zero-filled
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(bytes) : "memory");
 }
 
-// nrm[c] = |C_c|^2; warp per centre.
-__global__ void centre_norms(const float* __restrict__ C, int K, int D, float* __restrict__ nrm) {
-    const int lane = threadIdx.x & 31;
-    const int c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (c >= K) return;
-    float s = 0.f;
-    for (int j = lane; j < D; j += 32) s += C[(int64_t)c * D + j] * C[(int64_t)c * D + j];
-    s = warp_allsum(s);
-    if (lane == 0) nrm[c] = s;
+// (distance, slot) as one word whose unsigned order is distance first, then the lower slot.
+__device__ __forceinline__ uint64_t nearest_key(float v, int c) {
+    uint32_t u = __float_as_uint(v + 0.0f);  // -0 and +0 are the same distance
+    u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+    return ((uint64_t)u << 32) | (uint32_t)c;
 }
 
-// pa[p] = argmin over active c of nrm[c] - 2 G[p][c] (ties to the lower index); warp per point.
-__global__ void global_assign(const float* __restrict__ G, int64_t ldg, const float* __restrict__ nrm, int K,
-                              MergeBufs b, int32_t* __restrict__ pa) {
-    const int lane = threadIdx.x & 31;
-    const int p = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (p >= b.n_points[0]) return;
-    float best = INFINITY;
-    int bi = 0x7fffffff;
-    for (int c = lane; c < K; c += 32) {
-        if (!b.active[c]) continue;
-        const float v = nrm[c] - 2.0f * G[(int64_t)p * ldg + c];
-        if (v < best) best = v, bi = c;  // c increases along the lane's list
+// keys[p] = minimum over the active slots c of (nrm[c] - 2 <Pm_p, C_c>, c): TP x TC tiles of the
+// points' products with the slots, FP32 FMAs with D in order, operands by cp.async through a ring
+// of `kDistStages` slices of BK; each thread MP x MC products (rows a half-warp apart).  A distance
+// that is not below infinity takes no slot.
+constexpr int kDistStages = 4;
+
+template <int TP, int TC, int BK>
+constexpr size_t dist_smem() {
+    return sizeof(float) * kDistStages * (size_t)(TP + TC) * (BK + 4);
+}
+
+template <int TP, int TC, int THREADS, int BK>
+__global__ void __launch_bounds__(THREADS) global_nearest(const float* __restrict__ Pm, int KP,
+                                                          const float* __restrict__ C, int K, int D, MergeBufs b,
+                                                          const float* __restrict__ nrm,
+                                                          unsigned long long* __restrict__ keys) {
+    constexpr int LD = BK + 4;  // padded rows: eight rows of 16 bytes cover the banks once
+    constexpr int MP = TP / (THREADS / 16), MC = TC / 16;
+    extern __shared__ __align__(16) float sm[];
+    const int P = b.n_points[0];
+    const int p0 = blockIdx.y * TP, c0 = blockIdx.x * TC;
+    if (p0 >= P) return;
+    const int t = threadIdx.x, tc = t & 15, tp = t >> 4;
+    const int slices = (D + BK - 1) / BK;
+    auto load = [&](int s) {
+        float* dst = sm + (size_t)(s % kDistStages) * (TP + TC) * LD;
+        for (int i = t; i < (TP + TC) * (BK / 4); i += THREADS) {
+            const int row = i / (BK / 4), col = s * BK + 4 * (i % (BK / 4));
+            const bool point = row < TP;
+            const int g = point ? p0 + row : c0 + row - TP;
+            const bool in = col < D && g < (point ? KP : K);
+            const float* src = (point ? Pm : C) + (in ? (int64_t)g * D + col : 0);
+            cp_async16(dst + row * LD + 4 * (i % (BK / 4)), src, in);
+        }
+    };
+    float acc[MP][MC];
+#pragma unroll
+    for (int i = 0; i < MP; ++i)
+#pragma unroll
+        for (int j = 0; j < MC; ++j) acc[i][j] = 0.f;
+#pragma unroll
+    for (int s = 0; s < kDistStages - 1; ++s) {
+        if (s < slices) load(s);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    for (int s = 0; s < slices; ++s) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kDistStages - 2) : "memory");
+        __syncthreads();
+        if (s + kDistStages - 1 < slices) load(s + kDistStages - 1);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        const float* A = sm + (size_t)(s % kDistStages) * (TP + TC) * LD;
+        const float* B = A + TP * LD;
+#pragma unroll 4
+        for (int kk = 0; kk < BK; kk += 4) {
+            float4 a[MP], c[MC];
+#pragma unroll
+            for (int i = 0; i < MP; ++i)
+                a[i] = *reinterpret_cast<const float4*>(A + (tp + (THREADS / 16) * i) * LD + kk);
+#pragma unroll
+            for (int j = 0; j < MC; ++j) c[j] = *reinterpret_cast<const float4*>(B + (tc + 16 * j) * LD + kk);
+#pragma unroll
+            for (int i = 0; i < MP; ++i)
+#pragma unroll
+                for (int j = 0; j < MC; ++j) {
+                    float v = acc[i][j];
+                    v = fmaf(a[i].x, c[j].x, v);
+                    v = fmaf(a[i].y, c[j].y, v);
+                    v = fmaf(a[i].z, c[j].z, v);
+                    acc[i][j] = fmaf(a[i].w, c[j].w, v);
+                }
+        }
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float ob = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ob < best || (ob == best && oi < bi)) best = ob, bi = oi;
+    for (int i = 0; i < MP; ++i) {
+        const int p = p0 + tp + (THREADS / 16) * i;
+        uint64_t key = ~0ull;
+#pragma unroll
+        for (int j = 0; j < MC; ++j) {
+            const int c = c0 + tc + 16 * j;
+            if (c < K && b.active[c]) {
+                const float v = nrm[c] - 2.0f * acc[i][j];
+                if (v < INFINITY) key = min(key, nearest_key(v, c));
+            }
+        }
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) key = min(key, (uint64_t)__shfl_xor_sync(0xffffffffu, key, o));
+        if (tc == 0 && p < P && key != ~0ull) atomicMin(keys + p, (unsigned long long)key);
     }
-    if (lane == 0) pa[p] = bi;
 }
 
-// Block per centre: the weighted mean of its points (in point order) and their total weight;
-// an active centre without points keeps its position with weight 0; inactive slots are left.
-__global__ void __launch_bounds__(256) global_update(const float* __restrict__ Pm, int D, MergeBufs b,
-                                                     const int32_t* __restrict__ pa, float* __restrict__ C,
-                                                     float* __restrict__ W) {
-    const int c = blockIdx.x;
-    if (!b.active[c]) return;
+// Block per slot: the weighted mean of its points (in point order), their total weight and the
+// new row's squared norm; an active slot without points keeps its position with weight 0; inactive
+// slots are left.  The points' keys are read 256 at a time and the slot's own compacted in order.
+// `next` (the other half of the keys) is cleared for the next iteration; pa (nullable): every
+// point's slot.
+__global__ void __launch_bounds__(256) global_update(const float* __restrict__ Pm, int K, int KP, int D, MergeBufs b,
+                                                     const uint64_t* __restrict__ keys, uint64_t* __restrict__ next,
+                                                     int32_t* __restrict__ pa, float* __restrict__ C,
+                                                     float* __restrict__ W, float* __restrict__ nrm) {
+    __shared__ int s_p[256], s_n[8];
+    __shared__ float s_w[256];
+    __shared__ float s_row[1024];
+    const int c = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int P = b.n_points[0];
+    for (int p = c * 256 + t; p < KP; p += K * 256) next[p] = ~0ull;
+    if (pa)
+        for (int p = c * 256 + t; p < P; p += K * 256) pa[p] = keys[p] == ~0ull ? 0x7fffffff : (int32_t)(uint32_t)keys[p];
+    if (!b.active[c]) return;
     constexpr int kCols = 4;  // D <= 1024 = 4 x 256
     float acc[kCols] = {0.f, 0.f, 0.f, 0.f};
     float wsum = 0.f;
-    for (int p = 0; p < P; ++p) {
-        if (pa[p] != c) continue;
-        const float wp = b.pt_w[p];
-        wsum += wp;
+    for (int base = 0; base < P; base += 256) {
+        const int p = base + t;
+        const bool mine = p < P && (uint32_t)keys[p] == (uint32_t)c;
+        const uint32_t vote = __ballot_sync(0xffffffffu, mine);
+        if (lane == 0) s_n[warp] = __popc(vote);
+        __syncthreads();
+        int at = __popc(vote & ((1u << lane) - 1u)), members = 0;
 #pragma unroll
-        for (int u = 0; u < kCols; ++u) {
-            const int j = threadIdx.x + 256 * u;
-            if (j < D) acc[u] += wp * Pm[(int64_t)p * D + j];
+        for (int w = 0; w < 8; ++w) {
+            if (w < warp) at += s_n[w];
+            members += s_n[w];
+        }
+        if (mine) s_p[at] = p, s_w[at] = b.pt_w[p];
+        __syncthreads();
+#pragma unroll 4
+        for (int m = 0; m < members; ++m) {
+            const float wp = s_w[m];
+            const float* row = Pm + (int64_t)s_p[m] * D;
+            wsum += wp;
+#pragma unroll
+            for (int u = 0; u < kCols; ++u) {
+                const int j = t + 256 * u;
+                if (j < D) acc[u] += wp * row[j];
+            }
+        }
+        __syncthreads();
+    }
+    if (t == 0) W[c] = wsum;
+    if (!(wsum > 0.f)) return;
+#pragma unroll
+    for (int u = 0; u < kCols; ++u) {
+        const int j = t + 256 * u;
+        if (j < D) {
+            const float v = acc[u] / wsum;
+            C[(int64_t)c * D + j] = v;
+            s_row[j] = v;
         }
     }
-    if (wsum > 0.f) {
-#pragma unroll
-        for (int u = 0; u < kCols; ++u) {
-            const int j = threadIdx.x + 256 * u;
-            if (j < D) C[(int64_t)c * D + j] = acc[u] / wsum;
-        }
+    __syncthreads();
+    if (warp == 0) {
+        const float s = warp_norm2(s_row, D, lane);
+        if (lane == 0) nrm[c] = s;
     }
-    if (threadIdx.x == 0) W[c] = wsum;
+}
+
+template <int TP, int TC, int THREADS, int BK>
+latentam_status launch_nearest(const float* Pm, int KP, const float* C, int K, int D, const MergeBufs& mb,
+                               const float* nrm, uint64_t* keys, cudaStream_t st) {
+    constexpr size_t smem = dist_smem<TP, TC, BK>();
+    auto kern = global_nearest<TP, TC, THREADS, BK>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return cuda_error(e, "kmeans global_nearest smem attribute");
+    kern<<<dim3((K + TC - 1) / TC, (KP + TP - 1) / TP), THREADS, smem, st>>>(
+        Pm, KP, C, K, D, mb, nrm, reinterpret_cast<unsigned long long*>(keys));
+    LAT_CHECK_LAUNCH("kmeans global_nearest");
+    return LATENTAM_OK;
+}
+
+template <int NV, int R>
+latentam_status launch_pass(const KMeansArgs& a, const float* C, int warps, int nb, int32_t* assign, float* part,
+                            int32_t* pcnt, cudaStream_t st) {
+    const size_t smem = sizeof(float) * ((size_t)(warps + 1) * a.k * a.D + a.k);
+    auto kern = local_pass<NV, R>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return cuda_error(e, "kmeans local_pass smem attribute");
+    kern<<<nb, 32 * kRowWarps, smem, st>>>(a.F, a.n, a.D, a.valid, C, a.k, warps, assign, part, pcnt);
+    LAT_CHECK_LAUNCH("kmeans local_pass");
+    return LATENTAM_OK;
+}
+
+// Rows a warp of local_pass holds at D features (64 registers of embeddings a lane).
+int rows_per_warp(int D) { return D <= 256 ? 8 : D <= 512 ? 4 : 2; }
+
+latentam_status pass(const KMeansArgs& a, const float* C, int warps, int nb, int32_t* assign, float* part,
+                     int32_t* pcnt, cudaStream_t st) {
+    switch ((a.D + 127) / 128) {
+        case 1: return launch_pass<1, 8>(a, C, warps, nb, assign, part, pcnt, st);
+        case 2: return launch_pass<2, 8>(a, C, warps, nb, assign, part, pcnt, st);
+        case 3: return launch_pass<3, 4>(a, C, warps, nb, assign, part, pcnt, st);
+        case 4: return launch_pass<4, 4>(a, C, warps, nb, assign, part, pcnt, st);
+        case 5:
+        case 6: return launch_pass<6, 2>(a, C, warps, nb, assign, part, pcnt, st);
+        default: return launch_pass<8, 2>(a, C, warps, nb, assign, part, pcnt, st);
+    }
 }
 
 }  // namespace
 
-size_t kmeans_scratch_bytes(int64_t n, int D, int k, int K, int nb, bool need_mc, bool need_mw, bool need_assign) {
-    auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    const size_t KP = (size_t)K + k, ldg = ((size_t)K + 3) & ~(size_t)3;
-    size_t b = 0;
-    if (need_mc) b += up(4 * (size_t)k * D);
-    if (need_mw) b += up(4 * (size_t)k);
-    if (need_assign) b += up(4 * (size_t)std::max<int64_t>(n, 1));
-    b += up(4 * (size_t)nb * k * D) + up(4 * (size_t)nb * k);
-    b += up(4) + up(4 * KP) * 3 + up(4 * (size_t)K) * 3;
-    b += up(4 * KP * D) + up(4 * KP * ldg);
-    return b;
-}
-
 latentam_status stream_kmeans(latentam_ctx* ctx, const KMeansArgs& a, cudaStream_t st) {
-    const int k = a.k, K = a.K, D = a.D;
+    const int k = a.k, K = a.K, D = a.D, KP = K + k;
     const int64_t n = a.n;
     auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    const int nb = (int)std::max<int64_t>(1, std::min<int64_t>((n + 63) / 64, 2 * (int64_t)ctx->num_sms));
-    const int64_t R = (n + nb - 1) / nb;
-    const size_t KP = (size_t)K + k, ldg = ((size_t)K + 3) & ~(size_t)3;
-    char* base = static_cast<char*>(
-        ws(ctx, WS_KMEANS, kmeans_scratch_bytes(n, D, k, K, nb, !a.micro_C, !a.micro_W, !a.micro_assign)));
+    // Blocks and row warps of the local pass: two blocks per SM where the sums' copies leave room,
+    // fewer row warps where there are fewer rows than that many warps take.
+    const int R = rows_per_warp(D), most = local_warps(k, D), sms = ctx->num_sms;
+    const int64_t groups = (n + R - 1) / R;
+    const bool fused = most > 0;
+    const int warps = fused ? (int)std::max<int64_t>(1, std::min<int64_t>(most, (groups + sms - 1) / sms)) : 0;
+    const int per_sm = sizeof(float) * ((size_t)(warps + 1) * k * D + k) <= 111 * 1024 ? 2 : 1;
+    const int nb = (int)std::max<int64_t>(
+        1, fused ? std::min<int64_t>((groups + warps - 1) / warps, (int64_t)per_sm * sms)
+                 : std::min<int64_t>((n + 63) / 64, 2 * (int64_t)sms));
+    const size_t part_b = up(4 * (size_t)nb * k * D), pcnt_b = up(4 * (size_t)nb * k);
+    const size_t asg_b = fused || a.micro_assign ? 0 : up(4 * (size_t)std::max<int64_t>(n, 1));
+    const size_t bytes = (a.micro_C ? 0 : up(4 * (size_t)k * D)) + (a.micro_W ? 0 : up(4 * (size_t)k)) + up(4) +
+                         2 * up(4 * (size_t)KP) + up(16 * (size_t)KP) + 3 * up(4 * (size_t)K) +
+                         up(4 * (size_t)KP * D) + part_b + pcnt_b + asg_b;
+    char* base = static_cast<char*>(ws(ctx, WS_KMEANS, bytes));
     if (!base) return LATENTAM_ERR_OUT_OF_MEMORY;
     size_t o = 0;
     auto take = [&](size_t bytes) {
@@ -364,66 +682,59 @@ latentam_status stream_kmeans(latentam_ctx* ctx, const KMeansArgs& a, cudaStream
     float* mW = a.micro_W ? a.micro_W : reinterpret_cast<float*>(take(4 * (size_t)k));
     MergeBufs mb;
     mb.n_points = reinterpret_cast<int32_t*>(take(4));
-    mb.pt_src = reinterpret_cast<int32_t*>(take(4 * KP));
-    mb.pt_w = reinterpret_cast<float*>(take(4 * KP));
-    int32_t* pa = a.point_assign ? a.point_assign : reinterpret_cast<int32_t*>(take(4 * KP));
+    mb.pt_src = reinterpret_cast<int32_t*>(take(4 * (size_t)KP));
+    mb.pt_w = reinterpret_cast<float*>(take(4 * (size_t)KP));
+    uint64_t* keys = reinterpret_cast<uint64_t*>(take(16 * (size_t)KP));  // two halves, used in turn
     mb.slot_fill = reinterpret_cast<int32_t*>(take(4 * (size_t)K));
     mb.active = reinterpret_cast<int32_t*>(take(4 * (size_t)K));
     float* nrm = reinterpret_cast<float*>(take(4 * (size_t)K));
-    float* Pm = reinterpret_cast<float*>(take(4 * KP * D));
-    float* G = reinterpret_cast<float*>(take(4 * KP * ldg));
-    int32_t* asg = a.micro_assign ? a.micro_assign : reinterpret_cast<int32_t*>(take(4 * (size_t)std::max<int64_t>(n, 1)));
-    float* part = reinterpret_cast<float*>(take(4 * (size_t)nb * k * D));
-    float* pcnt = reinterpret_cast<float*>(take(4 * (size_t)nb * k));
+    float* Pm = reinterpret_cast<float*>(take(4 * (size_t)KP * D));
+    float* part = reinterpret_cast<float*>(take(part_b));
+    int32_t* pcnt = reinterpret_cast<int32_t*>(take(pcnt_b));
+    int32_t* asg = a.micro_assign || fused ? a.micro_assign : reinterpret_cast<int32_t*>(take(asg_b));
 
     // Both phases are chains of small dependent launches with no host round trip: each replays
     // a captured CUDA graph once the same shapes and buffers recur (the global phase's shapes
     // are the dictionary's, the same for every keyframe; the local phase's depend on the
     // number of targets).
-    const size_t sm_assign = 4 * ((size_t)k * D + k);
-    const int G_rows = kAccumThreads / (D / 4);
-    const size_t sm_accum = 4 * (size_t)G_rows * k * D;
-    const int ga = (int)std::max<int64_t>(1, std::min<int64_t>((n + 7) / 8, 4 * (int64_t)ctx->num_sms));
     auto local = [&](cudaStream_t s) -> latentam_status {
-        cudaFuncSetAttribute(local_assign, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_assign);
-        cudaFuncSetAttribute(local_accum, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_accum);
         local_init<<<k, 256, 0, s>>>(a.F, n, D, a.init_idx, mC);
         LAT_CHECK_LAUNCH("kmeans local_init");
         for (int it = 0; it < a.iters_local; ++it) {
-            if (n > 0) {
+            if (fused) {
+                LAT_TRY(pass(a, mC, warps, nb, it + 1 == a.iters_local ? asg : nullptr, part, pcnt, s));
+            } else {
+                const size_t sm_assign = 4 * ((size_t)k * D + k);
+                const size_t sm_accum = 4 * (size_t)(kAccumThreads / (D / 4)) * k * D;
+                const int ga = (int)std::max<int64_t>(1, std::min<int64_t>((n + 7) / 8, 4 * (int64_t)sms));
+                cudaFuncSetAttribute(local_assign, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_assign);
+                cudaFuncSetAttribute(local_accum, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_accum);
                 local_assign<<<ga, 256, sm_assign, s>>>(a.F, n, D, a.valid, mC, k, asg);
                 LAT_CHECK_LAUNCH("kmeans local_assign");
-                local_accum<<<nb, kAccumThreads, sm_accum, s>>>(a.F, n, D, asg, k, R, part, pcnt);
+                local_accum<<<nb, kAccumThreads, sm_accum, s>>>(a.F, n, D, asg, k, (n + nb - 1) / nb, part, pcnt);
                 LAT_CHECK_LAUNCH("kmeans local_accum");
-            } else {
-                cudaError_t e = cudaMemsetAsync(pcnt, 0, 4 * (size_t)nb * k, s);
-                if (e != cudaSuccess) return cuda_error(e, "clear kmeans counts");
-                e = cudaMemsetAsync(part, 0, 4 * (size_t)nb * k * D, s);
-                if (e != cudaSuccess) return cuda_error(e, "clear kmeans sums");
             }
-            local_finish<<<(unsigned)(((int64_t)k * D + 255) / 256), 256, 0, s>>>(part, pcnt, nb, k, D, mC, mW);
+            local_finish<<<(k * D + 31) / 32, 256, 0, s>>>(part, pcnt, nb, k, D, mC, mW);
             LAT_CHECK_LAUNCH("kmeans local_finish");
         }
         return LATENTAM_OK;
     };
     auto global = [&](cudaStream_t s) -> latentam_status {
-        cudaError_t e = cudaMemsetAsync(Pm, 0, 4 * KP * D, s);
-        if (e != cudaSuccess) return cuda_error(e, "clear kmeans points");
-        e = cudaMemsetAsync(pa, 0xff, 4 * KP, s);  // -1 past the last point
-        if (e != cudaSuccess) return cuda_error(e, "clear kmeans point assignment");
         global_merge<<<1, 1024, 0, s>>>(a.weights, K, mW, k, mb);
         LAT_CHECK_LAUNCH("kmeans global_merge");
-        global_points<<<(unsigned)KP, 256, 0, s>>>(a.centres, mC, D, mb, Pm);
-        LAT_CHECK_LAUNCH("kmeans global_points");
-        global_fill<<<K, 256, 0, s>>>(mC, D, mb, a.centres);
-        LAT_CHECK_LAUNCH("kmeans global_fill");
+        global_setup<<<KP, 256, 0, s>>>(a.centres, mC, K, KP, D, mb, Pm, nrm, keys, a.point_assign);
+        LAT_CHECK_LAUNCH("kmeans global_setup");
+        const int64_t small_tiles = (int64_t)((KP + 15) / 16) * ((K + 31) / 32);
         for (int it = 0; it < a.iters_global; ++it) {
-            centre_norms<<<(K + 7) / 8, 256, 0, s>>>(a.centres, K, D, nrm);
-            LAT_CHECK_LAUNCH("kmeans centre_norms");
-            LAT_TRY(sgemm_abt(Pm, (int64_t)KP, a.centres, K, D, G, (int64_t)ldg, 1.0f, s));
-            global_assign<<<(unsigned)((KP + 7) / 8), 256, 0, s>>>(G, (int64_t)ldg, nrm, K, mb, pa);
-            LAT_CHECK_LAUNCH("kmeans global_assign");
-            global_update<<<K, 256, 0, s>>>(Pm, D, mb, pa, a.centres, a.weights);
+            uint64_t *cur = keys + (it & 1 ? KP : 0), *next = keys + (it & 1 ? 0 : KP);
+            // 16 x 32 tiles while all of them are resident at once (four blocks per SM), else 64 x 64
+            if (small_tiles <= 4 * sms)
+                LAT_TRY((launch_nearest<16, 32, 128, 64>(Pm, KP, a.centres, K, D, mb, nrm, cur, s)));
+            else
+                LAT_TRY((launch_nearest<64, 64, 256, 32>(Pm, KP, a.centres, K, D, mb, nrm, cur, s)));
+            global_update<<<K, 256, 0, s>>>(Pm, K, KP, D, mb, cur, next,
+                                            it + 1 == a.iters_global ? a.point_assign : nullptr, a.centres, a.weights,
+                                            nrm);
             LAT_CHECK_LAUNCH("kmeans global_update");
         }
         return LATENTAM_OK;
@@ -432,14 +743,13 @@ latentam_status stream_kmeans(latentam_ctx* ctx, const KMeansArgs& a, cudaStream
                              (uint64_t)a.iters_local, reinterpret_cast<uint64_t>(a.F),
                              reinterpret_cast<uint64_t>(a.valid), reinterpret_cast<uint64_t>(a.init_idx),
                              reinterpret_cast<uint64_t>(mC), reinterpret_cast<uint64_t>(mW),
-                             reinterpret_cast<uint64_t>(asg), reinterpret_cast<uint64_t>(base),
+                             reinterpret_cast<uint64_t>(asg), reinterpret_cast<uint64_t>(part),
                              reinterpret_cast<uint64_t>(st), ctx->ws_generation};
     LAT_TRY(cached_launch(ctx, lkey, (int)(sizeof(lkey) / sizeof(lkey[0])), st, local));
     const uint64_t gkey[] = {0x6b6d2d676c6f6262ull /* tag: global phase */, (uint64_t)D, (uint64_t)k, (uint64_t)K,
                              (uint64_t)a.iters_global, reinterpret_cast<uint64_t>(a.centres),
                              reinterpret_cast<uint64_t>(a.weights), reinterpret_cast<uint64_t>(mC),
-                             reinterpret_cast<uint64_t>(mW), reinterpret_cast<uint64_t>(pa),
-                             reinterpret_cast<uint64_t>(Pm), reinterpret_cast<uint64_t>(G),
+                             reinterpret_cast<uint64_t>(mW), reinterpret_cast<uint64_t>(a.point_assign),
                              reinterpret_cast<uint64_t>(base), reinterpret_cast<uint64_t>(st), ctx->ws_generation};
     LAT_TRY(cached_launch(ctx, gkey, (int)(sizeof(gkey) / sizeof(gkey[0])), st, global));
     return LATENTAM_OK;

@@ -221,6 +221,22 @@ def test_rejects_unsupported_shapes(api, ctx):
     assert e.value.status == L.ERR_UNSUPPORTED_SHAPE
 
 
+@pytest.mark.parametrize("n,D,k,K", [(1, 4, 1, 1), (37, 132, 6, 33), (2500, 256, 32, 64), (333, 384, 9, 700),
+                                     (700, 640, 13, 90), (260, 1024, 13, 1100), (500, 1024, 32, 40)])
+def test_replay_tile_edges(api, ctx, n, D, k, K):
+    """Ragged rows, partial feature blocks of every row form (two, four and eight rows a warp, and
+    k x D too large for the one-pass form), both tile sizes of the re-clustering and their rims."""
+    rng = np.random.default_rng(n + D)
+    E = rng.normal(size=(17, D)) / np.sqrt(D)
+    F = (E[rng.integers(0, 17, size=n)] + rng.normal(0, 0.3, size=(n, D)) / np.sqrt(D)).astype(np.float32)
+    valid = (rng.uniform(size=n) > 0.2).astype(np.uint8)
+    valid[:k] = 1
+    C = (E[rng.integers(0, 17, size=K)] + rng.normal(0, 0.3, size=(K, D)) / np.sqrt(D)).astype(np.float32)
+    W = np.where(rng.uniform(size=K) < 0.9, rng.integers(1, 50, size=K), 0).astype(np.float32)
+    init = rng.choice(np.flatnonzero(valid), size=k, replace=False).astype(np.int32)
+    _replay(api, ctx, F, valid, C, W, init, 3, 3)
+
+
 def test_full_size_per_pixel(api, ctx):
     """640x480 per-pixel targets (307,200 rows, D = 512), 5 micro-clusters into K = 256 slots
     of which 100 are occupied, replay-validated."""
