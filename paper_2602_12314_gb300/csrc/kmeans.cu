@@ -5,7 +5,7 @@
 // empty slot, and the empty slots take the heaviest micro-centres first.
 //
 // Local phase (n rows, k <= 32 centres): one pass over the rows per Lloyd iteration.  A warp
-// holds four rows in registers (two past D = 512), finds each one's nearest centre against the
+// holds four rows in registers (eight up to D = 256), finds each one's nearest centre against the
 // centres staged in shared memory (squared distance as |c|^2 - 2 <x, c>, ties to the lower index)
 // and adds the rows to its own copy of the cluster sums in shared memory; copies and blocks are
 // summed in a fixed order (no atomics), so the result does not depend on scheduling.
@@ -49,13 +49,35 @@ __global__ void local_init(const float* __restrict__ F, int64_t n, int D, const 
     for (int j = threadIdx.x; j < D; j += blockDim.x) C[(int64_t)c * D + j] = ok ? F[(int64_t)r * D + j] : 0.f;
 }
 
-// Warps (each with a copy of the k x D sums beside the staged centres) of a block of local_pass;
-// 0: not even one copy fits.
-int local_warps(int k, int D) {
-    const size_t copy = sizeof(float) * (size_t)k * D, norms = 256;
-    if (2 * copy + norms > kRowSmem) return 0;
-    return (int)std::min<size_t>(kRowWarps, (kRowSmem - norms) / copy - 1);
+// Launch shape of the local pass.  Row warps per block (a power of two: eight, fewer when there are
+// fewer rows than that many warps take), the copies of the k x D sums they share (a power of two; 0
+// when k x D is too large for even one beside the staged centres), rows per warp and blocks.
+struct PassShape {
+    int warps, copies, rows, per_sm, nb;
+    size_t smem;
+};
+
+// Two blocks per SM up to D = 512 (64 registers of embeddings a lane at four rows of 512), one
+// above (128 registers), so that 128 KB of rows per SM are in flight either way; of the shapes
+// that fit, the one with the most copies.
+PassShape pass_shape(int64_t n, int k, int D, int sms) {
+    PassShape p{};
+    p.rows = D <= 256 ? 8 : 4;
+    const int64_t groups = (n + p.rows - 1) / p.rows;
+    p.warps = 1;
+    while (p.warps < kRowWarps && (int64_t)p.warps * sms < groups) p.warps *= 2;
+    auto bytes = [&](int copies) { return sizeof(float) * ((size_t)(copies + 1) * k * D + k); };
+    for (p.per_sm = D <= 512 ? 2 : 1; p.per_sm >= 1 && !p.copies; --p.per_sm)
+        for (p.copies = p.warps; p.copies && bytes(p.copies) > kRowSmem / p.per_sm; p.copies /= 2) {
+        }
+    ++p.per_sm;
+    p.smem = bytes(p.copies);
+    p.nb = (int)std::max<int64_t>(1, std::min<int64_t>((groups + p.warps - 1) / p.warps, (int64_t)p.per_sm * sms));
+    return p;
 }
+
+__device__ __forceinline__ void pair_sync(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
+__device__ __forceinline__ void pair_arrive(int id) { asm volatile("bar.arrive %0, 64;" ::"r"(id) : "memory"); }
 
 // One Lloyd pass: every valid row's nearest centre and the block's sums of its rows per cluster,
 // part[block] (k x D) and pcnt[block] (k).  Bound by the read of the embeddings (HBM, once per
@@ -64,35 +86,43 @@ int local_warps(int k, int D) {
 // products leave the butterfly together (log2 R scatter steps, then the R lane groups each finish
 // one row), in the summation tree of a plain butterfly.  Rows of one group that share their
 // cluster are added together before the read-modify-write of the sums.  NV: quads per lane
-// (D <= 128 NV).  `warps` of the block's eight take rows (as many as the sums' copies leave room
-// for, or as there are rows); all of them stage the centres and add up the copies.
+// (D <= 128 NV).  `warps` of the block's eight take rows, all of them stage the centres and add up
+// the copies.  With fewer copies of the sums than row warps, the warps of a copy add in turn, round
+// by round (warp w hands over to w + copies, the last one to the first one's next round), each
+// handover a named barrier of the two warps; every row warp runs every round.
+// At 307,200 x 512, k = 5: 252 + 185 us (assign, accumulate) -> 126 us, 5.0 TB/s.
 template <int NV, int R>
-__global__ void __launch_bounds__(32 * kRowWarps, 2) local_pass(const float* __restrict__ F, int64_t n, int D,
+__global__ void __launch_bounds__(32 * kRowWarps, NV <= 4 ? 2 : 1) local_pass(const float* __restrict__ F, int64_t n, int D,
                                                                 const uint8_t* __restrict__ valid,
                                                                 const float* __restrict__ C, int k,
-                                                                int warps, int32_t* __restrict__ assign,
+                                                                int warps, int copies,
+                                                                int32_t* __restrict__ assign,
                                                                 float* __restrict__ part, int32_t* __restrict__ pcnt) {
     extern __shared__ __align__(16) float sm[];
     __shared__ int s_cnt[kRowWarps][kMaxMicro];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int D4 = D / 4;
     float4* sC = reinterpret_cast<float4*>(sm);        // k x D
-    float4* sS = sC + (size_t)k * D4;                  // warps x k x D
-    float* sN = sm + (size_t)(warps + 1) * k * D;      // k
+    float4* sS = sC + (size_t)k * D4;                  // copies x k x D
+    float* sN = sm + (size_t)(copies + 1) * k * D;     // k
     for (int i = threadIdx.x; i < k * D4; i += blockDim.x) sC[i] = reinterpret_cast<const float4*>(C)[i];
-    for (int i = threadIdx.x; i < warps * k * D4; i += blockDim.x) sS[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = threadIdx.x; i < copies * k * D4; i += blockDim.x) sS[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncthreads();
     for (int c = warp; c < k; c += kRowWarps) {
         const float s = warp_norm2(sm + (size_t)c * D, D, lane);
         if (lane == 0) sN[c] = s;
     }
     __syncthreads();
-    float4* own = sS + (size_t)warp * k * D4;  // lane l only touches quads l, l + 32, ...
+    // lane l only touches quads l, l + 32, ... of its warp's copy
+    float4* own = sS + (size_t)(warp % copies) * k * D4;
+    const bool turns = copies < warps, last = warp + copies >= warps;
     int cnt = 0;                               // rows of cluster `lane`
     constexpr int G = 32 / R;                  // lanes that end with one row's dot product
     const float4* F4 = reinterpret_cast<const float4*>(F);
-    const int64_t step = (int64_t)gridDim.x * warps * R;
-    for (int64_t r0 = ((int64_t)blockIdx.x * warps + warp) * R; warp < warps && r0 < n; r0 += step) {
+    const int64_t step = (int64_t)gridDim.x * warps * R, begin = (int64_t)blockIdx.x * warps * R;
+    const int64_t rounds = warp < warps && begin < n ? (n - begin + step - 1) / step : 0;  // the same for all row warps
+    for (int64_t round = 0; round < rounds; ++round) {
+        const int64_t r0 = begin + round * step + warp * R;
         float4 x[R][NV];
         bool ok[R];
 #pragma unroll
@@ -155,6 +185,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) local_pass(const float* __r
                 }
             }
         };
+        if (turns && (warp >= copies || round > 0)) pair_sync(1 + warp);
         if (same) {
             if (a[0] >= 0) {
 #pragma unroll
@@ -171,12 +202,13 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) local_pass(const float* __r
             for (int r = 0; r < R; ++r)
                 if (a[r] >= 0) add(a[r], x[r]);
         }
+        if (turns && !(last && round + 1 == rounds)) pair_arrive(last ? 1 + warp % copies : 1 + warp + copies);
     }
     s_cnt[warp][lane] = cnt;
     __syncthreads();
     for (int i = threadIdx.x; i < k * D4; i += blockDim.x) {
         float4 t = sS[i];
-        for (int w = 1; w < warps; ++w) {
+        for (int w = 1; w < copies; ++w) {
             const float4 u = sS[(size_t)w * k * D4 + i];
             t.x += u.x, t.y += u.y, t.z += u.z, t.w += u.w;
         }
@@ -191,7 +223,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) local_pass(const float* __r
 
 // assign[r] = nearest of the k centres (-1 for an invalid row); warp per row.  Shared memory:
 // the centres (k x D) and their squared norms.  D % 4 == 0, D <= 1024.  With local_accum, the
-// form for k x D past what local_pass holds twice in shared memory (k = 32 at D > 860).
+// form for k x D past what local_pass holds twice in shared memory (k = 32 at D > 876).
 __global__ void __launch_bounds__(256) local_assign(const float* __restrict__ F, int64_t n, int D,
                                                     const uint8_t* __restrict__ valid, const float* __restrict__ C,
                                                     int k, int32_t* __restrict__ assign) {
@@ -296,22 +328,24 @@ __global__ void __launch_bounds__(kAccumThreads) local_accum(const float* __rest
 }
 
 // C[c][j] = (sum over blocks of part[b][c][j]) / count_c, kept when the cluster is empty;
-// W[c] = count_c.  Block per 32 columns of the k x D sums, warp w takes blocks w, w + 8, ... and the
+// W[c] = count_c.  Block per 32 columns of the k x D sums, warp w takes blocks w, w + 32, ... and the
 // warps' sums are added in order.  (One thread per column walking all blocks took 43 us over 304
 // blocks at k = 5, D = 512.)
-__global__ void __launch_bounds__(256) local_finish(const float* __restrict__ part, const int32_t* __restrict__ pcnt,
-                                                    int nb, int k, int D, float* __restrict__ C,
-                                                    float* __restrict__ W) {
-    __shared__ float s_sum[8][32];
-    __shared__ long long s_cnt[8][32];
+constexpr int kFinishWarps = 32;
+__global__ void __launch_bounds__(32 * kFinishWarps) local_finish(const float* __restrict__ part,
+                                                                  const int32_t* __restrict__ pcnt, int nb, int k,
+                                                                  int D, float* __restrict__ C,
+                                                                  float* __restrict__ W) {
+    __shared__ float s_sum[kFinishWarps][32];
+    __shared__ long long s_cnt[kFinishWarps][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int i = blockIdx.x * 32 + lane, kD = k * D;
     const int c = min(i, kD - 1) / D;
     float s = 0.f;
     long long m = 0;
     if (i < kD) {
-#pragma unroll 8
-        for (int b = warp; b < nb; b += 8) {
+#pragma unroll 4
+        for (int b = warp; b < nb; b += kFinishWarps) {
             s += part[(size_t)b * kD + i];
             m += pcnt[(size_t)b * k + c];
         }
@@ -320,7 +354,8 @@ __global__ void __launch_bounds__(256) local_finish(const float* __restrict__ pa
     s_cnt[warp][lane] = m;
     __syncthreads();
     if (warp != 0 || i >= kD) return;
-    for (int w = 1; w < 8; ++w) s += s_sum[w][lane], m += s_cnt[w][lane];
+#pragma unroll
+    for (int w = 1; w < kFinishWarps; ++w) s += s_sum[w][lane], m += s_cnt[w][lane];
     if (m > 0) C[i] = s / (float)m;
     if (i == c * D) W[c] = (float)m;
 }
@@ -471,8 +506,9 @@ __global__ void __launch_bounds__(THREADS) global_nearest(const float* __restric
     extern __shared__ __align__(16) float sm[];
     const int P = b.n_points[0];
     const int p0 = blockIdx.y * TP, c0 = blockIdx.x * TC;
-    if (p0 >= P) return;
     const int t = threadIdx.x, tc = t & 15, tp = t >> 4;
+    // nothing to do past the last point, or where every slot of the tile is empty
+    if (p0 >= P || !__syncthreads_or(t < TC && c0 + t < K && b.active[c0 + t])) return;
     const int slices = (D + BK - 1) / BK;
     auto load = [&](int s) {
         float* dst = sm + (size_t)(s % kDistStages) * (TP + TC) * LD;
@@ -620,30 +656,26 @@ latentam_status launch_nearest(const float* Pm, int KP, const float* C, int K, i
 }
 
 template <int NV, int R>
-latentam_status launch_pass(const KMeansArgs& a, const float* C, int warps, int nb, int32_t* assign, float* part,
+latentam_status launch_pass(const KMeansArgs& a, const float* C, const PassShape& p, int32_t* assign, float* part,
                             int32_t* pcnt, cudaStream_t st) {
-    const size_t smem = sizeof(float) * ((size_t)(warps + 1) * a.k * a.D + a.k);
     auto kern = local_pass<NV, R>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
     if (e != cudaSuccess) return cuda_error(e, "kmeans local_pass smem attribute");
-    kern<<<nb, 32 * kRowWarps, smem, st>>>(a.F, a.n, a.D, a.valid, C, a.k, warps, assign, part, pcnt);
+    kern<<<p.nb, 32 * kRowWarps, p.smem, st>>>(a.F, a.n, a.D, a.valid, C, a.k, p.warps, p.copies, assign, part, pcnt);
     LAT_CHECK_LAUNCH("kmeans local_pass");
     return LATENTAM_OK;
 }
 
-// Rows a warp of local_pass holds at D features (64 registers of embeddings a lane).
-int rows_per_warp(int D) { return D <= 256 ? 8 : D <= 512 ? 4 : 2; }
-
-latentam_status pass(const KMeansArgs& a, const float* C, int warps, int nb, int32_t* assign, float* part,
+latentam_status pass(const KMeansArgs& a, const float* C, const PassShape& p, int32_t* assign, float* part,
                      int32_t* pcnt, cudaStream_t st) {
     switch ((a.D + 127) / 128) {
-        case 1: return launch_pass<1, 8>(a, C, warps, nb, assign, part, pcnt, st);
-        case 2: return launch_pass<2, 8>(a, C, warps, nb, assign, part, pcnt, st);
-        case 3: return launch_pass<3, 4>(a, C, warps, nb, assign, part, pcnt, st);
-        case 4: return launch_pass<4, 4>(a, C, warps, nb, assign, part, pcnt, st);
+        case 1: return launch_pass<1, 8>(a, C, p, assign, part, pcnt, st);
+        case 2: return launch_pass<2, 8>(a, C, p, assign, part, pcnt, st);
+        case 3: return launch_pass<3, 4>(a, C, p, assign, part, pcnt, st);
+        case 4: return launch_pass<4, 4>(a, C, p, assign, part, pcnt, st);
         case 5:
-        case 6: return launch_pass<6, 2>(a, C, warps, nb, assign, part, pcnt, st);
-        default: return launch_pass<8, 2>(a, C, warps, nb, assign, part, pcnt, st);
+        case 6: return launch_pass<6, 4>(a, C, p, assign, part, pcnt, st);
+        default: return launch_pass<8, 4>(a, C, p, assign, part, pcnt, st);
     }
 }
 
@@ -653,16 +685,10 @@ latentam_status stream_kmeans(latentam_ctx* ctx, const KMeansArgs& a, cudaStream
     const int k = a.k, K = a.K, D = a.D, KP = K + k;
     const int64_t n = a.n;
     auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    // Blocks and row warps of the local pass: two blocks per SM where the sums' copies leave room,
-    // fewer row warps where there are fewer rows than that many warps take.
-    const int R = rows_per_warp(D), most = local_warps(k, D), sms = ctx->num_sms;
-    const int64_t groups = (n + R - 1) / R;
-    const bool fused = most > 0;
-    const int warps = fused ? (int)std::max<int64_t>(1, std::min<int64_t>(most, (groups + sms - 1) / sms)) : 0;
-    const int per_sm = sizeof(float) * ((size_t)(warps + 1) * k * D + k) <= 111 * 1024 ? 2 : 1;
-    const int nb = (int)std::max<int64_t>(
-        1, fused ? std::min<int64_t>((groups + warps - 1) / warps, (int64_t)per_sm * sms)
-                 : std::min<int64_t>((n + 63) / 64, 2 * (int64_t)sms));
+    const int sms = ctx->num_sms;
+    const PassShape shape = pass_shape(n, k, D, sms);
+    const bool fused = shape.copies > 0;
+    const int nb = fused ? shape.nb : (int)std::min<int64_t>((n + 63) / 64, 2 * (int64_t)sms);
     const size_t part_b = up(4 * (size_t)nb * k * D), pcnt_b = up(4 * (size_t)nb * k);
     const size_t asg_b = fused || a.micro_assign ? 0 : up(4 * (size_t)std::max<int64_t>(n, 1));
     const size_t bytes = (a.micro_C ? 0 : up(4 * (size_t)k * D)) + (a.micro_W ? 0 : up(4 * (size_t)k)) + up(4) +
@@ -702,7 +728,7 @@ latentam_status stream_kmeans(latentam_ctx* ctx, const KMeansArgs& a, cudaStream
         LAT_CHECK_LAUNCH("kmeans local_init");
         for (int it = 0; it < a.iters_local; ++it) {
             if (fused) {
-                LAT_TRY(pass(a, mC, warps, nb, it + 1 == a.iters_local ? asg : nullptr, part, pcnt, s));
+                LAT_TRY(pass(a, mC, shape, it + 1 == a.iters_local ? asg : nullptr, part, pcnt, s));
             } else {
                 const size_t sm_assign = 4 * ((size_t)k * D + k);
                 const size_t sm_accum = 4 * (size_t)(kAccumThreads / (D / 4)) * k * D;
@@ -714,7 +740,7 @@ latentam_status stream_kmeans(latentam_ctx* ctx, const KMeansArgs& a, cudaStream
                 local_accum<<<nb, kAccumThreads, sm_accum, s>>>(a.F, n, D, asg, k, (n + nb - 1) / nb, part, pcnt);
                 LAT_CHECK_LAUNCH("kmeans local_accum");
             }
-            local_finish<<<(k * D + 31) / 32, 256, 0, s>>>(part, pcnt, nb, k, D, mC, mW);
+            local_finish<<<(k * D + 31) / 32, 32 * kFinishWarps, 0, s>>>(part, pcnt, nb, k, D, mC, mW);
             LAT_CHECK_LAUNCH("kmeans local_finish");
         }
         return LATENTAM_OK;
@@ -729,7 +755,7 @@ latentam_status stream_kmeans(latentam_ctx* ctx, const KMeansArgs& a, cudaStream
             uint64_t *cur = keys + (it & 1 ? KP : 0), *next = keys + (it & 1 ? 0 : KP);
             // 16 x 32 tiles while all of them are resident at once (four blocks per SM), else 64 x 64
             if (small_tiles <= 4 * sms)
-                LAT_TRY((launch_nearest<16, 32, 128, 64>(Pm, KP, a.centres, K, D, mb, nrm, cur, s)));
+                LAT_TRY((launch_nearest<16, 32, 256, 64>(Pm, KP, a.centres, K, D, mb, nrm, cur, s)));
             else
                 LAT_TRY((launch_nearest<64, 64, 256, 32>(Pm, KP, a.centres, K, D, mb, nrm, cur, s)));
             global_update<<<K, 256, 0, s>>>(Pm, K, KP, D, mb, cur, next,
