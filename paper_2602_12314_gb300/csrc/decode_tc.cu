@@ -322,7 +322,7 @@ struct SoftmaxEpi {
     static constexpr bool SPLIT = SPLIT_, INPLACE = false;
     static constexpr int BN = 256, BK = SPLIT_ ? 16 : 64, ELEM = 2, STAGES = SPLIT_ ? 3 : 1, BOX_B = 256;
     static constexpr int EPI_WG = 4, E_BOXES = 0, O_BOXES = 4;
-    static constexpr int XROUNDS = 1;
+    static constexpr int XROUNDS = 1, WARP_STAGE = 0;
     static constexpr bool A_MN = false, B_MN = false;
     using Params = SoftmaxParams;
     static __device__ int run(const Params& p, const tc::EpiCtx& ec) {
@@ -399,11 +399,72 @@ struct FhatParams {
     double* acc;
     bf16* dF;     // n x D
     float* row;   // n x 4: a_p, b_p, <A_p, dA_p>, cos_p
-    float* Fout;  // n x D FP32 Fhat (inference form: no loss) or NULL
     // E4M3 form: row statistics of the softmax (the per-pixel scale 448 l_p) and the
     // per-feature scale inverses max_j |V_jc| / 448
     const float* stats;
     const float* inv_t;
+};
+
+// Fhat chunk c0 of this thread's row from TMEM (E4M3: times 1 / (scale_p scale_c), isp the pixel's)
+template <bool Q8>
+__device__ __forceinline__ void fhat32(const FhatParams& p, const tc::EpiCtx& ec, int c0, float isp, float (&h)[32]) {
+    tc::tmem_ld32(ec.taddr + c0, h);
+    if constexpr (Q8) {
+        const float4* it = reinterpret_cast<const float4*>(p.inv_t + ec.n0 + c0);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const float4 v = it[q];
+            h[4 * q] *= isp * v.x;
+            h[4 * q + 1] *= isp * v.y;
+            h[4 * q + 2] *= isp * v.z;
+            h[4 * q + 3] *= isp * v.w;
+        }
+    }
+}
+template <bool Q8>
+__device__ __forceinline__ float row_scale_inv(const FhatParams& p, int64_t pix, bool valid) {
+    if constexpr (Q8) return valid ? 1.0f / (448.0f * p.stats[2 * pix + 1]) : 0.f;
+    return 1.f;
+}
+
+// Inference form of G2: Fhat = A V out as FP32 rows, no loss and no row terms (independent column
+// tiles).  Each warp stages 32 rows x 32 columns (4 KB) in shared memory of its own and sends them
+// with a TMA store, so that every row leaves as whole 128-byte lines; without box buffers the
+// operand ring takes 144 KB (three stages of 64 K elements; 32 in the split form) instead of 72.
+// Bound by the FP32 rows written and the value matrix streamed through the ring for every tile.
+// 816,000 rows, M = 512, D = 768, BF16: 1,694 us with one row per thread stored in 16-byte pieces
+// and a 72 KB ring -> 678 us (the same bits).
+template <bool Q8 = false, bool SPLIT_ = false>
+struct FhatOutEpi {
+    static_assert(!SPLIT_ || !Q8, "the split form has no E4M3 operands");
+    static constexpr bool SPLIT = SPLIT_, INPLACE = false;
+    static constexpr int ELEM = Q8 ? 1 : 2, BK = SPLIT_ ? 32 : 64, STAGES = Q8 ? 6 : 3;
+    static constexpr int BN = 256, BOX_B = 256, EPI_WG = 4, XROUNDS = 0, E_BOXES = 0, O_BOXES = 0;
+    static constexpr int WARP_STAGE = 4096;
+    static constexpr bool A_MN = false, B_MN = !Q8;
+    using Params = FhatParams;
+    static __device__ int run(const Params& p, const tc::EpiCtx& ec) {
+        const int ncols = min(BN, p.D - ec.n0), lane = ec.row & 31;
+        const int64_t pix = (int64_t)ec.m0 + ec.row;
+        const float isp = row_scale_inv<Q8>(p, pix, pix < p.n);
+        for (int c0 = 32 * ec.g; c0 < ncols; c0 += 32 * EPI_WG) {
+            float h[32];
+            fhat32<Q8>(p, ec, c0, isp, h);
+            if (lane == 0) tc::bulk_wait_read();  // the previous chunk has left the staging rows
+            __syncwarp();
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                *reinterpret_cast<float4*>(ec.xstage + lane * 128 + ((q ^ (lane & 7)) << 4)) =
+                    make_float4(h[4 * q], h[4 * q + 1], h[4 * q + 2], h[4 * q + 3]);
+            tc::fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) {  // rows past the last one are not written
+                tc::tma_store_2d(ec.omap, ec.xstage, ec.n0 + c0, ec.m0 + ec.row);
+                tc::bulk_commit();
+            }
+        }
+        return 0;
+    }
 };
 
 // ETILE: the BF16 target rows come through shared memory (TMA, after the MMAs); otherwise
@@ -422,31 +483,12 @@ struct FhatEpi {
     // persistent, 64-byte K chunks (three ring stages fit beside two epilogue buffers)
     static constexpr int ELEM = Q8 ? 1 : 2, BK = SPLIT_ ? 16 : 64 / ELEM;
     static constexpr int BN = 256, STAGES = 3, BOX_B = 256, EPI_WG = ETILE ? 4 : 2, XROUNDS = 1;
+    static constexpr int WARP_STAGE = 0;
     // dFhat staged over the target
     static constexpr int E_BOXES = INPLACE ? 8 : ETILE ? BN / 64 : 0, O_BOXES = BN / 64;
     // B = V (atoms x features, features contiguous: MN-major) or, for E4M3, V^T (K-major)
     static constexpr bool A_MN = false, B_MN = !Q8;
     using Params = FhatParams;
-    // Fhat chunk c0 of this thread's row from TMEM (E4M3: times 1 / (scale_p scale_c))
-    static __device__ __forceinline__ void fhat32(const Params& p, const tc::EpiCtx& ec, int c0, float isp,
-                                                  float (&h)[32]) {
-        tc::tmem_ld32(ec.taddr + c0, h);
-        if constexpr (Q8) {
-            const float4* it = reinterpret_cast<const float4*>(p.inv_t + ec.n0 + c0);
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const float4 v = it[q];
-                h[4 * q] *= isp * v.x;
-                h[4 * q + 1] *= isp * v.y;
-                h[4 * q + 2] *= isp * v.z;
-                h[4 * q + 3] *= isp * v.w;
-            }
-        }
-    }
-    static __device__ __forceinline__ float row_scale_inv(const Params& p, int64_t pix, bool valid) {
-        if constexpr (Q8) return valid ? 1.0f / (448.0f * p.stats[2 * pix + 1]) : 0.f;
-        return 1.f;
-    }
     // body(c0, h, f) for each 32-column chunk of this thread's share of the slice: h = Fhat
     // (TMEM), f = target
     template <class Body>
@@ -460,7 +502,7 @@ struct FhatEpi {
                     ec.row32f(c0, f);
                 else
                     ec.row32(c0, f);
-                fhat32(p, ec, c0, isp, h);
+                fhat32<Q8>(p, ec, c0, isp, h);
                 body(c0, h, f);
             }
         } else {
@@ -468,7 +510,7 @@ struct FhatEpi {
             load_target32(p.F, p.F_dtype, frow + 32 * ec.g, f);
             for (int c0 = 32 * ec.g; c0 < ncols; c0 += step) {
                 if (c0 + step < ncols) load_target32(p.F, p.F_dtype, frow + c0 + step, fn);
-                fhat32(p, ec, c0, isp, h);
+                fhat32<Q8>(p, ec, c0, isp, h);
                 body(c0, h, f);
 #pragma unroll
                 for (int i = 0; i < 32; ++i) f[i] = fn[i];
@@ -481,22 +523,7 @@ struct FhatEpi {
         float* scr = ec.scratch;
         const int64_t pix = (int64_t)m0 + row;
         const bool valid = pix < p.n;
-        const float isp = row_scale_inv(p, pix, valid);
-        if (p.Fout) {  // inference form, launched without a cluster
-            ec.wait_out();
-            float h[32];
-            for (int c0 = 32 * g; c0 < ncols; c0 += 32 * EPI_WG) {
-                fhat32(p, ec, c0, isp, h);
-                if (valid) {
-                    float4* d4 = reinterpret_cast<float4*>(p.Fout + pix * p.D + ec.n0 + c0);
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) d4[q] = make_float4(h[4 * q], h[4 * q + 1], h[4 * q + 2], h[4 * q + 3]);
-                }
-            }
-            const float none[tc::kXchgVals] = {0.f, 0.f, 0.f, 0.f};
-            ec.exchange(none);
-            return 0;
-        }
+        const float isp = row_scale_inv<Q8>(p, pix, valid);
         // invalid rows read row 0 (discarded)
         const int64_t frow = (valid ? pix * p.D : 0) + ec.n0;
         // per-row and per-frame inputs first: their latency hides behind the first pass
@@ -1245,8 +1272,6 @@ latentam_status tc_fhat(latentam_ctx* ctx, const TcBuffers& b, int64_t n, int M,
     LAT_TRY(op_map(SPLIT, &mA, b.A, M, n, M, kTileM, BK));
     LAT_TRY(mn_map(SPLIT, &mV, b.Vb, D, M, D, BK, EpiF::BN / 64));
     const int cy = cdiv(D, 256), tiles = cdiv(n, kTileM), kc = cdiv(M, BK);
-    if (fp.Fout)  // no row terms: independent column tiles
-        return launch_persist<EpiF>(ctx, mA, mV, tiles, kc, cy, false, fp, b.err, st);
     CUtensorMap mdF;  // dFhat leaves through the TMA
     if (SPLIT && fp.F_dtype == LATENTAM_DTYPE_F32) {
         // FP32 targets by TMA, 32 columns at a time; dFhat written over them as 32-column planes
@@ -1278,7 +1303,6 @@ latentam_status tc_fhat8(latentam_ctx* ctx, const TcBuffers& b, int64_t n, int M
     LAT_TRY(u8_map(&mA, b.Aq, M, n, M, kTileM));
     LAT_TRY(u8_map(&mV, b.Vtq, M, D, M, 256));
     const int cy = cdiv(D, 256), tiles = cdiv(n, kTileM), kc = cdiv(M, 64);
-    if (fp.Fout) return launch_persist<FhatEpi<false, true>>(ctx, mA, mV, tiles, kc, cy, false, fp, b.err, st);
     CUtensorMap mdF;
     LAT_TRY(bf16_map(&mdF, fp.dF, D, n, D, kTileM));
     if (fp.F_dtype == LATENTAM_DTYPE_BF16) {
@@ -1287,6 +1311,28 @@ latentam_status tc_fhat8(latentam_ctx* ctx, const TcBuffers& b, int64_t n, int M
         return launch_persist<FhatEpi<true, true>>(ctx, mA, mV, tiles, kc, cy, true, fp, b.err, st, &mF, &mdF);
     }
     return launch_persist<FhatEpi<false, true>>(ctx, mA, mV, tiles, kc, cy, true, fp, b.err, st, nullptr, &mdF);
+}
+
+// The inference form: Fhat rows to F_hat (n x D).
+template <class Epi>
+latentam_status tc_fhat_out(latentam_ctx* ctx, const TcBuffers& b, int64_t n, int M, int D, float* F_hat,
+                            cudaStream_t st) {
+    constexpr bool Q8 = Epi::ELEM == 1;
+    CUtensorMap mA, mV, mO;
+    if (Q8) {
+        fp8_rows<<<cdiv(n * (M / 8), 256), 256, 0, st>>>(b.A, b.stats, n, M, b.Aq);
+        LAT_CHECK_LAUNCH("fp8_rows");
+        LAT_TRY(u8_map(&mA, b.Aq, M, n, M, kTileM));
+        LAT_TRY(u8_map(&mV, b.Vtq, M, D, M, 256));
+    } else {
+        LAT_TRY(op_map(Epi::SPLIT, &mA, b.A, M, n, M, kTileM, Epi::BK));
+        LAT_TRY(mn_map(Epi::SPLIT, &mV, b.Vb, D, M, D, Epi::BK, Epi::BN / 64));
+    }
+    LAT_TRY(f32_map(&mO, F_hat, D, n, 32));  // one warp's rows per box
+    const FhatParams fp{n, D, nullptr, LATENTAM_DTYPE_F32, nullptr, latentam_loss_cfg{}, nullptr, nullptr, nullptr,
+                        b.stats, b.inv_t};
+    return launch_persist<Epi>(ctx, mA, mV, cdiv(n, kTileM), cdiv(M, Epi::BK), cdiv(D, 256), false, fp, b.err, st,
+                               nullptr, &mO);
 }
 
 // The six contractions of the decode, its loss and its backward.  SPLIT: the FP32 form, every
@@ -1327,7 +1373,7 @@ latentam_status tc_loss_bwd(latentam_ctx* ctx, const DecodeArgs& a, cudaStream_t
         // G1: S = Q K^T -> softmax
         LAT_TRY(tc_forward<SPLIT>(ctx, a.Q, n, d, a.K, a.V, M, D, a.c, b, b.stats, st));
         // G2: Fhat = A V -> loss terms -> dFhat
-        FhatParams fp{n, D, a.F, a.F_dtype, a.mask, a.cfg, b.acc, b.dF, b.row, nullptr, nullptr, nullptr};
+        FhatParams fp{n, D, a.F, a.F_dtype, a.mask, a.cfg, b.acc, b.dF, b.row, nullptr, nullptr};
         LAT_TRY(tc_fhat<SPLIT>(ctx, b, n, M, D, fp, st));
         // G3: dA = dFhat V^T -> dS
         CUtensorMap mdF, mV, mdS, mK;
@@ -1460,12 +1506,10 @@ latentam_status tc_fwd(latentam_ctx* ctx, const float* Q, int64_t n, int d, cons
         e = cudaMemcpyAsync(row_stats, b.stats, sizeof(float) * 2 * n, cudaMemcpyDeviceToDevice, st);
         if (e != cudaSuccess) return cuda_error(e, "copy row statistics");
     }
-    if (F_hat) {
-        FhatParams fp{n, D, nullptr, LATENTAM_DTYPE_F32, nullptr, latentam_loss_cfg{}, b.acc, nullptr, b.row, F_hat,
-                      nullptr, nullptr};
-        LAT_TRY(tc_fhat<SPLIT>(ctx, b, n, M, D, fp, st));
-    }
-    return LATENTAM_OK;
+    if (!F_hat) return LATENTAM_OK;
+    if constexpr (!SPLIT)
+        if (fp8) return tc_fhat_out<FhatOutEpi<true>>(ctx, b, n, M, D, F_hat, st);
+    return tc_fhat_out<FhatOutEpi<false, SPLIT>>(ctx, b, n, M, D, F_hat, st);
 }
 
 }  // namespace

@@ -190,7 +190,10 @@ struct EpiCtx {
     uint32_t oplane = 0;   // split form: bytes from the hi to the lo plane of the staged output
     uint64_t* ofree = nullptr;  // split persistent form: completes when the staging buffers are free
     uint32_t ofree_phase = 0;
-    uint8_t* xstage = nullptr;  // one-tile kernel, run_x: 32 KB of free shared memory, or null
+    // one-tile kernel, run_x: 32 KB of free shared memory, or null; persistent form with
+    // Epi::WARP_STAGE: this warp's own staging bytes, stored by the warp itself to *omap
+    uint8_t* xstage = nullptr;
+    const CUtensorMap* omap = nullptr;
 
     // In-place split form (Epi::INPLACE): the tile's FP32 epilogue operand sits in the box
     // buffers as 32-column chunks (128 rows x 128 B, 128-byte swizzle, chunk c at c x 16 KB), and
@@ -804,6 +807,10 @@ __global__ void __launch_bounds__(gemm_threads(Epi::EPI_WG), Epi::MIN_BLOCKS)
 //   e_free[e]            buffer e free for tile lt's output (no operand) [u & 1]
 //   staged[e]            output of tile lt staged in buffer e          [u & 1]
 //   xbar[e]              cluster row exchange of tile lt               [u & 1]
+//
+// An epilogue with WARP_STAGE bytes per warp (a multiple of 1024) needs no box buffers: each warp
+// stages and TMA-stores its own 32 rows (EpiCtx::xstage, EpiCtx::omap) and waits for the read of
+// its last store itself.
 struct PersistGrid {
     int k_chunks;   // Epi::BK-wide K chunks per tile
     int row_tiles;  // 128-row tiles of A
@@ -828,8 +835,8 @@ __host__ __device__ constexpr int persist_threads(int epi_warpgroups) { return 9
 template <class Epi>
 __host__ __device__ constexpr size_t persist_smem_bytes() {
     return (size_t)Epi::STAGES * persist_stage_bytes<Epi>() + 2 * persist_box_bytes<Epi>() +
-           1024 /* alignment */ + 512 /* barriers */ + scratch_bytes(Epi::EPI_WG) +
-           (Epi::XROUNDS > 0 ? 2 * kXchgBytes : 0);  // one exchange buffer per accumulator
+           4 * Epi::EPI_WG * Epi::WARP_STAGE + 1024 /* alignment */ + 512 /* barriers */ +
+           scratch_bytes(Epi::EPI_WG) + (Epi::XROUNDS > 0 ? 2 * kXchgBytes : 0);  // one exchange buffer per accumulator
 }
 
 template <class Epi>
@@ -871,7 +878,8 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t* boxes = smem + PIPE_BYTES;  // [2][BOX_BYTES]
-    uint64_t* bars = reinterpret_cast<uint64_t*>(boxes + 2 * BOX_BYTES);
+    uint8_t* warp_stage = boxes + 2 * BOX_BYTES;  // [4 G][WARP_STAGE]
+    uint64_t* bars = reinterpret_cast<uint64_t*>(warp_stage + 4 * G * Epi::WARP_STAGE);
     uint64_t* full = bars;                // [STAGES]
     uint64_t* empty = full + STAGES;      // [STAGES]
     uint64_t* acc_full = empty + STAGES;  // [2]
@@ -1170,6 +1178,10 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
                 ec.ofree = &e_free[0];
                 ec.ofree_phase = (uint32_t)lt & 1u;
             }
+            if (Epi::WARP_STAGE > 0) {
+                ec.xstage = warp_stage + (warp - 3) * Epi::WARP_STAGE;
+                ec.omap = &tmO;
+            }
             int out_boxes = 0;
             if (*decision) {
                 out_boxes = Epi::run(ep, ec);  // split form: run() calls ec.wait_out() once, on every path
@@ -1191,6 +1203,7 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
                 mbar_arrive(&staged[sb]);
             }
         }
+        if (Epi::WARP_STAGE > 0) bulk_wait_read();  // each warp's last store has read its staging
     }
     __syncthreads();
     // no CTA leaves while a peer may still read or write its shared memory (the row exchange)

@@ -1,0 +1,59 @@
+"""The inference decode latentam_decode_fwd at the rims of its tiles against float64 PyTorch: ragged
+row counts (one row, a partial warp, several tiles per CTA), atoms that do not fill a 64-wide K
+chunk, one to four 256-feature column tiles, every tensor-core form.  Bars: the parity bars of the
+forms (relative 1e-4 per row for FP32; per-pixel cosine 0.999 for BF16 and 0.995 for FP8), and
+rows past the last one untouched."""
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def api():
+    from paper_2602_12314_gb300 import api as _api
+    return _api
+
+
+@pytest.fixture(scope="module")
+def ctx(api):
+    c = api.Context(0)
+    yield c
+    c.close()
+
+
+@pytest.mark.parametrize("precision", ["FP32", "BF16", "FP8"])
+@pytest.mark.parametrize("n,d,M,D", [(1, 16, 32, 128), (33, 32, 96, 384), (129, 64, 288, 640),
+                                     (45_003, 32, 160, 1024), (2_000, 32, 1024, 768)])
+def test_rows_match_float64(api, ctx, precision, n, d, M, D):
+    g = torch.Generator(device="cuda").manual_seed(n + M)
+    Q = torch.randn(n, d, generator=g, device="cuda")
+    K = torch.randn(M, d, generator=g, device="cuda") / d**0.5
+    V = torch.randn(M, D, generator=g, device="cuda") / d**0.5
+    prec = getattr(api, precision)
+    Fh, stats = api.decode_fwd(ctx, Q, K, V, precision=prec)
+    S = Q.double() @ K.double().T / d**0.5
+    want = torch.softmax(S, 1) @ V.double()
+    got = Fh.double()
+    if precision == "FP32":
+        err = ((got - want).norm(dim=1) / want.norm(dim=1)).max()
+        assert float(err) <= 1e-4
+    else:
+        cos = torch.nn.functional.cosine_similarity(got, want, dim=1).min()
+        assert float(cos) >= (0.999 if precision == "BF16" else 0.995)
+    assert torch.isfinite(stats).all()
+
+
+def test_rows_past_the_last_one_are_not_written(api, ctx):
+    import ctypes
+
+    from paper_2602_12314_gb300 import _lib as L
+    n, d, M, D = 70, 32, 64, 256
+    Q, K, V = (torch.randn(*s, device="cuda") for s in ((n, d), (M, d), (M, D)))
+    out = torch.full((128, D), 7.0, device="cuda")
+    p = lambda t: ctypes.c_void_p(t.data_ptr())  # noqa: E731
+    st = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    L.check(L.load().latentam_decode_fwd(ctx.handle, p(Q), n, d, p(K), p(V), M, D, 0.0, int(api.BF16), p(out), None,
+                                         st))
+    torch.cuda.synchronize()
+    assert bool((out[n:] == 7.0).all()) and bool((out[:n] != 7.0).any(dim=1).all())
