@@ -26,7 +26,7 @@ using namespace lat;
 namespace {
 
 constexpr int kMapThreads = 256;
-constexpr int64_t kScanChunk = 1ll << 24;  // the largest exclusive scan one call supports
+constexpr int64_t kMaxInsert = 1ll << 24;  // rows of one insertion
 
 struct Rows {  // SoA rows of Gaussians (any may be null where not used)
     float *means, *quats, *scales, *opac, *f, *m_f, *v_f;
@@ -52,11 +52,13 @@ struct latentam_map {
     int64_t loc_capacity[2];
     int cur;                  // the current local buffer
     int64_t local_count;
-    // scratch of one operation
+    int64_t fresh;            // at most this many local rows have no entry in the store yet
+    // scratch of one operation: slots and candidate flags per row, kept / selected rows per block
     int32_t* slot;
     uint32_t *flag, *pos;
     int64_t scratch_n;
-    uint32_t* total;          // device counters
+    uint32_t* total;          // device counters (2) and their pinned copy
+    uint32_t* host_total;
 };
 
 namespace {
@@ -183,12 +185,131 @@ __device__ __forceinline__ bool in_radius(const float* p, float cx, float cy, fl
     return s <= r2;
 }
 
-__device__ __forceinline__ void copy_row(const Rows& s, int64_t i, const Rows& t, int64_t j, int d) {
-    for (int k = 0; k < 3; ++k) t.means[3 * j + k] = s.means[3 * i + k];
-    for (int k = 0; k < 4; ++k) t.quats[4 * j + k] = s.quats[4 * i + k];
-    for (int k = 0; k < 3; ++k) t.scales[3 * j + k] = s.scales[3 * i + k];
-    t.opac[j] = s.opac[i];
-    for (int k = 0; k < d; ++k) t.f[(size_t)d * j + k] = s.f[(size_t)d * i + k];
+// ---- row movement ---------------------------------------------------------------------------
+//
+// A block looks at kMapThreads consecutive rows, lists the ones it moves in shared memory and copies
+// them element by element, so that neighbouring threads touch neighbouring words (a thread per
+// row left every 172- or 432-byte row to one thread's scattered words: 109 us to compact 111,000
+// local rows of d = 32, 96 MB, against 22 us).  Bound by HBM: each row read and written once.
+
+struct RowList {
+    int32_t src[kMapThreads];   // row, counted from the block's first
+    int64_t dst[kMapThreads];
+    int32_t warp[kMapThreads / 32];
+};
+
+// Lists the rows with `take` in order (every thread of the block); returns their number.  With
+// first >= 0 they go to consecutive rows from there, else each to its thread's `to`.
+__device__ __forceinline__ int list_rows(RowList& l, bool take, int64_t first, int64_t to) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t vote = __ballot_sync(0xffffffffu, take);
+    if (lane == 0) l.warp[warp] = __popc(vote);
+    __syncthreads();
+    int at = __popc(vote & ((1u << lane) - 1u)), n = 0;
+#pragma unroll
+    for (int w = 0; w < kMapThreads / 32; ++w) {
+        if (w < warp) at += l.warp[w];
+        n += l.warp[w];
+    }
+    if (take) {
+        l.src[at] = threadIdx.x;
+        l.dst[at] = first >= 0 ? first + at : to;
+    }
+    __syncthreads();
+    return n;
+}
+
+template <class T>
+__device__ __forceinline__ void move_field(const RowList& l, int n, int64_t i0, uint32_t w, const T* __restrict__ s,
+                                           T* __restrict__ t) {
+#pragma unroll 4
+    for (uint32_t e = threadIdx.x; e < (uint32_t)n * w; e += kMapThreads) {
+        const uint32_t r = e / w, k = e - r * w;
+        t[l.dst[r] * w + k] = s[(i0 + l.src[r]) * w + k];
+    }
+}
+
+enum class Moments { kNone, kCopy, kZero };
+
+// The listed rows of s (counted from i0) to t.  vec: d is a multiple of 4 and the d-wide arrays
+// are 16-byte aligned.
+template <Moments MO>
+__device__ __forceinline__ void move_rows(const RowList& l, int n, int64_t i0, const Rows& s, const Rows& t, int d,
+                                          bool vec) {
+    move_field(l, n, i0, 3, s.means, t.means);
+    move_field(l, n, i0, 4, s.quats, t.quats);
+    move_field(l, n, i0, 3, s.scales, t.scales);
+    move_field(l, n, i0, 1, s.opac, t.opac);
+    if (vec) {
+        const uint32_t w = (uint32_t)d / 4;
+        auto v4 = [](float* p) { return reinterpret_cast<float4*>(p); };
+        move_field<float4>(l, n, i0, w, v4(s.f), v4(t.f));
+        if (MO == Moments::kCopy) {
+            move_field<float4>(l, n, i0, w, v4(s.m_f), v4(t.m_f));
+            move_field<float4>(l, n, i0, w, v4(s.v_f), v4(t.v_f));
+        }
+    } else {
+        move_field(l, n, i0, (uint32_t)d, s.f, t.f);
+        if (MO == Moments::kCopy) {
+            move_field(l, n, i0, (uint32_t)d, s.m_f, t.m_f);
+            move_field(l, n, i0, (uint32_t)d, s.v_f, t.v_f);
+        }
+    }
+    if (MO == Moments::kZero)
+        for (uint32_t e = threadIdx.x; e < (uint32_t)n * d; e += kMapThreads) {
+            const uint32_t r = e / d, k = e - r * d;
+            t.m_f[l.dst[r] * d + k] = t.v_f[l.dst[r] * d + k] = 0.f;
+        }
+}
+
+bool vec_rows(int d, const Rows& s, const Rows& t) {
+    uintptr_t a = 0;
+    for (const float* p : {s.f, s.m_f, s.v_f, t.f, t.m_f, t.v_f}) a |= reinterpret_cast<uintptr_t>(p);
+    return d % 4 == 0 && (a & 15u) == 0;
+}
+
+// In-place exclusive scans of up to two lists of block counts (block b takes list b) and their
+// totals; 4096 counts at a time with a carry.
+__global__ void __launch_bounds__(1024) scan_counts(uint32_t* a, int64_t na, uint32_t* b, int64_t nb,
+                                                    uint32_t* __restrict__ total) {
+    __shared__ uint32_t s_warp[32], s_carry;
+    uint32_t* v = blockIdx.x ? b : a;
+    const int64_t n = blockIdx.x ? nb : na;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    if (t == 0) s_carry = 0;
+    __syncthreads();
+    for (int64_t base = 0; base < n; base += 4096) {
+        uint32_t x[4], sum = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int64_t i = base + 4 * t + k;
+            x[k] = i < n ? v[i] : 0u;
+            sum += x[k];
+        }
+        uint32_t incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t u = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += u;
+        }
+        if (lane == 31) s_warp[warp] = incl;
+        __syncthreads();
+        uint32_t run = s_carry + incl - sum, all = 0;
+        for (int w = 0; w < 32; ++w) {
+            if (w < warp) run += s_warp[w];
+            all += s_warp[w];
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int64_t i = base + 4 * t + k;
+            if (i < n) v[i] = run;
+            run += x[k];
+        }
+        __syncthreads();
+        if (t == 0) s_carry += all;
+        __syncthreads();
+    }
+    if (t == 0) total[blockIdx.x] = s_carry;
 }
 
 // Candidates: rows whose slot is empty (and, with gidx, that have no global entry yet) claim it.
@@ -210,94 +331,113 @@ __global__ void insert_claim(int64_t n, const float* __restrict__ means, const i
     cand[i] = c;
 }
 
-// win[i] = candidate i holds the lowest claim of its slot (written over cand).
-__global__ void insert_win(int64_t n, const int32_t* __restrict__ slot, const int32_t* __restrict__ claim,
-                           uint32_t* cand) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    if (cand[i]) cand[i] = claim[slot[i]] == (int32_t)i ? 1u : 2u;  // 1 = won, 2 = lost
+// cand[i] = 1 where candidate i holds the lowest claim of its slot, 2 where it lost; won[block] =
+// the block's winners.
+__global__ void __launch_bounds__(kMapThreads) insert_win(int64_t n, const int32_t* __restrict__ slot,
+                                                          const int32_t* __restrict__ claim, uint32_t* cand,
+                                                          uint32_t* __restrict__ won) {
+    const int64_t i = (int64_t)blockIdx.x * kMapThreads + threadIdx.x;
+    bool w = false;
+    if (i < n && cand[i]) {
+        w = claim[slot[i]] == (int32_t)i;
+        cand[i] = w ? 1u : 2u;
+    }
+    const int c = __syncthreads_count(w);
+    if (threadIdx.x == 0) won[blockIdx.x] = (uint32_t)c;
 }
 
-// Winners take index base + pos[i] and their slot; every claim is released.
-__global__ void insert_commit(int64_t n, Rows src, int d, const int32_t* __restrict__ slot,
-                              const uint32_t* __restrict__ win, const uint32_t* __restrict__ pos, int64_t base,
-                              int32_t* table, int32_t* claim, Rows dst, int32_t* __restrict__ out_index,
-                              int32_t* __restrict__ gidx_out) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const uint32_t w = win[i];
-    int32_t idx = -1;
+// Winners take the indices from base on, in input order (won: the scanned block counts), and their
+// slot; every claim is released.
+__global__ void __launch_bounds__(kMapThreads) insert_commit(int64_t n, Rows src, int d, bool vec,
+                                                             const int32_t* __restrict__ slot,
+                                                             const uint32_t* __restrict__ cand,
+                                                             const uint32_t* __restrict__ won, int64_t base,
+                                                             int32_t* table, int32_t* claim, Rows dst,
+                                                             int32_t* __restrict__ out_index,
+                                                             int32_t* __restrict__ gidx_out) {
+    __shared__ RowList l;
+    const int64_t i0 = (int64_t)blockIdx.x * kMapThreads, i = i0 + threadIdx.x;
+    const uint32_t w = i < n ? cand[i] : 0u;
     if (w) claim[slot[i]] = INT_MAX;
-    if (w == 1) {
-        idx = (int32_t)(base + pos[i]);
-        table[slot[i]] = idx;
-        copy_row(src, i, dst, idx, d);
-        if (gidx_out) gidx_out[i] = idx;
+    const int cnt = list_rows(l, w == 1, base + won[blockIdx.x], 0);
+    if (out_index && i < n && w != 1) out_index[i] = -1;
+    if ((int)threadIdx.x < cnt) {
+        const int64_t r = i0 + l.src[threadIdx.x];
+        const int32_t idx = (int32_t)l.dst[threadIdx.x];
+        table[slot[r]] = idx;
+        if (gidx_out) gidx_out[r] = idx;
+        if (out_index) out_index[r] = idx;
     }
-    if (out_index) out_index[i] = idx;
+    move_rows<Moments::kNone>(l, cnt, i0, src, dst, d, vec);
 }
 
-// flags of a 0/1 predicate: win[i] = 1 for winners only (losers 2 -> 0) before the scan.
-__global__ void winners_only(int64_t n, const uint32_t* __restrict__ cand, uint32_t* __restrict__ flag) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) flag[i] = cand[i] == 1 ? 1u : 0u;
+// Local -> Global for the rows with a store entry, and the first half of the prune: kept[block] =
+// the block's local rows inside the radius, whose store entries are marked with the epoch.
+__global__ void __launch_bounds__(kMapThreads) write_back(int64_t n, Rows local, int d, bool vec, Rows global,
+                                                          float cx, float cy, float cz, float r2,
+                                                          int32_t* __restrict__ epoch_mark, int32_t epoch,
+                                                          uint32_t* __restrict__ kept) {
+    __shared__ RowList l;
+    const int64_t i0 = (int64_t)blockIdx.x * kMapThreads, i = i0 + threadIdx.x;
+    const int32_t g = i < n ? local.gidx[i] : -1;
+    const bool k = i < n && in_radius(local.means + 3 * i, cx, cy, cz, r2);
+    if (k && g >= 0) epoch_mark[g] = epoch;
+    const int c = __syncthreads_count(k);
+    if (threadIdx.x == 0) kept[blockIdx.x] = (uint32_t)c;
+    const int cnt = list_rows(l, g >= 0, -1, g);
+    move_rows<Moments::kNone>(l, cnt, i0, local, global, d, vec);
 }
 
-__global__ void write_back_rows(int64_t n, Rows local, int d, Rows global) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int32_t g = local.gidx[i];
-    if (g >= 0) copy_row(local, i, global, g, d);
+// The kept local rows to consecutive rows of the other local buffer (kept: scanned block counts).
+__global__ void __launch_bounds__(kMapThreads) compact_local(int64_t n, Rows src, int d, bool vec, float cx, float cy,
+                                                             float cz, float r2, const uint32_t* __restrict__ kept,
+                                                             Rows dst) {
+    __shared__ RowList l;
+    const int64_t i0 = (int64_t)blockIdx.x * kMapThreads, i = i0 + threadIdx.x;
+    const bool k = i < n && in_radius(src.means + 3 * i, cx, cy, cz, r2);
+    const int cnt = list_rows(l, k, kept[blockIdx.x], 0);
+    move_rows<Moments::kCopy>(l, cnt, i0, src, dst, d, vec);
+    if ((int)threadIdx.x < cnt) dst.gidx[l.dst[threadIdx.x]] = src.gidx[i0 + l.src[threadIdx.x]];
 }
 
-__global__ void keep_flags(int64_t n, Rows local, float cx, float cy, float cz, float r2, int32_t* epoch_mark,
-                           int32_t epoch, uint32_t* __restrict__ keep) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const bool k = in_radius(local.means + 3 * i, cx, cy, cz, r2);
-    keep[i] = k ? 1u : 0u;
-    if (k && local.gidx[i] >= 0) epoch_mark[local.gidx[i]] = epoch;
+__device__ __forceinline__ bool selected(int64_t g, int64_t n, const float* means, float cx, float cy, float cz,
+                                         float r2, const int32_t* epoch_mark, int32_t epoch) {
+    return g < n && in_radius(means + 3 * g, cx, cy, cz, r2) && epoch_mark[g] != epoch;
 }
 
-__global__ void compact_local(int64_t n, Rows src, int d, const uint32_t* __restrict__ keep,
-                              const uint32_t* __restrict__ pos, Rows dst) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n || !keep[i]) return;
-    const int64_t j = pos[i];
-    copy_row(src, i, dst, j, d);
-    for (int k = 0; k < d; ++k) {
-        dst.m_f[(size_t)d * j + k] = src.m_f[(size_t)d * i + k];
-        dst.v_f[(size_t)d * j + k] = src.v_f[(size_t)d * i + k];
-    }
-    dst.gidx[j] = src.gidx[i];
+// sel[block] = the block's store rows inside the radius that are not local.
+__global__ void __launch_bounds__(kMapThreads) select_global(int64_t n, const float* __restrict__ means, float cx,
+                                                             float cy, float cz, float r2,
+                                                             const int32_t* __restrict__ epoch_mark, int32_t epoch,
+                                                             uint32_t* __restrict__ sel) {
+    const int64_t g = (int64_t)blockIdx.x * kMapThreads + threadIdx.x;
+    const int c = __syncthreads_count(selected(g, n, means, cx, cy, cz, r2, epoch_mark, epoch));
+    if (threadIdx.x == 0) sel[blockIdx.x] = (uint32_t)c;
 }
 
-__global__ void select_global(int64_t g0, int64_t n, const float* __restrict__ means, float cx, float cy, float cz,
-                              float r2, const int32_t* __restrict__ epoch_mark, int32_t epoch,
-                              uint32_t* __restrict__ sel) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int64_t g = g0 + i;
-    sel[i] = (in_radius(means + 3 * g, cx, cy, cz, r2) && epoch_mark[g] != epoch) ? 1u : 0u;
-}
-
-__global__ void append_global(int64_t g0, int64_t n, Rows global, int d, const uint32_t* __restrict__ sel,
-                              const uint32_t* __restrict__ pos, int64_t base, Rows dst) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n || !sel[i]) return;
-    const int64_t g = g0 + i, j = base + pos[i];
-    copy_row(global, g, dst, j, d);
-    for (int k = 0; k < d; ++k) dst.m_f[(size_t)d * j + k] = dst.v_f[(size_t)d * j + k] = 0.f;
-    dst.gidx[j] = (int32_t)g;
+// Those rows appended to the local buffer from row `base` on, in index order (sel: scanned block
+// counts, total: their sum).
+__global__ void __launch_bounds__(kMapThreads) append_global(int64_t n, Rows global, int d, bool vec, float cx,
+                                                             float cy, float cz, float r2,
+                                                             const int32_t* __restrict__ epoch_mark, int32_t epoch,
+                                                             const uint32_t* __restrict__ sel, uint32_t total,
+                                                             int64_t base, Rows dst) {
+    __shared__ RowList l;
+    const uint32_t first = sel[blockIdx.x];
+    if (first == (blockIdx.x + 1 < gridDim.x ? sel[blockIdx.x + 1] : total)) return;  // none of the block's rows
+    const int64_t i0 = (int64_t)blockIdx.x * kMapThreads, g = i0 + threadIdx.x;
+    const int cnt = list_rows(l, selected(g, n, global.means, cx, cy, cz, r2, epoch_mark, epoch), base + first, 0);
+    move_rows<Moments::kZero>(l, cnt, i0, global, dst, d, vec);
+    if ((int)threadIdx.x < cnt) dst.gidx[l.dst[threadIdx.x]] = (int32_t)(i0 + l.src[threadIdx.x]);
 }
 
 unsigned blocks(int64_t n) { return (unsigned)((n + kMapThreads - 1) / kMapThreads); }
 
-latentam_status read_total(latentam_map* m, cudaStream_t st, uint32_t* out) {
-    cudaError_t e = cudaMemcpyAsync(out, m->total, sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
+// The first `k` device totals (after everything enqueued on st), through pinned memory.
+latentam_status read_totals(latentam_map* m, int k, cudaStream_t st) {
+    cudaError_t e = cudaMemcpyAsync(m->host_total, m->total, sizeof(uint32_t) * k, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return cuda_error(e, "voxel map: read count");
-    return LATENTAM_OK;
+    return e == cudaSuccess ? LATENTAM_OK : cuda_error(e, "voxel map: read counts");
 }
 
 // Insert-if-free of n rows of `src` (rows with gidx >= 0 skipped when gidx is given); the
@@ -306,8 +446,8 @@ latentam_status insert_rows(latentam_ctx* ctx, latentam_map* m, int64_t n, const
                             int32_t* out_index, int64_t* n_inserted, cudaStream_t st) {
     if (n_inserted) *n_inserted = 0;
     if (n <= 0) return LATENTAM_OK;
-    if (n > kScanChunk) {
-        set_error("voxel map: at most %lld Gaussians per insertion", (long long)kScanChunk);
+    if (n > kMaxInsert) {
+        set_error("voxel map: at most %lld Gaussians per insertion", (long long)kMaxInsert);
         return LATENTAM_ERR_UNSUPPORTED_SHAPE;
     }
     LAT_TRY(grow_global(m, m->count + n));
@@ -315,17 +455,15 @@ latentam_status insert_rows(latentam_ctx* ctx, latentam_map* m, int64_t n, const
     insert_claim<<<blocks(n), kMapThreads, 0, st>>>(n, src.means, gidx, m->voxel_size, m->table_log2, m->table,
                                                     m->claim, m->slot, m->flag);
     LAT_CHECK_LAUNCH("insert_claim");
-    insert_win<<<blocks(n), kMapThreads, 0, st>>>(n, m->slot, m->claim, m->flag);
+    insert_win<<<blocks(n), kMapThreads, 0, st>>>(n, m->slot, m->claim, m->flag, m->pos);
     LAT_CHECK_LAUNCH("insert_win");
-    uint32_t* won = m->pos;  // the 0/1 winner flags, scanned in place into positions
-    winners_only<<<blocks(n), kMapThreads, 0, st>>>(n, m->flag, won);
-    LAT_CHECK_LAUNCH("winners_only");
-    LAT_TRY(scan_exclusive_u32(ctx, won, won, n, m->total, st));
-    insert_commit<<<blocks(n), kMapThreads, 0, st>>>(n, src, m->d, m->slot, m->flag, won, m->count, m->table,
-                                                     m->claim, m->g, out_index, gidx);
+    scan_counts<<<1, 1024, 0, st>>>(m->pos, blocks(n), nullptr, 0, m->total);
+    LAT_CHECK_LAUNCH("scan_counts");
+    insert_commit<<<blocks(n), kMapThreads, 0, st>>>(n, src, m->d, vec_rows(m->d, src, m->g), m->slot, m->flag, m->pos,
+                                                     m->count, m->table, m->claim, m->g, out_index, gidx);
     LAT_CHECK_LAUNCH("insert_commit");
-    uint32_t added = 0;
-    LAT_TRY(read_total(m, st, &added));
+    LAT_TRY(read_totals(m, 1, st));
+    const uint32_t added = m->host_total[0];
     m->count += added;
     if (n_inserted) *n_inserted = added;
     return LATENTAM_OK;
@@ -389,7 +527,8 @@ latentam_status latentam_map_create(latentam_ctx* ctx, int32_t d, int32_t table_
     const size_t T = (size_t)1 << table_log2;
     bool ok = cudaMalloc(&m->table, sizeof(int32_t) * T) == cudaSuccess &&
               cudaMalloc(&m->claim, sizeof(int32_t) * T) == cudaSuccess &&
-              cudaMalloc(&m->total, sizeof(uint32_t) * 2) == cudaSuccess;
+              cudaMalloc(&m->total, sizeof(uint32_t) * 2) == cudaSuccess &&
+              cudaHostAlloc(&m->host_total, sizeof(uint32_t) * 2, cudaHostAllocDefault) == cudaSuccess;
     if (ok) ok = cudaMemset(m->table, 0xff, sizeof(int32_t) * T) == cudaSuccess;  // -1
     if (ok) {
         // INT_MAX in every claim: fill through a host pattern once
@@ -428,6 +567,7 @@ latentam_status latentam_map_destroy(latentam_map* m) {
     for (void* p : {(void*)m->table, (void*)m->claim, (void*)m->epoch_mark, (void*)m->slot, (void*)m->flag,
                     (void*)m->pos, (void*)m->total})
         if (p) cudaFree(p);
+    if (m->host_total) cudaFreeHost(m->host_total);
     delete m;
     return LATENTAM_OK;
 }
@@ -472,6 +612,7 @@ latentam_status latentam_map_add_local(latentam_ctx* ctx, latentam_map* m, const
     if (e == cudaSuccess) e = cudaMemsetAsync(L.gidx + o, 0xff, sizeof(int32_t) * (size_t)n, st);  // -1
     if (e != cudaSuccess) return cuda_error(e, "voxel map: add local");
     m->local_count += n;
+    m->fresh += n;
     return LATENTAM_OK;
 }
 
@@ -485,45 +626,49 @@ latentam_status latentam_map_sync(latentam_ctx* ctx, latentam_map* m, const floa
     cudaStream_t st = (cudaStream_t)stream;
     const int d = m->d;
     const int64_t nl = m->local_count;
-    // Local -> Global: known Gaussians overwrite their entries, new ones are inserted if free
-    if (nl > 0) {
-        write_back_rows<<<blocks(nl), kMapThreads, 0, st>>>(nl, m->loc[m->cur], d, m->g);
-        LAT_CHECK_LAUNCH("write_back_rows");
-        Rows src = m->loc[m->cur];
-        LAT_TRY(insert_rows(ctx, m, nl, src, src.gidx, nullptr, nullptr, st));
-    }
-    // Global -> Local: prune, mark, select, then compact and append into the other buffer
     const float cx = centre[0], cy = centre[1], cz = centre[2];
     const float r2 = radius * radius;
+    // Local -> Global: new rows are inserted if free (only where some may have no store entry),
+    // known ones overwrite their entries; the prune's counts and marks come with the same pass
+    Rows local = m->loc[m->cur];
+    if (nl > 0 && m->fresh > 0) {
+        int64_t added = 0;
+        LAT_TRY(insert_rows(ctx, m, nl, local, local.gidx, nullptr, &added, st));
+        m->fresh -= added;
+    }
     m->epoch += 1;
-    LAT_TRY(grow_scratch(m, std::max<int64_t>(nl, std::min<int64_t>(m->count, kScanChunk))));
-    uint32_t kept = 0;
+    const int64_t nbl = blocks(nl), nbg = blocks(m->count);
+    LAT_TRY(grow_scratch(m, nbl + nbg));
+    uint32_t *kept = m->pos, *sel = m->pos + nbl;
     if (nl > 0) {
-        keep_flags<<<blocks(nl), kMapThreads, 0, st>>>(nl, m->loc[m->cur], cx, cy, cz, r2, m->epoch_mark, m->epoch,
-                                                       m->flag);
-        LAT_CHECK_LAUNCH("keep_flags");
-        LAT_TRY(scan_exclusive_u32(ctx, m->flag, m->pos, nl, m->total, st));
-        LAT_TRY(read_total(m, st, &kept));
-        const int other = m->cur ^ 1;
-        LAT_TRY(grow_local(m, other, kept, 0));
-        compact_local<<<blocks(nl), kMapThreads, 0, st>>>(nl, m->loc[m->cur], d, m->flag, m->pos, m->loc[other]);
+        write_back<<<blocks(nl), kMapThreads, 0, st>>>(nl, local, d, vec_rows(d, local, m->g), m->g, cx, cy, cz, r2,
+                                                       m->epoch_mark, m->epoch, kept);
+        LAT_CHECK_LAUNCH("write_back");
+    }
+    // Global -> Local: the store's unmarked rows inside the radius, one host read of both counts,
+    // then compact and append into the other buffer
+    if (m->count > 0) {
+        select_global<<<blocks(m->count), kMapThreads, 0, st>>>(m->count, m->g.means, cx, cy, cz, r2, m->epoch_mark,
+                                                                m->epoch, sel);
+        LAT_CHECK_LAUNCH("select_global");
+    }
+    scan_counts<<<2, 1024, 0, st>>>(kept, nbl, sel, nbg, m->total);
+    LAT_CHECK_LAUNCH("scan_counts");
+    LAT_TRY(read_totals(m, 2, st));
+    const int64_t n_kept = m->host_total[0], n_sel = m->host_total[1], n_new = n_kept + n_sel;
+    m->fresh = std::min(m->fresh, n_kept);
+    const int other = m->cur ^ 1;
+    LAT_TRY(grow_local(m, other, n_new, 0));
+    if (n_kept > 0) {
+        compact_local<<<blocks(nl), kMapThreads, 0, st>>>(nl, local, d, vec_rows(d, local, m->loc[other]), cx, cy, cz,
+                                                          r2, kept, m->loc[other]);
         LAT_CHECK_LAUNCH("compact_local");
     }
-    int64_t n_new = kept;
-    const int other = m->cur ^ 1;
-    for (int64_t g0 = 0; g0 < m->count; g0 += kScanChunk) {
-        const int64_t n = std::min<int64_t>(kScanChunk, m->count - g0);
-        select_global<<<blocks(n), kMapThreads, 0, st>>>(g0, n, m->g.means, cx, cy, cz, r2, m->epoch_mark, m->epoch,
-                                                         m->flag);
-        LAT_CHECK_LAUNCH("select_global");
-        LAT_TRY(scan_exclusive_u32(ctx, m->flag, m->pos, n, m->total, st));
-        uint32_t sel = 0;
-        LAT_TRY(read_total(m, st, &sel));
-        if (sel == 0) continue;
-        LAT_TRY(grow_local(m, other, n_new + sel, n_new));
-        append_global<<<blocks(n), kMapThreads, 0, st>>>(g0, n, m->g, d, m->flag, m->pos, n_new, m->loc[other]);
+    if (n_sel > 0) {
+        append_global<<<blocks(m->count), kMapThreads, 0, st>>>(m->count, m->g, d, vec_rows(d, m->g, m->loc[other]),
+                                                                cx, cy, cz, r2, m->epoch_mark, m->epoch, sel,
+                                                                (uint32_t)n_sel, n_kept, m->loc[other]);
         LAT_CHECK_LAUNCH("append_global");
-        n_new += sel;
     }
     m->cur = other;
     m->local_count = n_new;

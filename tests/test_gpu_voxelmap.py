@@ -115,6 +115,34 @@ def test_sync_sequence_matches_oracle(api, ctx, host_store):
     gm.close()
 
 
+@pytest.mark.parametrize("n,d", [(1, 3), (255, 4), (256, 5), (257, 12), (1300, 7)])
+def test_row_movement_at_block_rims(api, ctx, n, d):
+    """Row counts around one block, widths that are and are not whole 16-byte quads: a walk out of
+    the cloud and back (everything kept, partly kept, nothing kept, everything appended again),
+    rows added on the way that win or lose their slot."""
+    rng = np.random.default_rng(n)
+    gm = api.VoxelMap(ctx, d, table_log2=14, voxel_size=0.05, capacity=64)
+    om = vm.GlobalMap(d, 14, 0.05)
+    g0 = _gauss(rng, rng.uniform(-1, 1, size=(n, 3)), d)
+    gm.insert(*_args(g0))
+    om.insert(g0)
+    olocal = {k: [] for k in (*vm.FIELDS, "gidx")}
+    for step, x in enumerate((0.0, 0.0, 1.0, 9.0, 0.2)):
+        if step == 2:
+            new = _gauss(rng, np.concatenate([g0["means"][:3], rng.uniform(-1, 1, size=(20, 3))]), d)
+            gm.add_local(*_args(new))
+            for k in vm.FIELDS:
+                olocal[k] += [np.array(v, np.float32) for v in new[k]]
+            olocal["gidx"] += [-1] * len(new["means"])
+        loc = gm.sync([x, 0.0, 0.0], 1.2)
+        olocal = om.sync(olocal, np.asarray([x, 0, 0], np.float32), 1.2)
+        np.testing.assert_array_equal(_np(loc["gidx"]), np.array(olocal["gidx"], np.int32))
+        for k in vm.FIELDS:
+            np.testing.assert_array_equal(_np(loc[k]), np.array(olocal[k], np.float32).reshape(_np(loc[k]).shape))
+        _same_store(gm, om)
+    gm.close()
+
+
 def test_empty_map_and_zero_radius(api, ctx):
     gm = api.VoxelMap(ctx, 4, table_log2=8, voxel_size=0.1)
     loc = gm.sync([0, 0, 0], 1.0)
