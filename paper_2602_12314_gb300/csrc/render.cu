@@ -39,14 +39,41 @@ __device__ __forceinline__ float splat_alpha(float2 m, float4 q, float px, float
     return fminf(kAlphaMax, __fmul_rn(q.w, __expf(power)));
 }
 
-// a.xy += w v.xy as one packed FMA (two FP32 FMAs, each rounded as its own).
+// Two FP32 values for the packed arithmetic (each half rounded as its own).
+struct Pair {
+    uint64_t v;
+    __device__ __forceinline__ Pair() {}
+    __device__ __forceinline__ Pair(float a, float b) { asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b)); }
+    __device__ __forceinline__ explicit Pair(float a) : Pair(a, a) {}
+    __device__ __forceinline__ void get(float& a, float& b) const {
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+    }
+};
+__device__ __forceinline__ Pair fma2(Pair a, Pair b, Pair c) {
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(c.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return c;
+}
+__device__ __forceinline__ Pair mul2(Pair a, Pair b) {
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(a.v) : "l"(a.v), "l"(b.v));
+    return a;
+}
+__device__ __forceinline__ Pair add2(Pair a, Pair b) {
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(a.v) : "l"(a.v), "l"(b.v));
+    return a;
+}
+// a.xy += w v.xy
 __device__ __forceinline__ void fma2(float& a0, float& a1, float w, float v0, float v1) {
-    asm("{\n\t.reg .b64 a, w, v;\n\t"
-        "mov.b64 a, {%0, %1};\n\tmov.b64 w, {%2, %2};\n\tmov.b64 v, {%3, %4};\n\t"
-        "fma.rn.f32x2 a, w, v, a;\n\t"
-        "mov.b64 {%0, %1}, a;\n\t}"
-        : "+f"(a0), "+f"(a1)
-        : "f"(w), "f"(v0), "f"(v1));
+    fma2(Pair(w), Pair(v0, v1), Pair(a0, a1)).get(a0, a1);
+}
+
+// splat_alpha of the pixels (px, -npy.x) and (px, -npy.y): the same operations, two at a time.
+__device__ __forceinline__ void splat_alpha2(float2 m, float4 q, float px, Pair npy, float& a0, float& a1) {
+    const Pair dx(__fsub_rn(m.x, px)), dy = add2(Pair(m.y), npy);
+    float p0, p1;
+    fma2(dx, fma2(Pair(q.x), dx, mul2(Pair(q.y), dy)), mul2(mul2(Pair(q.z), dy), dy)).get(p0, p1);
+    mul2(Pair(q.w), Pair(__expf(p0), __expf(p1))).get(a0, a1);
+    a0 = p0 > 0.0f ? -1.0f : fminf(kAlphaMax, a0);
+    a1 = p1 > 0.0f ? -1.0f : fminf(kAlphaMax, a1);
 }
 
 // Pixels per thread of the forward: two (a tile is 128 threads), one at d = 64, where two pixels'
@@ -72,7 +99,8 @@ struct FwdSmem {
 // Front-to-back blend of one tile.  Bound by issue and by the shared-memory broadcasts of the staged
 // rows: a thread blends two vertically adjacent pixels, so that each row read from shared memory
 // meets two pixels' FMAs (packed two channels each) and the two transmittance chains overlap.
-// (1200 x 680, 600k Gaussians, d = 32: 174 us with one pixel per thread, 157 with two.)
+// The pixels' exponents and transmittances are taken with packed arithmetic, two pixels an
+// instruction.  (1200 x 680, 600k Gaussians, d = 32: 186 us with one pixel per thread, 151 with two.)
 template <int DQ>
 __device__ __forceinline__ void render_fwd_tile(const TileJob& job, FwdSmem<DQ>& sm) {
     constexpr int DV = DQ / 4, PX = fwd_px<DQ>(), NT = fwd_threads<DQ>();
@@ -81,6 +109,7 @@ __device__ __forceinline__ void render_fwd_tile(const TileJob& job, FwdSmem<DQ>&
     const int t = threadIdx.x;
     const int px = tx * kTile + t % kTile, py = ty * kTile + t / kTile * PX;
     const float fpx = (float)px;
+    const Pair npy(-(float)py, -(float)(py + 1));
     const int2 range = job.ranges[tile];
     float4 acc[PX][DV];
     float T[PX];
@@ -110,18 +139,26 @@ __device__ __forceinline__ void render_fwd_tile(const TileJob& job, FwdSmem<DQ>&
         for (int j = 0; j < cnt && !out; ++j) {
             const float2 m = sm.xy[j];
             const float4 q = sm.co[j];
-            float w[PX];
+            float w[PX], alphas[PX], left[PX];
             bool use[PX], any = false;
+            if (PX == 2) {
+                splat_alpha2(m, q, fpx, npy, alphas[0], alphas[PX - 1]);
+                const Pair t2(T[0], T[PX - 1]), a2(alphas[0], alphas[PX - 1]);
+                mul2(t2, add2(Pair(1.0f), Pair(-alphas[0], -alphas[PX - 1]))).get(left[0], left[PX - 1]);
+                mul2(a2, t2).get(w[0], w[PX - 1]);
+            } else {
+                alphas[0] = splat_alpha(m, q, fpx, (float)py);
+                left[0] = __fmul_rn(T[0], __fsub_rn(1.0f, alphas[0]));
+                w[0] = __fmul_rn(alphas[0], T[0]);
+            }
 #pragma unroll
             for (int i = 0; i < PX; ++i) {
-                const float alpha = splat_alpha(m, q, fpx, (float)(py + i));
-                const float test_T = __fmul_rn(T[i], __fsub_rn(1.0f, alpha));
+                const float alpha = alphas[i], test_T = left[i];
                 use[i] = !done[i] && !(alpha < kAlphaMin);
                 if (use[i] && test_T < kTMin) {
                     done[i] = true;
                     use[i] = false;
                 }
-                w[i] = __fmul_rn(alpha, T[i]);
                 if (use[i]) {
                     T[i] = test_T;
                     ++count[i];
@@ -155,7 +192,7 @@ __device__ __forceinline__ void render_fwd_tile(const TileJob& job, FwdSmem<DQ>&
 }
 
 template <int DQ>
-__global__ void __launch_bounds__(fwd_threads<DQ>()) render_fwd_kernel(CamParams cam, const int2* __restrict__ ranges,
+__global__ void __launch_bounds__(fwd_threads<DQ>(), 1) render_fwd_kernel(CamParams cam, const int2* __restrict__ ranges,
                                                                        const int32_t* __restrict__ pair_ids,
                                                                        const float2* __restrict__ xy,
                                                                        const float4* __restrict__ conic_opac,
@@ -182,9 +219,12 @@ __device__ __forceinline__ int next_item(int* counter, const int32_t* order, int
     return it < total ? order[it] : -1;
 }
 
-// Persistent render forward over every tile of every frame of a batch, longest lists first.
+// Persistent render forward over every tile of every frame of a batch, longest lists first.  (At
+// d = 32 held to five blocks per SM: over six 640 x 480 frames 475 us a launch against 492 at the
+// four that its registers would allow; the single frame above is shorter with four, 57 against
+// 70 us at 640 x 480, where the last tiles' own length counts.)
 template <int DQ>
-__global__ void __launch_bounds__(fwd_threads<DQ>()) render_fwd_batch_kernel(const __grid_constant__ BatchJobs jobs,
+__global__ void __launch_bounds__(fwd_threads<DQ>(), DQ == 32 ? 5 : 1) render_fwd_batch_kernel(const __grid_constant__ BatchJobs jobs,
                                                                              const int32_t* __restrict__ order,
                                                                              int total, int* __restrict__ counter) {
     __shared__ FwdSmem<DQ> sm;
