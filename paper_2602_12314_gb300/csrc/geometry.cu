@@ -32,165 +32,161 @@ __device__ __forceinline__ double block_sum_d(double v, double* red) {
     return s;
 }
 
-// Horizontal pass of the five moments of each channel: out[(k * 3 + ch) * n + p], k = x, y,
-// x^2, y^2, x y.  x = rendered image, y = observed image (both n x 3 interleaved).
-__global__ void ssim_moments_h(const float* __restrict__ X, const float* __restrict__ Y, int W, int H,
-                               float* __restrict__ out) {
-    const int64_t n = (int64_t)W * H;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= 3 * n) return;
-    const int ch = (int)(i / n);
-    const int64_t p = i % n;
-    const int py = (int)(p / W), px = (int)(p % W);
-    float s[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-    for (int k = -kHalf; k <= kHalf; ++k) {
-        const int x = px + k;
-        if (x < 0 || x >= W) continue;
-        const int64_t q = (int64_t)py * W + x;
-        const float a = X[3 * q + ch], b = Y[3 * q + ch], w = c_win[k + kHalf];
-        s[0] += w * a;
-        s[1] += w * b;
-        s[2] += w * a * a;
-        s[3] += w * b * b;
-        s[4] += w * a * b;
-    }
-#pragma unroll
-    for (int k = 0; k < 5; ++k) out[((int64_t)k * 3 + ch) * n + p] = s[k];
-}
+// Both blurs run on kTW x kTH output tiles with the halo in shared memory: a horizontal pass into
+// shared memory, then a vertical one.  Bound by shared-memory reads and issue; the images and the
+// partial planes between the two kernels stay in L2.  (As four passes over global planes, with the
+// depth loss and the totals in three more launches: 115 us at 640 x 480; these two take 53.)
+constexpr int kTW = 32, kTH = 16;                             // output tile
+constexpr int kIW = kTW + 2 * kHalf, kIH = kTH + 2 * kHalf;  // with its halo
+constexpr int kImgThreads = 256;
+constexpr int kPerThread = kTW * kTH / kImgThreads;
 
-// Vertical pass, the SSIM map and the partial derivatives ds/dm_x, ds/de_xx, ds/de_xy
-// (written to dpart[(k * 3 + ch) * n + p]); acc[1] += sum of SSIM values.
-__global__ void __launch_bounds__(256) ssim_map_v(const float* __restrict__ hm, int W, int H,
-                                                  float* __restrict__ dpart, double* __restrict__ acc) {
-    __shared__ double red[8];
+// sums[0..3] += |x - y| over the tile, SSIM, |Z_hat - Z| over the pixels with depth, their number.
+// dpart[(k * 3 + ch) * n + p] = ds/dm_x, ds/de_xx, ds/de_xy of each channel (x = rendered, y =
+// observed image, both n x 3 interleaved).
+__global__ void __launch_bounds__(kImgThreads) image_terms(const float* __restrict__ X, const float* __restrict__ Y,
+                                                           const float* __restrict__ Zh,
+                                                           const float* __restrict__ Zo, int W, int H,
+                                                           float* __restrict__ dpart, double* __restrict__ sums) {
+    __shared__ float s_x[kIH][kIW], s_y[kIH][kIW];
+    __shared__ float s_h[5][kIH][kTW];
+    __shared__ double red[kImgThreads / 32];
     const int64_t n = (int64_t)W * H;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    double ssim = 0.0;
-    if (i < 3 * n) {
-        const int ch = (int)(i / n);
-        const int64_t p = i % n;
-        const int py = (int)(p / W), px = (int)(p % W);
-        float m[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-        for (int k = -kHalf; k <= kHalf; ++k) {
-            const int y = py + k;
-            if (y < 0 || y >= H) continue;
-            const int64_t q = (int64_t)y * W + px;
-            const float w = c_win[k + kHalf];
-#pragma unroll
-            for (int j = 0; j < 5; ++j) m[j] += w * hm[((int64_t)j * 3 + ch) * n + q];
+    const int x0 = blockIdx.x * kTW, y0 = blockIdx.y * kTH, t = threadIdx.x;
+    double l1 = 0.0, ssim = 0.0, dz = 0.0, cz = 0.0;
+    for (int ch = 0; ch < 3; ++ch) {
+        __syncthreads();
+        for (int i = t; i < kIH * kIW; i += kImgThreads) {
+            const int r = i / kIW, c = i % kIW, gy = y0 + r - kHalf, gx = x0 + c - kHalf;
+            const bool in = gy >= 0 && gy < H && gx >= 0 && gx < W;
+            const int64_t q = 3 * ((int64_t)gy * W + gx) + ch;
+            s_x[r][c] = in ? X[q] : 0.f;
+            s_y[r][c] = in ? Y[q] : 0.f;
         }
-        const float mx = m[0], my = m[1];
-        const float sxx = m[2] - mx * mx, syy = m[3] - my * my, sxy = m[4] - mx * my;
-        const float A1 = 2.0f * mx * my + kC1, A2 = 2.0f * sxy + kC2;
-        const float B1 = mx * mx + my * my + kC1, B2 = sxx + syy + kC2;
-        const float s = (A1 * A2) / (B1 * B2);
-        ssim = s;
-        // s as a function of m_x, e_xx, e_xy (with sxx = e_xx - m_x^2, sxy = e_xy - m_x m_y)
-        const float ds_dmx = (2.0f * my * A2 - 2.0f * my * A1) / (B1 * B2) - s * (2.0f * mx / B1 - 2.0f * mx / B2);
-        const float ds_dexx = -s / B2;
-        const float ds_dexy = 2.0f * A1 / (B1 * B2);
-        dpart[((int64_t)0 * 3 + ch) * n + p] = ds_dmx;
-        dpart[((int64_t)1 * 3 + ch) * n + p] = ds_dexx;
-        dpart[((int64_t)2 * 3 + ch) * n + p] = ds_dexy;
-    }
-    const double b = block_sum_d(ssim, red);
-    if (threadIdx.x == 0) atomicAdd(&acc[1], b);
-}
-
-// Horizontal blur of the three partial-derivative maps.
-__global__ void ssim_partials_h(const float* __restrict__ dpart, int W, int H, float* __restrict__ out) {
-    const int64_t n = (int64_t)W * H;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= 9 * n) return;
-    const int64_t plane = i / n, p = i % n;
-    const int py = (int)(p / W), px = (int)(p % W);
-    float s = 0.f;
-    for (int k = -kHalf; k <= kHalf; ++k) {
-        const int x = px + k;
-        if (x < 0 || x >= W) continue;
-        s += c_win[k + kHalf] * dpart[plane * n + (int64_t)py * W + x];
-    }
-    out[i] = s;
-}
-
-// Vertical blur of the partials and the image gradient dC = lambda_rgb (lambda_I1 dL1 +
-// lambda_I2 dL_ssim); acc[0] += sum |x - y|.
-__global__ void __launch_bounds__(256) rgb_grad(const float* __restrict__ X, const float* __restrict__ Y,
-                                                const float* __restrict__ hpart, int W, int H,
-                                                latentam_image_cfg cfg, float* __restrict__ dC,
-                                                double* __restrict__ acc) {
-    __shared__ double red[8];
-    const int64_t n = (int64_t)W * H;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    double l1 = 0.0;
-    if (i < 3 * n) {
-        const int ch = (int)(i / n);
-        const int64_t p = i % n;
-        const int py = (int)(p / W), px = (int)(p % W);
-        float b[3] = {0.f, 0.f, 0.f};
-        for (int k = -kHalf; k <= kHalf; ++k) {
-            const int y = py + k;
-            if (y < 0 || y >= H) continue;
-            const float w = c_win[k + kHalf];
-            const int64_t q = (int64_t)y * W + px;
+        __syncthreads();
+        for (int i = t; i < kIH * kTW; i += kImgThreads) {
+            const int r = i / kTW, c = i % kTW;
+            float m[5] = {0.f, 0.f, 0.f, 0.f, 0.f};  // x, y, x^2, y^2, x y
 #pragma unroll
-            for (int j = 0; j < 3; ++j) b[j] += w * hpart[((int64_t)j * 3 + ch) * n + q];
+            for (int k = 0; k < kWin; ++k) {
+                const float a = s_x[r][c + k], b = s_y[r][c + k], w = c_win[k];
+                m[0] += w * a;
+                m[1] += w * b;
+                m[2] += w * a * a;
+                m[3] += w * b * b;
+                m[4] += w * a * b;
+            }
+#pragma unroll
+            for (int j = 0; j < 5; ++j) s_h[j][r][c] = m[j];
         }
-        const float x = X[3 * p + ch], y = Y[3 * p + ch];
-        const float inv = 1.0f / (3.0f * (float)n);
-        const float d_ssim = -inv * (b[0] + 2.0f * x * b[1] + y * b[2]);
-        const float diff = x - y;
-        const float d_l1 = inv * (diff > 0.f ? 1.f : (diff < 0.f ? -1.f : 0.f));
-        l1 = fabs((double)diff);
-        dC[3 * p + ch] = cfg.lambda_rgb * (cfg.lambda_I1 * d_l1 + cfg.lambda_I2 * d_ssim);
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < kPerThread; ++u) {
+            const int r = t / kTW + u * (kImgThreads / kTW), c = t % kTW;
+            if (x0 + c >= W || y0 + r >= H) continue;
+            const int64_t p = (int64_t)(y0 + r) * W + x0 + c;
+            float m[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int k = 0; k < kWin; ++k)
+#pragma unroll
+                for (int j = 0; j < 5; ++j) m[j] += c_win[k] * s_h[j][r + k][c];
+            const float mx = m[0], my = m[1];
+            const float sxx = m[2] - mx * mx, syy = m[3] - my * my, sxy = m[4] - mx * my;
+            const float A1 = 2.0f * mx * my + kC1, A2 = 2.0f * sxy + kC2;
+            const float B1 = mx * mx + my * my + kC1, B2 = sxx + syy + kC2;
+            const float s = (A1 * A2) / (B1 * B2);
+            // s as a function of m_x, e_xx, e_xy (with sxx = e_xx - m_x^2, sxy = e_xy - m_x m_y)
+            dpart[((int64_t)0 * 3 + ch) * n + p] =
+                (2.0f * my * A2 - 2.0f * my * A1) / (B1 * B2) - s * (2.0f * mx / B1 - 2.0f * mx / B2);
+            dpart[((int64_t)1 * 3 + ch) * n + p] = -s / B2;
+            dpart[((int64_t)2 * 3 + ch) * n + p] = 2.0f * A1 / (B1 * B2);
+            ssim += s;
+            l1 += fabs((double)(s_x[r + kHalf][c + kHalf] - s_y[r + kHalf][c + kHalf]));
+            if (ch == 0 && Zo[p] > 0.f) {
+                dz += fabs((double)Zh[p] - (double)Zo[p]);
+                cz += 1.0;
+            }
+        }
     }
-    const double s = block_sum_d(l1, red);
-    if (threadIdx.x == 0) atomicAdd(&acc[0], s);
+    const double v[4] = {l1, ssim, dz, cz};
+    for (int k = 0; k < 4; ++k) {
+        const double b = block_sum_d(v[k], red);
+        if (t == 0) atomicAdd(&sums[k], b);
+    }
 }
 
-// acc[2] += sum over valid pixels of |Z_hat - Z|, acc[3] += their count.
-__global__ void __launch_bounds__(256) depth_sums(const float* __restrict__ Zh, const float* __restrict__ Zo,
-                                                  int64_t n, double* __restrict__ acc) {
-    __shared__ double red[8];
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    double e = 0.0, c = 0.0;
-    if (p < n && Zo[p] > 0.f) {
-        e = fabs((double)Zh[p] - (double)Zo[p]);
-        c = 1.0;
+// The image gradients dC = lambda_rgb (lambda_I1 dL1 + lambda_I2 dL_ssim), with the blur of the
+// partial planes, and dZ; one thread writes the loss parts: [5] L1, [6] 1 - mean SSIM, [7] L_d, [8]
+// pixels with depth, [9] the total of Eq. full_obj (parts[3] holds lambda_f L_f).
+__global__ void __launch_bounds__(kImgThreads) image_grads(const float* __restrict__ X, const float* __restrict__ Y,
+                                                           const float* __restrict__ Zh,
+                                                           const float* __restrict__ Zo,
+                                                           const float* __restrict__ dpart, int W, int H,
+                                                           latentam_image_cfg cfg, const double* __restrict__ sums,
+                                                           float* __restrict__ dC, float* __restrict__ dZ,
+                                                           double* __restrict__ parts) {
+    __shared__ float s_in[3][kIH][kIW];
+    __shared__ float s_h[3][kIH][kTW];
+    const int64_t n = (int64_t)W * H;
+    const int x0 = blockIdx.x * kTW, y0 = blockIdx.y * kTH, t = threadIdx.x;
+    const double n_depth = sums[3];
+    if (blockIdx.x == 0 && blockIdx.y == 0 && t == 0) {
+        const double N3 = 3.0 * (double)n;
+        const double l1 = sums[0] / N3, ls = 1.0 - sums[1] / N3, ld = n_depth > 0.0 ? sums[2] / n_depth : 0.0;
+        parts[5] = l1;
+        parts[6] = ls;
+        parts[7] = ld;
+        parts[8] = n_depth;
+        parts[9] = (double)cfg.lambda_rgb * ((double)cfg.lambda_I1 * l1 + (double)cfg.lambda_I2 * ls) +
+                   (double)cfg.lambda_d * ld + parts[3];
     }
-    const double se = block_sum_d(e, red);
-    const double sc = block_sum_d(c, red);
-    if (threadIdx.x == 0) {
-        atomicAdd(&acc[2], se);
-        atomicAdd(&acc[3], sc);
+    for (int ch = 0; ch < 3; ++ch) {
+        __syncthreads();
+        for (int i = t; i < kIH * kIW; i += kImgThreads) {
+            const int r = i / kIW, c = i % kIW, gy = y0 + r - kHalf, gx = x0 + c - kHalf;
+            const bool in = gy >= 0 && gy < H && gx >= 0 && gx < W;
+            const int64_t q = (int64_t)gy * W + gx;
+#pragma unroll
+            for (int j = 0; j < 3; ++j) s_in[j][r][c] = in ? dpart[((int64_t)j * 3 + ch) * n + q] : 0.f;
+        }
+        __syncthreads();
+        for (int i = t; i < kIH * kTW; i += kImgThreads) {
+            const int r = i / kTW, c = i % kTW;
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                float h = 0.f;
+#pragma unroll
+                for (int k = 0; k < kWin; ++k) h += c_win[k] * s_in[j][r][c + k];
+                s_h[j][r][c] = h;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < kPerThread; ++u) {
+            const int r = t / kTW + u * (kImgThreads / kTW), c = t % kTW;
+            if (x0 + c >= W || y0 + r >= H) continue;
+            const int64_t p = (int64_t)(y0 + r) * W + x0 + c;
+            float b[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+            for (int k = 0; k < kWin; ++k)
+#pragma unroll
+                for (int j = 0; j < 3; ++j) b[j] += c_win[k] * s_h[j][r + k][c];
+            const float x = X[3 * p + ch], y = Y[3 * p + ch];
+            const float inv = 1.0f / (3.0f * (float)n);
+            const float d_ssim = -inv * (b[0] + 2.0f * x * b[1] + y * b[2]);
+            const float diff = x - y;
+            const float d_l1 = inv * (diff > 0.f ? 1.f : (diff < 0.f ? -1.f : 0.f));
+            dC[3 * p + ch] = cfg.lambda_rgb * (cfg.lambda_I1 * d_l1 + cfg.lambda_I2 * d_ssim);
+            if (ch == 0) {
+                float g = 0.f;
+                if (Zo[p] > 0.f && n_depth > 0.0) {
+                    const float e = Zh[p] - Zo[p];
+                    g = cfg.lambda_d * (e > 0.f ? 1.f : (e < 0.f ? -1.f : 0.f)) / (float)n_depth;
+                }
+                dZ[p] = g;
+            }
+        }
     }
-}
-
-__global__ void depth_grad(const float* __restrict__ Zh, const float* __restrict__ Zo, int64_t n,
-                           latentam_image_cfg cfg, const double* __restrict__ acc, float* __restrict__ dZ) {
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    float g = 0.f;
-    if (Zo[p] > 0.f && acc[3] > 0.0) {
-        const float diff = Zh[p] - Zo[p];
-        g = cfg.lambda_d * (diff > 0.f ? 1.f : (diff < 0.f ? -1.f : 0.f)) / (float)acc[3];
-    }
-    dZ[p] = g;
-}
-
-// parts[5] L1, [6] 1 - mean SSIM, [7] L_d, [8] pixels with depth, [9] the total of Eq. full_obj.
-__global__ void finalize_full(const double* __restrict__ acc, int64_t n, latentam_image_cfg cfg,
-                              double* __restrict__ parts) {
-    const double N3 = 3.0 * (double)n;
-    const double l1 = n > 0 ? acc[0] / N3 : 0.0;
-    const double ls = n > 0 ? 1.0 - acc[1] / N3 : 0.0;
-    const double ld = acc[3] > 0.0 ? acc[2] / acc[3] : 0.0;
-    parts[5] = l1;
-    parts[6] = ls;
-    parts[7] = ld;
-    parts[8] = acc[3];
-    parts[9] = (double)cfg.lambda_rgb * ((double)cfg.lambda_I1 * l1 + (double)cfg.lambda_I2 * ls) +
-               (double)cfg.lambda_d * ld + parts[3];
 }
 
 // ---- projection backward ------------------------------------------------------------------
@@ -335,30 +331,17 @@ latentam_status launch_image_loss(latentam_ctx* ctx, const float* C, const float
     }
     auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
     const size_t nn = (size_t)std::max<int64_t>(n, 1);
-    char* base = static_cast<char*>(ws(ctx, WS_FULL_AUX, up(sizeof(float) * 15 * nn) + up(sizeof(float) * 9 * nn) +
-                                                             up(sizeof(double) * 4)));
+    char* base = static_cast<char*>(ws(ctx, WS_FULL_AUX, up(sizeof(float) * 9 * nn) + up(sizeof(double) * 4)));
     if (!base) return LATENTAM_ERR_OUT_OF_MEMORY;
-    float* hm = reinterpret_cast<float*>(base);          // 15 planes, then the 9 blurred partial planes
-    float* dpart = reinterpret_cast<float*>(base + up(sizeof(float) * 15 * nn));
-    double* acc = reinterpret_cast<double*>(base + up(sizeof(float) * 15 * nn) + up(sizeof(float) * 9 * nn));
-    cudaError_t e = cudaMemsetAsync(acc, 0, sizeof(double) * 4, st);
+    float* dpart = reinterpret_cast<float*>(base);
+    double* sums = reinterpret_cast<double*>(base + up(sizeof(float) * 9 * nn));
+    cudaError_t e = cudaMemsetAsync(sums, 0, sizeof(double) * 4, st);
     if (e != cudaSuccess) return cuda_error(e, "memset image loss");
-    if (n > 0) {
-        ssim_moments_h<<<nblk(3 * n), 256, 0, st>>>(C, image, W, H, hm);
-        LAT_CHECK_LAUNCH("ssim_moments_h");
-        ssim_map_v<<<nblk(3 * n), 256, 0, st>>>(hm, W, H, dpart, acc);
-        LAT_CHECK_LAUNCH("ssim_map_v");
-        ssim_partials_h<<<nblk(9 * n), 256, 0, st>>>(dpart, W, H, hm);
-        LAT_CHECK_LAUNCH("ssim_partials_h");
-        rgb_grad<<<nblk(3 * n), 256, 0, st>>>(C, image, hm, W, H, cfg, dC, acc);
-        LAT_CHECK_LAUNCH("rgb_grad");
-        depth_sums<<<nblk(n), 256, 0, st>>>(Z, depth_obs, n, acc);
-        LAT_CHECK_LAUNCH("depth_sums");
-        depth_grad<<<nblk(n), 256, 0, st>>>(Z, depth_obs, n, cfg, acc, dZ);
-        LAT_CHECK_LAUNCH("depth_grad");
-    }
-    finalize_full<<<1, 1, 0, st>>>(acc, n, cfg, parts);
-    LAT_CHECK_LAUNCH("finalize_full");
+    const dim3 grid((unsigned)((W + kTW - 1) / kTW), (unsigned)((H + kTH - 1) / kTH));
+    image_terms<<<grid, kImgThreads, 0, st>>>(C, image, Z, depth_obs, W, H, dpart, sums);
+    LAT_CHECK_LAUNCH("image_terms");
+    image_grads<<<grid, kImgThreads, 0, st>>>(C, image, Z, depth_obs, dpart, W, H, cfg, sums, dC, dZ, parts);
+    LAT_CHECK_LAUNCH("image_grads");
     return LATENTAM_OK;
 }
 

@@ -89,11 +89,21 @@ constexpr int fwd_threads() {
 
 constexpr int kBatch = 128;  // Gaussians staged per round
 
-template <int DQ>
+template <int DQ, bool FULL = false>
 struct FwdSmem {
     float2 xy[kBatch];
     float4 co[kBatch];
     float4 f[kBatch][DQ / 4];
+    float4 cz[FULL ? kBatch : 1];  // colour, depth
+};
+
+// The further channels of the full Stage I render: colours (N x 3) and camera depths (N) blended
+// with the queries' weights into C (n x 3) and Z.
+struct FullImages {
+    const float* colours;
+    const float* depth;
+    float* C;
+    float* Z;
 };
 
 // Front-to-back blend of one tile.  Bound by issue and by the shared-memory broadcasts of the staged
@@ -101,8 +111,8 @@ struct FwdSmem {
 // meets two pixels' FMAs (packed two channels each) and the two transmittance chains overlap.
 // The pixels' exponents and transmittances are taken with packed arithmetic, two pixels an
 // instruction.  (1200 x 680, 600k Gaussians, d = 32: 186 us with one pixel per thread, 151 with two.)
-template <int DQ>
-__device__ __forceinline__ void render_fwd_tile(const TileJob& job, FwdSmem<DQ>& sm) {
+template <int DQ, bool FULL = false>
+__device__ __forceinline__ void render_fwd_tile(const TileJob& job, FwdSmem<DQ, FULL>& sm, const FullImages& full = {}) {
     constexpr int DV = DQ / 4, PX = fwd_px<DQ>(), NT = fwd_threads<DQ>();
     const int tile = job.tile;
     const int tx = tile % job.tiles_x, ty = tile / job.tiles_x;
@@ -111,7 +121,7 @@ __device__ __forceinline__ void render_fwd_tile(const TileJob& job, FwdSmem<DQ>&
     const float fpx = (float)px;
     const Pair npy(-(float)py, -(float)(py + 1));
     const int2 range = job.ranges[tile];
-    float4 acc[PX][DV];
+    float4 acc[PX][DV], acz[PX];
     float T[PX];
     int count[PX];
     bool done[PX], out = true;
@@ -119,6 +129,7 @@ __device__ __forceinline__ void render_fwd_tile(const TileJob& job, FwdSmem<DQ>&
     for (int i = 0; i < PX; ++i) {
 #pragma unroll
         for (int k = 0; k < DV; ++k) acc[i][k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        acz[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         T[i] = 1.0f;
         count[i] = 0;
         done[i] = !(px < job.W && py + i < job.H);
@@ -133,6 +144,9 @@ __device__ __forceinline__ void render_fwd_tile(const TileJob& job, FwdSmem<DQ>&
             sm.co[t] = stage_splat(job.conic_opac[g]);
 #pragma unroll
             for (int c = 0; c < DV; ++c) sm.f[t][c] = job.f[(size_t)g * DV + c];
+            if (FULL)
+                sm.cz[t] = make_float4(full.colours[3 * (size_t)g], full.colours[3 * (size_t)g + 1],
+                                       full.colours[3 * (size_t)g + 2], full.depth[g]);
         }
         __syncthreads();
         const int cnt = min(kBatch, range.y - start);
@@ -176,6 +190,15 @@ __device__ __forceinline__ void render_fwd_tile(const TileJob& job, FwdSmem<DQ>&
                             fma2(acc[i][c].z, acc[i][c].w, w[i], v.z, v.w);
                         }
                 }
+                if (FULL) {
+                    const float4 v = sm.cz[j];
+#pragma unroll
+                    for (int i = 0; i < PX; ++i)
+                        if (use[i]) {
+                            fma2(acz[i].x, acz[i].y, w[i], v.x, v.y);
+                            fma2(acz[i].z, acz[i].w, w[i], v.z, v.w);
+                        }
+                }
             }
             out = done[0] && done[PX - 1];
         }
@@ -186,6 +209,12 @@ __device__ __forceinline__ void render_fwd_tile(const TileJob& job, FwdSmem<DQ>&
             const size_t p = (size_t)(py + i) * job.W + px;
 #pragma unroll
             for (int c = 0; c < DV; ++c) job.Q[p * DV + c] = acc[i][c];
+            if (FULL) {
+                full.C[3 * p] = acz[i].x;
+                full.C[3 * p + 1] = acz[i].y;
+                full.C[3 * p + 2] = acz[i].z;
+                full.Z[p] = acz[i].w;
+            }
             job.T_final[p] = T[i];
             job.n_contrib[p] = count[i];
         }
@@ -233,22 +262,6 @@ __global__ void __launch_bounds__(fwd_threads<DQ>(), DQ == 32 ? 5 : 1) render_fw
         job.tile = item & 0xFFFFF;
         render_fwd_tile<DQ>(job, sm);
     }
-}
-
-// Reduce-scatter of 32 per-lane channels over the warp: lane l ends with the warp-wide
-// sum of channel l (31 shuffles instead of 32 x 5).
-__device__ __forceinline__ float warp_reduce_scatter32(float (&v)[32], int lane) {
-#pragma unroll
-    for (int half = 16; half >= 1; half >>= 1) {
-        const bool upper = (lane & half) != 0;
-#pragma unroll
-        for (int i = 0; i < half; ++i) {
-            const float send = upper ? v[i] : v[i + half];
-            const float keep = upper ? v[i + half] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, half);
-        }
-    }
-    return v[0];
 }
 
 // Backward of the query blend, df_i = sum_p w_ip dQ_p, as one small GEMM per strip (16 x 4 pixels) and
@@ -520,218 +533,279 @@ __global__ void __launch_bounds__(32 * kBwdWarps) render_bwd_batch_kernel(const 
 // passes dL/dalpha to o (e^power) and to power (alpha) unless it is clamped, and power to the
 // screen mean and the conic.
 
-constexpr int kBatchFull = 128;  // Gaussians staged per round (f rows, colour + depth, geometry)
-
 template <int DQ>
-__global__ void __launch_bounds__(kTilePixels) render_fwd_full_kernel(
+__global__ void __launch_bounds__(fwd_threads<DQ>(), 1) render_fwd_full_kernel(
     CamParams cam, const int2* __restrict__ ranges, const int32_t* __restrict__ pair_ids,
     const float2* __restrict__ xy, const float4* __restrict__ conic_opac, const float4* __restrict__ f,
-    const float* __restrict__ colours, const float* __restrict__ depth, float4* __restrict__ Q,
-    float* __restrict__ C, float* __restrict__ Z, float* __restrict__ T_final, int32_t* __restrict__ n_contrib) {
-    constexpr int DV = DQ / 4;
-    __shared__ float2 s_xy[kBatchFull];
-    __shared__ float4 s_co[kBatchFull];
-    __shared__ float4 s_cz[kBatchFull];
-    __shared__ float4 s_f[kBatchFull][DV];
+    float4* __restrict__ Q, FullImages full, float* __restrict__ T_final, int32_t* __restrict__ n_contrib) {
+    __shared__ FwdSmem<DQ, true> sm;
     const int tile = cam.tile_order ? cam.tile_order[blockIdx.x] : (int)blockIdx.x;
-    const int tx = tile % cam.tiles_x, ty = tile / cam.tiles_x;
-    const int t = threadIdx.x;
-    const int px = tx * kTile + (t % kTile), py = ty * kTile + (t / kTile);
-    const bool inside = px < cam.W && py < cam.H;
-    const float fpx = (float)px, fpy = (float)py;
-    const int2 range = ranges[tile];
-    float4 acc[DV];
+    const TileJob job{tile, cam.tiles_x, cam.W, cam.H, ranges, pair_ids, xy, conic_opac, f, Q, T_final, n_contrib,
+                      nullptr, nullptr};
+    render_fwd_tile<DQ, true>(job, sm, full);
+}
+
+// Backward of the full blend, a warp per strip as above but in FP32 throughout (the geometry terms
+// need <G, x_i>, a dot product over all channels, for every pixel and splat).  Per batch of 16
+// Gaussians: (1) each lane takes its own pixels front to back from the strip's dQ rows in its
+// registers: weight, <G, x_j>, dL/dalpha; the six geometry terms of its pixels are added over the
+// warp by a reduce-scatter and leave with one atomic per term; the weights go to shared memory;
+// (2) with lane = channel, the strip's dQ column in registers and the weights read as broadcasts,
+// df_j[lane] = sum_p w_jp dQ_p[lane] leaves as one 128-byte atomic per Gaussian.  Reading the
+// weights back instead of reducing 32 products over the warp takes 48 instructions where the 31
+// shuffles with their selects took about 190.  Bound by issue.
+// (640 x 480, 300k Gaussians, d = 32: 226 us with a block per tile and two warp reductions per
+// Gaussian, 190-204 with the warp per strip.)
+constexpr int kFullBatch = 16;
+
+template <int DQ>
+constexpr int full_px() {  // pixels per lane (two at d = 32 take 220 registers: 8 warps per SM, 235 us
+                            // against 190-204 at 640 x 480)
+    return DQ <= 16 ? 2 : 1;
+}
+
+template <int DQ>
+struct FullSmem {
+    float w[kFullBatch][32 * full_px<DQ>() + 4];
+    float4 f[kFullBatch][DQ / 4];
+    float4 cz[kFullBatch];
+    float4 co[kFullBatch];
+    float2 xy[kFullBatch];
+    int id[kFullBatch];
+};
+
+struct FullGrads {
+    const float* Q;   // rendered images and their gradients
+    const float* C;
+    const float* Z;
+    const float* dC;
+    const float* dZ;
+    float* dcol;      // N x 3
+    float* dgeo;      // N x 8: d mean2d x, y, d conic a, b, c, d opacity, d depth channel, unused
+};
+
+template <int DQ>
+__device__ __forceinline__ void render_bwd_full_strip(const TileJob& job, const FullImages& in, const FullGrads& out,
+                                                      int strip, FullSmem<DQ>& sm) {
+    constexpr int DV = DQ / 4, PX = full_px<DQ>(), SP = 32 * PX, ROWS = SP / kTile;
+    constexpr int LC = DQ < 32 ? DQ : 32;       // channel lanes
+    constexpr int CG = DQ > 32 ? DQ / 32 : 1;   // channels per lane
+    constexpr int PC = SP * LC / 32;            // pixels of a lane's column
+    const int tile = job.tile;
+    const int tx = tile % job.tiles_x, ty = tile / job.tiles_x;
+    const int lane = threadIdx.x & 31;
+    const int x0 = tx * kTile, y0 = ty * kTile + strip * ROWS;
+    const int px = x0 + (PX * lane) % kTile, py = y0 + PX * lane / kTile;
+    const float fpy = (float)py;
+    const int2 range = job.ranges[tile];
+    int remaining[PX];
+    int left = 0;
 #pragma unroll
-    for (int k = 0; k < DV; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-    float4 acz = make_float4(0.f, 0.f, 0.f, 0.f);
-    float T = 1.0f;
-    int count = 0;
-    bool done = !inside;
-    for (int start = range.x; start < range.y; start += kBatchFull) {
-        if (__syncthreads_count(done) == kTilePixels) break;
-        const int k = start + t;
-        if (t < kBatchFull && k < range.y) {
-            const int g = pair_ids[k];
-            s_xy[t] = xy[g];
-            s_co[t] = stage_splat(conic_opac[g]);
-            s_cz[t] = make_float4(colours[3 * g], colours[3 * g + 1], colours[3 * g + 2], depth[g]);
+    for (int i = 0; i < PX; ++i) {
+        remaining[i] = px + i < job.W && py < job.H ? job.n_contrib[(size_t)py * job.W + px + i] : 0;
+        left |= remaining[i];
+    }
+    if (range.x >= range.y || !__any_sync(0xffffffffu, left > 0)) return;
+    // the lane's own rows G (queries, then colour and depth) and GX = <G, X>
+    float4 g[PX][DV], gcz[PX];
+    float GX[PX], P[PX], T[PX];
 #pragma unroll
-            for (int c = 0; c < DV; ++c) s_f[t][c] = f[(size_t)g * DV + c];
-        }
-        __syncthreads();
-        const int cnt = min(kBatchFull, range.y - start);
-        for (int j = 0; j < cnt && !done; ++j) {
-            const float alpha = splat_alpha(s_xy[j], s_co[j], fpx, fpy);
-            if (alpha < kAlphaMin) continue;
-            const float test_T = __fmul_rn(T, __fsub_rn(1.0f, alpha));
-            if (test_T < kTMin) {
-                done = true;
-                break;
-            }
-            const float w = __fmul_rn(alpha, T);
+    for (int i = 0; i < PX; ++i) {
+        GX[i] = P[i] = 0.f;
+        T[i] = 1.0f;
+        gcz[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int c = 0; c < DV; ++c) g[i][c] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (px + i < job.W && py < job.H) {
+            const size_t p = (size_t)py * job.W + px + i;
 #pragma unroll
             for (int c = 0; c < DV; ++c) {
-                const float4 v = s_f[j][c];
-                acc[c].x += w * v.x;
-                acc[c].y += w * v.y;
-                acc[c].z += w * v.z;
-                acc[c].w += w * v.w;
+                const float4 v = job.dQ[p * DV + c], q = reinterpret_cast<const float4*>(out.Q)[p * DV + c];
+                g[i][c] = v;
+                GX[i] += v.x * q.x + v.y * q.y + v.z * q.z + v.w * q.w;
             }
-            const float4 v = s_cz[j];
-            acz.x += w * v.x;
-            acz.y += w * v.y;
-            acz.z += w * v.z;
-            acz.w += w * v.w;
-            T = test_T;
-            ++count;
+            gcz[i] = make_float4(out.dC[3 * p], out.dC[3 * p + 1], out.dC[3 * p + 2], out.dZ[p]);
+            GX[i] += gcz[i].x * out.C[3 * p] + gcz[i].y * out.C[3 * p + 1] + gcz[i].z * out.C[3 * p + 2] +
+                     gcz[i].w * out.Z[p];
         }
     }
-    if (inside) {
-        const size_t p = (size_t)py * cam.W + px;
+    // the lane's columns: channels lane % LC + 32 h of the strip's pixels (of half of them at
+    // d = 16), and channel lane % 4 of colour and depth of SP / 8 of them
+    const int first = PC * (lane / LC);
+    float col[CG][PC], colz[SP / 8];
 #pragma unroll
-        for (int c = 0; c < DV; ++c) Q[p * DV + c] = acc[c];
-        C[3 * p] = acz.x;
-        C[3 * p + 1] = acz.y;
-        C[3 * p + 2] = acz.z;
-        Z[p] = acz.w;
-        T_final[p] = T;
-        n_contrib[p] = count;
+    for (int h = 0; h < CG; ++h)
+#pragma unroll
+        for (int k = 0; k < PC; ++k) {
+            const int x = x0 + (first + k) % kTile, y = y0 + (first + k) / kTile;
+            const float* d = reinterpret_cast<const float*>(job.dQ);
+            col[h][k] = x < job.W && y < job.H ? d[((size_t)y * job.W + x) * DQ + 32 * h + lane % LC] : 0.f;
+        }
+#pragma unroll
+    for (int k = 0; k < SP / 8; ++k) {
+        const int i = (SP / 8) * (lane >> 2) + k, x = x0 + i % kTile, y = y0 + i / kTile;
+        const size_t p = (size_t)y * job.W + x;
+        colz[k] = x < job.W && y < job.H ? ((lane & 3) < 3 ? out.dC[3 * p + (lane & 3)] : out.dZ[p]) : 0.f;
+    }
+    for (int start = range.x; start < range.y; start += kFullBatch) {
+        const int cnt = min(kFullBatch, range.y - start);
+        __syncwarp();
+        if (lane < cnt) {
+            const int gid = job.pair_ids[start + lane];
+            sm.id[lane] = gid;
+            sm.xy[lane] = job.xy[gid];
+            sm.co[lane] = stage_splat(job.conic_opac[gid]);
+            sm.cz[lane] = make_float4(in.colours[3 * (size_t)gid], in.colours[3 * (size_t)gid + 1],
+                                      in.colours[3 * (size_t)gid + 2], in.depth[gid]);
+        }
+        __syncwarp();
+        for (int k = lane; k < cnt * DV; k += 32) sm.f[k / DV][k % DV] = job.f[(size_t)sm.id[k / DV] * DV + k % DV];
+        __syncwarp();
+        uint32_t hit = 0;  // Gaussians that reach the strip
+        for (int j = 0; j < cnt; ++j) {
+            const float2 m = sm.xy[j];
+            const float4 q = sm.co[j];
+            float w[PX], dx[PX], raw[PX], alpha[PX];
+            const float dy = __fsub_rn(m.y, fpy);
+            bool use[PX], any = false;
+#pragma unroll
+            for (int i = 0; i < PX; ++i) {
+                dx[i] = __fsub_rn(m.x, (float)(px + i));
+                const float power = __fmaf_rn(dx[i], __fmaf_rn(q.x, dx[i], __fmul_rn(q.y, dy)),
+                                              __fmul_rn(__fmul_rn(q.z, dy), dy));
+                raw[i] = __fmul_rn(q.w, __expf(power));
+                alpha[i] = fminf(kAlphaMax, raw[i]);
+                use[i] = remaining[i] > 0 && power <= 0.0f && alpha[i] >= kAlphaMin;
+                any = any || use[i];
+            }
+            if (!__any_sync(0xffffffffu, any)) continue;
+            hit |= 1u << j;
+            // <G, x_j>
+            float gx[PX];
+            {
+                const float4 v = sm.cz[j];
+#pragma unroll
+                for (int i = 0; i < PX; ++i)
+                    gx[i] = gcz[i].x * v.x + gcz[i].y * v.y + gcz[i].z * v.z + gcz[i].w * v.w;
+            }
+            Pair e[PX][2];  // two chains a pixel
+#pragma unroll
+            for (int i = 0; i < PX; ++i) e[i][0] = Pair(gx[i], 0.f), e[i][1] = Pair(0.f);
+#pragma unroll
+            for (int c = 0; c < DV; ++c) {
+                const float4 v = sm.f[j][c];
+#pragma unroll
+                for (int i = 0; i < PX; ++i) {
+                    e[i][0] = fma2(Pair(g[i][c].x, g[i][c].y), Pair(v.x, v.y), e[i][0]);
+                    e[i][1] = fma2(Pair(g[i][c].z, g[i][c].w), Pair(v.z, v.w), e[i][1]);
+                }
+            }
+            // d mean2d x, y, d conic a, b, c, d opacity of the lane's pixels
+            float geo[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            const float ca = -2.0f * q.x, cb = -q.y, cc = -2.0f * q.z;
+#pragma unroll
+            for (int i = 0; i < PX; ++i) {
+                w[i] = 0.f;
+                if (use[i]) {
+                    float x, x1;
+                    add2(e[i][0], e[i][1]).get(x, x1);
+                    x += x1;
+                    const float Tb = T[i];
+                    w[i] = __fmul_rn(alpha[i], Tb);
+                    T[i] = __fmul_rn(Tb, __fsub_rn(1.0f, alpha[i]));
+                    --remaining[i];
+                    P[i] += w[i] * x;
+                    const float dalpha = Tb * x - (GX[i] - P[i]) / (1.0f - alpha[i]);
+                    if (raw[i] <= kAlphaMax) {
+                        const float dpow = dalpha * raw[i];
+                        geo[0] += dpow * (-ca * dx[i] - cb * dy);
+                        geo[1] += dpow * (-cb * dx[i] - cc * dy);
+                        geo[2] += dpow * (-0.5f * dx[i] * dx[i]);
+                        geo[3] += dpow * (-dx[i] * dy);
+                        geo[4] += dpow * (-0.5f * dy * dy);
+                        geo[5] += dalpha * (raw[i] / q.w);
+                    }
+                }
+            }
+            if (PX == 2)
+                *reinterpret_cast<float2*>(&sm.w[j][2 * lane]) = make_float2(w[0], w[PX - 1]);
+            else
+                sm.w[j][lane] = w[0];
+            // eight values (six used) scattered over lane bits 16, 8, 4, then added over 2 and 1
+            const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
+            float v[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float lo = geo[k], hi = k + 4 < 6 ? geo[k + 4 < 6 ? k + 4 : 0] : 0.f;
+                const float r = __shfl_xor_sync(0xffffffffu, b4 ? lo : hi, 16);
+                v[k] = (b4 ? hi : lo) + r;
+            }
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const float r = __shfl_xor_sync(0xffffffffu, b3 ? v[k] : v[k + 2], 8);
+                v[k] = (b3 ? v[k + 2] : v[k]) + r;
+            }
+            float s = (b2 ? v[1] : v[0]) + __shfl_xor_sync(0xffffffffu, b2 ? v[0] : v[1], 4);
+            s += __shfl_xor_sync(0xffffffffu, s, 2);
+            s += __shfl_xor_sync(0xffffffffu, s, 1);
+            const int slot = (b4 ? 4 : 0) + (b3 ? 2 : 0) + (b2 ? 1 : 0);
+            if ((lane & 3) == 0 && slot < 6 && s != 0.0f) atomicAdd(out.dgeo + (size_t)sm.id[j] * 8 + slot, s);
+        }
+        __syncwarp();
+        for (; hit; hit &= hit - 1) {
+            const int j = __ffs(hit) - 1;
+            const size_t gid = (size_t)sm.id[j];
+            Pair a[CG][2];
+#pragma unroll
+            for (int h = 0; h < CG; ++h) a[h][0] = a[h][1] = Pair(0.f);
+#pragma unroll
+            for (int k = 0; k < PC; k += 4) {
+                const float4 v = *reinterpret_cast<const float4*>(&sm.w[j][first + k]);
+#pragma unroll
+                for (int h = 0; h < CG; ++h) {
+                    a[h][0] = fma2(Pair(v.x, v.y), Pair(col[h][k], col[h][k + 1]), a[h][0]);
+                    a[h][1] = fma2(Pair(v.z, v.w), Pair(col[h][k + 2], col[h][k + 3]), a[h][1]);
+                }
+            }
+            float az = 0.f;
+#pragma unroll
+            for (int k = 0; k < SP / 8; k += 4) {
+                const float4 v = *reinterpret_cast<const float4*>(&sm.w[j][(SP / 8) * (lane >> 2) + k]);
+                az += v.x * colz[k] + v.y * colz[k + 1] + v.z * colz[k + 2] + v.w * colz[k + 3];
+            }
+#pragma unroll
+            for (int h = 0; h < CG; ++h) {
+                float s, s1;
+                add2(a[h][0], a[h][1]).get(s, s1);
+                s += s1;
+                if (LC == 16) s += __shfl_xor_sync(0xffffffffu, s, 16);
+                if (lane < LC && s != 0.0f) atomicAdd(job.df + gid * DQ + 32 * h + lane, s);
+            }
+#pragma unroll
+            for (int o = 16; o >= 4; o >>= 1) az += __shfl_xor_sync(0xffffffffu, az, o);
+            if (lane < 4 && az != 0.0f) atomicAdd(lane < 3 ? out.dcol + gid * 3 + lane : out.dgeo + gid * 8 + 6, az);
+        }
+        left = 0;
+#pragma unroll
+        for (int i = 0; i < PX; ++i) left |= remaining[i];
+        if (!__any_sync(0xffffffffu, left > 0)) break;
     }
 }
 
-// Per-Gaussian gradients: df (N x DQ), dcol (N x 3) and dgeo (N x 8: d mean2d x, y, d conic
-// a, b, c, d opacity, d depth channel, unused), accumulated with one atomic per warp and channel.
 template <int DQ>
-__global__ void __launch_bounds__(kTilePixels) render_bwd_full_kernel(
+__global__ void __launch_bounds__(32 * kBwdWarps, DQ == 32 ? 4 : 1) render_bwd_full_kernel(
     CamParams cam, const int2* __restrict__ ranges, const int32_t* __restrict__ pair_ids,
-    const float2* __restrict__ xy, const float4* __restrict__ conic_opac, const float4* __restrict__ f,
-    const float* __restrict__ colours, const float* __restrict__ depth, const int32_t* __restrict__ n_contrib,
-    const float4* __restrict__ Qf, const float* __restrict__ Cf, const float* __restrict__ Zf,
-    const float4* __restrict__ dQ, const float* __restrict__ dC, const float* __restrict__ dZ,
-    float* __restrict__ df, float* __restrict__ dcol, float* __restrict__ dgeo) {
-    constexpr int DV = DQ / 4;
-    constexpr int NG = DQ / 32 > 0 ? DQ / 32 : 1;
-    __shared__ float2 s_xy[kBatchFull];
-    __shared__ float4 s_co[kBatchFull];
-    __shared__ float4 s_cz[kBatchFull];
-    __shared__ float4 s_f[kBatchFull][DV];
-    __shared__ int s_id[kBatchFull];
-    const int tile = cam.tile_order ? cam.tile_order[blockIdx.x] : (int)blockIdx.x;
-    const int tx = tile % cam.tiles_x, ty = tile / cam.tiles_x;
-    const int t = threadIdx.x, lane = t & 31;
-    const int px = tx * kTile + (t % kTile), py = ty * kTile + (t / kTile);
-    const bool inside = px < cam.W && py < cam.H;
-    const float fpx = (float)px, fpy = (float)py;
-    const int2 range = ranges[tile];
-    float g[DQ];
-    float4 gcz = make_float4(0.f, 0.f, 0.f, 0.f);  // dL/dC (3), dL/dZ
-    float GX = 0.f;
-    int remaining = 0;
-    if (inside) {
-        const size_t p = (size_t)py * cam.W + px;
-#pragma unroll
-        for (int c = 0; c < DV; ++c) {
-            const float4 v = dQ[p * DV + c], q = Qf[p * DV + c];
-            g[4 * c] = v.x;
-            g[4 * c + 1] = v.y;
-            g[4 * c + 2] = v.z;
-            g[4 * c + 3] = v.w;
-            GX += v.x * q.x + v.y * q.y + v.z * q.z + v.w * q.w;
-        }
-        gcz = make_float4(dC[3 * p], dC[3 * p + 1], dC[3 * p + 2], dZ[p]);
-        GX += gcz.x * Cf[3 * p] + gcz.y * Cf[3 * p + 1] + gcz.z * Cf[3 * p + 2] + gcz.w * Zf[p];
-        remaining = n_contrib[p];
-    } else {
-#pragma unroll
-        for (int c = 0; c < DQ; ++c) g[c] = 0.f;
-    }
-    float T = 1.0f, P = 0.0f;
-    bool done = remaining == 0;
-    for (int start = range.x; start < range.y; start += kBatchFull) {
-        if (__syncthreads_count(done) == kTilePixels) break;
-        const int k = start + t;
-        if (t < kBatchFull && k < range.y) {
-            const int gid = pair_ids[k];
-            s_xy[t] = xy[gid];
-            s_co[t] = stage_splat(conic_opac[gid]);
-            s_cz[t] = make_float4(colours[3 * gid], colours[3 * gid + 1], colours[3 * gid + 2], depth[gid]);
-#pragma unroll
-            for (int c = 0; c < DV; ++c) s_f[t][c] = f[(size_t)gid * DV + c];
-            s_id[t] = gid;
-        }
-        __syncthreads();
-        const int cnt = min(kBatchFull, range.y - start);
-        for (int j = 0; j < cnt; ++j) {
-            float w = 0.0f;
-            float geo[10] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            if (!done) {
-                const float2 m = s_xy[j];
-                const float4 q = s_co[j];
-                const float dx = __fsub_rn(m.x, fpx), dy = __fsub_rn(m.y, fpy);
-                const float power =
-                    __fmaf_rn(dx, __fmaf_rn(q.x, dx, __fmul_rn(q.y, dy)), __fmul_rn(__fmul_rn(q.z, dy), dy));
-                if (power <= 0.0f) {
-                    const float raw = __fmul_rn(q.w, __expf(power));
-                    const float alpha = fminf(kAlphaMax, raw);
-                    if (alpha >= kAlphaMin) {
-                        const float Tb = T;
-                        w = __fmul_rn(alpha, T);
-                        T = __fmul_rn(T, __fsub_rn(1.0f, alpha));
-                        if (--remaining == 0) done = true;
-                        // <G, x_j>
-                        float gx = gcz.x * s_cz[j].x + gcz.y * s_cz[j].y + gcz.z * s_cz[j].z + gcz.w * s_cz[j].w;
-#pragma unroll
-                        for (int c = 0; c < DV; ++c) {
-                            const float4 v = s_f[j][c];
-                            gx += g[4 * c] * v.x + g[4 * c + 1] * v.y + g[4 * c + 2] * v.z + g[4 * c + 3] * v.w;
-                        }
-                        P += w * gx;
-                        const float dalpha = Tb * gx - (GX - P) / (1.0f - alpha);
-                        geo[0] = w * gcz.x;
-                        geo[1] = w * gcz.y;
-                        geo[2] = w * gcz.z;
-                        geo[3] = w * gcz.w;
-                        if (raw <= kAlphaMax) {
-                            const float dpow = dalpha * raw;
-                            const float a = -2.0f * q.x, b = -q.y, cc = -2.0f * q.z;
-                            geo[4] = dpow * (-a * dx - b * dy);  // d mean2d x
-                            geo[5] = dpow * (-b * dx - cc * dy);
-                            geo[6] = dpow * (-0.5f * dx * dx);    // d conic a, b, c
-                            geo[7] = dpow * (-dx * dy);
-                            geo[8] = dpow * (-0.5f * dy * dy);
-                            geo[9] = dalpha * (raw / q.w);         // d opacity
-                        }
-                    }
-                }
-            }
-            if (__any_sync(0xffffffffu, w != 0.0f)) {
-                const int gid = s_id[j];
-#pragma unroll
-                for (int grp = 0; grp < NG; ++grp) {
-                    float v[32];
-                    if (DQ >= 32) {
-#pragma unroll
-                        for (int c = 0; c < 32; ++c) v[c] = w * g[grp * 32 + c];
-                    } else {
-#pragma unroll
-                        for (int c = 0; c < 32; ++c) v[c] = c < DQ ? w * g[c] : 0.0f;
-                    }
-                    const float s = warp_reduce_scatter32(v, lane);
-                    if (lane < (DQ < 32 ? DQ : 32)) atomicAdd(&df[(size_t)gid * DQ + grp * 32 + lane], s);
-                }
-                float v[32];
-#pragma unroll
-                for (int c = 0; c < 32; ++c) v[c] = c < 10 ? geo[c] : 0.0f;
-                const float s = warp_reduce_scatter32(v, lane);
-                if (lane < 3) atomicAdd(&dcol[(size_t)gid * 3 + lane], s);
-                else if (lane < 10) {
-                    // lanes 3..9: depth channel, mean2d x, y, conic a, b, c, opacity
-                    const int slot = lane == 3 ? 6 : lane - 4;
-                    atomicAdd(&dgeo[(size_t)gid * 8 + slot], s);
-                }
-            }
-        }
-    }
+    const float2* __restrict__ xy, const float4* __restrict__ conic_opac, const float4* __restrict__ f, FullImages in,
+    const int32_t* __restrict__ n_contrib, const float4* __restrict__ dQ, FullGrads out, float* __restrict__ df) {
+    __shared__ __align__(16) FullSmem<DQ> sm[kBwdWarps];
+    constexpr int strips = kTilePixels / (32 * full_px<DQ>());
+    const int item = blockIdx.x * kBwdWarps + (threadIdx.x >> 5);
+    const int t = item / strips;
+    if (t >= cam.tiles_x * cam.tiles_y) return;
+    const int tile = cam.tile_order ? cam.tile_order[t] : t;
+    const TileJob job{tile, cam.tiles_x, cam.W, cam.H, ranges, pair_ids, xy, conic_opac, f, nullptr, nullptr,
+                      const_cast<int32_t*>(n_contrib), dQ, df};
+    render_bwd_full_strip<DQ>(job, in, out, item % strips, sm[threadIdx.x >> 5]);
 }
 
 template <int DQ>
@@ -931,17 +1005,17 @@ latentam_status launch_render_full(const CamParams& cam, const latentam_projecte
                                    const float* f, int d, const float* colours, float* Q, float* C, float* Z,
                                    float* T_final, int32_t* n_contrib, cudaStream_t st) {
     const int tiles = cam.tiles_x * cam.tiles_y;
-    auto args = [&](auto kernel) {
-        kernel<<<tiles, kTilePixels, 0, st>>>(cam, reinterpret_cast<const int2*>(bins.tile_ranges), bins.pair_ids,
-                                              reinterpret_cast<const float2*>(proj.xy),
-                                              reinterpret_cast<const float4*>(proj.conic_opacity),
-                                              reinterpret_cast<const float4*>(f), colours, proj.depth,
-                                              reinterpret_cast<float4*>(Q), C, Z, T_final, n_contrib);
+    auto args = [&](auto kernel, int threads) {
+        kernel<<<tiles, threads, 0, st>>>(cam, reinterpret_cast<const int2*>(bins.tile_ranges), bins.pair_ids,
+                                          reinterpret_cast<const float2*>(proj.xy),
+                                          reinterpret_cast<const float4*>(proj.conic_opacity),
+                                          reinterpret_cast<const float4*>(f), reinterpret_cast<float4*>(Q),
+                                          FullImages{colours, proj.depth, C, Z}, T_final, n_contrib);
     };
     switch (d) {
-        case 16: args(render_fwd_full_kernel<16>); break;
-        case 32: args(render_fwd_full_kernel<32>); break;
-        case 64: args(render_fwd_full_kernel<64>); break;
+        case 16: args(render_fwd_full_kernel<16>, fwd_threads<16>()); break;
+        case 32: args(render_fwd_full_kernel<32>, fwd_threads<32>()); break;
+        case 64: args(render_fwd_full_kernel<64>, fwd_threads<64>()); break;
         default: set_error("query dimension d=%d not in {16, 32, 64}", d); return LATENTAM_ERR_UNSUPPORTED_SHAPE;
     }
     LAT_CHECK_LAUNCH("render_fwd_full_kernel");
@@ -958,17 +1032,17 @@ latentam_status launch_render_bwd_full(const CamParams& cam, const latentam_proj
     if (e == cudaSuccess) e = cudaMemsetAsync(dgeo, 0, sizeof(float) * (size_t)n * 8, st);
     if (e != cudaSuccess) return cuda_error(e, "memset full gradients");
     const int tiles = cam.tiles_x * cam.tiles_y;
-    auto args = [&](auto kernel) {
-        kernel<<<tiles, kTilePixels, 0, st>>>(
+    auto args = [&](auto kernel, int strips) {
+        kernel<<<(tiles * strips + kBwdWarps - 1) / kBwdWarps, 32 * kBwdWarps, 0, st>>>(
             cam, reinterpret_cast<const int2*>(bins.tile_ranges), bins.pair_ids, reinterpret_cast<const float2*>(proj.xy),
-            reinterpret_cast<const float4*>(proj.conic_opacity), reinterpret_cast<const float4*>(f), colours, proj.depth,
-            n_contrib, reinterpret_cast<const float4*>(Q), C, Z, reinterpret_cast<const float4*>(dQ), dC, dZ, df, dcol,
-            dgeo);
+            reinterpret_cast<const float4*>(proj.conic_opacity), reinterpret_cast<const float4*>(f),
+            FullImages{colours, proj.depth, nullptr, nullptr}, n_contrib, reinterpret_cast<const float4*>(dQ),
+            FullGrads{Q, C, Z, dC, dZ, dcol, dgeo}, df);
     };
     switch (d) {
-        case 16: args(render_bwd_full_kernel<16>); break;
-        case 32: args(render_bwd_full_kernel<32>); break;
-        case 64: args(render_bwd_full_kernel<64>); break;
+        case 16: args(render_bwd_full_kernel<16>, 8 / full_px<16>()); break;
+        case 32: args(render_bwd_full_kernel<32>, 8 / full_px<32>()); break;
+        case 64: args(render_bwd_full_kernel<64>, 8 / full_px<64>()); break;
         default: set_error("query dimension d=%d not in {16, 32, 64}", d); return LATENTAM_ERR_UNSUPPORTED_SHAPE;
     }
     LAT_CHECK_LAUNCH("render_bwd_full_kernel");
