@@ -956,9 +956,34 @@ latentam_status split_map_mn(CUtensorMap* m, const void* base, int64_t inner, in
     return LATENTAM_OK;
 }
 
+// Tensor map of a plain operand read MN-major in one box: a 3D view (64 elements, K row, 64-element
+// block) whose box of 64 x box_rows x nblk lands as [block][K row][128 B].
+latentam_status bf16_map_mn(CUtensorMap* m, const void* base, int64_t inner, int64_t rows, int64_t ld, int box_rows,
+                            int nblk) {
+    EncodeTiledFn enc;
+    LAT_TRY(encoder(&enc));
+    if ((reinterpret_cast<uintptr_t>(base) & 15u) || (ld * 2) % 16 || inner % 64) {
+        set_error("MN-major operand not 16-byte aligned or not made of 64-wide blocks");
+        return LATENTAM_ERR_INVALID_ARG;
+    }
+    const cuuint64_t dims[3] = {64, (cuuint64_t)rows, (cuuint64_t)(inner / 64)};
+    const cuuint64_t strides[2] = {(cuuint64_t)(ld * 2), 128};
+    const cuuint32_t box[3] = {64, (cuuint32_t)box_rows, (cuuint32_t)nblk};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) {
+        set_error("cuTensorMapEncodeTiled failed (%d) for an MN-major %lld x %lld operand", (int)r, (long long)rows,
+                  (long long)inner);
+        return LATENTAM_ERR_CUDA;
+    }
+    return LATENTAM_OK;
+}
+
 // Maps of the plain (BF16, 2D) or split (FP32, hi / lo planes) form: op_map for a K-major MMA
-// operand (split: both planes per box), mn_map for an MN-major B operand (split: both planes
-// and nblk 64-wide blocks per box), io_map for epilogue operands, staged outputs and MN-major A
+// operand (split: both planes per box), mn_map for an MN-major operand (nblk 64-wide blocks per
+// box, split: of both planes; a plain single block is a 2D box), io_map for epilogue operands, staged outputs and MN-major A
 // operands (split: one plane per box).
 latentam_status op_map(bool split, CUtensorMap* m, const void* base, int64_t inner, int64_t rows, int64_t ld,
                        int box_rows, int box_inner = tc::kChunkK) {
@@ -967,8 +992,9 @@ latentam_status op_map(bool split, CUtensorMap* m, const void* base, int64_t inn
 }
 latentam_status mn_map(bool split, CUtensorMap* m, const void* base, int64_t inner, int64_t rows, int64_t ld,
                        int box_rows, int nblk) {
-    return split ? split_map_mn(m, base, inner, rows, ld, box_rows, nblk)
-                 : bf16_map(m, base, inner, rows, ld, box_rows);
+    return split     ? split_map_mn(m, base, inner, rows, ld, box_rows, nblk)
+           : nblk > 1 ? bf16_map_mn(m, base, inner, rows, ld, box_rows, nblk)
+                      : bf16_map(m, base, inner, rows, ld, box_rows);
 }
 latentam_status io_map(bool split, CUtensorMap* m, const void* base, int64_t inner, int64_t rows, int64_t ld,
                        int box_rows, int box_inner = tc::kChunkK) {
@@ -1052,7 +1078,8 @@ template <class Epi>
 latentam_status launch_persist(latentam_ctx* ctx, const CUtensorMap& a, const CUtensorMap& b, int row_tiles,
                                int k_chunks, int gy, bool cluster, const typename Epi::Params& p, int* err,
                                cudaStream_t st, const CUtensorMap* emap = nullptr,
-                               const CUtensorMap* omap = nullptr) {
+                               const CUtensorMap* omap = nullptr, const void* a_mem = nullptr, int64_t a_rows = 0,
+                               int a_row_bytes = 0) {
     constexpr size_t smem = tc::persist_smem_bytes<Epi>();
     static_assert(smem <= 227 * 1024, "persistent tile does not fit in shared memory");
     if (row_tiles <= 0) return LATENTAM_OK;
@@ -1095,7 +1122,7 @@ latentam_status launch_persist(latentam_ctx* ctx, const CUtensorMap& a, const CU
         slots = cached[gy];
     }
     cfg.gridDim = dim3((unsigned)std::max(1, std::min(row_tiles, slots)), (unsigned)gy, 1);
-    const tc::PersistGrid pg{k_chunks, row_tiles};
+    const tc::PersistGrid pg{k_chunks, row_tiles, static_cast<const char*>(a_mem), a_rows, a_row_bytes};
     cudaError_t e = cudaLaunchKernelEx(&cfg, kern, a, b, emap ? *emap : a, omap ? *omap : a, pg, p, err);
     if (e != cudaSuccess) return cuda_error(e, "tc_persist_kernel launch");
     LAT_CHECK_LAUNCH("tc_persist_kernel");
@@ -1285,7 +1312,8 @@ latentam_status tc_fhat(latentam_ctx* ctx, const TcBuffers& b, int64_t n, int M,
         // BF16 targets: the tile's target rows are TMA-loaded into shared memory for the epilogue
         CUtensorMap mF;
         LAT_TRY(bf16_map(&mF, fp.F, D, n, D, kTileM));
-        return launch_persist<FhatEpi<true>>(ctx, mA, mV, tiles, kc, cy, true, fp, b.err, st, &mF, &mdF);
+        return launch_persist<FhatEpi<true>>(ctx, mA, mV, tiles, kc, cy, true, fp, b.err, st, &mF, &mdF, b.A, n,
+                                             2 * M);
     }
     return launch_persist<EpiF>(ctx, mA, mV, tiles, kc, cy, true, fp, b.err, st, nullptr, &mdF);
 }

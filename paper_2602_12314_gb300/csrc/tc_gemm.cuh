@@ -516,10 +516,10 @@ __global__ void __launch_bounds__(gemm_threads(Epi::EPI_WG), Epi::MIN_BLOCKS)
                     } else {
                         tma_load_2d(sa, &tmA, &full[s], kx, m0);
                     }
-                    if (B_MN) {
-#pragma unroll
-                        for (int b = 0; b < BN / 64; ++b)
-                            tma_load_2d(sb + b * MNBOX, &tmB, &full[s], n0 + 64 * b, kx);
+                    if (B_MN && BN > 64) {
+                        tma_load_3d(sb, &tmB, &full[s], 0, kx, n0 / 64);
+                    } else if (B_MN) {
+                        tma_load_2d(sb, &tmB, &full[s], n0, kx);
                     } else {
 #pragma unroll
                         for (int b = 0; b < BN / BOX_B; ++b)
@@ -814,6 +814,14 @@ __global__ void __launch_bounds__(gemm_threads(Epi::EPI_WG), Epi::MIN_BLOCKS)
 struct PersistGrid {
     int k_chunks;   // Epi::BK-wide K chunks per tile
     int row_tiles;  // 128-row tiles of A
+    // A as plain memory (a_rows x a_row_bytes, a multiple of 16) for the prefetch of a tile's rows
+    // into L2, or null: none.  (One tiled prefetch per K chunk, in every CTA, took as much of the TMA
+    // as the chunk's loads: the FP32 decode of 307,200 rows 964 us with it, 927 without.  One per
+    // tile and row block helps the BF16 form, 507 -> 503 us, and M = 1024, 2,170 -> 2,145; not the
+    // split form, 927 -> 930, nor FP32 targets in the BF16 form, 854 -> 861.)
+    const char* a;
+    int64_t a_rows;
+    int a_row_bytes;
 };
 
 template <class Epi>
@@ -940,14 +948,13 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
             bool ok = true;
             for (int lt = 0; lt < my_tiles && ok; ++lt) {
                 const int m0 = (first + lt * stride) * kTileM;
-                // the next tile's A rows go to L2 now, so that its ring refills at L2 latency
-                if (lt + 1 < my_tiles)
-                    for (int i = 0; i < nk; ++i) {
-                        if (SPLIT)
-                            tma_prefetch_3d(&tmA, i * BK, m0 + stride * kTileM, 0);  // both planes
-                        else
-                            tma_prefetch_2d(&tmA, i * BK, m0 + stride * kTileM);
-                    }
+                // where asked for, the next tile's A rows go to L2 now, so that its ring refills at
+                // L2 latency: one untiled prefetch of the whole rows
+                if (pg.a && blockIdx.y == 0 && lt + 1 < my_tiles) {
+                    const int64_t r0 = (int64_t)(first + (lt + 1) * stride) * kTileM;
+                    const int64_t rows = min((int64_t)kTileM, pg.a_rows - r0);
+                    bulk_prefetch_l2(pg.a + r0 * pg.a_row_bytes, (uint32_t)(rows * pg.a_row_bytes));
+                }
                 for (int i = 0; i < nk; ++i, ++it) {
                     const int s = it % STAGES;
                     if (it >= STAGES && !mbar_wait(&empty[s], ((uint32_t)(it / STAGES) & 1u) ^ 1u, abort_flag)) {
@@ -966,10 +973,8 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
                             tma_load_3d(sb, &tmB, &full[s], kx, n0, 0);
                     } else {
                         tma_load_2d(sa, &tmA, &full[s], kx, m0);
-                        if (B_MN) {
-#pragma unroll
-                            for (int b = 0; b < BN / 64; ++b)
-                                tma_load_2d(sb + b * MN_BOX, &tmB, &full[s], n0 + 64 * b, kx);
+                        if (B_MN) {  // the tile's 64-wide blocks in one box
+                            tma_load_3d(sb, &tmB, &full[s], 0, kx, n0 / 64);
                         } else {
 #pragma unroll
                             for (int b = 0; b < BN / BOX_B; ++b)
