@@ -322,7 +322,7 @@ struct SoftmaxEpi {
     static constexpr bool SPLIT = SPLIT_, INPLACE = false;
     static constexpr int BN = 256, BK = SPLIT_ ? 16 : 64, ELEM = 2, STAGES = SPLIT_ ? 3 : 1, BOX_B = 256;
     static constexpr int EPI_WG = 4, E_BOXES = 0, O_BOXES = 4;
-    static constexpr int XROUNDS = 1, WARP_STAGE = 0;
+    static constexpr int XROUNDS = 1, WARP_STAGE = 0, SLOTS = 0;
     static constexpr bool A_MN = false, B_MN = false;
     using Params = SoftmaxParams;
     static __device__ int run(const Params& p, const tc::EpiCtx& ec) {
@@ -440,7 +440,7 @@ struct FhatOutEpi {
     static constexpr bool SPLIT = SPLIT_, INPLACE = false;
     static constexpr int ELEM = Q8 ? 1 : 2, BK = SPLIT_ ? 32 : 64, STAGES = Q8 ? 6 : 3;
     static constexpr int BN = 256, BOX_B = 256, EPI_WG = 4, XROUNDS = 0, E_BOXES = 0, O_BOXES = 0;
-    static constexpr int WARP_STAGE = 4096;
+    static constexpr int WARP_STAGE = 4096, SLOTS = 0;
     static constexpr bool A_MN = false, B_MN = !Q8;
     using Params = FhatParams;
     static __device__ int run(const Params& p, const tc::EpiCtx& ec) {
@@ -476,14 +476,16 @@ struct FhatOutEpi {
 // ETILE (FP32 targets) the tile's target rows come by TMA as eight 32-column FP32 chunks filling
 // both box buffers and dFhat is written over them (INPLACE); without, the targets (FP32 or BF16)
 // are read per thread and dFhat is staged as two planes across the buffers.
-template <bool ETILE, bool Q8 = false, bool SPLIT_ = false>
+// SLOTS_ (plain ETILE): target boxes held, eight (two tiles) with three ring stages or four with five.
+template <bool ETILE, bool Q8 = false, bool SPLIT_ = false, int SLOTS_ = 8>
 struct FhatEpi {
     static_assert(!SPLIT_ || !Q8, "the split form has no E4M3 operands");
     static constexpr bool SPLIT = SPLIT_, INPLACE = SPLIT_ && ETILE;
     // persistent, 64-byte K chunks (three ring stages fit beside two epilogue buffers)
     static constexpr int ELEM = Q8 ? 1 : 2, BK = SPLIT_ ? 16 : 64 / ELEM;
-    static constexpr int BN = 256, STAGES = 3, BOX_B = 256, EPI_WG = ETILE ? 4 : 2, XROUNDS = 1;
-    static constexpr int WARP_STAGE = 0;
+    static constexpr int SLOTS = ETILE && !SPLIT_ ? SLOTS_ : 0;
+    static constexpr int BN = 256, STAGES = SLOTS == 4 ? 5 : 3, BOX_B = 256;
+    static constexpr int EPI_WG = ETILE ? 4 : 2, XROUNDS = 1, WARP_STAGE = 0;
     // dFhat staged over the target
     static constexpr int E_BOXES = INPLACE ? 8 : ETILE ? BN / 64 : 0, O_BOXES = BN / 64;
     // B = V (atoms x features, features contiguous: MN-major) or, for E4M3, V^T (K-major)
@@ -1190,18 +1192,20 @@ tc::GemmGrid pixel_split(int64_t n, int z, int* z_out, int chunk = tc::kChunkK) 
     return tc::GemmGrid{chunks, cpz};
 }
 
-// The split the tile grid starts from: about one wave of CTAs.
-int wave_split(int tiles_xy, int num_sms) { return std::max(1, (num_sms + tiles_xy - 1) / tiles_xy); }
+// The split that fills `waves` waves of one CTA per SM and does not start another (M = 1024, D = 768
+// on 152 SMs: 12 tiles; 13 parts left 4 CTAs to a second wave, 26 parts 8 to a third).
+int wave_split(int tiles_xy, int num_sms, int waves) { return std::max(1, waves * num_sms / tiles_xy); }
+constexpr int kMaxWaves = 3;  // the tuner tries 1 .. kMaxWaves
 
 // Autotuned launch shape of a pixel reduction: the first time a shape (n, M, D, which) is seen
-// outside stream capture, `launch(shape, z)` runs for every tile shape 0 .. nshapes - 1 with its
-// wave split z0[shape], half of it and twice it (one untimed warm-up run first), timed with CUDA
-// events on the stream, and the fastest (tile shape, split) is kept in the context.
+// outside stream capture, `launch(shape, z)` runs for every tile shape 0 .. nshapes - 1 (tiles[shape]
+// CTAs per part) with its splits of one to kMaxWaves waves (one untimed warm-up run first), timed
+// with CUDA events on the stream, and the fastest (tile shape, split) is kept in the context.
 template <class Launch>
-latentam_status tuned_shape(latentam_ctx* ctx, int64_t n, int M, int D, int which, int nshapes, const int* z0,
+latentam_status tuned_shape(latentam_ctx* ctx, int64_t n, int M, int D, int which, int nshapes, const int* tiles,
                             cudaStream_t st, Launch&& launch, int* shape_out, int* z_out) {
     *shape_out = 0;
-    *z_out = z0[0];
+    *z_out = wave_split(tiles[0], ctx->num_sms, 1);
     for (int i = 0; i < ctx->tune_used; ++i) {
         const auto& t = ctx->tune[i];
         if (t.n == n && t.M == M && t.D == D && t.which == which) {
@@ -1216,18 +1220,18 @@ latentam_status tuned_shape(latentam_ctx* ctx, int64_t n, int M, int D, int whic
     cudaEvent_t ev[2];
     for (auto& e : ev)
         if (cudaEventCreate(&e) != cudaSuccess) return cuda_error(cudaGetLastError(), "tuning events");
-    latentam_status s = launch(0, z0[0]);  // warm-up
+    latentam_status s = launch(0, *z_out);  // warm-up
     float best = 1e30f;
     for (int sh = 0; sh < nshapes && s == LATENTAM_OK; ++sh) {
-        const int cand[3] = {z0[sh], std::max(1, z0[sh] / 2), 2 * z0[sh]};
-        for (int i = 0; i < 3 && s == LATENTAM_OK; ++i) {
+        for (int w = 1; w <= kMaxWaves && s == LATENTAM_OK; ++w) {
+            const int z = wave_split(tiles[sh], ctx->num_sms, w);
             cudaEventRecord(ev[0], st);
-            s = launch(sh, cand[i]);
+            s = launch(sh, z);
             cudaEventRecord(ev[1], st);
             cudaEventSynchronize(ev[1]);
             float ms = 0.f;
             cudaEventElapsedTime(&ms, ev[0], ev[1]);
-            if (s == LATENTAM_OK && ms < best) best = ms, *shape_out = sh, *z_out = cand[i];
+            if (s == LATENTAM_OK && ms < best) best = ms, *shape_out = sh, *z_out = z;
         }
     }
     for (auto& e : ev) cudaEventDestroy(e);
@@ -1312,6 +1316,13 @@ latentam_status tc_fhat(latentam_ctx* ctx, const TcBuffers& b, int64_t n, int M,
         // BF16 targets: the tile's target rows are TMA-loaded into shared memory for the epilogue
         CUtensorMap mF;
         LAT_TRY(bf16_map(&mF, fp.F, D, n, D, kTileM));
+        // Past 512 atoms the operand ring takes longer than an epilogue with its target's load and
+        // store: one tile of target boxes and five stages.  (300,000 rows, whole decode with two
+        // tiles / one: M = 256 500 / 560 us, 512 x 768 1,099 / 1,115, 768 x 256 1,016 / 980,
+        // 1024 x 768 2,140 / 2,002.)
+        if (M > 512)
+            return launch_persist<FhatEpi<true, false, false, 4>>(ctx, mA, mV, tiles, kc, cy, true, fp, b.err, st, &mF,
+                                                                  &mdF, b.A, n, 2 * M);
         return launch_persist<FhatEpi<true>>(ctx, mA, mV, tiles, kc, cy, true, fp, b.err, st, &mF, &mdF, b.A, n,
                                              2 * M);
     }
@@ -1388,11 +1399,9 @@ latentam_status tc_loss_bwd(latentam_ctx* ctx, const DecodeArgs& a, cudaStream_t
     using EpiV1 = PartEpi<256, SPLIT, 1>;
     const int tilesV[2] = {cdiv(M, 2 * kTileM) * cdiv(D, 256), cdiv(M, kTileM) * cdiv(D, 256)};
     const int tilesK = cdiv(M, kTileM);
-    const int zV0[2] = {wave_split(tilesV[0], ctx->num_sms), wave_split(tilesV[1], ctx->num_sms)};
-    const int zK0 = wave_split(tilesK, ctx->num_sms);
     // partial sums for the largest split a tuner may try
-    const size_t part_floats = std::max({(size_t)2 * zV0[0] * M * D, (size_t)2 * zV0[1] * M * D,
-                                         (size_t)2 * zK0 * M * BNq});
+    auto most = [&](int tiles) { return (size_t)wave_split(tiles, ctx->num_sms, kMaxWaves); };
+    const size_t part_floats = std::max({most(tilesV[0]) * M * D, most(tilesV[1]) * M * D, most(tilesK) * M * BNq});
     b.part = static_cast<float*>(ws(ctx, WS_DEC_PART, sizeof(float) * part_floats));
     if (!b.part) return LATENTAM_ERR_OUT_OF_MEMORY;
     const int which = SPLIT ? 16 : 0;  // autotuner key offset of the split form
@@ -1425,11 +1434,13 @@ latentam_status tc_loss_bwd(latentam_ctx* ctx, const DecodeArgs& a, cudaStream_t
         DsParams dp{n,   M, b.A, b.row, b.dS, dq_fused ? a.dQ : nullptr, d, a.c, ty > 1 ? 1 : 0,
                     dk_fused ? reinterpret_cast<float*>(b.dS) : nullptr};
         const dim3 grow(cdiv(n, kTileM), 1, 1);
-        const tc::GemmGrid g3{cdiv(D, BK3), cdiv(D, BK3)};
+        // the column tiles of a row tile side by side: with the row tiles innermost, every column
+        // tile read all of dFhat from HBM again (1,254,528 rows, M = 1024: @@)
+        const tc::GemmGrid g3{cdiv(D, BK3), cdiv(D, BK3), ty};
         CUtensorMap mAe, mdSo;  // attention rows for the epilogue, dS out through the TMA
         LAT_TRY(io_map(SPLIT, &mAe, b.A, M, n, M, kTileM));
         LAT_TRY(io_map(SPLIT, &mdSo, b.dS, M, n, M, kTileM));
-        LAT_TRY((launch_gemm<DsEpi<SPLIT>>(mdF, mV, dim3(cdiv(n, kTileM), ty, 1), g3, dp, b.err, st, &mAe, &mdSo, 1,
+        LAT_TRY((launch_gemm<DsEpi<SPLIT>>(mdF, mV, dim3(cdiv(n, kTileM) * ty, 1, 1), g3, dp, b.err, st, &mAe, &mdSo, 1,
                                            dq_fused ? &mK : nullptr, dk_fused ? &mQt : nullptr)));
         if (a.dQ && !dq_fused) {
             LAT_TRY(op_map(SPLIT, &mdS, b.dS, M, n, M, kTileM));
@@ -1486,7 +1497,7 @@ latentam_status tc_loss_bwd(latentam_ctx* ctx, const DecodeArgs& a, cudaStream_t
                 return reduce_dV(zz);
             };
             int shape, z;
-            LAT_TRY(tuned_shape(ctx, n, M, D, 5 + which, 2, zV0, st, g5, &shape, &z));
+            LAT_TRY(tuned_shape(ctx, n, M, D, 5 + which, 2, tilesV, st, g5, &shape, &z));
             LAT_TRY(g5(shape, z));
         }
     }
@@ -1510,7 +1521,7 @@ latentam_status tc_loss_bwd(latentam_ctx* ctx, const DecodeArgs& a, cudaStream_t
                 return reduce_dK(zz);
             };
             int shape, z;
-            LAT_TRY(tuned_shape(ctx, n, M, D, 6 + which, 1, &zK0, st, g6, &shape, &z));
+            LAT_TRY(tuned_shape(ctx, n, M, D, 6 + which, 1, &tilesK, st, g6, &shape, &z));
             LAT_TRY(g6(0, z));
         }
     }

@@ -6,7 +6,8 @@
 // Warp roles (192 threads): warp 0 issues the TMA loads, warp 1 owns the TMEM allocation and
 // issues the MMAs (one thread), warps 2..5 run the epilogue; epilogue thread r owns tile row r
 // (TMEM lane r; warp w reads the lane quarter w % 4).
-// blockIdx.x: 128-row tile of A, blockIdx.y: BN-row tile of B, blockIdx.z: split of the K range.
+// blockIdx.x: 128-row tile of A, blockIdx.y: BN-row tile of B (or both in blockIdx.x, see
+// GemmGrid::y_inner), blockIdx.z: split of the K range.
 // When a row reduction spans several BN tiles, the tiles of one row block run as a thread-block
 // cluster along y and trade their per-row partial results through distributed shared memory.
 #pragma once
@@ -130,6 +131,9 @@ __device__ __forceinline__ float group_max(float v, float* scratch, int slot, in
 struct GemmGrid {
     int k_chunks;      // total 64-wide K chunks
     int chunks_per_z;  // chunks handled by one blockIdx.z
+    // > 0: blockIdx.x walks this many B tiles of one A tile before the next A tile (gridDim.y 1), so
+    // that the A tile is read from HBM once and the others find it in L2
+    int y_inner = 0;
 };
 
 // Epi must provide: static constexpr int BN, STAGES, BOX_B (rows per TMA box of a K-major B,
@@ -190,6 +194,9 @@ struct EpiCtx {
     uint32_t oplane = 0;   // split form: bytes from the hi to the lo plane of the staged output
     uint64_t* ofree = nullptr;  // split persistent form: completes when the staging buffers are free
     uint32_t ofree_phase = 0;
+    // persistent plain form with an epilogue operand: its boxes take the slots q0, q0 + 1, ... of a
+    // ring of `slots` (0: box b is at b), in the ring's round of parity ephase
+    int q0 = 0, slots = 0;
     // one-tile kernel, run_x: 32 KB of free shared memory, or null; persistent form with
     // Epi::WARP_STAGE: this warp's own staging bytes, stored by the warp itself to *omap
     uint8_t* xstage = nullptr;
@@ -272,12 +279,19 @@ struct EpiCtx {
         return xbuf[slot * (kXchgMsg / 4) + k * kTileM + row];
     }
 
+    __device__ __forceinline__ int box_at(int b) const {
+        const int s = q0 + b;
+        return slots > 0 && s >= slots ? s - slots : s;
+    }
     // Wait for box b of the epilogue operand (bounded; false if it gave up).
-    __device__ __forceinline__ bool wait_box(int b) const { return mbar_wait(&ebar[b], ephase, abort); }
+    __device__ __forceinline__ bool wait_box(int b) const {
+        const int s = box_at(b);
+        return mbar_wait(&ebar[s], ephase ^ (s < q0 ? 1u : 0u), abort);
+    }
     // Stage 32 values of this thread's row as BF16 at column c0 (a multiple of 32) of the output
     // (split form: the hi terms in the hi plane, the lo terms in the lo plane).
     __device__ __forceinline__ void put32(int c0, const float (&v)[32]) const {
-        uint8_t* base = otile + ((c0 - col0) >> 6) * (kTileM * 128) + row * 128;
+        uint8_t* base = otile + box_at((c0 - col0) >> 6) * (kTileM * 128) + row * 128;
         const int j0 = (c0 & 63) >> 3;
         if (oplane) {
 #pragma unroll
@@ -300,7 +314,7 @@ struct EpiCtx {
     // 32 values of this thread's row from column c0 (a multiple of 32) of the operand (split
     // form: hi + lo).
     __device__ __forceinline__ void row32(int c0, float (&v)[32]) const {
-        const uint8_t* base = etile + ((c0 - col0) >> 6) * (kTileM * 128) + row * 128;
+        const uint8_t* base = etile + box_at((c0 - col0) >> 6) * (kTileM * 128) + row * 128;
         const int j0 = (c0 & 63) >> 3;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -433,8 +447,9 @@ __global__ void __launch_bounds__(gemm_threads(Epi::EPI_WG), Epi::MIN_BLOCKS)
     if constexpr (X2 > 0) x2_on = x_on && Epi::x2_active(ep);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m0 = blockIdx.x * MSUB * kTileM;
-    const int n0 = blockIdx.y * BN;
+    const int tile_x = g.y_inner > 0 ? (int)blockIdx.x / g.y_inner : (int)blockIdx.x;
+    const int m0 = tile_x * MSUB * kTileM;
+    const int n0 = (g.y_inner > 0 ? (int)blockIdx.x % g.y_inner : (int)blockIdx.y) * BN;
     const int k_begin = blockIdx.z * g.chunks_per_z;
     const int k_end = min(g.k_chunks, k_begin + g.chunks_per_z);
     const int nk = k_end - k_begin;
@@ -757,7 +772,7 @@ __global__ void __launch_bounds__(gemm_threads(Epi::EPI_WG), Epi::MIN_BLOCKS)
                         if (threadIdx.x == 64) *decision = (*decision && !*abort_flag) ? 1 : 0;
                         epi_sync(128 * Epi::EPI_WG);
                         tc_fence_after();
-                        if (*decision) Epi::run_k(ep, ec, (int)blockIdx.x);
+                        if (*decision) Epi::run_k(ep, ec, tile_x);
                     }
                 }
             }
@@ -803,7 +818,7 @@ __global__ void __launch_bounds__(gemm_threads(Epi::EPI_WG), Epi::MIN_BLOCKS)
 //   full[s] / empty[s]   operand ring                                  [(it / STAGES) & 1]
 //   acc_full[e]          MMAs of tile lt done -> epilogue              [u & 1]
 //   acc_empty[e]         epilogue done reading TMEM -> MMA (tile lt+2) [(u - 1) & 1]
-//   e_full[e][k]         epilogue operand box k of tile lt loaded      [u & 1]
+//   e_full[slot]         epilogue operand box loaded                   [round of the slot]
 //   e_free[e]            buffer e free for tile lt's output (no operand) [u & 1]
 //   staged[e]            output of tile lt staged in buffer e          [u & 1]
 //   xbar[e]              cluster row exchange of tile lt               [u & 1]
@@ -825,10 +840,11 @@ struct PersistGrid {
 };
 
 template <class Epi>
-__host__ __device__ constexpr uint32_t persist_box_bytes() {  // one box buffer
-    // in place (split): the eight 16 KB operand chunks of one tile fill both buffers
-    return Epi::INPLACE ? 4 * kTileABytes
-                        : (uint32_t)(Epi::E_BOXES > Epi::O_BOXES ? Epi::E_BOXES : Epi::O_BOXES) * kTileABytes;
+__host__ __device__ constexpr uint32_t persist_box_bytes() {  // half of the box buffers
+    // in place (split): the eight 16 KB operand chunks of one tile fill both halves
+    return Epi::INPLACE        ? 4 * kTileABytes
+           : Epi::E_BOXES > 0 ? (uint32_t)Epi::SLOTS * kTileABytes / 2
+                              : (uint32_t)Epi::O_BOXES * kTileABytes;
 }
 
 // One ring stage: A (128 x BK) and B (BN x BK) elements of Epi::ELEM bytes (2: BF16, 1: E4M3),
@@ -875,6 +891,8 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
     static_assert(BN % BOX_B == 0 && BOX_B <= 256 && (BOX_B * 128) % 1024 == 0, "bad B box");
     static_assert(!B_MN || BN % 64 == 0, "an MN-major B tile is made of 64-wide boxes");
     constexpr bool INPLACE = Epi::INPLACE;  // split: FP32 operand chunks in, output over them
+    static_assert(E_BOXES == 0 || INPLACE || (E_BOXES == 4 && Epi::SLOTS >= 4 && Epi::SLOTS <= 8 && Epi::SLOTS % 2 == 0),
+                  "box ring");
     static_assert((E_BOXES <= 4 || INPLACE) && O_BOXES <= 4 && Epi::XROUNDS <= 1 && G <= 4, "epilogue shape");
     static_assert(ROWB == 128 || ROWB == 64 || ROWB == 32, "K chunk rows of 128, 64 or 32 bytes");
     static_assert(!A_MN, "the persistent tile reads A K-major");
@@ -921,7 +939,7 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
         for (int e = 0; e < 2; ++e) {
             mbar_init(&acc_full[e], 1);
             mbar_init(&acc_empty[e], 1);
-            for (int b = 0; b < (INPLACE ? 4 : E_BOXES); ++b) mbar_init(&e_full[4 * e + b], 1);
+            for (int b = 0; b < (E_BOXES > 0 ? 4 : 0); ++b) mbar_init(&e_full[4 * e + b], 1);
             mbar_init(&e_free[e], 1);
             mbar_init(&staged[e], 1);
             if (csize > 1) mbar_init(&xbars[e], 1);  // this CTA's expect-tx arrival
@@ -1054,10 +1072,56 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
                 bulk_wait_read();
             }
         }
+    } else if (warp == 2 && E_BOXES > 0) {
+        if (lane == 0 && nk > 0) {
+            // ---- box ring: staged outputs out, epilogue operands in ----
+            constexpr int NS = Epi::SLOTS > 0 ? Epi::SLOTS : 1, EB = E_BOXES > 0 ? E_BOXES : 1;
+            int sent = -1;  // last tile whose stores were issued (one bulk group per box)
+            int loaded = 0;  // boxes loaded
+            bool ok = true;
+            auto store_tile = [&](int t) -> bool {
+                if (!mbar_wait(&staged[t & 1], (uint32_t)(t >> 1) & 1u, abort_flag)) return false;
+                const int nb = nbox[t & 1];
+                const int m0t = (first + t * stride) * kTileM;
+                for (int b = 0; b < EB; ++b) {
+                    if (b < nb)
+                        tma_store_2d(&tmO, boxes + ((EB * t + b) % NS) * kTileABytes, n0 + 64 * b, m0t);
+                    bulk_commit();
+                }
+                sent = t;
+                return true;
+            };
+            for (; loaded < EB * my_tiles && ok; ++loaded) {
+                const int old = loaded - NS;  // the box that held the slot
+                if (old >= 0) {
+                    if (old / EB > sent && !store_tile(old / EB)) {
+                        ok = false;
+                        break;
+                    }
+                    switch (EB * (sent + 1) - old - 1) {  // groups issued after that box's
+                        case 0: bulk_wait_read_but<0>(); break;
+                        case 1: bulk_wait_read_but<1>(); break;
+                        case 2: bulk_wait_read_but<2>(); break;
+                        default: bulk_wait_read_but<3>(); break;
+                    }
+                }
+                const int s = loaded % NS, lt = loaded / EB;
+                mbar_expect_tx(&e_full[s], kTileABytes);
+                tma_load_2d(boxes + s * kTileABytes, &tmE, &e_full[s], n0 + 64 * (loaded % EB),
+                            (first + lt * stride) * kTileM);
+            }
+            while (ok && sent + 1 < my_tiles) ok = store_tile(sent + 1);
+            bulk_wait_read();
+            if (!ok) {
+                *abort_flag = 1;
+                for (int q = max(0, loaded - NS); q < loaded; ++q)  // never leave the CTA with copies in flight
+                    (void)mbar_wait(&e_full[q % NS], (uint32_t)(q / NS) & 1u, nullptr);
+            }
+        }
     } else if (warp == 2) {
         if (lane == 0 && nk > 0) {
-            // ---- box buffers: staged outputs out, epilogue operands in ----
-            int stored = 0, e_issued = -1;
+            // ---- box buffers: staged outputs out ----
+            int stored = 0;
             bool ok = true;
             // send the staged output of tile t (its buffer is t & 1) and wait until it was read
             auto store_tile = [&](int t) -> bool {
@@ -1079,27 +1143,13 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
                     }
                     stored = lt - 1;
                 }
-                const int e = lt & 1;
-                if (E_BOXES > 0) {
-                    const int m0 = (first + lt * stride) * kTileM;
-                    for (int b = 0; b < E_BOXES; ++b) {
-                        mbar_expect_tx(&e_full[4 * e + b], kTileABytes);
-                        tma_load_2d(boxes + e * BOX_BYTES + b * kTileABytes, &tmE, &e_full[4 * e + b], n0 + 64 * b,
-                                    m0);
-                    }
-                    e_issued = lt;
-                } else {
-                    mbar_arrive(&e_free[e]);
-                }
+                mbar_arrive(&e_free[lt & 1]);
             }
             if (ok) {
                 for (int t = stored; t < my_tiles && ok; ++t) ok = store_tile(t);
             }
             if (!ok) {
                 *abort_flag = 1;
-                for (int t = max(0, e_issued - 1); t <= e_issued; ++t)
-                    for (int b = 0; b < E_BOXES; ++b)
-                        (void)mbar_wait(&e_full[4 * (t & 1) + b], (uint32_t)(t >> 1) & 1u, nullptr);
                 bulk_wait_read();
             }
         }
@@ -1172,7 +1222,16 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
                       row, tile * kTileM, n0, 0, group, scratch, E_BOXES > 0 ? box : nullptr, box,
                       &e_full[4 * e], abort_flag, (int)crank, (int)csize, &xbars[e],
                       xbufs + e * (kXchgBytes / 4), (uint32_t)use & 1u, (uint32_t)use & 1u, G, 96};
-            if (INPLACE) {  // the operand chunks of this tile, the output written over them
+            if (E_BOXES > 0 && !INPLACE) {  // the tile's boxes in the ring, the output written over them
+                constexpr int NS = Epi::SLOTS > 0 ? Epi::SLOTS : 1;
+                const int q = E_BOXES * lt;
+                ec.etile = boxes;
+                ec.otile = boxes;
+                ec.ebar = e_full;
+                ec.slots = NS;
+                ec.q0 = q % NS;
+                ec.ephase = (uint32_t)(q / NS) & 1u;
+            } else if (INPLACE) {  // the operand chunks of this tile, the output written over them
                 ec.etile = boxes;
                 ec.otile = boxes;
                 ec.ebar = e_full;
