@@ -1192,20 +1192,36 @@ tc::GemmGrid pixel_split(int64_t n, int z, int* z_out, int chunk = tc::kChunkK) 
     return tc::GemmGrid{chunks, cpz};
 }
 
-// The split that fills `waves` waves of one CTA per SM and does not start another (M = 1024, D = 768
-// on 152 SMs: 12 tiles; 13 parts left 4 CTAs to a second wave, 26 parts 8 to a third).
-int wave_split(int tiles_xy, int num_sms, int waves) { return std::max(1, waves * num_sms / tiles_xy); }
-constexpr int kMaxWaves = 3;  // the tuner tries 1 .. kMaxWaves
+// Splits the tuner tries, the first one where it does not tune.
+constexpr int kSplits = 3;
+using Splits = int[kSplits];
+// dV: those that fill w, w + 1 and w + 2 waves of one CTA per SM and do not start another (M = 1024,
+// D = 768 on 152 SMs: 12 tiles; 13 parts left 4 CTAs to a second wave, 26 parts 8 to a third, and dV
+// over 1,254,528 rows took 1,480 us against 1,090 in 12 or 25 parts), with the smallest w whose
+// parts are no longer than kMaxPart pixels: a part is one FP32 chain, and at 104,000 pixels its
+// rounding shows (dV off by 1.2e-6 against 64 bits, half of that at 50,000).
+constexpr int64_t kMaxPart = 51200;
+void full_waves(int tiles_xy, int64_t n, int num_sms, Splits& z) {
+    int w = 1;
+    while ((int64_t)(w * num_sms / tiles_xy) * kMaxPart < n) ++w;
+    for (int i = 0; i < kSplits; ++i) z[i] = std::max(1, (w + i) * num_sms / tiles_xy);
+}
+// dK (sums with much cancellation: longer FP32 chains show): about one wave, half and two.
+void near_waves(int tiles_xy, int num_sms, Splits& z) {
+    z[0] = std::max(1, (num_sms + tiles_xy - 1) / tiles_xy);
+    z[1] = std::max(1, z[0] / 2);
+    z[2] = 2 * z[0];
+}
 
 // Autotuned launch shape of a pixel reduction: the first time a shape (n, M, D, which) is seen
-// outside stream capture, `launch(shape, z)` runs for every tile shape 0 .. nshapes - 1 (tiles[shape]
-// CTAs per part) with its splits of one to kMaxWaves waves (one untimed warm-up run first), timed
-// with CUDA events on the stream, and the fastest (tile shape, split) is kept in the context.
+// outside stream capture, `launch(shape, z)` runs for every tile shape 0 .. nshapes - 1 with its
+// splits cand[shape] (one untimed warm-up run first), timed with CUDA events on the stream, and the
+// fastest (tile shape, split) is kept in the context.
 template <class Launch>
-latentam_status tuned_shape(latentam_ctx* ctx, int64_t n, int M, int D, int which, int nshapes, const int* tiles,
+latentam_status tuned_shape(latentam_ctx* ctx, int64_t n, int M, int D, int which, int nshapes, const Splits* cand,
                             cudaStream_t st, Launch&& launch, int* shape_out, int* z_out) {
     *shape_out = 0;
-    *z_out = wave_split(tiles[0], ctx->num_sms, 1);
+    *z_out = cand[0][0];
     for (int i = 0; i < ctx->tune_used; ++i) {
         const auto& t = ctx->tune[i];
         if (t.n == n && t.M == M && t.D == D && t.which == which) {
@@ -1223,8 +1239,8 @@ latentam_status tuned_shape(latentam_ctx* ctx, int64_t n, int M, int D, int whic
     latentam_status s = launch(0, *z_out);  // warm-up
     float best = 1e30f;
     for (int sh = 0; sh < nshapes && s == LATENTAM_OK; ++sh) {
-        for (int w = 1; w <= kMaxWaves && s == LATENTAM_OK; ++w) {
-            const int z = wave_split(tiles[sh], ctx->num_sms, w);
+        for (int i = 0; i < kSplits && s == LATENTAM_OK; ++i) {
+            const int z = cand[sh][i];
             cudaEventRecord(ev[0], st);
             s = launch(sh, z);
             cudaEventRecord(ev[1], st);
@@ -1400,8 +1416,12 @@ latentam_status tc_loss_bwd(latentam_ctx* ctx, const DecodeArgs& a, cudaStream_t
     const int tilesV[2] = {cdiv(M, 2 * kTileM) * cdiv(D, 256), cdiv(M, kTileM) * cdiv(D, 256)};
     const int tilesK = cdiv(M, kTileM);
     // partial sums for the largest split a tuner may try
-    auto most = [&](int tiles) { return (size_t)wave_split(tiles, ctx->num_sms, kMaxWaves); };
-    const size_t part_floats = std::max({most(tilesV[0]) * M * D, most(tilesV[1]) * M * D, most(tilesK) * M * BNq});
+    Splits zV[2], zK[1];
+    full_waves(tilesV[0], n, ctx->num_sms, zV[0]);
+    full_waves(tilesV[1], n, ctx->num_sms, zV[1]);
+    near_waves(tilesK, ctx->num_sms, zK[0]);
+    auto most = [](const Splits& z) { return (size_t)*std::max_element(z, z + kSplits); };
+    const size_t part_floats = std::max({most(zV[0]) * M * D, most(zV[1]) * M * D, most(zK[0]) * M * BNq});
     b.part = static_cast<float*>(ws(ctx, WS_DEC_PART, sizeof(float) * part_floats));
     if (!b.part) return LATENTAM_ERR_OUT_OF_MEMORY;
     const int which = SPLIT ? 16 : 0;  // autotuner key offset of the split form
@@ -1435,7 +1455,7 @@ latentam_status tc_loss_bwd(latentam_ctx* ctx, const DecodeArgs& a, cudaStream_t
                     dk_fused ? reinterpret_cast<float*>(b.dS) : nullptr};
         const dim3 grow(cdiv(n, kTileM), 1, 1);
         // the column tiles of a row tile side by side: with the row tiles innermost, every column
-        // tile read all of dFhat from HBM again (1,254,528 rows, M = 1024: @@)
+        // tile read all of dFhat from HBM again (1,254,528 rows, M = 1024: dA -> dS 2,200 -> 1,929 us)
         const tc::GemmGrid g3{cdiv(D, BK3), cdiv(D, BK3), ty};
         CUtensorMap mAe, mdSo;  // attention rows for the epilogue, dS out through the TMA
         LAT_TRY(io_map(SPLIT, &mAe, b.A, M, n, M, kTileM));
@@ -1497,7 +1517,7 @@ latentam_status tc_loss_bwd(latentam_ctx* ctx, const DecodeArgs& a, cudaStream_t
                 return reduce_dV(zz);
             };
             int shape, z;
-            LAT_TRY(tuned_shape(ctx, n, M, D, 5 + which, 2, tilesV, st, g5, &shape, &z));
+            LAT_TRY(tuned_shape(ctx, n, M, D, 5 + which, 2, zV, st, g5, &shape, &z));
             LAT_TRY(g5(shape, z));
         }
     }
@@ -1521,7 +1541,7 @@ latentam_status tc_loss_bwd(latentam_ctx* ctx, const DecodeArgs& a, cudaStream_t
                 return reduce_dK(zz);
             };
             int shape, z;
-            LAT_TRY(tuned_shape(ctx, n, M, D, 6 + which, 1, &tilesK, st, g6, &shape, &z));
+            LAT_TRY(tuned_shape(ctx, n, M, D, 6 + which, 1, zK, st, g6, &shape, &z));
             LAT_TRY(g6(0, z));
         }
     }
