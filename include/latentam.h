@@ -203,9 +203,9 @@ LATENTAM_API latentam_status latentam_profile_read(latentam_ctx* ctx, double* ms
 LATENTAM_API latentam_status latentam_graphs_enable(latentam_ctx* ctx, int32_t enable);
 
 /* Test hook for the failure paths of the bounded device waits (no GPU fault is involved).
- * which = 0: the next binning's radix sort makes the look-back of one 1024-key block poll a
- * word that nothing writes, with a short limit (4096 polls), so that the wait gives up: that
- * binning leaves its tiles empty and the NEXT binning returns LATENTAM_ERR_TIMEOUT.
+ * which = 0: the next binning of more than 64 tiles makes the look-back of its last block of
+ * tiles poll a word that nothing writes, with a short limit (4096 polls), so that the wait gives
+ * up: that binning leaves its tiles empty and the NEXT binning returns LATENTAM_ERR_TIMEOUT.
  * which = 1: raises the flag a tensor-core kernel's bounded wait raises when it gives up, so
  * that the next synchronising call (binning, or a step reading its loss) reports it.
  * INVALID_ARG for other values. */
@@ -249,12 +249,13 @@ LATENTAM_API latentam_status latentam_project(latentam_ctx* ctx, const latentam_
                                  const latentam_camera* cam, const latentam_projected* out,
                                  latentam_stream stream);
 
-/* Bin and sort: emit one (tile, Gaussian) pair per covered tile in Gaussian index order,
- * stable radix sort of the pairs by tile, per-tile ranges, then each tile's list sorted by
+/* Bin and sort: count the Gaussians of each tile, scan the counts into per-tile ranges, place one
+ * (tile, Gaussian) pair per covered tile, then sort each tile's list by
  * (binary32 depth key, index): the front-to-back order, ties in index order.
- * SYNCHRONISES `stream` once to read the pair count P into bins->num_pairs; if
+ * WAITS once, for the work on `stream` up to the pair count P, which it reads into
+ * bins->num_pairs (the placing and the sort may still run when it returns); if
  * P > bins->capacity returns LATENTAM_ERR_CAPACITY and writes no pairs (retry with a larger
- * buffer).  Returns LATENTAM_ERR_TIMEOUT if a bounded wait of an EARLIER call's sort gave up
+ * buffer).  Returns LATENTAM_ERR_TIMEOUT if a bounded wait of an EARLIER call's scan gave up
  * (that call's tiles were left empty), or if a bounded wait of a tensor-core decode kernel
  * gave up since the last report (that call's loss was NaN); the flag is cleared when reported. */
 LATENTAM_API latentam_status latentam_sort(latentam_ctx* ctx, int32_t n, const latentam_projected* proj,

@@ -118,7 +118,7 @@ class Context:
         L.check(_lib().latentam_graphs_enable(self.handle, int(bool(enable))))
 
     def test_wait_timeout(self, which: int):
-        """Arms a bounded device wait to give up (latentam_test_wait_timeout): 0 = the radix
+        """Arms a bounded device wait to give up (latentam_test_wait_timeout): 0 = the
         look-back of the next binning, 1 = the tensor-core kernels' wait flag."""
         L.check(_lib().latentam_test_wait_timeout(self.handle, int(which)))
 

@@ -190,6 +190,16 @@ latentam_status ordered(latentam_ctx* ctx, CamParams* cp, const latentam_bins& b
     return LATENTAM_OK;
 }
 
+// The frame's binning together with the launch order of its tiles.
+latentam_status bin_ordered(latentam_ctx* ctx, int32_t n, const latentam_projected& proj, CamParams* cp,
+                            latentam_bins* bins, cudaStream_t st) {
+    const size_t tiles = (size_t)cp->tiles_x * cp->tiles_y;
+    int32_t* order = static_cast<int32_t*>(ws(ctx, WS_TILE_ORDER, sizeof(int32_t) * tiles));
+    if (!order) return LATENTAM_ERR_OUT_OF_MEMORY;
+    cp->tile_order = order;
+    return bin_and_sort(ctx, n, proj, *cp, bins, order, st);
+}
+
 void* frame_ws(latentam_ctx* ctx, int idx, size_t bytes) {
     if (bytes == 0) bytes = 256;
     if (ctx->frame_bytes[idx] >= bytes) return ctx->frame_ptr[idx];
@@ -542,8 +552,10 @@ latentam_status latentam_ctx_destroy(latentam_ctx* ctx) {
         if (ctx->slot_ptr[s]) cudaFree(ctx->slot_ptr[s]);
     for (int s = 0; s < LATENTAM_NUM_STAGES; ++s)
         for (int i = 0; i < ctx->prof[s].created; ++i) cudaEventDestroy(ctx->prof[s].ev[i]);
-    for (int i = 0; i < 8 * LATENTAM_MAX_BATCH; ++i)
+    for (int i = 0; i < 4 * LATENTAM_MAX_BATCH; ++i)
         if (ctx->frame_ptr[i]) cudaFree(ctx->frame_ptr[i]);
+    for (cudaEvent_t v : ctx->count_events)
+        if (v) cudaEventDestroy(v);
     if (ctx->bin_streams_ready) {
         for (cudaStream_t b : ctx->bin_streams) cudaStreamDestroy(b);
         for (cudaEvent_t v : ctx->bin_events) cudaEventDestroy(v);
@@ -591,7 +603,7 @@ latentam_status latentam_test_wait_timeout(latentam_ctx* ctx, int32_t which) {
         if (e != cudaSuccess) return cuda_error(e, "raise the tensor-core wait flag");
         return LATENTAM_OK;
     }
-    set_error("unknown wait %d (0: radix look-back of the next binning, 1: tensor-core flag)", which);
+    set_error("unknown wait %d (0: look-back of the next binning, 1: tensor-core flag)", which);
     return LATENTAM_ERR_INVALID_ARG;
 }
 
@@ -660,7 +672,7 @@ latentam_status latentam_sort(latentam_ctx* ctx, int32_t n, const latentam_proje
     LAT_TRY(check_projected(proj, n));
     LAT_TRY(check_bins(bins, false));
     StageTimer tm(ctx, LATENTAM_STAGE_SORT, (cudaStream_t)stream);
-    return bin_and_sort(ctx, n, *proj, cam_params(*cam), bins, (cudaStream_t)stream);
+    return bin_and_sort(ctx, n, *proj, cam_params(*cam), bins, nullptr, (cudaStream_t)stream);
 }
 
 latentam_status latentam_render_fwd(latentam_ctx* ctx, int32_t n, const latentam_projected* proj,
@@ -1020,14 +1032,13 @@ latentam_status latentam_backward_full(latentam_ctx* ctx, const latentam_gaussia
     latentam_status s;
     {
         StageTimer tm(ctx, LATENTAM_STAGE_SORT, st);
-        s = bin_and_sort(ctx, N, proj, cp, &bins, st);
+        s = bin_ordered(ctx, N, proj, &cp, &bins, st);
         if (s == LATENTAM_ERR_CAPACITY) {
             bins.pair_ids = static_cast<int32_t*>(ws(ctx, WS_STEP_PAIRS, sizeof(int32_t) * (size_t)bins.num_pairs));
             if (!bins.pair_ids) return LATENTAM_ERR_OUT_OF_MEMORY;
             bins.capacity = bins.num_pairs;
-            s = bin_and_sort(ctx, N, proj, cp, &bins, st);
+            s = bin_ordered(ctx, N, proj, &cp, &bins, st);
         }
-        if (s == LATENTAM_OK) s = ordered(ctx, &cp, bins, 0, (size_t)tiles, st);
     }
     LAT_TRY(s);
     // images, their gradients and the screen-space gradients
@@ -1148,14 +1159,15 @@ latentam_status latentam_step(latentam_ctx* ctx, const latentam_frame* frame, la
     bins.pair_ids = static_cast<int32_t*>(ctx->slot_ptr[WS_STEP_PAIRS]);
     bins.capacity = (int64_t)(ctx->slot_bytes[WS_STEP_PAIRS] / sizeof(int32_t));
     if (N > 0) REQUIRE(g.means && g.quats && g.scales && g.opacities, "null Gaussian attribute");
+    CamParams cp = cam_params(cam);
     {
         StageTimer tm(ctx, LATENTAM_STAGE_PROJECT, st);
-        LAT_TRY(launch_project(g, cam_params(cam), proj, st));
+        LAT_TRY(launch_project(g, cp, proj, st));
     }
     latentam_status s;
     {
         StageTimer tm(ctx, LATENTAM_STAGE_SORT, st);
-        s = bin_and_sort(ctx, N, proj, cam_params(cam), &bins, st);
+        s = bin_ordered(ctx, N, proj, &cp, &bins, st);
     }
     if (s == LATENTAM_ERR_CAPACITY) {
         bins.pair_ids = static_cast<int32_t*>(ws(ctx, WS_STEP_PAIRS, sizeof(int32_t) * (size_t)bins.num_pairs));
@@ -1164,7 +1176,7 @@ latentam_status latentam_step(latentam_ctx* ctx, const latentam_frame* frame, la
         // the projection buffers are intact; only the binning is redone
         pb = static_cast<char*>(ctx->slot_ptr[WS_STEP_PROJ]);
         StageTimer tm(ctx, LATENTAM_STAGE_SORT, st);
-        s = bin_and_sort(ctx, N, proj, cam_params(cam), &bins, st);
+        s = bin_ordered(ctx, N, proj, &cp, &bins, st);
     }
     LAT_TRY(s);
 
@@ -1184,11 +1196,6 @@ latentam_status latentam_step(latentam_ctx* ctx, const latentam_frame* frame, la
     float* dK = reinterpret_cast<float*>(gb + g_dk);
     float* dV = reinterpret_cast<float*>(gb + g_dv);
     double* lp = reinterpret_cast<double*>(gb + g_lp);
-    CamParams cp = cam_params(cam);
-    {
-        StageTimer tm(ctx, LATENTAM_STAGE_SORT, st);
-        LAT_TRY(ordered(ctx, &cp, bins, 0, (size_t)cp.tiles_x * cp.tiles_y, st));
-    }
     // mask-pooled targets: the plan of the mask set (once per call) and the pooled queries
     const int32_t S = frame->n_masks;
     const bool pooled = S > 0;
@@ -1342,18 +1349,8 @@ extern "C" latentam_status latentam_step_batch(latentam_ctx* ctx, const latentam
         total_pix += (int64_t)fr.camera.width * fr.camera.height;
     }
 
-    // projection and binning of every frame (once; the geometry is fixed during the step): the
-    // pair counts of all frames, one host synchronisation, then each frame's pairs, sort and
-    // ranges (binning slot k per frame, its scan offsets at offs + off_at[k])
-    size_t off_at[LATENTAM_MAX_BATCH + 1];
-    off_at[0] = 0;
-    bool any_gauss = false;
-    for (int k = 0; k < n_frames; ++k) {
-        off_at[k + 1] = off_at[k] + (((size_t)frames[k].gaussians.n + 1 + 63) & ~(size_t)63);
-        any_gauss = any_gauss || frames[k].gaussians.n > 0;
-    }
-    uint32_t* offs = static_cast<uint32_t*>(ws(ctx, WS_OFFSETS, sizeof(uint32_t) * off_at[n_frames]));
-    if (!offs) return LATENTAM_ERR_OUT_OF_MEMORY;
+    // projection and binning of every frame (once; the geometry is fixed during the step), each in
+    // its own binning slot; the host then reads the frames' pair counts in turn
     for (int k = 0; k < n_frames; ++k) {
         const latentam_batch_frame& fr = frames[k];
         const int N = fr.gaussians.n;
@@ -1400,25 +1397,20 @@ extern "C" latentam_status latentam_step_batch(latentam_ctx* ctx, const latentam
         for (int k = 0; k < n_frames && s == LATENTAM_OK; ++k) {
             s = launch_project(frames[k].gaussians, fs[k].cam, fs[k].proj, sk(k));
             if (s == LATENTAM_OK)
-                s = bin_count(ctx, frames[k].gaussians.n, fs[k].proj, fs[k].cam, &fs[k].bins, offs + off_at[k], k,
-                              sk(k));
-        }
-        if (s == LATENTAM_OK && any_gauss) {
-            cudaError_t e = cudaSuccess;
-            for (int i = 0; i < std::max(nside, 1) && e == cudaSuccess; ++i) e = cudaStreamSynchronize(sk(i));
-            if (e != cudaSuccess) s = cuda_error(e, "sync for the pair counts");
+                s = bin_launch(ctx, frames[k].gaussians.n, fs[k].proj, fs[k].cam, fs[k].bins, nullptr, k, sk(k));
         }
         for (int k = 0; k < n_frames && s == LATENTAM_OK; ++k) {
             const int N = frames[k].gaussians.n;
             latentam_bins& bins = fs[k].bins;
-            s = bin_finish(ctx, N, fs[k].proj, fs[k].cam, &bins, offs + off_at[k], k, sk(k));
+            s = bin_wait(ctx, N, fs[k].proj, fs[k].cam, &bins, k, sk(k));
             if (s == LATENTAM_ERR_CAPACITY) {
                 bins.pair_ids =
                     static_cast<int32_t*>(frame_ws(ctx, 2 * k + 1, sizeof(int32_t) * (size_t)bins.num_pairs));
                 if (!bins.pair_ids) s = LATENTAM_ERR_OUT_OF_MEMORY;
                 if (s != LATENTAM_ERR_OUT_OF_MEMORY) {
                     bins.capacity = bins.num_pairs;
-                    s = bin_finish(ctx, N, fs[k].proj, fs[k].cam, &bins, offs + off_at[k], k, sk(k));
+                    s = bin_launch(ctx, N, fs[k].proj, fs[k].cam, bins, nullptr, k, sk(k));
+                    if (s == LATENTAM_OK) s = bin_wait(ctx, N, fs[k].proj, fs[k].cam, &bins, k, sk(k));
                 }
             }
         }

@@ -46,13 +46,8 @@ inline CamParams cam_params(const latentam_camera& c) {
 
 // Workspace slots owned by the context.
 enum Slot : int {
-    WS_SORT_K0 = 0,
-    WS_SORT_K1,
-    WS_SORT_V0,
-    WS_SORT_V1,
-    WS_SORT_HIST,
-    WS_SCAN_SUMS,
-    WS_OFFSETS,
+    WS_BIN_WORDS = 0,  // counters of binning slot 0: per-tile counts, look-back words
+    WS_BIN_LONG,       // its merge buffers for lists too long for shared memory
     WS_COUNTERS,
     WS_DEC_A,      // n x M attention (FP32 form) / bf16 copies (tensor form)
     WS_DEC_DF,     // n x D Fhat, then dFhat
@@ -99,10 +94,12 @@ struct latentam_ctx {
     int profiling;
     lat::StageProfile prof[LATENTAM_NUM_STAGES];
     // per-frame buffers of the batched step: [2k] projection + tile ranges, [2k+1] pairs,
-    // [2 LATENTAM_MAX_BATCH + 6k + j] the scratch of binning slot k (j: scan sums, sort keys 0 / 1,
-    // sort values, long-list merge buffers, radix counters)
-    void* frame_ptr[8 * LATENTAM_MAX_BATCH];
-    size_t frame_bytes[8 * LATENTAM_MAX_BATCH];
+    // [2 LATENTAM_MAX_BATCH + 2k + j] the scratch of binning slot k (j: counters, long-list merge
+    // buffers)
+    void* frame_ptr[4 * LATENTAM_MAX_BATCH];
+    size_t frame_bytes[4 * LATENTAM_MAX_BATCH];
+    // per binning slot: recorded once its pair count has been written for the host (first use creates it)
+    cudaEvent_t count_events[LATENTAM_MAX_BATCH];
     // streams on which the keyframes of a batch are binned concurrently, created on first use
     cudaStream_t bin_streams[8];
     cudaEvent_t bin_events[9];  // [0] fork, [1 + i] join of stream i
@@ -121,7 +118,7 @@ struct latentam_ctx {
     lat::GraphCache* graphs;
     lat::GraphCache* sort_graphs;  // the binning before and after its host read (see cached_launch)
     uint32_t* host_counts;         // pinned: [4..5] the device flags read with a step's loss, [8 + 4 k ..] the
-                                   // counts of binning slot k read back by the host
+                                   // counts of binning slot k (written by its kernels)
     // autotuned split factors of the pixel reductions (see latentam_autotune_enable)
     int autotune;
     struct TuneEntry {
@@ -185,35 +182,19 @@ void count_launch();
 latentam_status launch_project(const latentam_gaussians& g, const CamParams& cam,
                                const latentam_projected& out, cudaStream_t st);
 
-// Exclusive scan of n uint32 values; *total_dev (device, nullable) receives the sum.  sums: the
-// block-sum scratch (scan_scratch_words(n) words), the context's workspace when null.
-latentam_status scan_exclusive_u32(latentam_ctx* ctx, const uint32_t* in, uint32_t* out, int64_t n,
-                                   uint32_t* total_dev, cudaStream_t st,
-                                   uint32_t* sums = nullptr);
-// Stable LSD radix sort of n (key, value) pairs on key bits [0, bits), bits <= 32, n < 2^30.
-// keys[0]/vals[0] hold the input (vals_iota: value = index, vals[0] is then only scratch);
-// keys[1]/vals[1] are scratch.  *result receives the index of the buffer pair holding the
-// sorted output.  *err (device) is set if a bounded cross-block wait gave up.  counters: the
-// digit-count, ticket and look-back scratch (radix_scratch_words(n, bits) words), the context's
-// workspace when null.
-latentam_status radix_sort_pairs(latentam_ctx* ctx, uint32_t* const keys[2], uint32_t* const vals[2], bool vals_iota,
-                                 int64_t n, int bits, int* result, uint32_t* err, cudaStream_t st,
-                                 uint32_t* counters = nullptr);
-// 32-bit words of the scratch of scan_exclusive_u32 over n items and of radix_sort_pairs over n
-// keys of `bits` bits (the buffers the optional `sums` / `counters` arguments must hold).
-size_t scan_scratch_words(int64_t n);
-size_t radix_scratch_words(int64_t n, int bits);
-latentam_status bin_and_sort(latentam_ctx* ctx, int32_t n, const latentam_projected& proj,
-                             const CamParams& cam, latentam_bins* bins, cudaStream_t st);
-// The two halves of bin_and_sort, for several keyframes binned with one host synchronisation:
-// bin_count enqueues the pair count of binning slot `slot` (0 .. LATENTAM_MAX_BATCH - 1) into
-// its pinned host words, the offsets into off[n + 1]; once the stream has been synchronised,
-// bin_finish reads them and enqueues the pairs, their sort and the ranges (LATENTAM_ERR_CAPACITY
-// when bins->capacity is short: bin_finish may then be called again with a larger buffer).
-latentam_status bin_count(latentam_ctx* ctx, int32_t n, const latentam_projected& proj, const CamParams& cam,
-                          latentam_bins* bins, uint32_t* off, int slot, cudaStream_t st);
-latentam_status bin_finish(latentam_ctx* ctx, int32_t n, const latentam_projected& proj, const CamParams& cam,
-                           latentam_bins* bins, const uint32_t* off, int slot, cudaStream_t st);
+// Per-tile lists of the visible Gaussians in depth order, in two halves so that several keyframes
+// can be binned at the same time.  bin_launch enqueues the whole binning in binning slot `slot`
+// (0 .. LATENTAM_MAX_BATCH - 1), with `order` (may be null) also the tiles' launch order (see
+// launch_tile_order); bin_wait waits until its pair count is known and reads it: with
+// LATENTAM_ERR_CAPACITY, when bins->capacity is short, nothing was binned (every tile is empty)
+// and both are called again with a larger buffer.
+latentam_status bin_launch(latentam_ctx* ctx, int32_t n, const latentam_projected& proj, const CamParams& cam,
+                           const latentam_bins& bins, int32_t* order, int slot, cudaStream_t st);
+latentam_status bin_wait(latentam_ctx* ctx, int32_t n, const latentam_projected& proj, const CamParams& cam,
+                         latentam_bins* bins, int slot, cudaStream_t st);
+// Both on slot 0.
+latentam_status bin_and_sort(latentam_ctx* ctx, int32_t n, const latentam_projected& proj, const CamParams& cam,
+                             latentam_bins* bins, int32_t* order, cudaStream_t st);
 
 // The tiles of a binned frame in decreasing order of list length (power-of-two classes), into
 // order[tiles]: the per-tile kernels start the longest tiles first.

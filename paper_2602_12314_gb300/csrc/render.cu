@@ -852,34 +852,8 @@ latentam_status render_bwd_t(const CamParams& cam, const latentam_projected& pro
     return LATENTAM_OK;
 }
 
-// Longest tiles first: class b holds the tiles whose list length has its highest set bit at b
-// (empty tiles last); within a class the order is that of the atomics (it only schedules).
-__global__ void __launch_bounds__(1024) tile_order_kernel(const int2* __restrict__ ranges, int tiles,
-                                                          int32_t* __restrict__ order) {
-    __shared__ int s_cnt[33], s_pos[33];
-    const int t = threadIdx.x;
-    if (t < 33) s_cnt[t] = 0;
-    __syncthreads();
-    auto cls = [&](int i) {
-        const int2 r = ranges[i];
-        const int len = r.y - r.x;
-        return len > 0 ? 32 - __clz(len) : 0;  // 1..31, 0 for an empty tile
-    };
-    for (int i = t; i < tiles; i += blockDim.x) atomicAdd(&s_cnt[cls(i)], 1);
-    __syncthreads();
-    if (t == 0) {
-        int run = 0;
-        for (int c = 32; c >= 0; --c) {
-            s_pos[c] = run;
-            run += s_cnt[c];
-        }
-    }
-    __syncthreads();
-    for (int i = t; i < tiles; i += blockDim.x) order[atomicAdd(&s_pos[cls(i)], 1)] = i;
-}
-
 // Longest tiles first over every frame of a batch (the same length classes as
-// tile_order_kernel); entries are (frame << 20) | tile.
+// a single frame's launch order); entries are (frame << 20) | tile.
 __global__ void __launch_bounds__(1024) batch_order_kernel(const __grid_constant__ BatchJobs jobs,
                                                            int32_t* __restrict__ order) {
     __shared__ int s_cnt[33], s_pos[33];
@@ -981,13 +955,6 @@ latentam_status launch_render_bwd_batch(const BatchJobs& jobs, int d, const int3
         case 64: return render_bwd_batch_t<64>(jobs, order, total, counter, st);
         default: set_error("query dimension d=%d not in {16, 32, 64}", d); return LATENTAM_ERR_UNSUPPORTED_SHAPE;
     }
-}
-
-latentam_status launch_tile_order(const CamParams& cam, const latentam_bins& bins, int32_t* order, cudaStream_t st) {
-    const int tiles = cam.tiles_x * cam.tiles_y;
-    tile_order_kernel<<<1, 1024, 0, st>>>(reinterpret_cast<const int2*>(bins.tile_ranges), tiles, order);
-    LAT_CHECK_LAUNCH("tile_order_kernel");
-    return LATENTAM_OK;
 }
 
 latentam_status launch_render_fwd(const CamParams& cam, const latentam_projected& proj, const latentam_bins& bins,

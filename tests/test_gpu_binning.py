@@ -1,0 +1,71 @@
+"""Tile lists of synthetic projections at the edges of the binning kernels, exactly (integers): scan
+blocks of 64 tiles (one tile, 64, 65, more than 32 blocks), splats of many tiles beside splats of
+none, lists above 4,096 keys with more pairs than the merge buffers start with (the second sort),
+depth ties, no pairs at all, and a buffer that is too small."""
+import ctypes
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def api():
+    from paper_2602_12314_gb300 import api as _api
+    return _api
+
+
+def _camera(width, height):
+    from paper_2602_12314_gb300 import _lib as L
+    c = L.Camera(fx=50.0, fy=50.0, cx=width / 2, cy=height / 2, z_near=0.01, width=width, height=height)
+    c.R[:] = [1, 0, 0, 0, 1, 0, 0, 0, 1]
+    return c
+
+
+def _scene(api, n, cam, span, seed, visible):
+    """Random rects of up to span x span tiles; depths with ties."""
+    tx, ty = (cam.width + 15) // 16, (cam.height + 15) // 16
+    g = np.random.default_rng(seed)
+    x0, y0 = g.integers(0, tx, n), g.integers(0, ty, n)
+    x1, y1 = np.minimum(tx, x0 + g.integers(1, span + 1, n)), np.minimum(ty, y0 + g.integers(1, span + 1, n))
+    rect = np.stack([x0, y0, x1, y1], 1).astype(np.int32)
+    touched = ((x1 - x0) * (y1 - y0) * (g.random(n) < visible)).astype(np.int32)
+    depth = (g.integers(1, 200, n) / 16).astype(np.float32)
+    dev = lambda a: torch.as_tensor(a, device="cuda")
+    proj = api.Projection(dev(np.zeros((n, 2), np.float32)), dev(np.zeros((n, 4), np.float32)), dev(depth), dev(rect),
+                          dev(touched))
+    own = np.repeat(np.arange(n), touched)
+    k = np.arange(len(own)) - np.repeat(np.cumsum(touched) - touched, touched)
+    w = (x1 - x0)[own]
+    tile = (y0[own] + k // w) * tx + x0[own] + k % w
+    at = np.lexsort((own, depth[own], tile))
+    ends = np.cumsum(np.bincount(tile, minlength=tx * ty))
+    ranges = np.stack([np.concatenate([[0], ends[:-1]]), ends], 1)
+    ranges[ranges[:, 0] == ranges[:, 1]] = 0
+    return proj, own[at], ranges
+
+
+@pytest.mark.parametrize("n,width,height,span,visible", [
+    (1, 16, 16, 1, 1.0), (700, 128, 128, 3, 0.7), (999, 1040, 16, 70, 0.5), (20_000, 1200, 680, 9, 0.3),
+    (3_000, 700, 500, 40, 0.9), (90_001, 64, 64, 4, 1.0), (4_097, 16, 16, 1, 1.0), (515, 640, 480, 8, 0.0)])
+def test_lists_equal_a_sort(api, n, width, height, span, visible):
+    from paper_2602_12314_gb300 import _lib as L
+    cam = _camera(width, height)
+    proj, ids, ranges = _scene(api, n, cam, span, n, visible)
+    P = len(ids)
+    with api.Context(0) as ctx:
+        for rep in range(4):  # plain launches, then the captured and the replayed ones
+            bins = api.sort(ctx, proj, cam, capacity=max(P, 1))
+            assert bins.num_pairs == P
+            np.testing.assert_array_equal(bins.tile_ranges.cpu().numpy(), ranges)
+            np.testing.assert_array_equal(bins.pair_ids[:P].cpu().numpy(), ids)
+        if P > 1:
+            bins = api.TileBins(torch.full((P,), -1, dtype=torch.int32, device="cuda"), bins.tile_ranges, 0)
+            bs, ps = bins.struct(), proj.struct()
+            bs.capacity = P - 1
+            assert L.load().latentam_sort(ctx.handle, n, ctypes.byref(ps), ctypes.byref(cam), ctypes.byref(bs),
+                                          api._stream()) == L.ERR_CAPACITY
+            assert bs.num_pairs == P and int(bins.tile_ranges.abs().sum()) == 0
+            assert bool((bins.pair_ids == -1).all())

@@ -1,6 +1,5 @@
 """The training decode past 512 atoms, three and four column tiles a row (BF16: one tile of target
-boxes and five operand stages; dQ in two sums, dQ and dK from the staged dS tile or, for BF16 at
-d = 64, as GEMMs), against float64 PyTorch with the forms' bars: BF16 gradients by norm 2e-2 and
+boxes and five operand stages; dV split into whole waves over the pixels), against float64 PyTorch with the forms' bars: BF16 gradients by norm 2e-2 and
 loss parts 5e-3, FP32 1e-3 and 1e-4; row counts that leave partial tiles and give every CTA several."""
 import pytest
 
