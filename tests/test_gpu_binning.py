@@ -1,6 +1,6 @@
 """Tile lists of synthetic projections at the edges of the binning kernels, exactly (integers): scan
 blocks of 64 tiles (one tile, 64, 65, more than 32 blocks), splats of many tiles beside splats of
-none, lists above 4,096 keys with more pairs than the merge buffers start with (the second sort),
+none, lists of 255 to 258 keys (counted or sorted by the network), lists above 4,096 keys with more pairs than the merge buffers start with (the second sort),
 depth ties, no pairs at all, and a buffer that is too small."""
 import ctypes
 
@@ -49,7 +49,8 @@ def _scene(api, n, cam, span, seed, visible):
 
 @pytest.mark.parametrize("n,width,height,span,visible", [
     (1, 16, 16, 1, 1.0), (700, 128, 128, 3, 0.7), (999, 1040, 16, 70, 0.5), (20_000, 1200, 680, 9, 0.3),
-    (3_000, 700, 500, 40, 0.9), (90_001, 64, 64, 4, 1.0), (4_097, 16, 16, 1, 1.0), (515, 640, 480, 8, 0.0)])
+    (3_000, 700, 500, 40, 0.9), (90_001, 64, 64, 4, 1.0), (4_097, 16, 16, 1, 1.0), (255, 16, 16, 1, 1.0),
+    (256, 16, 16, 1, 1.0), (257, 16, 16, 1, 1.0), (4_096, 16, 16, 1, 1.0), (515, 640, 480, 8, 0.0)])
 def test_lists_equal_a_sort(api, n, width, height, span, visible):
     from paper_2602_12314_gb300 import _lib as L
     cam = _camera(width, height)
