@@ -323,6 +323,7 @@ struct SoftmaxEpi {
     static constexpr int BN = 256, BK = SPLIT_ ? 16 : 64, ELEM = 2, STAGES = SPLIT_ ? 3 : 1, BOX_B = 256;
     static constexpr int EPI_WG = 4, E_BOXES = 0, O_BOXES = 4;
     static constexpr int XROUNDS = 1, WARP_STAGE = 0, SLOTS = 0;
+    static constexpr bool PAIR = false;
     static constexpr bool A_MN = false, B_MN = false;
     using Params = SoftmaxParams;
     static __device__ int run(const Params& p, const tc::EpiCtx& ec) {
@@ -430,18 +431,21 @@ __device__ __forceinline__ float row_scale_inv(const FhatParams& p, int64_t pix,
 // Inference form of G2: Fhat = A V out as FP32 rows, no loss and no row terms (independent column
 // tiles).  Each warp stages 32 rows x 32 columns (4 KB) in shared memory of its own and sends them
 // with a TMA store, so that every row leaves as whole 128-byte lines; without box buffers the
-// operand ring takes 144 KB (three stages of 64 K elements; 32 in the split form) instead of 72.
-// Bound by the FP32 rows written and the value matrix streamed through the ring for every tile.
-// 816,000 rows, M = 512, D = 768, BF16: 1,694 us with one row per thread stored in 16-byte pieces
-// and a 72 KB ring -> 678 us (the same bits).
-template <bool Q8 = false, bool SPLIT_ = false>
+// operand ring takes 144 KB (three stages of 64 K elements; 32 in the split form) instead of 72; on
+// CTA pairs (PAIR_) 128 KB are four stages of the same K, each CTA holding half of the value tile.
+// Bound by the FP32 rows written and, meanwhile, by the latency of the operand loads (816,000 rows,
+// M = 512, D = 768, BF16 pairs: 717 us; without the stores 395, the rate of the MMAs; with one K
+// chunk 520; with three stages 790, with two 990), so the attention rows of the next tile are
+// prefetched into L2 (717 -> 665).  One row per thread stored in 16-byte pieces with a 72 KB
+// ring took 1,694 us, single CTAs with 144 KB 755; the bits are the same.
+template <bool Q8 = false, bool SPLIT_ = false, bool PAIR_ = false>
 struct FhatOutEpi {
-    static_assert(!SPLIT_ || !Q8, "the split form has no E4M3 operands");
+    static_assert(!Q8 || (!SPLIT_ && !PAIR_), "the E4M3 form is neither split nor paired");
     static constexpr bool SPLIT = SPLIT_, INPLACE = false;
-    static constexpr int ELEM = Q8 ? 1 : 2, BK = SPLIT_ ? 32 : 64, STAGES = Q8 ? 6 : 3;
-    static constexpr int BN = 256, BOX_B = 256, EPI_WG = 4, XROUNDS = 0, E_BOXES = 0, O_BOXES = 0;
+    static constexpr int ELEM = Q8 ? 1 : 2, BK = SPLIT_ ? 32 : 64, STAGES = PAIR_ ? 4 : Q8 ? 6 : 3;
+    static constexpr int BN = 256, BOX_B = PAIR_ ? 128 : 256, EPI_WG = 4, XROUNDS = 0, E_BOXES = 0, O_BOXES = 0;
     static constexpr int WARP_STAGE = 4096, SLOTS = 0;
-    static constexpr bool A_MN = false, B_MN = !Q8;
+    static constexpr bool A_MN = false, B_MN = !Q8, PAIR = PAIR_;
     using Params = FhatParams;
     static __device__ int run(const Params& p, const tc::EpiCtx& ec) {
         const int ncols = min(BN, p.D - ec.n0), lane = ec.row & 31;
@@ -476,15 +480,17 @@ struct FhatOutEpi {
 // ETILE (FP32 targets) the tile's target rows come by TMA as eight 32-column FP32 chunks filling
 // both box buffers and dFhat is written over them (INPLACE); without, the targets (FP32 or BF16)
 // are read per thread and dFhat is staged as two planes across the buffers.
-// SLOTS_ (plain ETILE): target boxes held, eight (two tiles) with three ring stages or four with five.
-template <bool ETILE, bool Q8 = false, bool SPLIT_ = false, int SLOTS_ = 8>
+// SLOTS_ (plain ETILE): target boxes held, eight (two tiles) with three ring stages or four with five,
+// or, on CTA pairs (PAIR_), four with four stages of twice the K.
+template <bool ETILE, bool Q8 = false, bool SPLIT_ = false, int SLOTS_ = 8, bool PAIR_ = false>
 struct FhatEpi {
     static_assert(!SPLIT_ || !Q8, "the split form has no E4M3 operands");
     static constexpr bool SPLIT = SPLIT_, INPLACE = SPLIT_ && ETILE;
-    // persistent, 64-byte K chunks (three ring stages fit beside two epilogue buffers)
-    static constexpr int ELEM = Q8 ? 1 : 2, BK = SPLIT_ ? 16 : 64 / ELEM;
     static constexpr int SLOTS = ETILE && !SPLIT_ ? SLOTS_ : 0;
-    static constexpr int BN = 256, STAGES = SLOTS == 4 ? 5 : 3, BOX_B = 256;
+    static constexpr bool PAIR = PAIR_;
+    // persistent, 64-byte K chunks (three ring stages fit beside two epilogue buffers), 128-byte ones in a pair
+    static constexpr int ELEM = Q8 ? 1 : 2, BK = SPLIT_ ? 16 : PAIR ? 64 : 64 / ELEM;
+    static constexpr int BN = 256, STAGES = PAIR ? 4 : SLOTS == 4 ? 5 : 3, BOX_B = PAIR ? 128 : 256;
     static constexpr int EPI_WG = ETILE ? 4 : 2, XROUNDS = 1, WARP_STAGE = 0;
     // dFhat staged over the target
     static constexpr int E_BOXES = INPLACE ? 8 : ETILE ? BN / 64 : 0, O_BOXES = BN / 64;
@@ -727,6 +733,35 @@ struct DsEpi {
             ec.put32(c0, dA);
         }
         return cend > ec.col0 ? (cend - ec.col0 + 63) / 64 : 0;
+    }
+};
+
+// G3 of the plain form past 512 atoms, where nothing trails it: persistent CTA pairs (cta_group::2),
+// the attention rows through the box ring and dS stored over them.  The CTAs of a row tile's column
+// tiles run side by side, so dFhat comes from HBM once.  Bound by the bytes (dFhat and A in, dS out)
+// and, as the inference form, by the latency of the operand loads meanwhile.  Whole decode of
+// 200,000 rows, D = 768, M = 1024: 1,168 -> 1,112 us against the one-tile kernel.
+struct DsPairEpi {
+    static constexpr bool SPLIT = false, INPLACE = false, PAIR = true;
+    static constexpr int ELEM = 2, BK = 64, STAGES = 4, BN = 256, BOX_B = 128;
+    static constexpr int EPI_WG = 4, XROUNDS = 0, WARP_STAGE = 0, SLOTS = 4, E_BOXES = 4, O_BOXES = 4;
+    static constexpr bool A_MN = false, B_MN = false;
+    using Params = DsParams;
+    static __device__ int run(const Params& p, const tc::EpiCtx& ec) {
+        const int64_t pix = (int64_t)ec.m0 + ec.row;
+        const bool valid = pix < p.n;
+        const float rd = valid ? p.row[4 * pix + 2] : 0.f;
+        for (int b = 0; b < E_BOXES; ++b) (void)ec.wait_box(b);
+        const int cend = min(BN, p.M - ec.n0);
+        float dA[32], a[32];
+        for (int c0 = 32 * ec.g; c0 < cend; c0 += 32 * EPI_WG) {
+            ec.row32(c0, a);
+            tc::tmem_ld32(ec.taddr + c0, dA);
+#pragma unroll
+            for (int i = 0; i < 32; ++i) dA[i] = valid ? a[i] * (dA[i] - rd) : 0.f;
+            ec.put32(c0, dA);
+        }
+        return (cend + 63) / 64;
     }
 };
 
@@ -1103,27 +1138,29 @@ latentam_status launch_persist(latentam_ctx* ctx, const CUtensorMap& a, const CU
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
-    int slots = ctx->num_sms / gy;  // one CTA per SM
-    if (cluster && gy > 1) {
+    const int cx = Epi::PAIR ? 2 : 1, cy = cluster ? gy : 1;  // cluster shape
+    int slots = ctx->num_sms / gy;                            // one CTA per SM: CTAs (pairs) along x
+    if (cx * cy > 1) {
         attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 1;
-        attr[0].val.clusterDim.y = (unsigned)gy;
+        attr[0].val.clusterDim.x = (unsigned)cx;
+        attr[0].val.clusterDim.y = (unsigned)cy;
         attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         static int cached[tc::kMaxCluster + 1] = {0};
-        if (cached[gy] == 0) {
-            cfg.gridDim = dim3((unsigned)std::max(1, ctx->num_sms / gy), (unsigned)gy, 1);
+        if (cached[cy] == 0) {
+            cfg.gridDim = dim3((unsigned)(cx * std::max(1, ctx->num_sms / (cx * cy))), (unsigned)cy, 1);
             int nc = 0;
             if (cudaOccupancyMaxActiveClusters(&nc, kern, &cfg) != cudaSuccess || nc <= 0) {
                 (void)cudaGetLastError();
-                nc = std::max(1, ctx->num_sms / gy);
+                nc = std::max(1, ctx->num_sms / (cx * cy));
             }
-            cached[gy] = nc;
+            cached[cy] = nc;
         }
-        slots = cached[gy];
+        slots = cached[cy] * cy / gy;
     }
-    cfg.gridDim = dim3((unsigned)std::max(1, std::min(row_tiles, slots)), (unsigned)gy, 1);
+    const int units = (row_tiles + cx - 1) / cx;  // row tiles, or pairs of them
+    cfg.gridDim = dim3((unsigned)(cx * std::max(1, std::min(units, slots))), (unsigned)gy, 1);
     const tc::PersistGrid pg{k_chunks, row_tiles, static_cast<const char*>(a_mem), a_rows, a_row_bytes};
     cudaError_t e = cudaLaunchKernelEx(&cfg, kern, a, b, emap ? *emap : a, omap ? *omap : a, pg, p, err);
     if (e != cudaSuccess) return cuda_error(e, "tc_persist_kernel launch");
@@ -1304,8 +1341,8 @@ latentam_status tc_forward(latentam_ctx* ctx, const float* Q, int64_t n, int d, 
     return launch_persist<Epi>(ctx, mQ, mK, cdiv(n, kTileM), kc, cy, true, sp, b.err, st, nullptr, &mA);
 }
 
-// G2: Fhat = A V (A in 32-wide K chunks, 64-byte swizzle), B = V read MN-major in 64 x 32
-// boxes (features x atoms).
+// G2: Fhat = A V (A in K chunks of Epi::BK atoms), B = V read MN-major in boxes of 64-feature blocks
+// x BK atoms.
 latentam_status tc_fhat8(latentam_ctx* ctx, const TcBuffers& b, int64_t n, int M, int D, const FhatParams& fp,
                          cudaStream_t st);
 
@@ -1313,36 +1350,41 @@ template <bool SPLIT>
 latentam_status tc_fhat(latentam_ctx* ctx, const TcBuffers& b, int64_t n, int M, int D, const FhatParams& fp,
                         cudaStream_t st) {
     if (!SPLIT && b.Aq) return tc_fhat8(ctx, b, n, M, D, fp, st);
-    using EpiF = FhatEpi<false, false, SPLIT>;  // targets read per thread (FP32 or BF16)
-    constexpr int BK = EpiF::BK;
-    CUtensorMap mA, mV;
-    LAT_TRY(op_map(SPLIT, &mA, b.A, M, n, M, kTileM, BK));
-    LAT_TRY(mn_map(SPLIT, &mV, b.Vb, D, M, D, BK, EpiF::BN / 64));
-    const int cy = cdiv(D, 256), tiles = cdiv(n, kTileM), kc = cdiv(M, BK);
-    CUtensorMap mdF;  // dFhat leaves through the TMA
+    const int cy = cdiv(D, 256), tiles = cdiv(n, kTileM);
+    CUtensorMap mF, mdF;  // target rows (where they come by TMA) and dFhat, which leaves through it
+    auto launch = [&](auto epi, const CUtensorMap* mE, bool prefetch) -> latentam_status {
+        using Epi = decltype(epi);
+        CUtensorMap mA, mV;
+        LAT_TRY(op_map(SPLIT, &mA, b.A, M, n, M, kTileM, Epi::BK));
+        LAT_TRY(mn_map(SPLIT, &mV, b.Vb, D, M, D, Epi::BK, Epi::BOX_B / 64));
+        return launch_persist<Epi>(ctx, mA, mV, tiles, cdiv(M, Epi::BK), cy, true, fp, b.err, st, mE, &mdF,
+                                   prefetch ? b.A : nullptr, n, 2 * M);
+    };
     if (SPLIT && fp.F_dtype == LATENTAM_DTYPE_F32) {
         // FP32 targets by TMA, 32 columns at a time; dFhat written over them as 32-column planes
-        CUtensorMap mF;
         LAT_TRY(f32_map(&mF, fp.F, D, n, kTileM));
         LAT_TRY(io_map(true, &mdF, fp.dF, D, n, D, kTileM, 32));
-        return launch_persist<FhatEpi<true, false, true>>(ctx, mA, mV, tiles, kc, cy, true, fp, b.err, st, &mF, &mdF);
+        return launch(FhatEpi<true, false, true>{}, &mF, false);
     }
     LAT_TRY(io_map(SPLIT, &mdF, fp.dF, D, n, D, kTileM));
     if (!SPLIT && fp.F_dtype == LATENTAM_DTYPE_BF16) {
         // BF16 targets: the tile's target rows are TMA-loaded into shared memory for the epilogue
-        CUtensorMap mF;
         LAT_TRY(bf16_map(&mF, fp.F, D, n, D, kTileM));
         // Past 512 atoms the operand ring takes longer than an epilogue with its target's load and
-        // store: one tile of target boxes and five stages.  (300,000 rows, whole decode with two
+        // store: one tile of target boxes and twice the ring.  (300,000 rows, whole decode with two
         // tiles / one: M = 256 500 / 560 us, 512 x 768 1,099 / 1,115, 768 x 256 1,016 / 980,
         // 1024 x 768 2,140 / 2,002.)
-        if (M > 512)
-            return launch_persist<FhatEpi<true, false, false, 4>>(ctx, mA, mV, tiles, kc, cy, true, fp, b.err, st, &mF,
-                                                                  &mdF, b.A, n, 2 * M);
-        return launch_persist<FhatEpi<true>>(ctx, mA, mV, tiles, kc, cy, true, fp, b.err, st, &mF, &mdF, b.A, n,
-                                             2 * M);
+        // There, on CTA pairs unless the cluster of a row tile's pairs gets too large for what they
+        // save (200,000 rows, whole decode single / pairs: M = 544 x 256 578 / 571, x 512 713 / 725,
+        // x 1024 1,066 / 1,132; 768 x 512 804 / 793, x 768 992 / 971, x 1024 1,152 / 1,191; 1024 x
+        // 768 1,231 / 1,169).  Up to 512 atoms, where the epilogues bind, pairs lose (300,000 rows,
+        // 256 x 512 501 / 531; FP32 targets and operands 933 / 952).
+        if (M > 512 && (D <= 256 || (M >= 768 && D <= 768)))
+            return launch(FhatEpi<true, false, false, 4, true>{}, &mF, true);
+        if (M > 512) return launch(FhatEpi<true, false, false, 4>{}, &mF, true);
+        return launch(FhatEpi<true>{}, &mF, true);
     }
-    return launch_persist<EpiF>(ctx, mA, mV, tiles, kc, cy, true, fp, b.err, st, nullptr, &mdF);
+    return launch(FhatEpi<false, false, SPLIT>{}, nullptr, false);  // targets read per thread (FP32 or BF16)
 }
 
 // G2 on E4M3 operands: the attention rows scaled per pixel (from the softmax row statistics)
@@ -1381,13 +1423,13 @@ latentam_status tc_fhat_out(latentam_ctx* ctx, const TcBuffers& b, int64_t n, in
         LAT_TRY(u8_map(&mV, b.Vtq, M, D, M, 256));
     } else {
         LAT_TRY(op_map(Epi::SPLIT, &mA, b.A, M, n, M, kTileM, Epi::BK));
-        LAT_TRY(mn_map(Epi::SPLIT, &mV, b.Vb, D, M, D, Epi::BK, Epi::BN / 64));
+        LAT_TRY(mn_map(Epi::SPLIT, &mV, b.Vb, D, M, D, Epi::BK, Epi::BOX_B / 64));
     }
     LAT_TRY(f32_map(&mO, F_hat, D, n, 32));  // one warp's rows per box
     const FhatParams fp{n, D, nullptr, LATENTAM_DTYPE_F32, nullptr, latentam_loss_cfg{}, nullptr, nullptr, nullptr,
                         b.stats, b.inv_t};
     return launch_persist<Epi>(ctx, mA, mV, cdiv(n, kTileM), cdiv(M, Epi::BK), cdiv(D, 256), false, fp, b.err, st,
-                               nullptr, &mO);
+                               nullptr, &mO, Epi::PAIR && !Epi::SPLIT ? b.A : nullptr, n, 2 * M);
 }
 
 // The six contractions of the decode, its loss and its backward.  SPLIT: the FP32 form, every
@@ -1460,8 +1502,18 @@ latentam_status tc_loss_bwd(latentam_ctx* ctx, const DecodeArgs& a, cudaStream_t
         CUtensorMap mAe, mdSo;  // attention rows for the epilogue, dS out through the TMA
         LAT_TRY(io_map(SPLIT, &mAe, b.A, M, n, M, kTileM));
         LAT_TRY(io_map(SPLIT, &mdSo, b.dS, M, n, M, kTileM));
-        LAT_TRY((launch_gemm<DsEpi<SPLIT>>(mdF, mV, dim3(cdiv(n, kTileM) * ty, 1, 1), g3, dp, b.err, st, &mAe, &mdSo, 1,
-                                           dq_fused ? &mK : nullptr, dk_fused ? &mQt : nullptr)));
+        // pairs need long enough main loops (200,000 rows, whole decode one-tile kernel / pairs: M =
+        // 1024 x 256 795 / 797 us, x 512 962 / 916, x 768 1,168 / 1,112; 768 x 128 599 / 628, x 512
+        // 787 / 756; 544 x 512 726 / 714)
+        if (!SPLIT && M > 512 && D >= 512) {
+            CUtensorMap mVh;
+            LAT_TRY(bf16_map(&mVh, b.Vb, D, M, D, DsPairEpi::BOX_B));
+            LAT_TRY(launch_persist<DsPairEpi>(ctx, mdF, mVh, cdiv(n, kTileM), cdiv(D, 64), ty, false, dp, b.err, st,
+                                              &mAe, &mdSo, b.dF, n, 2 * D));
+        } else {
+            LAT_TRY((launch_gemm<DsEpi<SPLIT>>(mdF, mV, dim3(cdiv(n, kTileM) * ty, 1, 1), g3, dp, b.err, st, &mAe,
+                                               &mdSo, 1, dq_fused ? &mK : nullptr, dk_fused ? &mQt : nullptr)));
+        }
         if (a.dQ && !dq_fused) {
             LAT_TRY(op_map(SPLIT, &mdS, b.dS, M, n, M, kTileM));
             DqParams qp{n, d, a.c, a.dQ};
@@ -1568,6 +1620,11 @@ latentam_status tc_fwd(latentam_ctx* ctx, const float* Q, int64_t n, int d, cons
     if (!F_hat) return LATENTAM_OK;
     if constexpr (!SPLIT)
         if (fp8) return tc_fhat_out<FhatOutEpi<true>>(ctx, b, n, M, D, F_hat, st);
+    // CTA pairs once the operand loads outweigh what the two CTAs wait for each other (whole decode
+    // of 300,000 rows, D = 512, single / pairs: BF16 M = 192 196 / 196 us, 256 195 / 217, 384
+    // 290 / 275, 512 317 / 302; FP32 128 209 / 235, 192 269 / 265, 256 316 / 298, 512 522 / 489,
+    // 1024 1,054 / 925)
+    if (M >= (SPLIT ? 256 : 384)) return tc_fhat_out<FhatOutEpi<false, SPLIT, true>>(ctx, b, n, M, D, F_hat, st);
     return tc_fhat_out<FhatOutEpi<false, SPLIT>>(ctx, b, n, M, D, F_hat, st);
 }
 

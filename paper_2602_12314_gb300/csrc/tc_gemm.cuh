@@ -201,6 +201,7 @@ struct EpiCtx {
     // Epi::WARP_STAGE: this warp's own staging bytes, stored by the warp itself to *omap
     uint8_t* xstage = nullptr;
     const CUtensorMap* omap = nullptr;
+    int xstep = 1, xbase = 0;  // CTA q of the row exchange is the cluster's CTA q * xstep + xbase
 
     // In-place split form (Epi::INPLACE): the tile's FP32 epilogue operand sits in the box
     // buffers as 32-column chunks (128 rows x 128 B, 128-byte swizzle, chunk c at c x 16 KB), and
@@ -265,8 +266,8 @@ struct EpiCtx {
             for (int q = 0; q < csize; ++q) {
                 if (q == crank) continue;
                 const int slot = 1 + (crank < q ? crank : crank - 1);  // this CTA's slot at q
-                bulk_copy_to_peer(peer_addr(xbuf + slot * (kXchgMsg / 4), (uint32_t)q), xbuf, kXchgMsg,
-                                  peer_addr(xbar, (uint32_t)q));
+                const uint32_t to = (uint32_t)(q * xstep + xbase);
+                bulk_copy_to_peer(peer_addr(xbuf + slot * (kXchgMsg / 4), to), xbuf, kXchgMsg, peer_addr(xbar, to));
             }
         }
         const bool ok = mbar_wait_long(xbar, xphase);
@@ -342,13 +343,13 @@ struct EpiCtx {
 };
 
 // One MMA step of the product: A x B (plain) or, split, A_hi B_hi + A_hi B_lo + A_lo B_hi.
-template <bool SPLIT>
+template <bool SPLIT, bool PAIR = false>
 __device__ __forceinline__ void mma_step(uint32_t d, uint64_t a_hi, uint64_t a_lo, uint64_t b_hi, uint64_t b_lo,
                                          uint32_t idesc, uint32_t acc) {
-    mma_bf16(d, a_hi, b_hi, idesc, acc);
+    mma_bf16<PAIR>(d, a_hi, b_hi, idesc, acc);
     if (SPLIT) {
-        mma_bf16(d, a_hi, b_lo, idesc, 1u);
-        mma_bf16(d, a_lo, b_hi, idesc, 1u);
+        mma_bf16<PAIR>(d, a_hi, b_lo, idesc, 1u);
+        mma_bf16<PAIR>(d, a_lo, b_hi, idesc, 1u);
     }
 }
 
@@ -826,6 +827,12 @@ __global__ void __launch_bounds__(gemm_threads(Epi::EPI_WG), Epi::MIN_BLOCKS)
 // An epilogue with WARP_STAGE bytes per warp (a multiple of 1024) needs no box buffers: each warp
 // stages and TMA-stores its own 32 rows (EpiCtx::xstage, EpiCtx::omap) and waits for the read of
 // its last store itself.
+// An epilogue with PAIR runs on CTA pairs (neighbours in x, one cluster with the row exchange's CTAs
+// along y): a pair takes two row tiles at a time and the even CTA issues 256-row MMAs for both
+// (cta_group::2), each CTA holding its own 128 rows of A and half of the tile's B.  So a CTA loads
+// and reads 128 + BN / 2 instead of 128 + BN operand rows per K chunk.  full[] and acc_empty[] are
+// then the even CTA's (both CTAs' copies, both epilogues); empty[] and acc_full[] are signalled in
+// both.
 struct PersistGrid {
     int k_chunks;   // Epi::BK-wide K chunks per tile
     int row_tiles;  // 128-row tiles of A
@@ -847,11 +854,11 @@ __host__ __device__ constexpr uint32_t persist_box_bytes() {  // half of the box
                               : (uint32_t)Epi::O_BOXES * kTileABytes;
 }
 
-// One ring stage: A (128 x BK) and B (BN x BK) elements of Epi::ELEM bytes (2: BF16, 1: E4M3),
+// One ring stage: A (128 x BK) and B (BN x BK, a CTA of a pair half) elements of Epi::ELEM bytes (2: BF16, 1: E4M3),
 // each in both planes in the split form ([A hi][A lo][B hi][B lo]).
 template <class Epi>
 __host__ __device__ constexpr uint32_t persist_stage_bytes() {
-    return (uint32_t)planes<Epi>() * (kTileM + Epi::BN) * Epi::BK * Epi::ELEM;
+    return (uint32_t)planes<Epi>() * (kTileM + (Epi::PAIR ? Epi::BN / 2 : Epi::BN)) * Epi::BK * Epi::ELEM;
 }
 
 __host__ __device__ constexpr int persist_threads(int epi_warpgroups) { return 96 + 128 * epi_warpgroups; }
@@ -878,18 +885,21 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
     constexpr bool SPLIT = Epi::SPLIT;
     constexpr int PL = planes<Epi>();
     constexpr uint32_t A_BYTES = (uint32_t)kTileM * ROWB;          // per plane
-    constexpr uint32_t B_BYTES = (uint32_t)Epi::BN * BK * ELEM;    // per plane
+    constexpr bool PAIR = Epi::PAIR;
+    constexpr int NB = PAIR ? BN / 2 : BN;                   // B rows held by this CTA
+    constexpr uint32_t B_BYTES = (uint32_t)NB * BK * ELEM;   // per plane
     constexpr uint32_t STAGE_BYTES = persist_stage_bytes<Epi>();
     constexpr uint32_t PIPE_BYTES = STAGES * STAGE_BYTES;
     constexpr uint32_t MN_BOX = 64u * BK * 2;  // one 64 (MN) x BK (K) box of an MN-major operand
     constexpr uint32_t BOX_BYTES = persist_box_bytes<Epi>();
     constexpr bool A_MN = Epi::A_MN, B_MN = Epi::B_MN;
-    constexpr uint32_t IDESC = ELEM == 1 ? idesc_e4m3(kTileM, BN) : idesc_bf16(kTileM, BN, A_MN, B_MN);
+    constexpr int MMA_M = PAIR ? 2 * kTileM : kTileM;
+    constexpr uint32_t IDESC = ELEM == 1 ? idesc_e4m3(MMA_M, BN) : idesc_bf16(MMA_M, BN, A_MN, B_MN);
     constexpr int E_BOXES = Epi::E_BOXES, O_BOXES = Epi::O_BOXES;
     static_assert(BN % 16 == 0 && BN <= 256, "two accumulators of BN <= 256 columns fill TMEM");
     static_assert(ELEM == 2 || (ELEM == 1 && !B_MN), "E4M3 operands are read K-major");
-    static_assert(BN % BOX_B == 0 && BOX_B <= 256 && (BOX_B * 128) % 1024 == 0, "bad B box");
-    static_assert(!B_MN || BN % 64 == 0, "an MN-major B tile is made of 64-wide boxes");
+    static_assert(NB % BOX_B == 0 && BOX_B <= 256 && (BOX_B * 128) % 1024 == 0, "bad B box");
+    static_assert(!B_MN || NB % 64 == 0, "an MN-major B tile is made of 64-wide boxes");
     constexpr bool INPLACE = Epi::INPLACE;  // split: FP32 operand chunks in, output over them
     static_assert(E_BOXES == 0 || INPLACE || (E_BOXES == 4 && Epi::SLOTS >= 4 && Epi::SLOTS <= 8 && Epi::SLOTS % 2 == 0),
                   "box ring");
@@ -898,7 +908,7 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
     static_assert(!A_MN, "the persistent tile reads A K-major");
     static_assert(!SPLIT || (ELEM == 2 && (E_BOXES == 0 || INPLACE)), "split form: BF16 planes");
     static_assert(!INPLACE || (SPLIT && E_BOXES == 8 && 2 * BOX_BYTES == 8 * 16384), "in-place chunks fill both buffers");
-    static_assert(!SPLIT || B_MN || BOX_B == BN, "a split K-major B tile is one box");
+    static_assert(!SPLIT || B_MN || BOX_B == NB, "a split K-major B tile is one box");
     static_assert(STAGE_BYTES % 1024 == 0 && A_BYTES % 1024 == 0, "stages stay 1024-byte aligned");
 
     extern __shared__ uint8_t smem_raw[];
@@ -922,14 +932,19 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
     float* scratch = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + 512);
     float* xbufs = scratch + scratch_bytes(G) / 4;
 
-    uint32_t csize = 1;
-    if (Epi::XROUNDS > 0) asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(csize));
-    const uint32_t crank = csize > 1 ? cluster_rank() : 0u;
+    uint32_t nct = 1;  // CTAs of the cluster: csize of the row exchange, times two for pairs
+    if (Epi::XROUNDS > 0 || PAIR) asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(nct));
+    const uint32_t rank = nct > 1 ? cluster_rank() : 0u;
+    const uint32_t half = PAIR ? rank & 1u : 0u, even = rank & ~1u;  // of the pair
+    const uint32_t csize = PAIR ? nct >> 1 : nct, crank = PAIR ? rank >> 1 : rank;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n0 = blockIdx.y * BN;
     const int nk = pg.k_chunks;
     const int first = blockIdx.x, stride = gridDim.x;
-    const int my_tiles = first < pg.row_tiles ? (pg.row_tiles - first + stride - 1) / stride : 0;
+    // the CTAs of a pair take equally many tiles; the odd one's last may lie past the rows (it loads
+    // zeros and stores nothing)
+    const int first_own = PAIR ? first & ~1 : first;
+    const int my_tiles = first_own < pg.row_tiles ? (pg.row_tiles - first_own + stride - 1) / stride : 0;
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < STAGES; ++i) {
@@ -938,7 +953,7 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
         }
         for (int e = 0; e < 2; ++e) {
             mbar_init(&acc_full[e], 1);
-            mbar_init(&acc_empty[e], 1);
+            mbar_init(&acc_empty[e], PAIR ? 2 : 1);
             for (int b = 0; b < (E_BOXES > 0 ? 4 : 0); ++b) mbar_init(&e_full[4 * e + b], 1);
             mbar_init(&e_free[e], 1);
             mbar_init(&staged[e], 1);
@@ -952,11 +967,11 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
         if (E_BOXES > 0) prefetch_tmap(&tmE);
         if (O_BOXES > 0) prefetch_tmap(&tmO);
     }
-    if (warp == 1) tmem_alloc(tmem_slot, 512);
+    if (warp == 1) tmem_alloc<PAIR>(tmem_slot, 512);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (csize > 1) cluster_sync_all();
+    if (nct > 1) cluster_sync_all();
     const uint32_t tmem_base = *tmem_slot;
 
     if (warp == 0) {
@@ -964,6 +979,8 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
             // ---- TMA producer: operand ring ----
             int it = 0;
             bool ok = true;
+            const uint32_t full0 = PAIR ? peer_addr(full, even) : 0u;  // the even CTA's full[0]
+            const int nh = n0 + (int)half * NB;                        // this CTA's B rows
             for (int lt = 0; lt < my_tiles && ok; ++lt) {
                 const int m0 = (first + lt * stride) * kTileM;
                 // where asked for, the next tile's A rows go to L2 now, so that its ring refills at
@@ -971,7 +988,7 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
                 if (pg.a && blockIdx.y == 0 && lt + 1 < my_tiles) {
                     const int64_t r0 = (int64_t)(first + (lt + 1) * stride) * kTileM;
                     const int64_t rows = min((int64_t)kTileM, pg.a_rows - r0);
-                    bulk_prefetch_l2(pg.a + r0 * pg.a_row_bytes, (uint32_t)(rows * pg.a_row_bytes));
+                    if (rows > 0) bulk_prefetch_l2(pg.a + r0 * pg.a_row_bytes, (uint32_t)(rows * pg.a_row_bytes));
                 }
                 for (int i = 0; i < nk; ++i, ++it) {
                     const int s = it % STAGES;
@@ -980,10 +997,28 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
                         break;
                     }
                     const int kx = i * BK;
-                    mbar_expect_tx(&full[s], STAGE_BYTES);
+                    if (half == 0) mbar_expect_tx(&full[s], (PAIR ? 2 : 1) * STAGE_BYTES);
                     uint8_t* sa = smem + s * STAGE_BYTES;
                     uint8_t* sb = sa + PL * A_BYTES;
-                    if (SPLIT) {  // one box holds both planes (see tc_gemm_kernel)
+                    if (PAIR) {
+                        const uint32_t bar = full0 + 8u * (uint32_t)s;
+                        if (SPLIT) {
+                            tma_load_3d_pair(sa, &tmA, bar, kx, m0, 0);
+                            if (B_MN)
+                                tma_load_4d_pair(sb, &tmB, bar, 0, kx, nh / 64, 0);
+                            else
+                                tma_load_3d_pair(sb, &tmB, bar, kx, nh, 0);
+                        } else {
+                            tma_load_2d_pair(sa, &tmA, bar, kx, m0);
+                            if (B_MN) {
+                                tma_load_3d_pair(sb, &tmB, bar, 0, kx, nh / 64);
+                            } else {
+#pragma unroll
+                                for (int b = 0; b < NB / BOX_B; ++b)
+                                    tma_load_2d_pair(sb + b * BOX_B * ROWB, &tmB, bar, kx, nh + b * BOX_B);
+                            }
+                        }
+                    } else if (SPLIT) {  // one box holds both planes (see tc_gemm_kernel)
                         tma_load_3d(sa, &tmA, &full[s], kx, m0, 0);
                         if (B_MN)
                             tma_load_4d(sb, &tmB, &full[s], 0, kx, n0 / 64, 0);
@@ -1003,9 +1038,15 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
             }
             if (!ok) {
                 *abort_flag = 1;
-                // never leave the CTA with copies in flight
-                for (int j = max(0, it - STAGES); j < it; ++j)
-                    (void)mbar_wait(&full[j % STAGES], (uint32_t)(j / STAGES) & 1u, nullptr);
+                // never leave the CTA with copies in flight (those of a pair's odd CTA report to the
+                // even one, which waits for them where it issued its own: give the others 1 ms)
+                if (half == 0) {
+                    for (int j = max(0, it - STAGES); j < it; ++j)
+                        (void)mbar_wait(&full[j % STAGES], (uint32_t)(j / STAGES) & 1u, nullptr);
+                } else {
+                    const uint64_t t0 = global_timer_ns();
+                    while (global_timer_ns() - t0 < 1000000ull) __nanosleep(1000);
+                }
             }
         }
     } else if (warp == 2 && INPLACE) {
@@ -1154,8 +1195,14 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
             }
         }
     } else if (warp == 1) {
-        if (lane == 0 && nk > 0) {
-            // ---- MMA issuer ----
+        if (lane == 0 && nk > 0 && half == 0) {
+            // ---- MMA issuer (of a pair: the even CTA) ----
+            auto commit = [&](uint64_t* bar) {
+                if (PAIR)
+                    mma_commit_pair(bar, (uint16_t)(3u << even));
+                else
+                    mma_commit(bar);
+            };
             int it = 0;
             bool ok = true;
             for (int lt = 0; lt < my_tiles && ok; ++lt) {
@@ -1183,22 +1230,25 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
                         const uint64_t da = kdesc(sa + kk * 32);
                         const uint64_t db = B_MN ? mn128_desc(sb + kk * 16 * 128, MN_BOX) : kdesc(sb + kk * 32);
                         if (ELEM == 1) {
-                            mma_e4m3(dst, da, db, IDESC, (i > 0 || kk > 0) ? 1u : 0u);
+                            mma_e4m3<PAIR>(dst, da, db, IDESC, (i > 0 || kk > 0) ? 1u : 0u);
                         } else {
                             const uint64_t dal = kdesc(sa + A_BYTES + kk * 32);
                             const uint64_t dbl =
                                 B_MN ? mn128_desc(sb + B_BYTES + kk * 16 * 128, MN_BOX) : kdesc(sb + B_BYTES + kk * 32);
-                            mma_step<SPLIT>(dst, da, dal, db, dbl, IDESC, (i > 0 || kk > 0) ? 1u : 0u);
+                            mma_step<SPLIT, PAIR>(dst, da, dal, db, dbl, IDESC, (i > 0 || kk > 0) ? 1u : 0u);
                         }
                     }
-                    mma_commit(&empty[s]);
+                    commit(&empty[s]);
                 }
                 if (!ok) break;
-                mma_commit(&acc_full[buf]);
+                commit(&acc_full[buf]);
             }
             if (!ok) *abort_flag = 1;
             // every MMA issued by this thread has completed before TMEM is released
-            mma_commit(drain);
+            if (PAIR)
+                mma_commit_pair(drain);
+            else
+                mma_commit(drain);
             (void)mbar_wait(drain, 0, nullptr);
         }
     } else {
@@ -1242,6 +1292,10 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
                 ec.ofree = &e_free[0];
                 ec.ofree_phase = (uint32_t)lt & 1u;
             }
+            if (PAIR) {
+                ec.xstep = 2;
+                ec.xbase = (int)half;
+            }
             if (Epi::WARP_STAGE > 0) {
                 ec.xstage = warp_stage + (warp - 3) * Epi::WARP_STAGE;
                 ec.omap = &tmO;
@@ -1261,7 +1315,10 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
             fence_proxy_async();
             epi_sync(128 * G);
             if (threadIdx.x == 96) {
-                mbar_arrive(&acc_empty[e]);
+                if (PAIR)
+                    mbar_arrive_cluster(peer_addr(&acc_empty[e], even));
+                else
+                    mbar_arrive(&acc_empty[e]);
                 const int sb = SPLIT ? 0 : e;
                 nbox[sb] = *abort_flag ? 0 : out_boxes;
                 mbar_arrive(&staged[sb]);
@@ -1270,12 +1327,13 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
         if (Epi::WARP_STAGE > 0) bulk_wait_read();  // each warp's last store has read its staging
     }
     __syncthreads();
-    // no CTA leaves while a peer may still read or write its shared memory (the row exchange)
-    if (csize > 1) cluster_sync_all();
+    // no CTA leaves while a peer may still read or write its shared memory (the row exchange, a
+    // pair's operands and barriers)
+    if (nct > 1) cluster_sync_all();
     if (*abort_flag && threadIdx.x == 0) atomicExch(err, 1);
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, 512);
+        tmem_dealloc<PAIR>(tmem_base, 512);
     }
 }
 

@@ -24,6 +24,7 @@ def ctx(api):
 
 @pytest.mark.parametrize("precision", ["FP32", "BF16", "FP8"])
 @pytest.mark.parametrize("n,d,M,D", [(1, 16, 32, 128), (33, 32, 96, 384), (129, 64, 288, 640),
+                                     (300, 32, 64, 256),
                                      (45_003, 32, 160, 1024), (2_000, 32, 1024, 768)])
 def test_rows_match_float64(api, ctx, precision, n, d, M, D):
     g = torch.Generator(device="cuda").manual_seed(n + M)

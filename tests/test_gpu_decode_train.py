@@ -1,6 +1,7 @@
 """The training decode past 512 atoms, three and four column tiles a row (BF16: one tile of target
-boxes and five operand stages; dV split into whole waves over the pixels), against float64 PyTorch with the forms' bars: BF16 gradients by norm 2e-2 and
-loss parts 5e-3, FP32 1e-3 and 1e-4; row counts that leave partial tiles and give every CTA several."""
+boxes; single CTAs or CTA pairs, an odd last row tile; dV split into whole waves over the pixels),
+against float64 PyTorch with the forms' bars: BF16 gradients by norm 2e-2 and loss parts 5e-3, FP32
+1e-3 and 1e-4; row counts that leave partial tiles and give every CTA several."""
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -15,7 +16,8 @@ def api():
 
 @pytest.mark.parametrize("precision,grad_bar,loss_bar", [("BF16", 2e-2, 5e-3), ("FP32", 1e-3, 1e-4)])
 @pytest.mark.parametrize("n,d,M,D", [(130, 32, 544, 128), (41_001, 16, 544, 384), (33_000, 32, 800, 640),
-                                     (20_011, 64, 1024, 1024)])
+                                     (20_011, 64, 1024, 1024),
+                                     (300, 16, 1024, 768), (33_001, 32, 768, 512)])
 def test_gradients_match_float64(api, n, d, M, D, precision, grad_bar, loss_bar):
     g = torch.Generator(device="cuda").manual_seed(n)
     Q = torch.randn(n, d, generator=g, device="cuda")
