@@ -316,13 +316,22 @@ struct SoftmaxParams {
 // and combine their (row max, partial denominator) pairs before normalising.
 // SPLIT_: the FP32 form (queries, keys and A as hi / lo BF16 planes, three MMAs per product):
 // 16-wide K chunks over the d query columns, three ring stages.
+// Bound by latency: a tile is 512 cycles of MMAs between dependent waits (accumulator, row maximum,
+// row sum, cluster exchange, staging), with the A rows written at 2.9 - 4 TB/s.  So the plain form
+// keeps its tile of keys in shared memory and two tiles of queries on the way, two teams of epilogue
+// warps take the tiles in turn, and the exponentials run in packed arithmetic with flushed
+// results below 2^-126 (14 -> 10 warp instructions per 32 logits; the same bits, as the sums keep
+// their order).  Whole decode, together: 300,000 rows M = 1024 D = 768 1,602 -> 1,554 us, M = 512
+// 1,003 -> 985, inference of 816,000 rows M = 512 966 -> 908; two teams with the plain loops alone gave 1,600 -> 1,589.  The split form, whose two
+// staged planes take both buffers, lost 1% with either and keeps one team and the plain loops.
 template <bool SPLIT_ = false>
 struct SoftmaxEpi {
     // plain: one K chunk (the padded queries) per tile
     static constexpr bool SPLIT = SPLIT_, INPLACE = false;
-    static constexpr int BN = 256, BK = SPLIT_ ? 16 : 64, ELEM = 2, STAGES = SPLIT_ ? 3 : 1, BOX_B = 256;
+    static constexpr int BN = 256, BK = SPLIT_ ? 16 : 64, ELEM = 2, STAGES = SPLIT_ ? 3 : 2, BOX_B = 256;
     static constexpr int EPI_WG = 4, E_BOXES = 0, O_BOXES = 4;
-    static constexpr int XROUNDS = 1, WARP_STAGE = 0, SLOTS = 0;
+    static constexpr int XROUNDS = 1, XVALS = 2, TEAMS = SPLIT_ ? 1 : 2, WARP_STAGE = 0, SLOTS = 0;
+    static constexpr bool BRES = !SPLIT_;
     static constexpr bool PAIR = false;
     static constexpr bool A_MN = false, B_MN = false;
     using Params = SoftmaxParams;
@@ -330,32 +339,65 @@ struct SoftmaxEpi {
         const uint32_t taddr = ec.taddr;
         const int row = ec.row, m0 = ec.m0, g = ec.g;
         const int ncols = min(BN, p.M - ec.n0);  // atoms of this CTA's slice
+        constexpr int TG = EPI_WG / TEAMS;  // warpgroups on this tile
         float* scr = ec.scratch;
         const int64_t pix = (int64_t)m0 + row;
         const bool valid = pix < p.n;
         float mx = -INFINITY;
-        for (int c0 = 32 * g; c0 < ncols; c0 += 32 * EPI_WG) {
+        for (int c0 = 32 * g; c0 < ncols; c0 += 32 * TG) {
             float v[32];
             tc::tmem_ld32(taddr + c0, v);
 #pragma unroll
             for (int i = 0; i < 32; ++i) mx = fmaxf(mx, v[i]);
         }
-        mx = tc::group_max<EPI_WG>(mx, scr, 0, g, row);
+        mx = tc::group_max<TG>(mx, scr, 0, g, row, ec.bar);
         float cm = p.c * mx;  // c > 0
         // the exponentials are taken once and written back over S in TMEM (this thread's lane
-        // and chunks only), then scaled by the row's normaliser on the way out
+        // and chunks only), then scaled by the row's normaliser on the way out; the chunks' sums are
+        // added in chunk order, whatever the teams
         float sum = 0.f;
-        for (int c0 = 32 * g; c0 < ncols; c0 += 32 * EPI_WG) {
-            float v[32];
-            tc::tmem_ld32(taddr + c0, v);
+        if constexpr (SPLIT) {
+            for (int c0 = 32 * g; c0 < ncols; c0 += 32 * TG) {
+                float v[32];
+                tc::tmem_ld32(taddr + c0, v);
 #pragma unroll
-            for (int i = 0; i < 32; ++i) {
-                v[i] = __expf(p.c * v[i] - cm);
-                sum += v[i];
+                for (int i = 0; i < 32; ++i) {
+                    v[i] = __expf(p.c * v[i] - cm);
+                    sum += v[i];
+                }
+                tc::tmem_st32(taddr + c0, v);
             }
-            tc::tmem_st32(taddr + c0, v);
+            sum = tc::group_sum<TG>(sum, scr, 1, g, row);
+        } else {
+            const Pair scale(p.c), shift(-cm), log2e(1.44269504088896341f);
+            float part0 = 0.f, part1 = 0.f;  // of the chunks g and g + TG modulo EPI_WG
+            for (int c0 = 32 * g; c0 < ncols; c0 += 32 * TG) {
+                float v[32];
+                tc::tmem_ld32(taddr + c0, v);
+                const bool second = ((c0 >> 5) / TG) & 1;
+                float s = second ? part1 : part0;
+#pragma unroll
+                for (int i = 0; i < 32; i += 2) {
+                    float x0, x1;
+                    mul2(fma2(scale, Pair(v[i], v[i + 1]), shift), log2e).get(x0, x1);
+                    v[i] = tc::exp2_ftz(x0);
+                    v[i + 1] = tc::exp2_ftz(x1);
+                    s += v[i];
+                    s += v[i + 1];
+                }
+                tc::tmem_st32(taddr + c0, v);
+                if (second)
+                    part1 = s;
+                else
+                    part0 = s;
+            }
+            float* sums = scr + TG * tc::kTileM;
+            sums[g * tc::kTileM + row] = part0;
+            sums[(g + TG) * tc::kTileM + row] = part1;
+            tc::epi_sync(128 * TG, ec.bar);
+#pragma unroll
+            for (int q = 0; q < EPI_WG; ++q) sum += sums[q * tc::kTileM + row];
         }
-        sum = tc::group_sum<EPI_WG>(sum, scr, 1, g, row);
         const float mine[tc::kXchgVals] = {cm, sum, 0.f, 0.f};
         ec.exchange(mine);
         float rescale = 1.f;  // exp(cm - global max) when the row spans a cluster
@@ -372,7 +414,7 @@ struct SoftmaxEpi {
         }
         const float il = rescale / sum;
         ec.wait_out();
-        for (int c0 = 32 * g; c0 < ncols; c0 += 32 * EPI_WG) {
+        for (int c0 = 32 * g; c0 < ncols; c0 += 32 * TG) {
             float v[32];
             tc::tmem_ld32(taddr + c0, v);
 #pragma unroll
@@ -444,7 +486,8 @@ struct FhatOutEpi {
     static constexpr bool SPLIT = SPLIT_, INPLACE = false;
     static constexpr int ELEM = Q8 ? 1 : 2, BK = SPLIT_ ? 32 : 64, STAGES = PAIR_ ? 4 : Q8 ? 6 : 3;
     static constexpr int BN = 256, BOX_B = PAIR_ ? 128 : 256, EPI_WG = 4, XROUNDS = 0, E_BOXES = 0, O_BOXES = 0;
-    static constexpr int WARP_STAGE = 4096, SLOTS = 0;
+    static constexpr int WARP_STAGE = 4096, SLOTS = 0, XVALS = 0, TEAMS = 1;
+    static constexpr bool BRES = false;
     static constexpr bool A_MN = false, B_MN = !Q8, PAIR = PAIR_;
     using Params = FhatParams;
     static __device__ int run(const Params& p, const tc::EpiCtx& ec) {
@@ -491,7 +534,8 @@ struct FhatEpi {
     // persistent, 64-byte K chunks (three ring stages fit beside two epilogue buffers), 128-byte ones in a pair
     static constexpr int ELEM = Q8 ? 1 : 2, BK = SPLIT_ ? 16 : PAIR ? 64 : 64 / ELEM;
     static constexpr int BN = 256, STAGES = PAIR ? 4 : SLOTS == 4 ? 5 : 3, BOX_B = PAIR ? 128 : 256;
-    static constexpr int EPI_WG = ETILE ? 4 : 2, XROUNDS = 1, WARP_STAGE = 0;
+    static constexpr int EPI_WG = ETILE ? 4 : 2, XROUNDS = 1, XVALS = 4, TEAMS = 1, WARP_STAGE = 0;
+    static constexpr bool BRES = false;
     // dFhat staged over the target
     static constexpr int E_BOXES = INPLACE ? 8 : ETILE ? BN / 64 : 0, O_BOXES = BN / 64;
     // B = V (atoms x features, features contiguous: MN-major) or, for E4M3, V^T (K-major)
@@ -744,7 +788,9 @@ struct DsEpi {
 struct DsPairEpi {
     static constexpr bool SPLIT = false, INPLACE = false, PAIR = true;
     static constexpr int ELEM = 2, BK = 64, STAGES = 4, BN = 256, BOX_B = 128;
-    static constexpr int EPI_WG = 4, XROUNDS = 0, WARP_STAGE = 0, SLOTS = 4, E_BOXES = 4, O_BOXES = 4;
+    static constexpr int EPI_WG = 4, XROUNDS = 0, XVALS = 0, TEAMS = 1, WARP_STAGE = 0;
+    static constexpr bool BRES = false;
+    static constexpr int SLOTS = 4, E_BOXES = 4, O_BOXES = 4;
     static constexpr bool A_MN = false, B_MN = false;
     using Params = DsParams;
     static __device__ int run(const Params& p, const tc::EpiCtx& ec) {

@@ -44,6 +44,29 @@ inline CamParams cam_params(const latentam_camera& c) {
     return p;
 }
 
+// Two FP32 values for the packed arithmetic (each half rounded as its own).
+struct Pair {
+    uint64_t v;
+    __device__ __forceinline__ Pair() {}
+    __device__ __forceinline__ Pair(float a, float b) { asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b)); }
+    __device__ __forceinline__ explicit Pair(float a) : Pair(a, a) {}
+    __device__ __forceinline__ void get(float& a, float& b) const {
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+    }
+};
+__device__ __forceinline__ Pair fma2(Pair a, Pair b, Pair c) {
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(c.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return c;
+}
+__device__ __forceinline__ Pair mul2(Pair a, Pair b) {
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(a.v) : "l"(a.v), "l"(b.v));
+    return a;
+}
+__device__ __forceinline__ Pair add2(Pair a, Pair b) {
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(a.v) : "l"(a.v), "l"(b.v));
+    return a;
+}
+
 // Workspace slots owned by the context.
 enum Slot : int {
     WS_BIN_WORDS = 0,  // counters of binning slot 0: per-tile counts, look-back words

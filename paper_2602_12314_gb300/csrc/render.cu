@@ -39,28 +39,6 @@ __device__ __forceinline__ float splat_alpha(float2 m, float4 q, float px, float
     return fminf(kAlphaMax, __fmul_rn(q.w, __expf(power)));
 }
 
-// Two FP32 values for the packed arithmetic (each half rounded as its own).
-struct Pair {
-    uint64_t v;
-    __device__ __forceinline__ Pair() {}
-    __device__ __forceinline__ Pair(float a, float b) { asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b)); }
-    __device__ __forceinline__ explicit Pair(float a) : Pair(a, a) {}
-    __device__ __forceinline__ void get(float& a, float& b) const {
-        asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-    }
-};
-__device__ __forceinline__ Pair fma2(Pair a, Pair b, Pair c) {
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(c.v) : "l"(a.v), "l"(b.v), "l"(c.v));
-    return c;
-}
-__device__ __forceinline__ Pair mul2(Pair a, Pair b) {
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(a.v) : "l"(a.v), "l"(b.v));
-    return a;
-}
-__device__ __forceinline__ Pair add2(Pair a, Pair b) {
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(a.v) : "l"(a.v), "l"(b.v));
-    return a;
-}
 // a.xy += w v.xy
 __device__ __forceinline__ void fma2(float& a0, float& a1, float w, float v0, float v1) {
     fma2(Pair(w), Pair(v0, v1), Pair(a0, a1)).get(a0, a1);

@@ -24,8 +24,8 @@ __host__ __device__ constexpr int scratch_bytes(int groups) { return 4 * groups 
 constexpr int kScratchBytes = scratch_bytes(2);
 constexpr int kMaxCluster = 4;                         // CTAs of a cluster that trade row partials
 constexpr int kXchgVals = 4;                           // values per row per CTA in one exchange
-constexpr int kXchgMsg = kXchgVals * kTileM * 4;       // one CTA's partials of a tile (bytes)
-constexpr int kXchgBytes = kMaxCluster * kXchgMsg;     // one outgoing + (kMaxCluster - 1) incoming
+// one exchange of `vals` values per row: one outgoing + (kMaxCluster - 1) incoming blocks
+__host__ __device__ constexpr int xchg_bytes(int vals) { return kMaxCluster * vals * kTileM * 4; }
 constexpr int kChunkK = 64;                       // BF16 elements per 128-byte row
 constexpr uint32_t kTileABytes = kTileM * 128;    // 16 KB
 
@@ -84,23 +84,14 @@ __host__ __device__ constexpr size_t gemm_smem_bytes() {
 
 __host__ __device__ constexpr int gemm_threads(int epi_warpgroups) { return 64 + 128 * epi_warpgroups; }
 
-// Barrier among the epilogue threads only (named barrier 1).
-__device__ __forceinline__ void epi_sync(int nthreads) {
-    asm volatile("bar.sync 1, %0;" ::"r"(nthreads) : "memory");
+// Barrier among the epilogue threads only (named barrier 1; a second team's: 6).
+__device__ __forceinline__ void epi_sync(int nthreads, int bar = 1) {
+    if (bar == 1)
+        asm volatile("bar.sync 1, %0;" ::"r"(nthreads) : "memory");
+    else
+        asm volatile("bar.sync 6, %0;" ::"r"(nthreads) : "memory");
 }
 
-// Sum (or max) of one value per row over the G epilogue warpgroups, through shared memory.
-// `slot` (0..3) must differ between reductions of the same tile.
-template <int G>
-__device__ __forceinline__ float group_sum(float v, float* scratch, int slot, int g, int row) {
-    if (G == 1) return v;
-    scratch[(slot * G + g) * kTileM + row] = v;
-    epi_sync(128 * G);
-    float s = 0.f;
-#pragma unroll
-    for (int k = 0; k < G; ++k) s += scratch[(slot * G + k) * kTileM + row];
-    return s;
-}
 // The four per-row values v[0..3] summed over the G epilogue warpgroups with one barrier
 // (slots 0..3).
 template <int G>
@@ -117,11 +108,23 @@ __device__ __forceinline__ void group_sum4(float (&v)[4], float* scratch, int g,
         v[k] = s;
     }
 }
+// Sum, or maximum, of one value per row over the G epilogue warpgroups (of a team), through shared
+// memory; `slot` (0..3) must differ between reductions of the same tile.
 template <int G>
-__device__ __forceinline__ float group_max(float v, float* scratch, int slot, int g, int row) {
+__device__ __forceinline__ float group_sum(float v, float* scratch, int slot, int g, int row) {
     if (G == 1) return v;
     scratch[(slot * G + g) * kTileM + row] = v;
     epi_sync(128 * G);
+    float s = 0.f;
+#pragma unroll
+    for (int k = 0; k < G; ++k) s += scratch[(slot * G + k) * kTileM + row];
+    return s;
+}
+template <int G>
+__device__ __forceinline__ float group_max(float v, float* scratch, int slot, int g, int row, int bar = 1) {
+    if (G == 1) return v;
+    scratch[(slot * G + g) * kTileM + row] = v;
+    epi_sync(128 * G, bar);
     float s = -INFINITY;
 #pragma unroll
     for (int k = 0; k < G; ++k) s = fmaxf(s, scratch[(slot * G + k) * kTileM + row]);
@@ -192,7 +195,7 @@ struct EpiCtx {
     int col0 = 0;          // one-tile kernel, epilogue pass: first tile column of the pass's boxes
     uint32_t eplane = 0;   // split form: bytes from the hi to the lo plane of the epilogue operand
     uint32_t oplane = 0;   // split form: bytes from the hi to the lo plane of the staged output
-    uint64_t* ofree = nullptr;  // split persistent form: completes when the staging buffers are free
+    uint64_t* ofree = nullptr;  // persistent form: completes when the staging for this output is free
     uint32_t ofree_phase = 0;
     // persistent plain form with an epilogue operand: its boxes take the slots q0, q0 + 1, ... of a
     // ring of `slots` (0: box b is at b), in the ring's round of parity ephase
@@ -201,6 +204,8 @@ struct EpiCtx {
     // Epi::WARP_STAGE: this warp's own staging bytes, stored by the warp itself to *omap
     uint8_t* xstage = nullptr;
     const CUtensorMap* omap = nullptr;
+    int bar = 1;               // named barrier of the epilogue threads that share this tile
+    int xvals = kXchgVals;     // values per row of an exchange
     int xstep = 1, xbase = 0;  // CTA q of the row exchange is the cluster's CTA q * xstep + xbase
 
     // In-place split form (Epi::INPLACE): the tile's FP32 epilogue operand sits in the box
@@ -239,7 +244,7 @@ struct EpiCtx {
         asm volatile("bar.sync %0, 128;" ::"r"(2 + g) : "memory");
     }
 
-    // Split persistent form: wait until the previous tile's staged output has been read by its
+    // Persistent form: wait until the output staged where this tile's goes has been read by its
     // TMA stores (call before the first put32; a no-op elsewhere).  Bounded.
     __device__ __forceinline__ bool wait_out() const {
         if (!ofree) return true;
@@ -257,17 +262,19 @@ struct EpiCtx {
         if (csize <= 1) return true;
         if (g == 0) {
 #pragma unroll
-            for (int k = 0; k < kXchgVals; ++k) xbuf[k * kTileM + row] = v[k];
+            for (int k = 0; k < kXchgVals; ++k)
+                if (k < xvals) xbuf[k * kTileM + row] = v[k];
             fence_proxy_async();
         }
-        epi_sync(128 * ngroups);
+        epi_sync(128 * ngroups, bar);
+        const int msg = xvals * kTileM;  // floats
         if ((int)threadIdx.x == leader) {
-            mbar_expect_tx(xbar, (uint32_t)((csize - 1) * kXchgMsg));
+            mbar_expect_tx(xbar, (uint32_t)((csize - 1) * msg * 4));
             for (int q = 0; q < csize; ++q) {
                 if (q == crank) continue;
                 const int slot = 1 + (crank < q ? crank : crank - 1);  // this CTA's slot at q
                 const uint32_t to = (uint32_t)(q * xstep + xbase);
-                bulk_copy_to_peer(peer_addr(xbuf + slot * (kXchgMsg / 4), to), xbuf, kXchgMsg, peer_addr(xbar, to));
+                bulk_copy_to_peer(peer_addr(xbuf + slot * msg, to), xbuf, (uint32_t)msg * 4u, peer_addr(xbar, to));
             }
         }
         const bool ok = mbar_wait_long(xbar, xphase);
@@ -277,7 +284,7 @@ struct EpiCtx {
     // Partial k of this thread's row from CTA q (q != crank) of the cluster.
     __device__ __forceinline__ float xval(int q, int k) const {
         const int slot = 1 + (q < crank ? q : q - 1);
-        return xbuf[slot * (kXchgMsg / 4) + k * kTileM + row];
+        return xbuf[(slot * xvals + k) * kTileM + row];
     }
 
     __device__ __forceinline__ int box_at(int b) const {
@@ -820,13 +827,20 @@ __global__ void __launch_bounds__(gemm_threads(Epi::EPI_WG), Epi::MIN_BLOCKS)
 //   acc_full[e]          MMAs of tile lt done -> epilogue              [u & 1]
 //   acc_empty[e]         epilogue done reading TMEM -> MMA (tile lt+2) [(u - 1) & 1]
 //   e_full[slot]         epilogue operand box loaded                   [round of the slot]
-//   e_free[e]            buffer e free for tile lt's output (no operand) [u & 1]
+//   e_free[e]            staging free for tile lt's output (no operand) [u & 1]
 //   staged[e]            output of tile lt staged in buffer e          [u & 1]
 //   xbar[e]              cluster row exchange of tile lt               [u & 1]
+//                        (two teams: xbar[e + 2 (u & 1)]               [(u >> 1) & 1])
 //
 // An epilogue with WARP_STAGE bytes per warp (a multiple of 1024) needs no box buffers: each warp
 // stages and TMA-stores its own 32 rows (EpiCtx::xstage, EpiCtx::omap) and waits for the read of
 // its last store itself.
+// With Epi::TEAMS = 2 the epilogue warpgroups form two teams that take the tiles in turn, each with
+// its own barrier and row-reduction scratch, so that one team computes while the other waits for
+// its row reductions, exchange and staging.  The exchanges of tiles lt and lt + 2 are then not
+// separated by another one, so each accumulator has two exchange buffers, used in turn: a peer
+// that is a tile ahead of this team writes the one it does not read.
+//
 // An epilogue with PAIR runs on CTA pairs (neighbours in x, one cluster with the row exchange's CTAs
 // along y): a pair takes two row tiles at a time and the even CTA issues 256-row MMAs for both
 // (cta_group::2), each CTA holding its own 128 rows of A and half of the tile's B.  So a CTA loads
@@ -858,16 +872,23 @@ __host__ __device__ constexpr uint32_t persist_box_bytes() {  // half of the box
 // each in both planes in the split form ([A hi][A lo][B hi][B lo]).
 template <class Epi>
 __host__ __device__ constexpr uint32_t persist_stage_bytes() {
-    return (uint32_t)planes<Epi>() * (kTileM + (Epi::PAIR ? Epi::BN / 2 : Epi::BN)) * Epi::BK * Epi::ELEM;
+    return (uint32_t)planes<Epi>() * (kTileM + (Epi::BRES ? 0 : Epi::PAIR ? Epi::BN / 2 : Epi::BN)) * Epi::BK *
+           Epi::ELEM;
+}
+
+// With Epi::BRES (one K chunk) the tile of B is loaded once and stays behind the ring.
+template <class Epi>
+__host__ __device__ constexpr uint32_t persist_b_bytes() {
+    return Epi::BRES ? (uint32_t)planes<Epi>() * Epi::BN * Epi::BK * Epi::ELEM : 0u;
 }
 
 __host__ __device__ constexpr int persist_threads(int epi_warpgroups) { return 96 + 128 * epi_warpgroups; }
 
 template <class Epi>
 __host__ __device__ constexpr size_t persist_smem_bytes() {
-    return (size_t)Epi::STAGES * persist_stage_bytes<Epi>() + 2 * persist_box_bytes<Epi>() +
+    return (size_t)Epi::STAGES * persist_stage_bytes<Epi>() + persist_b_bytes<Epi>() + 2 * persist_box_bytes<Epi>() +
            4 * Epi::EPI_WG * Epi::WARP_STAGE + 1024 /* alignment */ + 512 /* barriers */ +
-           scratch_bytes(Epi::EPI_WG) + (Epi::XROUNDS > 0 ? 2 * kXchgBytes : 0);  // one exchange buffer per accumulator
+           scratch_bytes(Epi::EPI_WG) + (Epi::XROUNDS > 0 ? 2 * Epi::TEAMS * xchg_bytes(Epi::XVALS) : 0);
 }
 
 template <class Epi>
@@ -878,7 +899,8 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
     constexpr int BN = Epi::BN;
     constexpr int STAGES = Epi::STAGES;
     constexpr int BOX_B = Epi::BOX_B;
-    constexpr int G = Epi::EPI_WG;
+    constexpr int G = Epi::EPI_WG, TEAMS = Epi::TEAMS, GT = G / TEAMS;  // GT: warpgroups per tile
+    constexpr int NX = 2 * TEAMS;    // exchange buffers
     constexpr int BK = Epi::BK;      // K elements per chunk
     constexpr int ELEM = Epi::ELEM;  // 2: BF16 operands (kind::f16), 1: E4M3 (kind::f8f6f4)
     constexpr int ROWB = BK * ELEM;  // bytes per K-major row: 128, 64 or 32 (that swizzle)
@@ -889,7 +911,8 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
     constexpr int NB = PAIR ? BN / 2 : BN;                   // B rows held by this CTA
     constexpr uint32_t B_BYTES = (uint32_t)NB * BK * ELEM;   // per plane
     constexpr uint32_t STAGE_BYTES = persist_stage_bytes<Epi>();
-    constexpr uint32_t PIPE_BYTES = STAGES * STAGE_BYTES;
+    constexpr bool BRES = Epi::BRES;
+    constexpr uint32_t PIPE_BYTES = STAGES * STAGE_BYTES + persist_b_bytes<Epi>();
     constexpr uint32_t MN_BOX = 64u * BK * 2;  // one 64 (MN) x BK (K) box of an MN-major operand
     constexpr uint32_t BOX_BYTES = persist_box_bytes<Epi>();
     constexpr bool A_MN = Epi::A_MN, B_MN = Epi::B_MN;
@@ -906,6 +929,8 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
     static_assert((E_BOXES <= 4 || INPLACE) && O_BOXES <= 4 && Epi::XROUNDS <= 1 && G <= 4, "epilogue shape");
     static_assert(ROWB == 128 || ROWB == 64 || ROWB == 32, "K chunk rows of 128, 64 or 32 bytes");
     static_assert(!A_MN, "the persistent tile reads A K-major");
+    static_assert(!BRES || (!PAIR && !SPLIT && !B_MN && BOX_B == BN), "the resident B tile is one plain K-major box");
+    static_assert(TEAMS == 1 || (TEAMS == 2 && G % 2 == 0 && E_BOXES == 0), "two teams share no operand boxes");
     static_assert(!SPLIT || (ELEM == 2 && (E_BOXES == 0 || INPLACE)), "split form: BF16 planes");
     static_assert(!INPLACE || (SPLIT && E_BOXES == 8 && 2 * BOX_BYTES == 8 * 16384), "in-place chunks fill both buffers");
     static_assert(!SPLIT || B_MN || BOX_B == NB, "a split K-major B tile is one box");
@@ -923,12 +948,13 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
     uint64_t* e_full = acc_empty + 2;     // [2][4]
     uint64_t* e_free = e_full + 8;        // [2]
     uint64_t* staged = e_free + 2;        // [2]
-    uint64_t* xbars = staged + 2;         // [2]
-    uint64_t* drain = xbars + 2;          // [1]
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+    uint64_t* xbars = staged + 2;         // [NX]
+    uint64_t* drain = xbars + NX;         // [1]
+    uint64_t* bfull = drain + 1;          // [1]: the resident B tile
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bfull + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    volatile int* decision = abort_flag + 1;
-    volatile int* nbox = decision + 1;  // [2]: output boxes staged in each buffer
+    volatile int* decision = abort_flag + 1;  // [TEAMS]
+    volatile int* nbox = decision + TEAMS;    // [2]: output boxes staged in each buffer
     float* scratch = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + 512);
     float* xbufs = scratch + scratch_bytes(G) / 4;
 
@@ -957,8 +983,10 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
             for (int b = 0; b < (E_BOXES > 0 ? 4 : 0); ++b) mbar_init(&e_full[4 * e + b], 1);
             mbar_init(&e_free[e], 1);
             mbar_init(&staged[e], 1);
-            if (csize > 1) mbar_init(&xbars[e], 1);  // this CTA's expect-tx arrival
         }
+        for (int x = 0; x < NX; ++x)
+            if (csize > 1) mbar_init(&xbars[x], 1);  // this CTA's expect-tx arrival
+        if (BRES) mbar_init(bfull, 1);
         mbar_init(drain, 1);
         *abort_flag = 0;
         fence_mbar_init();
@@ -981,6 +1009,10 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
             bool ok = true;
             const uint32_t full0 = PAIR ? peer_addr(full, even) : 0u;  // the even CTA's full[0]
             const int nh = n0 + (int)half * NB;                        // this CTA's B rows
+            if (BRES) {
+                mbar_expect_tx(bfull, persist_b_bytes<Epi>());
+                tma_load_2d(smem + STAGES * STAGE_BYTES, &tmB, bfull, 0, n0);
+            }
             for (int lt = 0; lt < my_tiles && ok; ++lt) {
                 const int m0 = (first + lt * stride) * kTileM;
                 // where asked for, the next tile's A rows go to L2 now, so that its ring refills at
@@ -1026,7 +1058,8 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
                             tma_load_3d(sb, &tmB, &full[s], kx, n0, 0);
                     } else {
                         tma_load_2d(sa, &tmA, &full[s], kx, m0);
-                        if (B_MN) {  // the tile's 64-wide blocks in one box
+                        if (BRES) {
+                        } else if (B_MN) {  // the tile's 64-wide blocks in one box
                             tma_load_3d(sb, &tmB, &full[s], 0, kx, n0 / 64);
                         } else {
 #pragma unroll
@@ -1036,6 +1069,7 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
                     }
                 }
             }
+            if (BRES && !mbar_wait(bfull, 0, nullptr)) ok = false;
             if (!ok) {
                 *abort_flag = 1;
                 // never leave the CTA with copies in flight (those of a pair's odd CTA report to the
@@ -1106,7 +1140,7 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
                 }
                 bulk_commit();
                 bulk_wait_read();
-                mbar_arrive(&e_free[0]);  // tile t + 1 may stage
+                mbar_arrive(&e_free[(t + 1) & 1]);  // tile t + 1 may stage
             }
             if (!ok) {
                 *abort_flag = 1;
@@ -1204,7 +1238,7 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
                     mma_commit(bar);
             };
             int it = 0;
-            bool ok = true;
+            bool ok = !BRES || mbar_wait(bfull, 0, abort_flag);
             for (int lt = 0; lt < my_tiles && ok; ++lt) {
                 const int buf = lt & 1, use = lt >> 1;
                 if (use > 0 && !mbar_wait(&acc_empty[buf], (uint32_t)(use - 1) & 1u, abort_flag)) {
@@ -1221,7 +1255,8 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
                     }
                     tc_fence_after();
                     const uint32_t sa = smem_u32(smem + s * STAGE_BYTES);  // A hi (then A lo)
-                    const uint32_t sb = sa + PL * A_BYTES;                 // B hi (then B lo)
+                    const uint32_t sb =  // B hi (then B lo)
+                        BRES ? smem_u32(smem + STAGES * STAGE_BYTES) : sa + PL * A_BYTES;
                     auto kdesc = [&](uint32_t a) {
                         return ROWB == 128 ? sw128_desc(a) : ROWB == 64 ? sw64_desc(a) : sw32_desc(a);
                     };
@@ -1254,24 +1289,28 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
     } else {
         // ---- epilogue warps (3 ..) ----
         const int quarter = warp & 3;
-        const int group = (warp - 3) >> 2;
+        const int team = TEAMS == 1 ? 0 : ((warp - 3) >> 2) / GT, group = ((warp - 3) >> 2) - team * GT;
         const int row = quarter * 32 + lane;
-        for (int lt = 0; lt < my_tiles; ++lt) {
+        const int bar = team == 0 ? 1 : 6, head = 96 + 128 * GT * team;  // head: the team's first thread
+        float* tscratch = scratch + team * (scratch_bytes(GT) / 4);
+        for (int lt = team; lt < my_tiles; lt += TEAMS) {
             const int e = lt & 1, use = lt >> 1;
             const int tile = first + lt * stride;
-            bool ready = nk > 0 && mbar_wait(&acc_full[e], (uint32_t)use & 1u, abort_flag);
-            if (!SPLIT && ready && E_BOXES == 0 && O_BOXES > 0)
-                ready = mbar_wait(&e_free[e], (uint32_t)use & 1u, abort_flag);
+            const bool ready = nk > 0 && mbar_wait(&acc_full[e], (uint32_t)use & 1u, abort_flag);
             tc_fence_after();
             if (!ready) *abort_flag = 1;
-            epi_sync(128 * G);
-            if (threadIdx.x == 96) *decision = *abort_flag ? 0 : 1;
-            epi_sync(128 * G);
+            epi_sync(128 * GT, bar);
+            if ((int)threadIdx.x == head) decision[team] = *abort_flag ? 0 : 1;
+            epi_sync(128 * GT, bar);
             uint8_t* box = boxes + e * BOX_BYTES;
+            const int xi = TEAMS == 2 ? e + 2 * (use & 1) : e;
             EpiCtx ec{tmem_base + (uint32_t)(e * BN) + ((uint32_t)(quarter * 32) << 16),
-                      row, tile * kTileM, n0, 0, group, scratch, E_BOXES > 0 ? box : nullptr, box,
-                      &e_full[4 * e], abort_flag, (int)crank, (int)csize, &xbars[e],
-                      xbufs + e * (kXchgBytes / 4), (uint32_t)use & 1u, (uint32_t)use & 1u, G, 96};
+                      row, tile * kTileM, n0, 0, group, tscratch, E_BOXES > 0 ? box : nullptr, box,
+                      &e_full[4 * e], abort_flag, (int)crank, (int)csize, &xbars[xi],
+                      xbufs + xi * (xchg_bytes(Epi::XVALS) / 4), (uint32_t)use & 1u,
+                      (uint32_t)(TEAMS == 2 ? use >> 1 : use) & 1u, GT, head};
+            ec.bar = bar;
+            ec.xvals = Epi::XVALS;
             if (E_BOXES > 0 && !INPLACE) {  // the tile's boxes in the ring, the output written over them
                 constexpr int NS = Epi::SLOTS > 0 ? Epi::SLOTS : 1;
                 const int q = E_BOXES * lt;
@@ -1286,11 +1325,13 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
                 ec.otile = boxes;
                 ec.ebar = e_full;
                 ec.ephase = (uint32_t)lt & 1u;
-            } else if (SPLIT) {  // both buffers hold this tile's output; run() waits for them (wait_out)
-                ec.otile = boxes;
-                ec.oplane = BOX_BYTES;
-                ec.ofree = &e_free[0];
-                ec.ofree_phase = (uint32_t)lt & 1u;
+            } else if (O_BOXES > 0) {  // run() waits for the staging before it writes it (wait_out)
+                if (SPLIT) {  // both buffers hold this tile's output
+                    ec.otile = boxes;
+                    ec.oplane = BOX_BYTES;
+                }
+                ec.ofree = &e_free[e];
+                ec.ofree_phase = (uint32_t)use & 1u;
             }
             if (PAIR) {
                 ec.xstep = 2;
@@ -1301,20 +1342,20 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
                 ec.omap = &tmO;
             }
             int out_boxes = 0;
-            if (*decision) {
-                out_boxes = Epi::run(ep, ec);  // split form: run() calls ec.wait_out() once, on every path
+            if (decision[team]) {
+                out_boxes = Epi::run(ep, ec);  // calls ec.wait_out() once, on every path
             } else {
                 if (Epi::XROUNDS > 0) {
                     const float zero[kXchgVals] = {0.f, 0.f, 0.f, 0.f};
                     (void)ec.exchange(zero);
                 }
-                if (SPLIT && !INPLACE) (void)ec.wait_out();
+                (void)ec.wait_out();
             }
             // TMEM and the staged output are handed over once every epilogue thread is done
             tc_fence_before();
             fence_proxy_async();
-            epi_sync(128 * G);
-            if (threadIdx.x == 96) {
+            epi_sync(128 * GT, bar);
+            if ((int)threadIdx.x == head) {
                 if (PAIR)
                     mbar_arrive_cluster(peer_addr(&acc_empty[e], even));
                 else
