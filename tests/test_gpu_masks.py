@@ -98,6 +98,31 @@ def test_pool_degenerate_inputs(api, ctx):
     assert Qe.shape == (1, 16) and float(Qe.abs().max()) == 0.0
 
 
+@pytest.mark.parametrize("lens", [[1, 63, 64, 65, 0, 255, 256, 257, 1025, 128], [1, 300, 2, 0] + 40 * [3]],
+                         ids=["large", "small"])
+@pytest.mark.parametrize("d", [16, 32, 64])
+def test_pool_chunk_edges(api, ctx, d, lens):
+    """Mask lengths around the 64 entries of a warp and the 256 of a chunk (four warps a chunk), and
+    small masks (one), with invalid pixels, against float64 (means of values of about 1 over up
+    to 1,025 rows: 1e-6)."""
+    rng = np.random.default_rng(d)
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    npix = 500
+    pix = rng.integers(-3, npix + 3, off[-1]).astype(np.int32)
+    Q, G = rng.standard_normal((npix, d)).astype(np.float32), rng.standard_normal((len(lens), d)).astype(np.float32)
+    want, dwant = np.zeros((len(lens), d)), np.zeros((npix, d))
+    for m in range(len(lens)):
+        idx = pix[off[m]:off[m + 1]]
+        idx = idx[(idx >= 0) & (idx < npix)]
+        if len(idx):
+            want[m] = Q[idx].astype(np.float64).mean(0)
+            np.add.at(dwant, idx, G[m].astype(np.float64) / len(idx))
+    got = api.pool_queries(ctx, _dev(Q), off, pix).cpu().numpy()
+    np.testing.assert_allclose(got, want, rtol=0, atol=1e-6)
+    dgot = api.pool_queries_bwd(ctx, _dev(G), off, pix, npix).cpu().numpy()
+    np.testing.assert_allclose(dgot, dwant, rtol=1e-5, atol=1e-5)
+
+
 def test_pool_rejects_bad_arguments(api, ctx):
     from paper_2602_12314_gb300 import _lib as L
     Q = torch.zeros((10, 24), device="cuda")
