@@ -834,7 +834,7 @@ __global__ void __launch_bounds__(gemm_threads(Epi::EPI_WG), Epi::MIN_BLOCKS)
 //
 // An epilogue with WARP_STAGE bytes per warp (a multiple of 1024) needs no box buffers: each warp
 // stages and TMA-stores its own 32 rows (EpiCtx::xstage, EpiCtx::omap) and waits for the read of
-// its last store itself.
+// its last store itself.  Warp 2 and the barriers staged[] and e_free[] take no part then.
 // With Epi::TEAMS = 2 the epilogue warpgroups form two teams that take the tiles in turn, each with
 // its own barrier and row-reduction scratch, so that one team computes while the other waits for
 // its row reductions, exchange and staging.  The exchanges of tiles lt and lt + 2 are then not
@@ -929,6 +929,7 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
     static_assert((E_BOXES <= 4 || INPLACE) && O_BOXES <= 4 && Epi::XROUNDS <= 1 && G <= 4, "epilogue shape");
     static_assert(ROWB == 128 || ROWB == 64 || ROWB == 32, "K chunk rows of 128, 64 or 32 bytes");
     static_assert(!A_MN, "the persistent tile reads A K-major");
+    static_assert((O_BOXES > 0) == (Epi::WARP_STAGE == 0), "outputs leave through the boxes or the warps' own staging");
     static_assert(!BRES || (!PAIR && !SPLIT && !B_MN && BOX_B == BN), "the resident B tile is one plain K-major box");
     static_assert(TEAMS == 1 || (TEAMS == 2 && G % 2 == 0 && E_BOXES == 0), "two teams share no operand boxes");
     static_assert(!SPLIT || (ELEM == 2 && (E_BOXES == 0 || INPLACE)), "split form: BF16 planes");
@@ -1121,6 +1122,8 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
                 bulk_wait_read();
             }
         }
+    } else if (warp == 2 && O_BOXES == 0) {
+        // nothing staged here: each epilogue warp sends its own output (WARP_STAGE)
     } else if (warp == 2 && SPLIT) {
         if (lane == 0 && nk > 0) {
             // ---- split form: one staged output per tile, its hi plane in buffer 0 and its lo
@@ -1360,9 +1363,12 @@ __global__ void __launch_bounds__(persist_threads(Epi::EPI_WG), 1)
                     mbar_arrive_cluster(peer_addr(&acc_empty[e], even));
                 else
                     mbar_arrive(&acc_empty[e]);
-                const int sb = SPLIT ? 0 : e;
-                nbox[sb] = *abort_flag ? 0 : out_boxes;
-                mbar_arrive(&staged[sb]);
+                // (an arrival that no wait_out of a later tile paces could lap warp 2's parity wait)
+                if (O_BOXES > 0) {
+                    const int sb = SPLIT ? 0 : e;
+                    nbox[sb] = *abort_flag ? 0 : out_boxes;
+                    mbar_arrive(&staged[sb]);
+                }
             }
         }
         if (Epi::WARP_STAGE > 0) bulk_wait_read();  // each warp's last store has read its staging

@@ -58,3 +58,29 @@ def test_rows_past_the_last_one_are_not_written(api, ctx):
                                          st))
     torch.cuda.synchronize()
     assert bool((out[n:] == 7.0).all()) and bool((out[:n] != 7.0).any(dim=1).all())
+
+
+@pytest.mark.parametrize("precision,M", [("FP32", 32), ("BF16", 32), ("FP8", 32), ("FP32", 256), ("BF16", 384)])
+def test_many_short_tiles_per_cta_leave_no_wait_behind(api, ctx, precision, M):
+    """Two dozen of the shortest tiles per CTA (one feature tile, few atoms), launched back to back:
+    the warps that send their own output must not run ahead of any other warp's wait.  A wait that
+    gives up raises the flag that the next binning reports."""
+    from workloads import random_scene
+    n, d, D = 24 * 152 * 128 + 77, 16, 128
+    g = torch.Generator(device="cuda").manual_seed(M)
+    Q = torch.randn(n, d, generator=g, device="cuda")
+    K = torch.randn(M, d, generator=g, device="cuda") / d**0.5
+    V = torch.randn(M, D, generator=g, device="cuda") / d**0.5
+    prec = getattr(api, precision)
+    first, _ = api.decode_fwd(ctx, Q, K, V, precision=prec, want_stats=False)
+    for _ in range(20):
+        again, _ = api.decode_fwd(ctx, Q, K, V, precision=prec, want_stats=False)
+    assert torch.equal(first, again)
+    s = random_scene(5, n=200, d=16, M=32, D=128, width=48, height=40, log_scale=-2.6)
+    api.sort(ctx, api.project(ctx, s.means, s.quats, s.scales, s.opacities, s.camera), s.camera)  # raises if flagged
+    want = torch.softmax(Q.double() @ K.double().T / d**0.5, 1) @ V.double()
+    if precision == "FP32":
+        assert float(((first - want).norm(dim=1) / want.norm(dim=1)).max()) <= 1e-4
+    else:
+        cos = torch.nn.functional.cosine_similarity(first.double(), want, dim=1).min()
+        assert float(cos) >= (0.999 if precision == "BF16" else 0.995)
