@@ -256,8 +256,9 @@ LATENTAM_API latentam_status latentam_project(latentam_ctx* ctx, const latentam_
  * bins->num_pairs (the placing and the sort may still run when it returns); if
  * P > bins->capacity returns LATENTAM_ERR_CAPACITY and writes no pairs (retry with a larger
  * buffer).  Returns LATENTAM_ERR_TIMEOUT if a bounded wait of an EARLIER call's scan gave up
- * (that call's tiles were left empty), or if a bounded wait of a tensor-core decode kernel
- * gave up since the last report (that call's loss was NaN); the flag is cleared when reported. */
+ * (that call's tiles were left empty, its pair count was right), or if a bounded wait of a
+ * tensor-core decode kernel gave up since the last report (that call's loss was NaN); the flag is
+ * cleared when reported. */
 LATENTAM_API latentam_status latentam_sort(latentam_ctx* ctx, int32_t n, const latentam_projected* proj,
                               const latentam_camera* cam, latentam_bins* bins,
                               latentam_stream stream);

@@ -119,9 +119,10 @@ __global__ void __launch_bounds__(kBinThreads) count_tiles(int N, const int32_t*
 // Ranges of 64 consecutive tiles per block, the blocks in ticket order (so that every block before
 // one belongs to a block already running), each adding the pairs of the earlier blocks: one warp
 // reads 32 of their words at a time until it meets an inclusive one.  The waits are bounded
-// (spin_limit polls): a walk that gives up raises *err and uses what it summed; the later
-// steps then leave every tile empty.  stall_block >= 0 (a test of that path) makes that block's
-// first look-back poll the word that nothing writes, so that its wait runs out.
+// (spin_limit polls): a walk that gives up raises *err, so that the later steps leave every tile
+// empty, and adds up the earlier tiles' counts itself, so that the pair count stays exact.
+// stall_block >= 0 (a test of that path) makes that block's first look-back poll the word that
+// nothing writes, so that its wait runs out.
 __global__ void __launch_bounds__(kScanTiles) tile_scan(BinWords w, int tiles, int2* __restrict__ ranges,
                                                         uint32_t* __restrict__ total, volatile uint32_t* host,
                                                         uint32_t* err, int spin_limit, int stall_block) {
@@ -170,6 +171,12 @@ __global__ void __launch_bounds__(kScanTiles) tile_scan(BinWords w, int tiles, i
             for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
             sum += x;
             if (full) break;
+        }
+        if (!ok) {
+            sum = 0;
+            for (int i = lane; i < b * kScanTiles; i += 32) sum += w.count[i];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
         }
         if (lane == 0) {
             if (!ok) atomicExch(err, 1u);

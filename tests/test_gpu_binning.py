@@ -70,3 +70,24 @@ def test_lists_equal_a_sort(api, n, width, height, span, visible):
                                           api._stream()) == L.ERR_CAPACITY
             assert bs.num_pairs == P and int(bins.tile_ranges.abs().sum()) == 0
             assert bool((bins.pair_ids == -1).all())
+
+
+def test_pair_count_is_exact_when_a_look_back_gives_up(api):
+    """The last block's look-back is made to give up: no tile keeps a list, the pair count is still that
+    of the splats (a call that finds its buffer too small asks for the right size), and the next
+    binning reports the wait, the one after it is complete."""
+    from paper_2602_12314_gb300 import _lib as L
+    cam = _camera(1200, 680)  # 3,225 tiles: 51 scan blocks
+    proj, ids, ranges = _scene(api, 20_000, cam, 9, 7, 0.3)
+    P = len(ids)
+    with api.Context(0) as ctx:
+        ctx.test_wait_timeout(0)
+        bins = api.sort(ctx, proj, cam, capacity=P)
+        assert bins.num_pairs == P and int(bins.tile_ranges.abs().sum()) == 0
+        with pytest.raises(L.LatentamError) as e:
+            api.sort(ctx, proj, cam, capacity=P)
+        assert e.value.status == L.ERR_TIMEOUT
+        bins = api.sort(ctx, proj, cam, capacity=P)
+        assert bins.num_pairs == P
+        np.testing.assert_array_equal(bins.tile_ranges.cpu().numpy(), ranges)
+        np.testing.assert_array_equal(bins.pair_ids[:P].cpu().numpy(), ids)
