@@ -438,7 +438,8 @@ typedef struct latentam_map latentam_map;
 /* The local map (device pointers owned by the map, valid until the next call that changes it):
  * count rows of means (x3), quats (x4), scales (x3), opacities, queries f (x d) and the Adam
  * moments of f (x d, zero for rows appended from the store), and gidx, each row's index in the
- * global store (-1: not in the store). */
+ * global store (-1: not in the store; a row set to -1 is inserted like a new one by the next
+ * synchronisation). */
 typedef struct {
     float *means, *quats, *scales, *opacities, *f, *m_f, *v_f;
     int32_t* gidx;

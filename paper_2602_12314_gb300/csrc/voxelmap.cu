@@ -52,12 +52,13 @@ struct latentam_map {
     int64_t loc_capacity[2];
     int cur;                  // the current local buffer
     int64_t local_count;
-    int64_t fresh;            // at most this many local rows have no entry in the store yet
+    bool fresh;               // rows were added, or the last synchronisation met rows without a store
+                              // entry: the next one inserts first
     // scratch of one operation: slots and candidate flags per row, kept / selected rows per block
     int32_t* slot;
     uint32_t *flag, *pos;
     int64_t scratch_n;
-    uint32_t* total;          // device counters (2) and their pinned copy
+    uint32_t* total;          // device counters (3) and their pinned copy
     uint32_t* host_total;
 };
 
@@ -372,16 +373,18 @@ __global__ void __launch_bounds__(kMapThreads) insert_commit(int64_t n, Rows src
 }
 
 // Local -> Global for the rows with a store entry, and the first half of the prune: kept[block] =
-// the block's local rows inside the radius, whose store entries are marked with the epoch.
+// the block's local rows inside the radius, whose store entries are marked with the epoch.  A row
+// without an entry leaves the epoch in *unstored.
 __global__ void __launch_bounds__(kMapThreads) write_back(int64_t n, Rows local, int d, bool vec, Rows global,
                                                           float cx, float cy, float cz, float r2,
                                                           int32_t* __restrict__ epoch_mark, int32_t epoch,
-                                                          uint32_t* __restrict__ kept) {
+                                                          uint32_t* __restrict__ kept, uint32_t* unstored) {
     __shared__ RowList l;
     const int64_t i0 = (int64_t)blockIdx.x * kMapThreads, i = i0 + threadIdx.x;
     const int32_t g = i < n ? local.gidx[i] : -1;
     const bool k = i < n && in_radius(local.means + 3 * i, cx, cy, cz, r2);
     if (k && g >= 0) epoch_mark[g] = epoch;
+    if (i < n && g < 0) *unstored = (uint32_t)epoch;
     const int c = __syncthreads_count(k);
     if (threadIdx.x == 0) kept[blockIdx.x] = (uint32_t)c;
     const int cnt = list_rows(l, g >= 0, -1, g);
@@ -527,8 +530,9 @@ latentam_status latentam_map_create(latentam_ctx* ctx, int32_t d, int32_t table_
     const size_t T = (size_t)1 << table_log2;
     bool ok = cudaMalloc(&m->table, sizeof(int32_t) * T) == cudaSuccess &&
               cudaMalloc(&m->claim, sizeof(int32_t) * T) == cudaSuccess &&
-              cudaMalloc(&m->total, sizeof(uint32_t) * 2) == cudaSuccess &&
-              cudaHostAlloc(&m->host_total, sizeof(uint32_t) * 2, cudaHostAllocDefault) == cudaSuccess;
+              cudaMalloc(&m->total, sizeof(uint32_t) * 3) == cudaSuccess &&
+              cudaMemset(m->total, 0, sizeof(uint32_t) * 3) == cudaSuccess &&
+              cudaHostAlloc(&m->host_total, sizeof(uint32_t) * 3, cudaHostAllocDefault) == cudaSuccess;
     if (ok) ok = cudaMemset(m->table, 0xff, sizeof(int32_t) * T) == cudaSuccess;  // -1
     if (ok) {
         // INT_MAX in every claim: fill through a host pattern once
@@ -612,7 +616,7 @@ latentam_status latentam_map_add_local(latentam_ctx* ctx, latentam_map* m, const
     if (e == cudaSuccess) e = cudaMemsetAsync(L.gidx + o, 0xff, sizeof(int32_t) * (size_t)n, st);  // -1
     if (e != cudaSuccess) return cuda_error(e, "voxel map: add local");
     m->local_count += n;
-    m->fresh += n;
+    m->fresh = true;
     return LATENTAM_OK;
 }
 
@@ -628,35 +632,46 @@ latentam_status latentam_map_sync(latentam_ctx* ctx, latentam_map* m, const floa
     const int64_t nl = m->local_count;
     const float cx = centre[0], cy = centre[1], cz = centre[2];
     const float r2 = radius * radius;
-    // Local -> Global: new rows are inserted if free (only where some may have no store entry),
-    // known ones overwrite their entries; the prune's counts and marks come with the same pass
+    // Local -> Global: new rows are inserted if free, known ones overwrite their entries; the prune's
+    // counts and marks come with the same pass.  Global -> Local: the store's unmarked rows inside
+    // the radius; one host read of both counts, then compact and append into the other buffer.
+    // The insertion runs first where some rows are known to lack an entry, and is skipped elsewhere.
+    // gidx is the caller's to write, so the pass looks at every row's: where it meets one without
+    // an entry all the same, the rows are inserted and the pass is taken again.
     Rows local = m->loc[m->cur];
-    if (nl > 0 && m->fresh > 0) {
-        int64_t added = 0;
-        LAT_TRY(insert_rows(ctx, m, nl, local, local.gidx, nullptr, &added, st));
-        m->fresh -= added;
+    const int64_t nbl = blocks(nl);
+    int64_t nbg = 0;
+    uint32_t *kept = nullptr, *sel = nullptr;
+    auto count_pass = [&]() -> latentam_status {
+        m->epoch += 1;
+        nbg = blocks(m->count);
+        LAT_TRY(grow_scratch(m, nbl + nbg));
+        kept = m->pos, sel = m->pos + nbl;
+        if (nl > 0) {
+            write_back<<<blocks(nl), kMapThreads, 0, st>>>(nl, local, d, vec_rows(d, local, m->g), m->g, cx, cy, cz,
+                                                           r2, m->epoch_mark, m->epoch, kept, m->total + 2);
+            LAT_CHECK_LAUNCH("write_back");
+        }
+        if (m->count > 0) {
+            select_global<<<blocks(m->count), kMapThreads, 0, st>>>(m->count, m->g.means, cx, cy, cz, r2,
+                                                                    m->epoch_mark, m->epoch, sel);
+            LAT_CHECK_LAUNCH("select_global");
+        }
+        scan_counts<<<2, 1024, 0, st>>>(kept, nbl, sel, nbg, m->total);
+        LAT_CHECK_LAUNCH("scan_counts");
+        return read_totals(m, 3, st);
+    };
+    auto insert_new = [&] { return insert_rows(ctx, m, nl, local, local.gidx, nullptr, nullptr, st); };
+    auto unstored = [&] { return m->host_total[2] == (uint32_t)m->epoch; };
+    const bool first = m->fresh;
+    if (first) LAT_TRY(insert_new());
+    LAT_TRY(count_pass());
+    if (!first && unstored()) {
+        LAT_TRY(insert_new());
+        LAT_TRY(count_pass());
     }
-    m->epoch += 1;
-    const int64_t nbl = blocks(nl), nbg = blocks(m->count);
-    LAT_TRY(grow_scratch(m, nbl + nbg));
-    uint32_t *kept = m->pos, *sel = m->pos + nbl;
-    if (nl > 0) {
-        write_back<<<blocks(nl), kMapThreads, 0, st>>>(nl, local, d, vec_rows(d, local, m->g), m->g, cx, cy, cz, r2,
-                                                       m->epoch_mark, m->epoch, kept);
-        LAT_CHECK_LAUNCH("write_back");
-    }
-    // Global -> Local: the store's unmarked rows inside the radius, one host read of both counts,
-    // then compact and append into the other buffer
-    if (m->count > 0) {
-        select_global<<<blocks(m->count), kMapThreads, 0, st>>>(m->count, m->g.means, cx, cy, cz, r2, m->epoch_mark,
-                                                                m->epoch, sel);
-        LAT_CHECK_LAUNCH("select_global");
-    }
-    scan_counts<<<2, 1024, 0, st>>>(kept, nbl, sel, nbg, m->total);
-    LAT_CHECK_LAUNCH("scan_counts");
-    LAT_TRY(read_totals(m, 2, st));
+    m->fresh = unstored();
     const int64_t n_kept = m->host_total[0], n_sel = m->host_total[1], n_new = n_kept + n_sel;
-    m->fresh = std::min(m->fresh, n_kept);
     const int other = m->cur ^ 1;
     LAT_TRY(grow_local(m, other, n_new, 0));
     if (n_kept > 0) {

@@ -214,3 +214,39 @@ def test_latent_map_optimises_the_active_local_map(api, ctx):
     # the rendered ones among the active Gaussians learned (the rest of the sphere is out of view)
     assert len(changed) > 1000 and set(changed.tolist()) <= seen
     vmap.close()
+
+
+@pytest.mark.parametrize("n,moved,kept", [(1, [0], []), (1, [], [0]), (700, [3, 255, 256, 699], [5, 512]), (700, [], [])])
+def test_rows_set_to_minus_one_are_inserted_like_new_ones(api, ctx, n, moved, kept):
+    """A caller sets gidx to -1 of local rows: those moved to a free voxel are inserted by the next
+    synchronisation, those whose slot is taken (by their own entry) stay without one, the others
+    are written back; the same three synchronisations on, and at a smaller radius."""
+    d = 8
+    rng = np.random.default_rng(n)
+    x = np.arange(n) * 0.02 + 0.005
+    g = _gauss(rng, np.stack([x, np.full(n, 0.005), np.full(n, 0.005)], 1), d)
+    gm = api.VoxelMap(ctx, d, table_log2=16, voxel_size=0.01)
+    om = vm.GlobalMap(d, 16, 0.01)
+    gm.insert(*_args(g))
+    om.insert(g)
+    assert om.count == n
+    olocal = {k: [] for k in (*vm.FIELDS, "gidx")}
+    for step, radius in enumerate((1e3, 1e3, 1e3, 2.0)):
+        if step:
+            loc = gm.local()
+            loc["f"].mul_(0.5)
+            olocal["f"] = [v * np.float32(0.5) for v in olocal["f"]]
+        if step == 1:
+            for i in moved + kept:
+                loc["gidx"][i] = olocal["gidx"][i] = -1
+            for i in moved:
+                loc["means"][i, 2] += 1.0
+                olocal["means"][i][2] += np.float32(1.0)
+        loc = gm.sync([0.0, 0.0, 0.0], radius)
+        olocal = om.sync(olocal, np.zeros(3, np.float32), radius)
+        assert om.count == n + (len(moved) if step else 0)
+        np.testing.assert_array_equal(_np(loc["gidx"]), np.array(olocal["gidx"], np.int32))
+        for k in vm.FIELDS:
+            np.testing.assert_array_equal(_np(loc[k]), np.array(olocal[k], np.float32).reshape(_np(loc[k]).shape))
+        _same_store(gm, om)
+    gm.close()
