@@ -84,3 +84,29 @@ def test_many_short_tiles_per_cta_leave_no_wait_behind(api, ctx, precision, M):
     else:
         cos = torch.nn.functional.cosine_similarity(first.double(), want, dim=1).min()
         assert float(cos) >= (0.999 if precision == "BF16" else 0.995)
+
+
+@pytest.mark.parametrize("precision", ["FP32", "BF16"])
+@pytest.mark.parametrize("n,D", [(44_900, 768), (300, 256), (128, 128)])
+def test_cta_pairs_with_several_and_odd_row_tiles(api, ctx, precision, n, D):
+    """The paired form (M = 512): 351 row tiles are several per CTA and an odd number, three and one
+    leave the last pair's odd CTA past the rows; nothing is written there."""
+    import ctypes
+
+    from paper_2602_12314_gb300 import _lib as L
+    d, M = 32, 512
+    g = torch.Generator(device="cuda").manual_seed(n)
+    Q = torch.randn(n, d, generator=g, device="cuda")
+    K = torch.randn(M, d, generator=g, device="cuda") / d**0.5
+    V = torch.randn(M, D, generator=g, device="cuda") / d**0.5
+    out = torch.full((n + 256, D), 7.0, device="cuda")
+    p = lambda t: ctypes.c_void_p(t.data_ptr())  # noqa: E731
+    st = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    L.check(L.load().latentam_decode_fwd(ctx.handle, p(Q), n, d, p(K), p(V), M, D, 0.0,
+                                         int(getattr(api, precision)), p(out), None, st))
+    want = torch.softmax(Q.double() @ K.double().T / d**0.5, 1) @ V.double()
+    assert bool((out[n:] == 7.0).all())
+    if precision == "FP32":
+        assert float(((out[:n] - want).norm(dim=1) / want.norm(dim=1)).max()) <= 1e-4
+    else:
+        assert float(torch.nn.functional.cosine_similarity(out[:n].double(), want, dim=1).min()) >= 0.999

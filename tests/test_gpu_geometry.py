@@ -116,3 +116,9 @@ def test_full_step_first_update_and_descent(api, ctx):
         np.testing.assert_allclose(got[well], (x0 - lr * np.sign(g))[well], rtol=0, atol=1e-3 * lr + 1e-6, err_msg=k)
     last = st.step(19)
     assert last["total"] < first["total"] - 1e-2  # random targets: a slow but steady descent
+
+
+def test_full_backward_d64_scene(api, ctx):
+    """d = 64: two channels a lane in the backward, one pixel a thread in the forward."""
+    s = random_scene(34, n=300, d=64, M=32, D=128, width=33, height=27, log_scale=-2.3)
+    _compare(api, ctx, s, 5)
