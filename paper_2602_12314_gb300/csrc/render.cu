@@ -2,9 +2,10 @@
 // blending of Eq. (alpha_blending) applied to the d-dimensional query vectors f_i, and its
 // backward with respect to f.
 //
-// Forward: one CTA per 16x16 tile; the tile's Gaussians are staged through shared memory in
-// batches (mean, exponent coefficients/opacity, query as float4 rows), so every query row is read
-// from L2/HBM once per tile and broadcast to the 256 pixels.  Backward: one warp per 16x4 strip.
+// One CTA per 16x16 tile, in the forward and the backward; the tile's Gaussians are staged through
+// shared memory in batches (mean, exponent coefficients/opacity, query as float4 rows), so every query
+// row is read from L2/HBM once per tile and broadcast to the 256 pixels.  (The backward of the full
+// blend runs one warp per strip of a tile.)
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -242,43 +243,36 @@ __global__ void __launch_bounds__(fwd_threads<DQ>(), DQ == 32 ? 5 : 1) render_fw
     }
 }
 
-// Backward of the query blend, df_i = sum_p w_ip dQ_p, as one small GEMM per strip (16 x 4 pixels) and
-// batch of 32 Gaussians on the tensor cores, a warp to itself: each lane recomputes the weights of
-// two horizontally adjacent pixels front to back (the forward's arithmetic, so the same
-// contributions are taken: a pixel stops after its n_contrib-th one) into the warp's shared-memory
-// matrix W^T (Gaussians x pixels), each weight as two BF16 terms w = hi + lo (hi = bf16(w),
-// lo = bf16(w - hi)); the strip's dQ rows are held the same way, for d <= 32 as B fragments in
-// registers for the whole list.  mma.sync m16n8k16 (BF16 in, FP32 accumulate) then sums
-// W_hi dQ_hi + W_hi dQ_lo + W_lo dQ_hi over the 64 pixels (each product within 2^-16 of the FP32
-// one), and lane pairs trade halves so that the non-zero sums go to df as 16-byte atomics.
-// Bound by issue and latency of the weight chains: warps share nothing, so there are no block
-// barriers, each strip stops at its own last contribution, and 10 KB of shared memory per warp
-// leaves the registers to limit the warps in flight.  (A block per tile with a 256 x 64 weight
-// matrix and the tile's dQ in shared memory held two blocks per SM and three barriers a batch.)
-// A per-strip contraction of 32 x 64 x d does not amortise TMEM allocation and completion waits;
-// the warp-level MMA runs in the registers of the warp that computed the weights.
-// (848 x 480, 200k Gaussians, d = 32: 74 us with the block per tile, 48 with the warp per strip.)
-constexpr int kBwdBatch = 32;
-constexpr int kStripRows = 4;
-constexpr int kStrips = kTile / kStripRows;       // strips per tile
-constexpr int kStripPixels = kTile * kStripRows;  // 64: two per lane
-constexpr int kWtStride = kStripPixels + 8;       // bf16 per W^T row (144 B: ldmatrix rows on distinct banks)
+// Backward of the query blend, df_i = sum_p w_ip dQ_p, as one small GEMM per tile and batch on
+// the tensor cores: the weights w_ip of a batch of kBwdBatch Gaussians are first recomputed front
+// to back by the pixel threads (the forward's arithmetic, so the same contributions are taken: a
+// pixel stops after its n_contrib-th one) into a shared-memory matrix W^T (Gaussians x pixels),
+// each weight as two BF16 terms w = hi + lo (hi = bf16(w), lo = bf16(w - hi)); the tile's dQ
+// rows are held the same way.  Then warp (m, h) takes Gaussians 16m..16m+15 and channel half h
+// and sums over the tile's 256 pixels with mma.sync m16n8k16 (BF16 in, FP32 accumulate) as
+// W_hi dQ_hi + W_hi dQ_lo + W_lo dQ_hi (each product within 2^-16 of the FP32 one), and each
+// non-zero (Gaussian, channel) sum goes to df with one atomic per tile.  A per-tile contraction
+// of 64 x 256 x d does not amortise TMEM allocation and completion waits; the warp-level MMA
+// runs in the registers of the warps that computed the weights.  Bound by the serial weight chains
+// between the three barriers of a batch (848 x 480, 200k Gaussians, d = 32: 74 us).  A warp per
+// 16 x 4 strip without block barriers, whose sums left as 16-byte atomics, took 48 us there and
+// stopped with a misaligned address on other scenes (20,000 splats of about 27 pixels at 640 x 480;
+// room keyframes at d = 64), although every index and address it formed was in bounds and aligned.
+constexpr int kBwdBatch = 64;
+constexpr int kWtStride = kTilePixels + 8;  // bf16 per W^T row (528 B: ldmatrix rows on distinct banks)
 
 template <int DQ>
-struct BwdSmem {
-    __nv_bfloat16 w[2][kBwdBatch][kWtStride];  // W^T hi, lo
-    // dQ hi, lo; for d <= 32 one plane at a time passes through w on its way to the registers
-    __nv_bfloat16 dq[DQ <= 32 ? 1 : 2][DQ <= 32 ? 1 : kStripPixels][DQ + 8];
-    float4 co[kBwdBatch];
-    float2 xy[kBwdBatch];
-    int id[kBwdBatch];
-    __device__ __forceinline__ __nv_bfloat16* dq_row(int plane, int pixel) {
-        return DQ <= 32 ? &w[0][0][0] + pixel * (DQ + 8) : &dq[DQ <= 32 ? 0 : plane][DQ <= 32 ? 0 : pixel][0];
-    }
-};
-static_assert(sizeof(__nv_bfloat16) * kStripPixels * (32 + 8) <= sizeof(BwdSmem<32>::w), "a dQ plane fits in w");
-static_assert(sizeof(BwdSmem<16>) % 16 == 0 && sizeof(BwdSmem<32>) % 16 == 0 && sizeof(BwdSmem<64>) % 16 == 0,
-              "16-byte rows");
+constexpr int dq_stride() {
+    return DQ + 8;  // bf16 per dQ row (16 B of padding: ldmatrix rows on distinct banks)
+}
+
+template <int DQ>
+constexpr size_t render_bwd_smem() {
+    // W^T hi / lo, dQ hi / lo, staged splats
+    return 2 * sizeof(__nv_bfloat16) * (size_t)kBwdBatch * kWtStride +
+           2 * sizeof(__nv_bfloat16) * (size_t)kTilePixels * dq_stride<DQ>() +
+           (sizeof(float4) + sizeof(float2) + sizeof(int)) * kBwdBatch;
+}
 
 __device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t (&r)[4]) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
@@ -300,203 +294,157 @@ __device__ __forceinline__ uint32_t smem_addr(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-// The m16n8 accumulator tile (rows = Gaussians r0 .. r0 + 15 of the batch, columns = channels
-// c0 .. c0 + 7) added to dst rows of `ld` floats: an even lane ends with four consecutive channels of
-// its upper row, an odd lane of its lower row.  vec: dst and ld are multiples of 16 bytes.
-__device__ __forceinline__ void add_tile(const float (&c)[4], const int* id, int r0, int rows, int c0, float* dst,
-                                         int ld, bool vec, int lane) {
-    const bool odd = lane & 1;
-    const float s0 = odd ? c[0] : c[2], s1 = odd ? c[1] : c[3];
-    const float o0 = __shfl_xor_sync(0xffffffffu, s0, 1), o1 = __shfl_xor_sync(0xffffffffu, s1, 1);
-    const float4 v = odd ? make_float4(o0, o1, c[2], c[3]) : make_float4(c[0], c[1], o0, o1);
-    const int r = r0 + (lane >> 2) + (odd ? 8 : 0);
-    if (r >= rows) return;
-    float* p = dst + (size_t)id[r] * ld + c0 + 4 * ((lane & 3) >> 1);
-    if (vec) {
-        if (v.x != 0.0f || v.y != 0.0f || v.z != 0.0f || v.w != 0.0f) atomicAdd(reinterpret_cast<float4*>(p), v);
-    } else {
-        if (v.x != 0.0f) atomicAdd(p, v.x);
-        if (v.y != 0.0f) atomicAdd(p + 1, v.y);
-        if (v.z != 0.0f) atomicAdd(p + 2, v.z);
-        if (v.w != 0.0f) atomicAdd(p + 3, v.w);
-    }
-}
-
-// Backward of one strip by one warp.
+// Backward of one tile (256 threads); smem is the dynamic shared memory of render_bwd_smem.
 template <int DQ>
-__device__ __forceinline__ void render_bwd_strip(const TileJob& job, int strip, BwdSmem<DQ>& sm) {
-    constexpr int DV = DQ / 4, NT = DQ / 8, KT = kStripPixels / 16;
-    constexpr bool REG = DQ <= 32;  // dQ fragments in registers
+__device__ __forceinline__ void render_bwd_tile(const TileJob& job, float4* smem) {
+    constexpr int DV = DQ / 4;
+    constexpr int DQS = dq_stride<DQ>();
+    constexpr int NT = DQ / 16;  // n-tiles of 8 channels per warp (a warp covers DQ / 2 channels)
+    using bf16 = __nv_bfloat16;
+    bf16* wt_hi = reinterpret_cast<bf16*>(smem);      // [Gaussian][pixel]
+    bf16* wt_lo = wt_hi + (size_t)kBwdBatch * kWtStride;
+    bf16* dq_hi = wt_lo + (size_t)kBwdBatch * kWtStride;  // [pixel][channel]
+    bf16* dq_lo = dq_hi + (size_t)kTilePixels * DQS;
+    float4* s_co = reinterpret_cast<float4*>(dq_lo + (size_t)kTilePixels * DQS);
+    float2* s_xy = reinterpret_cast<float2*>(s_co + kBwdBatch);
+    int* s_id = reinterpret_cast<int*>(s_xy + kBwdBatch);
+    static_assert(((size_t)kBwdBatch * kWtStride * 2 * 2 + (size_t)kTilePixels * DQS * 2 * 2) % 16 == 0,
+                  "staged splats stay 16-byte aligned");
+
     const int tile = job.tile;
     const int tx = tile % job.tiles_x, ty = tile / job.tiles_x;
-    const int lane = threadIdx.x & 31;
-    const int px = tx * kTile + (2 * lane) % kTile, py = ty * kTile + strip * kStripRows + lane / (kTile / 2);
-    const float fpx[2] = {(float)px, (float)(px + 1)}, fpy = (float)py;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int px = tx * kTile + (t % kTile), py = ty * kTile + (t / kTile);
+    const bool inside = px < job.W && py < job.H;
+    const float fpx = (float)px, fpy = (float)py;
     const int2 range = job.ranges[tile];
-    const bool vec = (reinterpret_cast<uintptr_t>(job.df) & 15u) == 0;
-    int remaining[2];
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-        remaining[i] = px + i < job.W && py < job.H ? job.n_contrib[(size_t)py * job.W + px + i] : 0;
-    if (range.x >= range.y || !__any_sync(0xffffffffu, (remaining[0] | remaining[1]) > 0)) return;
-    // the strip's dQ rows (pixel 2 lane + i) as hi / lo terms
-    uint32_t bh[REG ? KT : 1][REG ? NT : 1][2], bl[REG ? KT : 1][REG ? NT : 1][2];
+    int remaining = 0;
     {
-        uint32_t lo[2][DQ / 2];
-        __syncwarp();
+        // this pixel's dQ row as hi / lo terms
+        float4 g[DV];
+        if (inside) {
+            const size_t p = (size_t)py * job.W + px;
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const bool in = px + i < job.W && py < job.H;
-            const size_t p = (size_t)py * job.W + px + i;
-#pragma unroll
-            for (int c = 0; c < DV; ++c) {
-                const float4 g = in ? job.dQ[p * DV + c] : make_float4(0.f, 0.f, 0.f, 0.f);
-                uint32_t h0, h1;
-                tc_split(g.x, g.y, h0, lo[i][2 * c]);
-                tc_split(g.z, g.w, h1, lo[i][2 * c + 1]);
-                *reinterpret_cast<uint2*>(sm.dq_row(0, 2 * lane + i) + 4 * c) = make_uint2(h0, h1);
-            }
-        }
-        auto put_lo = [&](int plane) {
-#pragma unroll
-            for (int i = 0; i < 2; ++i)
-#pragma unroll
-                for (int c = 0; c < DV; ++c)
-                    *reinterpret_cast<uint2*>(sm.dq_row(plane, 2 * lane + i) + 4 * c) =
-                        make_uint2(lo[i][2 * c], lo[i][2 * c + 1]);
-        };
-        auto fragments = [&](uint32_t (&b)[REG ? KT : 1][REG ? NT : 1][2]) {
-#pragma unroll
-            for (int kt = 0; kt < (REG ? KT : 0); ++kt)
-#pragma unroll
-                for (int n = 0; n < NT; ++n)
-                    ldsm_x2_trans(smem_addr(sm.dq_row(0, 16 * kt + (lane & 15)) + 8 * n), b[kt][n]);
-        };
-        if (REG) {
-            __syncwarp();
-            fragments(bh);
-            __syncwarp();
-            put_lo(0);
-            __syncwarp();
-            fragments(bl);
+            for (int c = 0; c < DV; ++c) g[c] = job.dQ[p * DV + c];
+            remaining = job.n_contrib[p];
         } else {
-            put_lo(1);
+#pragma unroll
+            for (int c = 0; c < DV; ++c) g[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int c = 0; c < DV; c += 2) {
+            uint32_t h[4], l[4];
+            const float4 a = g[c], b = c + 1 < DV ? g[c + 1] : make_float4(0.f, 0.f, 0.f, 0.f);
+            tc_split(a.x, a.y, h[0], l[0]);
+            tc_split(a.z, a.w, h[1], l[1]);
+            tc_split(b.x, b.y, h[2], l[2]);
+            tc_split(b.z, b.w, h[3], l[3]);
+            if (c + 1 < DV) {
+                *reinterpret_cast<uint4*>(dq_hi + (size_t)t * DQS + 4 * c) = make_uint4(h[0], h[1], h[2], h[3]);
+                *reinterpret_cast<uint4*>(dq_lo + (size_t)t * DQS + 4 * c) = make_uint4(l[0], l[1], l[2], l[3]);
+            } else {
+                *reinterpret_cast<uint2*>(dq_hi + (size_t)t * DQS + 4 * c) = make_uint2(h[0], h[1]);
+                *reinterpret_cast<uint2*>(dq_lo + (size_t)t * DQS + 4 * c) = make_uint2(l[0], l[1]);
+            }
         }
     }
-    float T[2] = {1.0f, 1.0f};
-    // the splats of the next batch are fetched while this one is worked on
-    int gid = 0;
-    float2 nxy = make_float2(0.f, 0.f);
-    float4 nco = make_float4(0.f, 0.f, 0.f, 0.f);
-    auto fetch = [&](int start) {
-        if (start + lane < range.y) {
-            gid = job.pair_ids[start + lane];
-            nxy = job.xy[gid];
-            nco = job.conic_opac[gid];
-        }
-    };
-    fetch(range.x);
+    const int mt = warp & 3, nh = warp >> 2;  // GEMM role: Gaussian rows 16 mt.., channel half nh
+    float T = 1.0f;
+    bool done = remaining == 0;
     for (int start = range.x; start < range.y; start += kBwdBatch) {
+        if (__syncthreads_count(done) == kTilePixels) break;
         const int cnt = min(kBwdBatch, range.y - start);
-        __syncwarp();
-        sm.xy[lane] = nxy;
-        sm.co[lane] = stage_splat(nco);
-        sm.id[lane] = gid;
-        __syncwarp();
-        fetch(start + kBwdBatch);
-        // 1. the lane's weights for the batch (identical arithmetic to the forward pass)
-#pragma unroll 2
-        for (int j = 0; j < cnt; ++j) {
-            const float2 m = sm.xy[j];
-            const float4 q = sm.co[j];
-            float w[2];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const float alpha = splat_alpha(m, q, fpx[i], fpy);
-                const bool use = remaining[i] > 0 && alpha >= kAlphaMin;
-                w[i] = use ? __fmul_rn(alpha, T[i]) : 0.0f;
-                if (use) {
-                    T[i] = __fmul_rn(T[i], __fsub_rn(1.0f, alpha));
-                    --remaining[i];
+        if (t < cnt) {
+            const int gid = job.pair_ids[start + t];
+            s_xy[t] = job.xy[gid];
+            s_co[t] = stage_splat(job.conic_opac[gid]);
+            s_id[t] = gid;
+        }
+        __syncthreads();
+        // 1. this pixel's weights for the batch (identical arithmetic to the forward pass); the
+        //    columns of the Gaussians past the batch are zero
+        for (int j = 0; j < kBwdBatch; ++j) {
+            float w = 0.0f;
+            if (j < cnt && !done) {
+                const float alpha = splat_alpha(s_xy[j], s_co[j], fpx, fpy);
+                if (alpha >= kAlphaMin) {
+                    w = __fmul_rn(alpha, T);
+                    T = __fmul_rn(T, __fsub_rn(1.0f, alpha));
+                    if (--remaining == 0) done = true;
                 }
             }
-            uint32_t h, l;
-            tc_split(w[0], w[1], h, l);
-            *reinterpret_cast<uint32_t*>(&sm.w[0][j][2 * lane]) = h;
-            *reinterpret_cast<uint32_t*>(&sm.w[1][j][2 * lane]) = l;
+            const __nv_bfloat16 wh = __float2bfloat16_rn(w);
+            wt_hi[(size_t)j * kWtStride + t] = wh;
+            wt_lo[(size_t)j * kWtStride + t] = __float2bfloat16_rn(w - __bfloat162float(wh));
         }
-        __syncwarp();
-        // 2. df rows (16 Gaussians) x channels over the strip's 64 pixels; rows past the batch hold
-        //    leftovers and are not added
-        for (int r0 = 0; r0 < cnt; r0 += 16) {
+        __syncthreads();
+        // 2. warp (mt, nh): df rows 16 mt.. (Gaussians) x channels nh DQ/2.. over the 256 pixels
+        if (16 * mt < cnt) {
             float acc[NT][4];
 #pragma unroll
             for (int n = 0; n < NT; ++n) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
-#pragma unroll
-            for (int kt = 0; kt < KT; ++kt) {
+            const int ar = 16 * mt + (lane & 15), ac = (lane >> 4) * 8;  // A fragment row / column
+            const int br = lane & 15;                                     // B fragment row (pixel)
+#pragma unroll 4
+            for (int kt = 0; kt < kTilePixels / 16; ++kt) {
                 uint32_t ah[4], al[4];
-                ldsm_x4(smem_addr(&sm.w[0][r0 + (lane & 15)][16 * kt + (lane >> 4) * 8]), ah);
-                ldsm_x4(smem_addr(&sm.w[1][r0 + (lane & 15)][16 * kt + (lane >> 4) * 8]), al);
+                ldsm_x4(smem_addr(wt_hi + (size_t)ar * kWtStride + 16 * kt + ac), ah);
+                ldsm_x4(smem_addr(wt_lo + (size_t)ar * kWtStride + 16 * kt + ac), al);
 #pragma unroll
                 for (int n = 0; n < NT; ++n) {
-                    uint32_t fh[2], fl[2];
-                    if (REG) {
-                        fh[0] = bh[REG ? kt : 0][REG ? n : 0][0], fh[1] = bh[REG ? kt : 0][REG ? n : 0][1];
-                        fl[0] = bl[REG ? kt : 0][REG ? n : 0][0], fl[1] = bl[REG ? kt : 0][REG ? n : 0][1];
-                    } else {
-                        ldsm_x2_trans(smem_addr(sm.dq_row(0, 16 * kt + (lane & 15)) + 8 * n), fh);
-                        ldsm_x2_trans(smem_addr(sm.dq_row(1, 16 * kt + (lane & 15)) + 8 * n), fl);
-                    }
-                    mma_bf16_16816(acc[n], ah, fh);
-                    mma_bf16_16816(acc[n], ah, fl);
-                    mma_bf16_16816(acc[n], al, fh);
+                    const int col = nh * (DQ / 2) + 8 * n;
+                    uint32_t bh[2], bl[2];
+                    ldsm_x2_trans(smem_addr(dq_hi + (size_t)(16 * kt + br) * DQS + col), bh);
+                    ldsm_x2_trans(smem_addr(dq_lo + (size_t)(16 * kt + br) * DQS + col), bl);
+                    mma_bf16_16816(acc[n], ah, bh);
+                    mma_bf16_16816(acc[n], ah, bl);
+                    mma_bf16_16816(acc[n], al, bh);
                 }
             }
-            // 3. the non-zero sums of the strip
+            // 3. one atomic per non-zero (Gaussian, channel) of the tile
+            const int g0 = 16 * mt + (lane >> 2);
 #pragma unroll
-            for (int n = 0; n < NT; ++n) add_tile(acc[n], sm.id, r0, cnt, 8 * n, job.df, DQ, vec, lane);
+            for (int n = 0; n < NT; ++n) {
+                const int c = nh * (DQ / 2) + 8 * n + 2 * (lane & 3);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int g = g0 + 8 * h;
+                    if (g >= cnt) continue;
+                    float* dst = job.df + (size_t)s_id[g] * DQ + c;
+                    if (acc[n][2 * h] != 0.0f) atomicAdd(dst, acc[n][2 * h]);
+                    if (acc[n][2 * h + 1] != 0.0f) atomicAdd(dst + 1, acc[n][2 * h + 1]);
+                }
+            }
         }
-        if (!__any_sync(0xffffffffu, (remaining[0] | remaining[1]) > 0)) break;
+        // the next batch's staging and W writes come after the barrier at the loop head
     }
 }
 
-constexpr int kBwdWarps = 4;  // warps per block, each with strips of its own
-
 template <int DQ>
-__global__ void __launch_bounds__(32 * kBwdWarps) render_bwd_kernel(CamParams cam, const int2* __restrict__ ranges,
-                                                                    const int32_t* __restrict__ pair_ids,
-                                                                    const float2* __restrict__ xy,
-                                                                    const float4* __restrict__ conic_opac,
-                                                                    const int32_t* __restrict__ n_contrib,
-                                                                    const float4* __restrict__ dQ,
-                                                                    float* __restrict__ df) {
+__global__ void __launch_bounds__(kTilePixels) render_bwd_kernel(CamParams cam, const int2* __restrict__ ranges,
+                                                                 const int32_t* __restrict__ pair_ids,
+                                                                 const float2* __restrict__ xy,
+                                                                 const float4* __restrict__ conic_opac,
+                                                                 const int32_t* __restrict__ n_contrib,
+                                                                 const float4* __restrict__ dQ, float* __restrict__ df) {
     extern __shared__ float4 smem_f4[];
-    const int item = blockIdx.x * kBwdWarps + (threadIdx.x >> 5);
-    const int t = item / kStrips;
-    if (t >= cam.tiles_x * cam.tiles_y) return;
-    const int tile = cam.tile_order ? cam.tile_order[t] : t;
+    const int tile = cam.tile_order ? cam.tile_order[blockIdx.x] : (int)blockIdx.x;
     const TileJob job{tile, cam.tiles_x, cam.W, cam.H, ranges, pair_ids, xy, conic_opac, nullptr, nullptr, nullptr,
                       const_cast<int32_t*>(n_contrib), dQ, df};
-    render_bwd_strip<DQ>(job, item % kStrips, reinterpret_cast<BwdSmem<DQ>*>(smem_f4)[threadIdx.x >> 5]);
+    render_bwd_tile<DQ>(job, smem_f4);
 }
 
-// Persistent render backward over every strip of every tile of a batch, longest lists first, each
-// warp with a ticket of its own (frames that share their queries add into the same df).
+// Persistent render backward over every tile of every frame of a batch, longest lists first
+// (frames that share their queries add into the same df).
 template <int DQ>
-__global__ void __launch_bounds__(32 * kBwdWarps) render_bwd_batch_kernel(const __grid_constant__ BatchJobs jobs,
-                                                                          const int32_t* __restrict__ order,
-                                                                          int total, int* __restrict__ counter) {
+__global__ void __launch_bounds__(kTilePixels) render_bwd_batch_kernel(const __grid_constant__ BatchJobs jobs,
+                                                                       const int32_t* __restrict__ order, int total,
+                                                                       int* __restrict__ counter) {
     extern __shared__ float4 smem_f4[];
-    BwdSmem<DQ>& sm = reinterpret_cast<BwdSmem<DQ>*>(smem_f4)[threadIdx.x >> 5];
-    for (;;) {
-        int it = 0;
-        if ((threadIdx.x & 31) == 0) it = atomicAdd(counter, 1);
-        it = __shfl_sync(0xffffffffu, it, 0);
-        if (it >= total * kStrips) return;
-        const int item = order[it / kStrips];
+    for (int item = next_item(counter, order, total); item >= 0; item = next_item(counter, order, total)) {
         TileJob job = jobs.fr[item >> 20];
         job.tile = item & 0xFFFFF;
-        render_bwd_strip<DQ>(job, it % kStrips, sm);
+        render_bwd_tile<DQ>(job, smem_f4);
     }
 }
 
@@ -523,7 +471,7 @@ __global__ void __launch_bounds__(fwd_threads<DQ>(), 1) render_fwd_full_kernel(
     render_fwd_tile<DQ, true>(job, sm, full);
 }
 
-// Backward of the full blend, a warp per strip as above but in FP32 throughout (the geometry terms
+// Backward of the full blend, a warp per strip of a tile and FP32 throughout (the geometry terms
 // need <G, x_i>, a dot product over all channels, for every pixel and splat).  Per batch of 16
 // Gaussians: (1) each lane takes its own pixels front to back from the strip's dQ rows in its
 // registers: weight, <G, x_j>, dL/dalpha; the six geometry terms of its pixels are added over the
@@ -535,6 +483,7 @@ __global__ void __launch_bounds__(fwd_threads<DQ>(), 1) render_fwd_full_kernel(
 // (640 x 480, 300k Gaussians, d = 32: 226 us with a block per tile and two warp reductions per
 // Gaussian, 190-204 with the warp per strip.)
 constexpr int kFullBatch = 16;
+constexpr int kBwdWarps = 4;  // warps per block, each with strips of its own
 
 template <int DQ>
 constexpr int full_px() {  // pixels per lane (two at d = 32 take 220 registers: 8 warps per SM, 235 us
@@ -821,9 +770,10 @@ latentam_status render_bwd_t(const CamParams& cam, const latentam_projected& pro
         if (e != cudaSuccess) return cuda_error(e, "memset df");
     }
     const int tiles = cam.tiles_x * cam.tiles_y;
-    constexpr size_t smem = sizeof(BwdSmem<DQ>) * kBwdWarps;
+    constexpr size_t smem = render_bwd_smem<DQ>();
+    static_assert(smem <= 227 * 1024, "render backward tile does not fit in shared memory");
     LAT_TRY(bwd_smem<render_bwd_kernel<DQ>>(smem));
-    render_bwd_kernel<DQ><<<(tiles * kStrips + kBwdWarps - 1) / kBwdWarps, 32 * kBwdWarps, smem, st>>>(
+    render_bwd_kernel<DQ><<<tiles, kTilePixels, smem, st>>>(
         cam, reinterpret_cast<const int2*>(bins.tile_ranges), bins.pair_ids, reinterpret_cast<const float2*>(proj.xy),
         reinterpret_cast<const float4*>(proj.conic_opacity), n_contrib, reinterpret_cast<const float4*>(dQ), df);
     LAT_CHECK_LAUNCH("render_bwd_kernel");
@@ -892,11 +842,10 @@ latentam_status render_fwd_batch_t(const BatchJobs& jobs, const int32_t* order, 
 template <int DQ>
 latentam_status render_bwd_batch_t(const BatchJobs& jobs, const int32_t* order, int total, int* counter,
                                    cudaStream_t st) {
-    constexpr size_t smem = sizeof(BwdSmem<DQ>) * kBwdWarps;
-    constexpr int threads = 32 * kBwdWarps;
+    constexpr size_t smem = render_bwd_smem<DQ>();
     LAT_TRY(bwd_smem<render_bwd_batch_kernel<DQ>>(smem));
-    const int grid = persistent_grid<render_bwd_batch_kernel<DQ>>(threads, smem, total);
-    render_bwd_batch_kernel<DQ><<<grid, threads, smem, st>>>(jobs, order, total, counter);
+    const int grid = persistent_grid<render_bwd_batch_kernel<DQ>>(kTilePixels, smem, total);
+    render_bwd_batch_kernel<DQ><<<grid, kTilePixels, smem, st>>>(jobs, order, total, counter);
     LAT_CHECK_LAUNCH("render_bwd_batch_kernel");
     return LATENTAM_OK;
 }
