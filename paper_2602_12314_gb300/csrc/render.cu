@@ -65,6 +65,13 @@ template <int DQ>
 constexpr int fwd_threads() {
     return kTilePixels / fwd_px<DQ>();
 }
+// Blocks per SM that the registers must leave room for: at d = 64 two of 256 threads (without the
+// bound the compiler takes 154 to 178 registers, one block: 1296 x 968, 1M Gaussians, the whole view
+// 1,022 us against 766).
+template <int DQ>
+constexpr int fwd_blocks() {
+    return DQ == 64 ? 2 : 1;
+}
 
 constexpr int kBatch = 128;  // Gaussians staged per round
 
@@ -200,7 +207,7 @@ __device__ __forceinline__ void render_fwd_tile(const TileJob& job, FwdSmem<DQ, 
 }
 
 template <int DQ>
-__global__ void __launch_bounds__(fwd_threads<DQ>(), 1) render_fwd_kernel(CamParams cam, const int2* __restrict__ ranges,
+__global__ void __launch_bounds__(fwd_threads<DQ>(), fwd_blocks<DQ>()) render_fwd_kernel(CamParams cam, const int2* __restrict__ ranges,
                                                                        const int32_t* __restrict__ pair_ids,
                                                                        const float2* __restrict__ xy,
                                                                        const float4* __restrict__ conic_opac,
@@ -232,7 +239,7 @@ __device__ __forceinline__ int next_item(int* counter, const int32_t* order, int
 // four that its registers would allow; the single frame above is shorter with four, 57 against
 // 70 us at 640 x 480, where the last tiles' own length counts.)
 template <int DQ>
-__global__ void __launch_bounds__(fwd_threads<DQ>(), DQ == 32 ? 5 : 1) render_fwd_batch_kernel(const __grid_constant__ BatchJobs jobs,
+__global__ void __launch_bounds__(fwd_threads<DQ>(), DQ == 32 ? 5 : fwd_blocks<DQ>()) render_fwd_batch_kernel(const __grid_constant__ BatchJobs jobs,
                                                                              const int32_t* __restrict__ order,
                                                                              int total, int* __restrict__ counter) {
     __shared__ FwdSmem<DQ> sm;
@@ -460,7 +467,7 @@ __global__ void __launch_bounds__(kTilePixels) render_bwd_batch_kernel(const __g
 // screen mean and the conic.
 
 template <int DQ>
-__global__ void __launch_bounds__(fwd_threads<DQ>(), 1) render_fwd_full_kernel(
+__global__ void __launch_bounds__(fwd_threads<DQ>(), fwd_blocks<DQ>()) render_fwd_full_kernel(
     CamParams cam, const int2* __restrict__ ranges, const int32_t* __restrict__ pair_ids,
     const float2* __restrict__ xy, const float4* __restrict__ conic_opac, const float4* __restrict__ f,
     float4* __restrict__ Q, FullImages full, float* __restrict__ T_final, int32_t* __restrict__ n_contrib) {
