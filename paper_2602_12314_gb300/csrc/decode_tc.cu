@@ -558,14 +558,19 @@ struct FhatEpi {
                 body(c0, h, f);
             }
         } else {
+            // two target buffers in turn, so that a load is waited for one chunk after it was issued (100,000
+            // rows, M = 256, D = 512, FP32 with BF16 targets: 143 us; copied from one to the other 179, with spills)
             float fn[32];
             load_target32(p.F, p.F_dtype, frow + 32 * ec.g, f);
-            for (int c0 = 32 * ec.g; c0 < ncols; c0 += step) {
-                if (c0 + step < ncols) load_target32(p.F, p.F_dtype, frow + c0 + step, fn);
+            for (int c0 = 32 * ec.g; c0 < ncols; c0 += 2 * step) {
+                const int c1 = c0 + step;
+                if (c1 < ncols) load_target32(p.F, p.F_dtype, frow + c1, fn);
                 fhat32<Q8>(p, ec, c0, isp, h);
                 body(c0, h, f);
-#pragma unroll
-                for (int i = 0; i < 32; ++i) f[i] = fn[i];
+                if (c1 >= ncols) break;
+                if (c1 + step < ncols) load_target32(p.F, p.F_dtype, frow + c1 + step, f);
+                fhat32<Q8>(p, ec, c1, isp, h);
+                body(c1, h, fn);
             }
         }
     }
