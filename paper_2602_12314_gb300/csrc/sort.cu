@@ -41,8 +41,11 @@ __device__ __forceinline__ void st_relaxed_gpu(uint64_t* p, uint64_t v) {
 }
 
 // The counters of one binning, in one zeroed block of memory (see bin_words): per tile the splats
-// counted and the splats placed, the look-back words (one more, never written: what an armed test
-// stall polls), the block ticket.
+// counted and the splats placed, kTileWords apart (packed, the atomics of a few hundred tiles meet in
+// a few L2 lines: 610,000 pairs in 300 tiles 103 us to count and 91 to place, 40 and 42 at 8 words, 17
+// and 21 at a line of 32), the look-back words (one more, never written: what an armed test stall
+// polls), the block ticket.
+constexpr int kTileWords = 32;
 struct BinWords {
     uint64_t* status;
     uint32_t *count, *placed, *ticket;
@@ -50,7 +53,7 @@ struct BinWords {
 
 size_t bin_words_bytes(int64_t tiles) {
     const int64_t nb = (tiles + kScanTiles - 1) / kScanTiles;
-    return 8 * (size_t)(nb + 1) + 4 * (size_t)(2 * tiles + 1);
+    return 8 * (size_t)(nb + 1) + 4 * (size_t)(kTileWords * tiles + 1);
 }
 
 BinWords bin_words(void* base, int64_t tiles) {
@@ -58,19 +61,33 @@ BinWords bin_words(void* base, int64_t tiles) {
     BinWords w;
     w.status = static_cast<uint64_t*>(base);
     w.count = reinterpret_cast<uint32_t*>(w.status + nb + 1);
-    w.placed = w.count + tiles;
-    w.ticket = w.placed + tiles;
+    w.placed = w.count + 1;
+    w.ticket = w.count + kTileWords * tiles;
     return w;
 }
 
-// body(g, tile) for every pair of a warp's 32 splats (lane l holds splat g, g < N), 32 pairs at a
-// time: each lane finds its pair's splat in the prefix sums of the counts, so that a splat of many
-// tiles does not leave 31 lanes waiting and the pairs' atomics overlap.  A splat's pairs are its
-// first tiles_touched tiles in row order, those of the image.  For full warps.
+// Warps that share the pairs of 32 splats (a power of two): one where the splats alone give every SM
+// eight warps, up to 64 where a few splats may cover the image (5 splats of 22,500 pairs: 156 us to
+// count and 438 to place with one warp, the whole binning 545 -> 40).
+int pair_parts(int N, int sms) {
+    const int64_t groups = ((int64_t)N + 31) / 32;
+    int parts = 1;
+    while (parts < 64 && groups * parts * 2 <= 8 * (int64_t)sms) parts *= 2;
+    return parts;
+}
+
+// body(g, tile) for every pair of 32 consecutive splats, of those of warp `index` (of the grid; parts
+// warps to 32 splats), 32 pairs at a time: each lane finds its pair's splat in the prefix sums of the
+// counts, so that a splat of many tiles does not leave 31 lanes waiting and the pairs' atomics
+// overlap.  A splat's pairs are its first tiles_touched tiles in row order, those of the image.  For
+// full warps.
 template <class Body>
-__device__ __forceinline__ void warp_pairs(int g, int N, const int32_t* __restrict__ touched,
+__device__ __forceinline__ void warp_pairs(int index, int parts, int N, const int32_t* __restrict__ touched,
                                            const int4* __restrict__ rect, int tiles_x, int tiles, Body&& body) {
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, part = index & (parts - 1);
+    const int64_t first = (int64_t)(index / parts) * 32;
+    if (first >= N) return;
+    const int g = (int)first + lane;
     int n = g < N ? touched[g] : 0;
     int x0 = 0, y0 = 0, w = 1;
     if (n > 0) {
@@ -86,7 +103,7 @@ __device__ __forceinline__ void warp_pairs(int g, int N, const int32_t* __restri
         if (lane >= o) incl += u;
     }
     const int all = __shfl_sync(0xffffffffu, incl, 31), before = incl - n;
-    for (int i0 = 0; i0 < all; i0 += 32) {
+    for (int i0 = 32 * part; i0 < all; i0 += 32 * parts) {
         const int i = i0 + lane;
         int own = 0;  // splats of the warp whose pairs all come before pair i
 #pragma unroll
@@ -104,16 +121,16 @@ __device__ __forceinline__ void warp_pairs(int g, int N, const int32_t* __restri
 
 // Also hands the slot's error words of earlier calls to the host (err: a look-back that gave up;
 // tc_flag: a tensor-core kernel's wait).
-__global__ void __launch_bounds__(kBinThreads) count_tiles(int N, const int32_t* __restrict__ touched,
+__global__ void __launch_bounds__(kBinThreads) count_tiles(int N, int parts, const int32_t* __restrict__ touched,
                                                            const int4* __restrict__ rect, int tiles_x, int tiles,
                                                            uint32_t* __restrict__ count, const uint32_t* err,
                                                            const int* tc_flag, volatile uint32_t* host) {
-    const int g = blockIdx.x * kBinThreads + threadIdx.x;
-    if (g == 0) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
         host[2] = *err;
         host[3] = (uint32_t)*tc_flag;
     }
-    warp_pairs(g, N, touched, rect, tiles_x, tiles, [&](int, int t) { atomicAdd(count + t, 1u); });
+    warp_pairs((int)(blockIdx.x * (kBinThreads / 32) + threadIdx.x / 32), parts, N, touched, rect, tiles_x, tiles,
+               [&](int, int t) { atomicAdd(count + (size_t)t * kTileWords, 1u); });
 }
 
 // Ranges of 64 consecutive tiles per block, the blocks in ticket order (so that every block before
@@ -132,7 +149,7 @@ __global__ void __launch_bounds__(kScanTiles) tile_scan(BinWords w, int tiles, i
     if (t == 0) s_block = atomicAdd(w.ticket, 1u);
     __syncthreads();
     const int b = (int)s_block, tile = b * kScanTiles + t;
-    const uint32_t c = tile < tiles ? w.count[tile] : 0u;
+    const uint32_t c = tile < tiles ? w.count[(size_t)tile * kTileWords] : 0u;
     uint32_t incl = c;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -174,7 +191,7 @@ __global__ void __launch_bounds__(kScanTiles) tile_scan(BinWords w, int tiles, i
         }
         if (!ok) {
             sum = 0;
-            for (int i = lane; i < b * kScanTiles; i += 32) sum += w.count[i];
+            for (int i = lane; i < b * kScanTiles; i += 32) sum += w.count[(size_t)i * kTileWords];
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
         }
@@ -229,7 +246,7 @@ __global__ void __launch_bounds__(1024) tile_order_kernel(const int2* __restrict
 
 // Pairs into their tiles' ranges; with `order`, block 0 writes the tiles' launch order instead.
 // Nothing is written past `limit` pairs or after a look-back that gave up.
-__global__ void __launch_bounds__(kBinThreads) place_pairs(int N, const int32_t* __restrict__ touched,
+__global__ void __launch_bounds__(kBinThreads) place_pairs(int N, int parts, const int32_t* __restrict__ touched,
                                                            const int4* __restrict__ rect, int tiles_x, int tiles,
                                                            const int2* __restrict__ ranges,
                                                            uint32_t* __restrict__ placed,
@@ -244,13 +261,13 @@ __global__ void __launch_bounds__(kBinThreads) place_pairs(int N, const int32_t*
         }
         --block;
     }
-    const int g = block * kBinThreads + threadIdx.x;
     if (*total > limit || *err) return;
-    warp_pairs(g, N, touched, rect, tiles_x, tiles, [&](int own, int t) {
-        const int2 r = ranges[t];
-        const int at = r.x + (int)atomicAdd(placed + t, 1u);
-        if (at < r.y) ids[at] = own;
-    });
+    warp_pairs(block * (kBinThreads / 32) + (int)threadIdx.x / 32, parts, N, touched, rect, tiles_x, tiles,
+               [&](int own, int t) {
+                   const int2 r = ranges[t];
+                   const int at = r.x + (int)atomicAdd(placed + (size_t)t * kTileWords, 1u);
+                   if (at < r.y) ids[at] = own;
+               });
 }
 
 // Per-tile depth order.  Each list is sorted on the 64-bit key (binary32 depth bits, index), i.e.
@@ -458,7 +475,8 @@ latentam_status bin_launch(latentam_ctx* ctx, int32_t N, const latentam_projecte
     LAT_TRY(bin_slot(ctx, slot, num_tiles, &b));
     const BinWords w = bin_words(b.words, num_tiles);
     const int nb = (tiles + kScanTiles - 1) / kScanTiles;
-    const unsigned blocks = (unsigned)((N + kBinThreads - 1) / kBinThreads);
+    const int parts = pair_parts(N, ctx->num_sms);
+    const unsigned blocks = (unsigned)((((int64_t)N + 31) / 32 * parts + kBinThreads / 32 - 1) / (kBinThreads / 32));
     const int4* rect = reinterpret_cast<const int4*>(proj.rect);
     // an armed test stall applies to the last block of the scan (once)
     const bool stall = ctx->test_stall_sort && nb > 1;
@@ -467,7 +485,7 @@ latentam_status bin_launch(latentam_ctx* ctx, int32_t N, const latentam_projecte
     auto count = [&](cudaStream_t s) -> latentam_status {
         cudaError_t e = cudaMemsetAsync(b.words, 0, bin_words_bytes(num_tiles), s);
         if (e != cudaSuccess) return cuda_error(e, "clear the binning counters");
-        count_tiles<<<blocks, kBinThreads, 0, s>>>(N, proj.tiles_touched, rect, cam.tiles_x, tiles, w.count, b.cnt + 2,
+        count_tiles<<<blocks, kBinThreads, 0, s>>>(N, parts, proj.tiles_touched, rect, cam.tiles_x, tiles, w.count, b.cnt + 2,
                                                    ctx->dev_flags, b.host);
         LAT_CHECK_LAUNCH("count_tiles");
         tile_scan<<<nb, kScanTiles, 0, s>>>(w, tiles, ranges, b.cnt + 1, b.host, b.cnt + 2,
@@ -486,7 +504,7 @@ latentam_status bin_launch(latentam_ctx* ctx, int32_t N, const latentam_projecte
     if (e != cudaSuccess) return cuda_error(e, "record the pair count");
     const uint32_t limit = pair_limit(bins);
     auto place = [&](cudaStream_t s) -> latentam_status {
-        place_pairs<<<blocks + (order ? 1 : 0), kBinThreads, 0, s>>>(N, proj.tiles_touched, rect, cam.tiles_x, tiles,
+        place_pairs<<<blocks + (order ? 1 : 0), kBinThreads, 0, s>>>(N, parts, proj.tiles_touched, rect, cam.tiles_x, tiles,
                                                                      ranges, w.placed, b.cnt + 1, limit, b.cnt + 2,
                                                                      bins.pair_ids, order);
         LAT_CHECK_LAUNCH("place_pairs");

@@ -91,3 +91,19 @@ def test_pair_count_is_exact_when_a_look_back_gives_up(api):
         assert bins.num_pairs == P
         np.testing.assert_array_equal(bins.tile_ranges.cpu().numpy(), ranges)
         np.testing.assert_array_equal(bins.pair_ids[:P].cpu().numpy(), ids)
+
+
+@pytest.mark.parametrize("n,width,height,span", [(1, 2000, 1500, 125), (5, 2000, 1500, 125), (33, 640, 480, 40),
+                                                 (1216, 640, 480, 12), (1217, 300, 200, 9), (2433, 320, 240, 20),
+                                                 (20_000, 320, 240, 3)])
+def test_splats_shared_by_several_warps(api, n, width, height, span):
+    """Few splats of many tiles, at the counts where one warp more or fewer shares 32 splats' pairs."""
+    cam = _camera(width, height)
+    proj, ids, ranges = _scene(api, n, cam, span, 3 * n, 0.9)
+    P = len(ids)
+    with api.Context(0) as ctx:
+        for _ in range(3):
+            bins = api.sort(ctx, proj, cam, capacity=max(P, 1))
+            assert bins.num_pairs == P
+            np.testing.assert_array_equal(bins.tile_ranges.cpu().numpy(), ranges)
+            np.testing.assert_array_equal(bins.pair_ids[:P].cpu().numpy(), ids)
