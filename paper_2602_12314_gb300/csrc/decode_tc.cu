@@ -496,6 +496,7 @@ struct FhatOutEpi {
         const float isp = row_scale_inv<Q8>(p, pix, pix < p.n);
         for (int c0 = 32 * ec.g; c0 < ncols; c0 += 32 * EPI_WG) {
             float h[32];
+            __syncwarp();  // the TMEM load is for whole warps
             fhat32<Q8>(p, ec, c0, isp, h);
             if (lane == 0) tc::bulk_wait_read();  // the previous chunk has left the staging rows
             __syncwarp();

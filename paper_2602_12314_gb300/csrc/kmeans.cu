@@ -185,6 +185,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, NV <= 4 ? 2 : 1) local_pass(co
                 }
             }
         };
+        __syncwarp();  // named barriers are for whole warps
         if (turns && (warp >= copies || round > 0)) pair_sync(1 + warp);
         if (same) {
             if (a[0] >= 0) {
@@ -202,6 +203,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, NV <= 4 ? 2 : 1) local_pass(co
             for (int r = 0; r < R; ++r)
                 if (a[r] >= 0) add(a[r], x[r]);
         }
+        __syncwarp();
         if (turns && !(last && round + 1 == rounds)) pair_arrive(last ? 1 + warp % copies : 1 + warp + copies);
     }
     s_cnt[warp][lane] = cnt;

@@ -250,6 +250,7 @@ struct EpiCtx {
         if (!ofree) return true;
         const bool ok = mbar_wait(ofree, ofree_phase, abort);
         if (!ok) *abort = 1;
+        __syncwarp();  // (the lanes leave the wait at different polls; TMEM loads follow)
         return ok;
     }
 
