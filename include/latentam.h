@@ -222,7 +222,8 @@ LATENTAM_API latentam_status latentam_test_wait_timeout(latentam_ctx* ctx, int32
  * waves, for dK about one wave, half and two); each candidate is timed together with the
  * reduction of its partial sums.  The fastest is kept for the context's lifetime (32 shapes).  Results differ between
  * candidates only by FP32 summation order.  Disabling clears the choices and uses the first
- * tile shape with its one-wave split. */
+ * tile shape with its first split: for dV the fewest whole waves of CTAs whose parts are no longer
+ * than 51,200 pixels, for dK about one wave. */
 LATENTAM_API latentam_status latentam_autotune_enable(latentam_ctx* ctx, int32_t enable);
 
 /* One choice of the autotuner. */

@@ -319,11 +319,13 @@ struct SoftmaxParams {
 // Bound by latency: a tile is 512 cycles of MMAs between dependent waits (accumulator, row maximum,
 // row sum, cluster exchange, staging), with the A rows written at 2.9 - 4 TB/s.  So the plain form
 // keeps its tile of keys in shared memory and two tiles of queries on the way, two teams of epilogue
-// warps take the tiles in turn, and the exponentials run in packed arithmetic with flushed
-// results below 2^-126 (14 -> 10 warp instructions per 32 logits; the same bits, as the sums keep
-// their order).  Whole decode, together: 300,000 rows M = 1024 D = 768 1,602 -> 1,554 us, M = 512
-// 1,003 -> 985, inference of 816,000 rows M = 512 966 -> 908; two teams with the plain loops alone gave 1,600 -> 1,589.  The split form, whose two
-// staged planes take both buffers, lost 1% with either and keeps one team and the plain loops.
+// warps take the tiles in turn, and the exponentials run in packed arithmetic (14 -> 10 warp
+// instructions per 32 logits; the sums keep their order, so the bits are the plain loops' except that
+// exponentials below 2^-126, of logits more than 87 below their row's maximum in the slice, are zero).
+// Whole decode, together: 300,000 rows M = 1024 D = 768 1,602 -> 1,554 us, M = 512 1,003 -> 985,
+// inference of 816,000 rows M = 512 966 -> 908; two teams with the plain loops alone gave 1,600 ->
+// 1,589.  The split form, whose two staged planes take both buffers, lost 1% with either and keeps one
+// team and the plain loops.
 template <bool SPLIT_ = false>
 struct SoftmaxEpi {
     // plain: one K chunk (the padded queries) per tile

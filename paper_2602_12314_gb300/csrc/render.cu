@@ -207,14 +207,11 @@ __device__ __forceinline__ void render_fwd_tile(const TileJob& job, FwdSmem<DQ, 
 }
 
 template <int DQ>
-__global__ void __launch_bounds__(fwd_threads<DQ>(), fwd_blocks<DQ>()) render_fwd_kernel(CamParams cam, const int2* __restrict__ ranges,
-                                                                       const int32_t* __restrict__ pair_ids,
-                                                                       const float2* __restrict__ xy,
-                                                                       const float4* __restrict__ conic_opac,
-                                                                       const float4* __restrict__ f,
-                                                                       float4* __restrict__ Q,
-                                                                       float* __restrict__ T_final,
-                                                                       int32_t* __restrict__ n_contrib) {
+__global__ void __launch_bounds__(fwd_threads<DQ>(), fwd_blocks<DQ>())
+    render_fwd_kernel(CamParams cam, const int2* __restrict__ ranges, const int32_t* __restrict__ pair_ids,
+                      const float2* __restrict__ xy, const float4* __restrict__ conic_opac,
+                      const float4* __restrict__ f, float4* __restrict__ Q, float* __restrict__ T_final,
+                      int32_t* __restrict__ n_contrib) {
     __shared__ FwdSmem<DQ> sm;
     const int tile = cam.tile_order ? cam.tile_order[blockIdx.x] : (int)blockIdx.x;
     const TileJob job{tile, cam.tiles_x, cam.W, cam.H, ranges, pair_ids, xy, conic_opac, f, Q, T_final, n_contrib,
@@ -239,9 +236,9 @@ __device__ __forceinline__ int next_item(int* counter, const int32_t* order, int
 // four that its registers would allow; the single frame above is shorter with four, 57 against
 // 70 us at 640 x 480, where the last tiles' own length counts.)
 template <int DQ>
-__global__ void __launch_bounds__(fwd_threads<DQ>(), DQ == 32 ? 5 : fwd_blocks<DQ>()) render_fwd_batch_kernel(const __grid_constant__ BatchJobs jobs,
-                                                                             const int32_t* __restrict__ order,
-                                                                             int total, int* __restrict__ counter) {
+__global__ void __launch_bounds__(fwd_threads<DQ>(), DQ == 32 ? 5 : fwd_blocks<DQ>())
+    render_fwd_batch_kernel(const __grid_constant__ BatchJobs jobs, const int32_t* __restrict__ order, int total,
+                            int* __restrict__ counter) {
     __shared__ FwdSmem<DQ> sm;
     for (int item = next_item(counter, order, total); item >= 0; item = next_item(counter, order, total)) {
         TileJob job = jobs.fr[item >> 20];

@@ -276,11 +276,11 @@ __global__ void __launch_bounds__(kBinThreads) place_pairs(int N, int parts, con
 // the keys below its own, which is its place: one pass of broadcast reads with no barrier instead
 // of up to 36 network steps (83,000 pairs in 1,200 tiles 18.1 -> 16.8 us, 251,000 in 3,225 32.4 ->
 // 22.8, 890 in 12 10.5 -> 6.5, launch included; counting up to 128 keys only: 16.8, 24.1, 10.2).
-// Lists of up to kTsCap keys are sorted in shared memory by a bitonic network; longer ones are cut into kTsCap runs sorted the same way and merged pairwise through the
-// scratch buffers (two arrays of `scratch` keys, each tile using its own segment; with more pairs
-// than that they are left for a second launch with larger ones).  Lists of up to `longer` keys are
-// left as they are.  A binning that failed (*err) or
-// does not fit leaves every tile empty.
+// Lists of up to kTsCap keys are sorted in shared memory by a bitonic network; longer ones are cut into
+// kTsCap runs sorted the same way and merged pairwise through the scratch buffers (two arrays of
+// `scratch` keys, each tile using its own segment; with more pairs than that they are left for a
+// second launch with larger ones).  Lists of up to `longer` keys are left as they are.  A binning that
+// failed (*err) or does not fit leaves every tile empty.
 constexpr int kTsThreads = 256;
 constexpr int kTsCap = 4096;
 
