@@ -1552,7 +1552,8 @@ latentam_status tc_loss_bwd(latentam_ctx* ctx, const DecodeArgs& a, cudaStream_t
         const dim3 grow(cdiv(n, kTileM), 1, 1);
         // the column tiles of a row tile side by side: with the row tiles innermost, every column
         // tile read all of dFhat from HBM again (1,254,528 rows, M = 1024: dA -> dS 2,200 -> 1,929 us)
-        const tc::GemmGrid g3{cdiv(D, BK3), cdiv(D, BK3), ty};
+        const int rows3 = cdiv(n, kTileM);
+        const tc::GemmGrid g3{cdiv(D, BK3), cdiv(D, BK3), rows3 <= 65535};
         CUtensorMap mAe, mdSo;  // attention rows for the epilogue, dS out through the TMA
         LAT_TRY(io_map(SPLIT, &mAe, b.A, M, n, M, kTileM));
         LAT_TRY(io_map(SPLIT, &mdSo, b.dS, M, n, M, kTileM));
@@ -1565,8 +1566,9 @@ latentam_status tc_loss_bwd(latentam_ctx* ctx, const DecodeArgs& a, cudaStream_t
             LAT_TRY(launch_persist<DsPairEpi>(ctx, mdF, mVh, cdiv(n, kTileM), cdiv(D, 64), ty, false, dp, b.err, st,
                                               &mAe, &mdSo, b.dF, n, 2 * D));
         } else {
-            LAT_TRY((launch_gemm<DsEpi<SPLIT>>(mdF, mV, dim3(cdiv(n, kTileM) * ty, 1, 1), g3, dp, b.err, st, &mAe,
-                                               &mdSo, 1, dq_fused ? &mK : nullptr, dk_fused ? &mQt : nullptr)));
+            LAT_TRY((launch_gemm<DsEpi<SPLIT>>(mdF, mV, g3.b_first ? dim3(ty, rows3, 1) : dim3(rows3, ty, 1), g3, dp,
+                                               b.err, st, &mAe, &mdSo, 1, dq_fused ? &mK : nullptr,
+                                               dk_fused ? &mQt : nullptr)));
         }
         if (a.dQ && !dq_fused) {
             LAT_TRY(op_map(SPLIT, &mdS, b.dS, M, n, M, kTileM));

@@ -6,8 +6,8 @@
 // Warp roles (192 threads): warp 0 issues the TMA loads, warp 1 owns the TMEM allocation and
 // issues the MMAs (one thread), warps 2..5 run the epilogue; epilogue thread r owns tile row r
 // (TMEM lane r; warp w reads the lane quarter w % 4).
-// blockIdx.x: 128-row tile of A, blockIdx.y: BN-row tile of B (or both in blockIdx.x, see
-// GemmGrid::y_inner), blockIdx.z: split of the K range.
+// blockIdx.x: 128-row tile of A, blockIdx.y: BN-row tile of B (or the other way round, see
+// GemmGrid::b_first), blockIdx.z: split of the K range.
 // When a row reduction spans several BN tiles, the tiles of one row block run as a thread-block
 // cluster along y and trade their per-row partial results through distributed shared memory.
 #pragma once
@@ -134,9 +134,9 @@ __device__ __forceinline__ float group_max(float v, float* scratch, int slot, in
 struct GemmGrid {
     int k_chunks;      // total 64-wide K chunks
     int chunks_per_z;  // chunks handled by one blockIdx.z
-    // > 0: blockIdx.x walks this many B tiles of one A tile before the next A tile (gridDim.y 1), so
-    // that the A tile is read from HBM once and the others find it in L2
-    int y_inner = 0;
+    // blockIdx.x walks the B tiles, blockIdx.y the A tiles (at most 65,535), so that the CTAs of one A
+    // tile run side by side: it is read from HBM once and the others find it in L2
+    bool b_first = false;
 };
 
 // Epi must provide: static constexpr int BN, STAGES, BOX_B (rows per TMA box of a K-major B,
@@ -456,9 +456,9 @@ __global__ void __launch_bounds__(gemm_threads(Epi::EPI_WG), Epi::MIN_BLOCKS)
     if constexpr (X2 > 0) x2_on = x_on && Epi::x2_active(ep);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int tile_x = g.y_inner > 0 ? (int)blockIdx.x / g.y_inner : (int)blockIdx.x;
+    const int tile_x = g.b_first ? (int)blockIdx.y : (int)blockIdx.x;
     const int m0 = tile_x * MSUB * kTileM;
-    const int n0 = (g.y_inner > 0 ? (int)blockIdx.x % g.y_inner : (int)blockIdx.y) * BN;
+    const int n0 = (g.b_first ? (int)blockIdx.x : (int)blockIdx.y) * BN;
     const int k_begin = blockIdx.z * g.chunks_per_z;
     const int k_end = min(g.k_chunks, k_begin + g.chunks_per_z);
     const int nk = k_end - k_begin;
