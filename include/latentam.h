@@ -218,10 +218,10 @@ LATENTAM_API latentam_status latentam_test_wait_timeout(latentam_ctx* ctx, int32
  * reduction sums the tiles in order) is chosen by timing its candidates with CUDA
  * events on the caller's stream (this synchronises that stream once): for dV the CTA tile
  * (256 atoms x 256 features, the pixel block read once for both 128-atom halves, or 128 x 256
- * on twice the CTAs), for both the pixel split (for dV three that fill whole
- * waves, for dK about one wave, half and two); each candidate is timed together with the
- * reduction of its partial sums.  The fastest is kept for the context's lifetime (32 shapes).  Results differ between
- * candidates only by FP32 summation order.  Disabling clears the choices and uses the first
+ * on twice the CTAs), for both the pixel split (for dV three that fill whole waves and, of few
+ * enough pixels, half a wave, for dK about one wave, half and two); each candidate is timed
+ * together with the reduction of its partial sums.  The fastest is kept for the context's lifetime
+ * (32 shapes).  Results differ between candidates only by FP32 summation order.  Disabling clears the choices and uses the first
  * tile shape with its first split: for dV the fewest whole waves of CTAs whose parts are no longer
  * than 51,200 pixels, for dK about one wave. */
 LATENTAM_API latentam_status latentam_autotune_enable(latentam_ctx* ctx, int32_t enable);

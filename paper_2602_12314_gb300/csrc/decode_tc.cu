@@ -1283,25 +1283,30 @@ tc::GemmGrid pixel_split(int64_t n, int z, int* z_out, int chunk = tc::kChunkK) 
     return tc::GemmGrid{chunks, cpz};
 }
 
-// Splits the tuner tries, the first one where it does not tune.
-constexpr int kSplits = 3;
+// Splits the tuner tries (an equal one is not tried again), the first one where it does not tune.
+constexpr int kSplits = 4;
 using Splits = int[kSplits];
 // dV: those that fill w, w + 1 and w + 2 waves of one CTA per SM and do not start another (M = 1024,
 // D = 768 on 152 SMs: 12 tiles; 13 parts left 4 CTAs to a second wave, 26 parts 8 to a third, and dV
 // over 1,254,528 rows took 1,480 us against 1,090 in 12 or 25 parts), with the smallest w whose
 // parts are no longer than kMaxPart pixels: a part is one FP32 chain, and at 104,000 pixels its
-// rounding shows (dV off by 1.2e-6 against 64 bits, half of that at 50,000).
+// rounding shows (dV off by 1.2e-6 against 64 bits, half of that at 50,000).  And half a wave where its
+// parts are short enough too: few rows leave more time in the sum of the parts (18,247 rows, M = 320, D =
+// 256, whole decode without it 123 -> 128 us in FP32, 96 -> 100 in BF16).
 constexpr int64_t kMaxPart = 51200;
 void full_waves(int tiles_xy, int64_t n, int num_sms, Splits& z) {
     int w = 1;
     while ((int64_t)(w * num_sms / tiles_xy) * kMaxPart < n) ++w;
-    for (int i = 0; i < kSplits; ++i) z[i] = std::max(1, (w + i) * num_sms / tiles_xy);
+    for (int i = 0; i < 3; ++i) z[i] = std::max(1, (w + i) * num_sms / tiles_xy);
+    const int half = std::max(1, num_sms / (2 * tiles_xy));
+    z[3] = half * kMaxPart >= n ? half : z[0];
 }
 // dK (sums with much cancellation: longer FP32 chains show): about one wave, half and two.
 void near_waves(int tiles_xy, int num_sms, Splits& z) {
     z[0] = std::max(1, (num_sms + tiles_xy - 1) / tiles_xy);
     z[1] = std::max(1, z[0] / 2);
     z[2] = 2 * z[0];
+    z[3] = z[0];
 }
 
 // Autotuned launch shape of a pixel reduction: the first time a shape (n, M, D, which) is seen
@@ -1332,6 +1337,7 @@ latentam_status tuned_shape(latentam_ctx* ctx, int64_t n, int M, int D, int whic
     for (int sh = 0; sh < nshapes && s == LATENTAM_OK; ++sh) {
         for (int i = 0; i < kSplits && s == LATENTAM_OK; ++i) {
             const int z = cand[sh][i];
+            if (std::find(cand[sh], cand[sh] + i, z) != cand[sh] + i) continue;
             cudaEventRecord(ev[0], st);
             s = launch(sh, z);
             cudaEventRecord(ev[1], st);
